@@ -213,31 +213,41 @@ def _step_call(s):
                x["seed"], s["step"], mp=s["mp"], vo=s["vo"], so=s["so"])
 
 
-def prepare(case, seed):
-    c = dict(DEFAULTS, **case)
+def _inputs(c, seed):
+    """(vocabulary map, n-grams or None, one step's tensors, the acceptance head's logits or None)."""
     g = torch.Generator(device="cuda")
     g.manual_seed(seed)
     vmap = _vocab_map(c, g)
-    s = dict(case=c, ctx=_context(c, vmap), step=0)
+    if c["path"] == "cache":
+        # enough batches that a batch comes round again only after the trims have evicted it
+        n = -(-c["entries"] // c["batch"])
+        runs = [_runs(c, c["batch"], vmap, g) for _ in range(n + 2)]
+        return vmap, runs, _proposals(c, vmap, tuple(torch.cat(t) for t in zip(*runs)), g, logits=False), None
+    runs = _runs(c, c["entries"], vmap, g) if c["entries"] else None
+    x = _proposals(c, vmap, runs, g)
+    head = None
+    if c["path"] == "adaptive":
+        # the acceptance head is unsure of later tokens: 0.95, 0.9, ... on average
+        B, K = c["B"], c["K"]
+        head = 2.5 + torch.randn(B, K, generator=g, device="cuda") - 0.2 * torch.arange(K, device="cuda")
+    return vmap, runs, x, head
+
+
+def prepare(case, seed):
+    c = dict(DEFAULTS, **case)
+    vmap, runs, x, head = _inputs(c, seed)
+    s = {"case": c, "ctx": _context(c, vmap), "step": 0, "in": x, "head": head}
     ctx, B, K, path = s["ctx"], c["B"], c["K"], c["path"]
     s["mp"], s["vo"], s["so"] = od.alloc_map_out(ctx, B, K), od.alloc_verify_out(ctx, B, K), od.alloc_sample_out(ctx, B)
     if path == "cache":
-        # enough batches that a batch comes round again only after the trims have evicted it
-        n = -(-c["entries"] // c["batch"])
-        s["batches"] = [_runs(c, c["batch"], vmap, g) for _ in range(n + 2)]
-        s["in"] = _proposals(c, vmap, tuple(torch.cat(t) for t in zip(*s["batches"])), g, logits=False)
+        s["batches"] = runs
         ctx.cache_configure(c["entries"], 1 if c["lfu"] else 0, c["batch"])
-        for i in range(n):
+        for i in range(len(runs) - 2):
             _upkeep(s)
         return s
-    runs = _runs(c, c["entries"], vmap, g) if c["entries"] else None
     if runs is not None:
         ctx.cache_build(*(t.cpu().numpy() for t in runs))
-    s["in"] = x = _proposals(c, vmap, runs, g)
-    if path == "adaptive":
-        # the acceptance head is unsure of later tokens: 0.95, 0.9, ... on average
-        s["head"] = 2.5 + torch.randn(B, K, generator=g, device="cuda") - 0.2 * torch.arange(K, device="cuda")
-    elif path == "graph":
+    if path == "graph":
         _step_call(s)
         s["graph"] = torch.cuda.CUDAGraph()
         with torch.cuda.graph(s["graph"]):
@@ -352,3 +362,122 @@ def tolerance(case):
     if case["path"] == "distill":
         return {"rel": 1e-6, "max": 2.5e-4, "differ": 0.0}
     return {"rel": 1e-6, "max": 1e-5, "differ": 0.01}
+
+
+# ---- the same in 64 bits, from the definitions --------------------------------------------
+
+def _uniform(seed, position, tag):
+    """Philox4x32-10, key = seed, counter = (0, 0, position, tag): 24 bits of the first word as a number in [0, 1)."""
+    w = 0xFFFFFFFF
+    c, k = [0, 0, position, tag], [seed & w, seed >> 32 & w]
+    for _ in range(10):
+        a, b = 0xD2511F53 * c[0], 0xCD9E8D57 * c[2]
+        c = [(b >> 32) ^ c[1] ^ k[0], b & w, (a >> 32) ^ c[3] ^ k[1], a & w]
+        k = [(k[0] + 0x9E3779B9) & w, (k[1] + 0xBB67AE85) & w]
+    return (c[0] >> 8) / 16777216.0
+
+
+def _translate(vmap, table, ids, n, q):
+    """One proposal: its pieces (target id, q', first draft position, length), and the position it stops at or None."""
+    pieces, pos = [], 0
+    while pos < n:
+        for L in (4, 3, 2):
+            t = table.get(tuple(ids[pos:pos + L])) if pos + L <= n else None
+            if t is not None:
+                pieces.append((t, math.prod(q[pos:pos + L]), pos, L))
+                break
+        else:
+            L = 1
+            if vmap[ids[pos]] < 0:
+                return pieces, pos
+            pieces.append((vmap[ids[pos]], q[pos], pos, 1))
+        pos += L
+    return pieces, None
+
+
+def _exact_step(c, vmap, runs, x, draft_len, loss=None, grad=None):
+    """The step's probabilities; with `loss` and `grad`, the distillation terms of the translated positions too."""
+    B, K = c["B"], c["K"]
+    z = lambda *shape: torch.zeros(*shape, dtype=torch.float64)
+    o = dict(q_prime=z(B, K), row_max=z(B, K + 1), row_sum=z(B, K + 1), p_sel=z(B, K), ratio=z(B, K), resid_mass=z(B))
+    table = {}
+    if runs is not None:
+        for r, L, t in zip(*(v.tolist() for v in runs)):
+            table.setdefault(tuple(r[:L]), t)
+    to = vmap.tolist()
+    mapped = torch.nonzero(vmap >= 0).squeeze(1).cuda()
+    image = vmap.cuda().long()[mapped]
+    host = {k: x[k].tolist() for k in ("draft_ids", "seed")}
+    q_sel, T = x["q_sel"].double().tolist(), x["temperature"].double().tolist()
+    for b in range(B):
+        ids = host["draft_ids"][b]
+        pieces, stop = _translate(to, table, ids, draft_len[b], q_sel[b])
+        m = len(pieces)
+        v = x["logits"][b, :m + 1].double()
+        M = v.amax(1)
+        e = torch.exp((v - M[:, None]) / T[b])
+        S = e.sum(1)
+        o["row_max"][b, :m + 1], o["row_sum"][b, :m + 1] = M.cpu(), S.cpu()
+        p = e / S[:, None]
+        n, open_ = 0, True
+        for i, (t, q, _, _) in enumerate(pieces):
+            o["q_prime"][b, i] = q
+            o["p_sel"][b, i] = p[i, t]
+            o["ratio"][b, i] = min(1.0, float(p[i, t]) / q)
+            open_ = open_ and _uniform(host["seed"][b], i, 0) < o["ratio"][b, i]
+            n += open_
+        mass = 1.0
+        if n < m or stop is not None:
+            t, q, first, L = pieces[n] if n < m else (None, 0.0, stop, 1)
+            row = x["q_rows"][b, first].double()
+            q_t = torch.zeros(c["v_p"], dtype=torch.float64, device="cuda")
+            q_t[image] = row[mapped]
+            if L > 1:
+                if to[ids[first]] >= 0:
+                    q_t[to[ids[first]]] = row[ids[first]] - q
+                q_t[t] = q
+            mass = float((p[n] - q_t).clamp(min=0).sum()) or 1.0
+        o["resid_mass"][b] = mass
+        for i, (t, q, first, L) in enumerate(pieces if loss is not None else []):
+            for j in range(first, first + L):
+                row = x["q_rows"][b, j].double()
+                if L > 1:
+                    w = float(p[i, t]) if c["verified_weight"] else LAMBDA
+                    loss[b, j] = -w * torch.log(row[ids[j]])
+                    d = w * row
+                    d[ids[j]] -= w
+                else:
+                    q_m = row[mapped]
+                    f = torch.log(q_m.clamp(min=1e-300)) - ((v[i, image] - M[i]) / T[b] - torch.log(S[i]))
+                    loss[b, j] = (q_m * f).sum()
+                    g = torch.zeros_like(row)
+                    g[mapped] = f + 1
+                    d = row * (g - (row * g).sum())
+                if grad is not None:
+                    grad[b, j] = d.cpu()
+    return o
+
+
+def exact(case, seed):
+    c = dict(DEFAULTS, **case)
+    if c["path"] in ("cache", "host"):      # whole values
+        return None
+    vmap, runs, x, head = _inputs(c, seed)
+    draft_len, reject = x["draft_len"].tolist(), None
+    if head is not None:
+        reject = (1 - torch.cumprod(torch.sigmoid(head.double()), 1)).cpu()
+        over = reject > GAMMA
+        draft_len = torch.where(over.any(1), over.int().argmax(1) + 1, c["K"]).tolist()
+    if c["path"] == "distill":
+        loss = torch.zeros(c["B"], c["K"], dtype=torch.float64)
+        grad = torch.zeros(c["B"], c["K"], c["v_q"], dtype=torch.float64) if c["grad"] else None
+        _exact_step(c, vmap, runs, x, draft_len, loss, grad)
+        return loss, grad
+    o = _exact_step(c, vmap, runs, x, draft_len)
+    mp = dict(dict.fromkeys(("tgt_ids", "span_start", "span_len", "m", "tail_kind", "counters")), q_prime=o["q_prime"])
+    vo = dict(dict.fromkeys(("n_accepted", "n_draft_accepted", "flags")),
+              **{k: o[k] for k in ("row_max", "row_sum", "p_sel", "ratio")})
+    so = dict(dict.fromkeys(("out_token", "flags")), resid_mass=None if c["path"] == "shard" else o["resid_mass"])
+    if c["path"] == "shard":                # a shard's records are relative to a reference of its own choice
+        return mp, vo, so, None, None
+    return (mp, vo, so) if head is None else (mp, vo, so, None, reject, None)
