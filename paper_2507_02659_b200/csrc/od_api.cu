@@ -45,7 +45,7 @@ int32_t dev_alloc(T **p, size_t n)
 void free_all(od_ctx *c)
 {
     od_cache_free_dynamic(c);
-    void *ptrs[] = {c->d_vocab_map, c->d_inv_map, c->d_keys, c->d_vals, c->d_partials,
+    void *ptrs[] = {c->d_vocab_map, c->d_inv_map, c->d_distill_lists, c->d_keys, c->d_vals, c->d_partials,
                     c->d_tile_sums,
                     c->d_samp_ticket, c->s_logits, c->s_q_rows, c->s_q_sel, c->s_temperature,
                     c->s_draft_ids, c->s_draft_len, c->s_seed, c->s_tgt_ids, c->s_span_start,
@@ -134,13 +134,19 @@ int32_t od_create(od_ctx **ctx, int32_t device, int32_t draft_vocab, int32_t tar
         delete c;
         return OD_ERR_CUDA;
     }
+    if (od_distill_prepare_device(draft_vocab) != cudaSuccess) {
+        delete c;
+        return OD_ERR_CUDA;
+    }
     // od_verify scratch serves one launch: at most OD_VERIFY_MAX_B sequences
     const size_t vb = max_batch < OD_VERIFY_MAX_B ? max_batch : OD_VERIFY_MAX_B;
     const size_t rows = vb * (max_k + 1);
     int32_t st = OD_OK;
     if (st == OD_OK) st = dev_alloc(&c->d_vocab_map, (size_t)draft_vocab);
     if (st == OD_OK) st = dev_alloc(&c->d_inv_map, (size_t)target_vocab + 8);
-
+    char *lists = nullptr;
+    if (st == OD_OK) st = dev_alloc(&lists, od_distill_lists_bytes(draft_vocab, target_vocab));
+    c->d_distill_lists = lists;
     if (st == OD_OK) st = dev_alloc(&c->d_partials, rows * OD_VERIFY_SEG_MAX);
     if (st == OD_OK) st = dev_alloc(&c->d_tile_sums, (size_t)max_batch * c->tiles_per_row);
     if (st == OD_OK) st = dev_alloc(&c->d_samp_ticket, (size_t)max_batch);
@@ -166,6 +172,7 @@ int32_t od_destroy(od_ctx *c)
 int32_t od_set_vocab_map(od_ctx *c, const int32_t *host_map)
 {
     if (!c || !host_map) return OD_ERR_INVALID_ARG;
+    try {
     std::vector<int32_t> inv((size_t)c->v_p, -1);
     for (int32_t d = 0; d < c->v_q; ++d) {
         const int32_t t = host_map[d];
@@ -182,8 +189,14 @@ int32_t od_set_vocab_map(od_ctx *c, const int32_t *host_map)
     for (int32_t d = 0; d < c->v_q; ++d) fwd[d] = host_map[d] < 0 ? -1 : host_map[d];
     OD_CUDA(cudaMemcpy(c->d_vocab_map, fwd.data(), fwd.size() * sizeof(int32_t), cudaMemcpyHostToDevice));
     OD_CUDA(cudaMemcpy(c->d_inv_map, inv.data(), inv.size() * sizeof(int32_t), cudaMemcpyHostToDevice));
+    std::vector<char> lists(od_distill_lists_bytes(c->v_q, c->v_p));
+    od_distill_plan(c->v_q, c->v_p, inv.data(), lists.data());
+    OD_CUDA(cudaMemcpy(c->d_distill_lists, lists.data(), lists.size(), cudaMemcpyHostToDevice));
     c->have_map = true;
     return OD_OK;
+    } catch (const std::bad_alloc &) {
+        return OD_ERR_NOMEM;
+    }
 }
 
 int32_t od_cache_build(od_ctx *c, const int32_t *host_runs, const int32_t *host_len,

@@ -16,6 +16,10 @@
 #define OD_VERIFY_SEG_MAX 64        // most segments (partials) one logit row is cut into
 #define OD_VERIFY_MAX_B 2048        // sequences per od_verify launch (longer batches go in slices)
 
+#define OD_DISTILL_LEVELS 4         // the distillation kernel cuts the draft ids into 1, 2, 4 or 8 chunks
+#define OD_DISTILL_MAX_CHUNKS 8     // (a portable cluster)
+#define OD_DISTILL_MAX_CHUNK_IDS 56320   // 220 KB of shared memory
+
 struct od_ctx {
     int device;
     int32_t v_q, v_p, max_batch, max_k;
@@ -24,6 +28,7 @@ struct od_ctx {
     // vocabulary map (device)
     int32_t *d_vocab_map;           // [v_q]
     int32_t *d_inv_map;             // [v_p], -1 outside the image
+    void *d_distill_lists;          // gather lists of the distillation kernel (od_distill_lists)
     bool have_map;
 
     // n-gram cache: open addressing over groups of 32 slots
@@ -166,6 +171,37 @@ cudaError_t od_launch_distill(od_ctx *c, int32_t B, int32_t K_max, const float *
                               int64_t row_stride, int64_t seq_stride, const float *row_max,
                               const float *row_sum, const float *p_sel, const float *temperature,
                               float lambda, int32_t lambda_mode, float *loss, float *grad, cudaStream_t s);
+
+// The gather lists of the distillation kernel, one block of memory: per level (1, 2, 4, 8 chunks
+// of the draft ids) the mapped ids chunk by chunk, in target-id order inside a chunk, in groups
+// of 32: an entry is (target id - the group's base) << 16 | (draft id - the chunk's first), or
+// 0xFFFF in the low half where the group has no more.
+struct OdDistillLists {
+    int64_t groups;                 // room for this many groups in each level, a multiple of the chunks
+    uint32_t *word;                 // [levels][groups][32]
+    int32_t *base;                  // [levels][groups]
+    int32_t *ofs;                   // [levels][max chunks][2] a chunk's groups within its level: the first, one past the last
+    uint32_t *bits;                 // [ceil(v_q / 32)] bit d: draft id d is mapped
+};
+inline OdDistillLists od_distill_lists(void *base, int32_t v_q, int32_t v_p)
+{
+    OdDistillLists l;
+    // a group ends full, or at a gap of over 65535 target ids, or with its chunk; a chunk is whole
+    // multiples of 32 ids
+    l.groups = OD_DISTILL_MAX_CHUNKS * (((int64_t)v_q + 255) / 256 + (int64_t)v_p / 65536 + 1);
+    l.word = (uint32_t *)base;
+    l.base = (int32_t *)(l.word + OD_DISTILL_LEVELS * l.groups * 32);
+    l.ofs = l.base + OD_DISTILL_LEVELS * l.groups;
+    l.bits = (uint32_t *)(l.ofs + OD_DISTILL_LEVELS * OD_DISTILL_MAX_CHUNKS * 2);
+    return l;
+}
+inline size_t od_distill_lists_bytes(int32_t v_q, int32_t v_p)
+{
+    const OdDistillLists l = od_distill_lists(nullptr, v_q, v_p);
+    return (size_t)((uintptr_t)(l.bits + (v_q + 31) / 32) - (uintptr_t)nullptr);
+}
+void od_distill_plan(int32_t v_q, int32_t v_p, const int32_t *inv, void *out);   // host
+cudaError_t od_distill_prepare_device(int32_t v_q);
 
 void od_cache_free_dynamic(od_ctx *c);   // frees what od_cache_configure allocated beyond keys / vals
 

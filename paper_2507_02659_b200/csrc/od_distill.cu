@@ -12,19 +12,34 @@
 // ln p_i(t) = (x_t - M_i)/T - ln S_i reuses the row statistics od_verify produced, so
 // the target row is only gathered at the mapped ids, never streamed again.
 //
-// One block of 512 threads per (sequence, draft position), two resident per SM so
-// that a whole batch is one wave; two sweeps over the draft vocabulary: sums, with
-// q(d) g(d) parked in the gradient row, then the gradient (which re-reads q and the
-// parked values from cache). Reads are coalesced except the one gathered logit per
-// mapped id, which touches practically every sector of the target row. Bound by HBM:
-// the drafter's row and the target row in, the gradient row out.
+// Bound by HBM: the drafter's row and the target row in, the gradient row out. What has to be
+// kept from adding to that is the gather, one logit per mapped id, scattered over the target
+// row: in draft-id order each takes a line and a 32-byte sector of its own, and the load/store
+// units and L2 bound the kernel. So the logits are gathered in TARGET-id order, from lists that
+// belong to the context (od_distill_plan): the 32 lanes of a load then sit within 7 lines or so;
+// they are put down in shared memory at their draft ids, and everything after that is
+// coalesced.
+//
+// A position is cut into `C` chunks of draft ids, one block of a thread-block cluster each, so
+// that three blocks share a multiprocessor and a few positions still fill the chip. Three
+// passes: the gather; over the chunk, loss and sum_e q(e) g(e), whose block sums are exchanged over
+// distributed shared memory; over the chunk again, the gradient (q from L2, g worked out again).
+//
+// Measured on 64 x 6 positions of v_q = 32000, v_p = 128256 bf16, 0.6 of them translated: 47.4 ->
+// 32.9 us (the bytes alone: 20.7); 5 x 10 positions with v_p = 152064 fp32: 22.7 -> 12.3 us. Per
+// block on the former (stamps): 1.1 us to find the piece, 11 the gather (HBM at its rate), 4 the
+// sums, 2.3 the exchange, 2 the gradient. The blocks go through these passes together, which
+// is what is left. Not kept: probabilities instead of logits in shared memory (two random
+// accesses per id instead of one: 38 us), q(d) parked there and four to five blocks of fewer
+// threads (39 to 59 us), bulk prefetches of the rows into L2 (no change), one chunk at 64 KB (45 us).
 #include <float.h>
 
 #include "od_common.cuh"
 
 namespace {
 
-constexpr int THREADS = 512;
+constexpr int THREADS = 512;                     // three blocks to a multiprocessor at 40 registers
+constexpr int WARPS = THREADS / 32;
 
 struct DistillArgs {
     int32_t B, K_max, v_q, v_p;
@@ -34,6 +49,10 @@ struct DistillArgs {
     int64_t row_stride, seq_stride;
     const float *row_max, *row_sum, *p_sel, *temperature;
     const int32_t *vocab_map;
+    // the context's lists for this launch's number of chunks (od_distill_plan); chunk = draft ids per block
+    const int32_t *list_base, *list_ofs;
+    const uint32_t *list_word, *mapped_bits;
+    int32_t chunk;
     float lambda;
     int32_t lambda_mode;
     float *loss, *grad;
@@ -46,6 +65,74 @@ __device__ __forceinline__ float lg2_approx(float x)
     float y;
     asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
+}
+
+// the terms of one mapped id with probability qd and target logit x: loss += q f, qg += q (f + 1);
+// returns g = f + 1 (0 for an id without (normal) mass)
+struct KlRow {
+    float M, scale, lg2_S;
+};
+__device__ __forceinline__ float kl_term(const KlRow &r, float qd, float x, float &loss, float &qg)
+{
+    // in base 2: ln q - ln p(t) = ln 2 * (lg2 q - ((x_t - M) * log2(e)/T - lg2 S))
+    const bool ok = qd >= FLT_MIN;
+    const float f = ok ? 0.6931471805599453f * (lg2_approx(qd) - fmaf(x - r.M, r.scale, -r.lg2_S)) : 0.f;
+    const float g = ok ? f + 1.f : 0.f;
+    loss += qd * f;
+    qg += qd * g;
+    return g;
+}
+
+// What a block finds out about its position (b, j) first: the piece of the translated proposal
+// that covers it, if any (thread i looks at piece i, so the loads go out together).
+__device__ __forceinline__ void find_piece(const DistillArgs &a, int b, int j, int *s_piece, int &piece, int &plen)
+{
+    int mb = a.m[b];
+    mb = mb < 0 ? 0 : (mb > a.K_max ? a.K_max : mb);
+    if (threadIdx.x == 0) { s_piece[0] = -1; s_piece[1] = 0; }
+    __syncthreads();
+    if ((int)threadIdx.x < mb) {
+        const size_t o = (size_t)b * a.K_max + threadIdx.x;
+        const int s0 = a.span_start[o], L = a.span_len[o];
+        if (j >= s0 && j < s0 + L) { s_piece[0] = (int)threadIdx.x; s_piece[1] = L; }
+    }
+    __syncthreads();
+    piece = s_piece[0]; plen = s_piece[1];
+}
+
+// Positions without a Kullback-Leibler term, ids [lo, hi) of the gradient row: nothing translated
+// there (loss 0), or a sub-token of a cached n-gram (-w ln q(d_j)). `first`: this block writes the loss.
+template <bool VEC4>
+__device__ __forceinline__ void write_grad_plain(float *grad, const float *q, int lo, int hi, float w, int dj)
+{
+    if (VEC4) {
+        for (int d = lo + (int)threadIdx.x * 4; d < hi; d += THREADS * 4) {
+            float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (q) {
+                const float4 v = __ldg((const float4 *)(q + d));
+                o.x = w * (v.x - (d == dj ? 1.f : 0.f)); o.y = w * (v.y - (d + 1 == dj ? 1.f : 0.f));
+                o.z = w * (v.z - (d + 2 == dj ? 1.f : 0.f)); o.w = w * (v.w - (d + 3 == dj ? 1.f : 0.f));
+            }
+            __stcs((float4 *)(grad + d), o);
+        }
+    } else {
+        for (int d = lo + (int)threadIdx.x; d < hi; d += THREADS) grad[d] = q ? w * (__ldg(q + d) - (d == dj ? 1.f : 0.f)) : 0.f;
+    }
+}
+template <bool VEC4>
+__device__ __forceinline__ void plain_position(const DistillArgs &a, int b, int j, int piece, bool ngram, const float *q,
+                                               float *grad, int lo, int hi, bool first)
+{
+    const size_t o = (size_t)b * a.K_max + j;
+    if (!ngram) {                                            // not translated: no loss, no gradient
+        if (first && threadIdx.x == 0) a.loss[o] = 0.f;
+        if (grad) write_grad_plain<VEC4>(grad, nullptr, lo, hi, 0.f, -1);
+        return;
+    }
+    const int32_t dj = a.draft_ids[o];
+    const float w = a.lambda_mode == 0 ? a.lambda : a.p_sel[(size_t)b * a.K_max + piece];
+    if (first && threadIdx.x == 0) a.loss[o] = (dj >= 0 && dj < a.v_q) ? -w * logf(q[dj]) : 0.f;
+    if (grad) write_grad_plain<VEC4>(grad, q, lo, hi, w, dj);
 }
 
 __device__ __forceinline__ double block_sum(double v, double *s_red)
@@ -61,156 +148,285 @@ __device__ __forceinline__ double block_sum(double v, double *s_red)
     return t;
 }
 
-// VEC4: the draft vocabulary is a multiple of 4 and the rows are 16-byte aligned, so the
-// coalesced accesses (map, q, gradient) move four ids per instruction.
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+// v to the shared-memory address of `p` in block `rank` of the cluster
+__device__ __forceinline__ void cluster_store(double *p, uint32_t rank, double v)
+{
+    uint32_t at;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(at) : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(rank));
+    asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(at), "d"(v) : "memory");
+}
+// A logit as it is stored
+template <int DTYPE>
+struct Logit {
+    typedef float raw;
+    static __device__ __forceinline__ float load(const float *p) { return *p; }
+    static __device__ __forceinline__ float4 load4(const float *p) { return *(const float4 *)p; }
+};
+template <>
+struct Logit<OD_BF16> {
+    typedef unsigned short raw;
+    static __device__ __forceinline__ float load(const raw *p) { return __uint_as_float((uint32_t)*p << 16); }
+    static __device__ __forceinline__ float4 load4(const raw *p)
+    {
+        const uint2 v = *(const uint2 *)p;
+        return make_float4(od_bf16_lo(v.x), od_bf16_hi(v.x), od_bf16_lo(v.y), od_bf16_hi(v.y));
+    }
+};
+
+// Grid (C, K, B), clusters of C blocks. VEC4: the draft vocabulary is a multiple of 4 and the
+// rows are 16-byte aligned, so the coalesced accesses (q, gradient) move four ids per
+// instruction; chunks are multiples of 32 ids.
 template <int DTYPE, bool VEC4>
-__global__ void __launch_bounds__(THREADS, 2)
+__global__ void __launch_bounds__(THREADS, 3)
 od_distill_kernel(const DistillArgs a)
 {
-    __shared__ double s_red[THREADS / 32];
-    const int b = blockIdx.y, j = blockIdx.x;
-    const int K = a.K_max;
-    int mb = a.m[b];
-    mb = mb < 0 ? 0 : (mb > K ? K : mb);
-    // the piece of the translated proposal that covers draft position j, if any
-    // (thread i looks at piece i, so the loads go out together)
-    __shared__ int s_piece, s_plen;
-    if (threadIdx.x == 0) { s_piece = -1; s_plen = 0; }
-    __syncthreads();
-    if ((int)threadIdx.x < mb) {
-        const int s0 = a.span_start[(size_t)b * K + threadIdx.x], L = a.span_len[(size_t)b * K + threadIdx.x];
-        if (j >= s0 && j < s0 + L) { s_piece = (int)threadIdx.x; s_plen = L; }
-    }
-    __syncthreads();
-    const int piece = s_piece, plen = s_plen;
-    const float *q = a.q_rows + ((size_t)b * K + j) * a.v_q;
-    float *grad = a.grad ? a.grad + ((size_t)b * K + j) * a.v_q : nullptr;
-    const float T = a.temperature[b];
-    if (piece < 0 || !(T > 0.f)) {                           // not translated: no loss, no gradient
-        if (threadIdx.x == 0) a.loss[(size_t)b * K + j] = 0.f;
-        if (grad)
-            for (int d = threadIdx.x; d < a.v_q; d += THREADS) grad[d] = 0.f;
-        return;
-    }
-    if (plen >= 2) {
-        // ---- a sub-token of a cached n-gram: -w ln q(d_j)
-        const int32_t dj = a.draft_ids[(size_t)b * K + j];
-        const float w = a.lambda_mode == 0 ? a.lambda : a.p_sel[(size_t)b * K + piece];
-        if (threadIdx.x == 0) a.loss[(size_t)b * K + j] = (dj >= 0 && dj < a.v_q) ? -w * logf(q[dj]) : 0.f;
-        if (grad)
-            for (int d = threadIdx.x; d < a.v_q; d += THREADS) grad[d] = w * (__ldg(q + d) - (d == dj ? 1.f : 0.f));
-        return;
-    }
-    // ---- a directly mapped token: KL(q' || p_i) over the mapped ids
-    const size_t esz = DTYPE == OD_BF16 ? 2 : 4;
-    const char *row = (const char *)a.logits + ((size_t)b * a.seq_stride + (size_t)piece * a.row_stride) * esz;
-    // The gathers below touch practically every 32-byte sector of the target row in no
-    // particular order: have the copy engine bring the row into L2 as one sequential
-    // transfer first (a no-op when od_verify has just streamed it).
-    if (threadIdx.x == 0) {
-        const uint32_t bytes = (uint32_t)((size_t)a.v_p * esz / 16 * 16);
-        if (bytes) asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(row), "r"(bytes) : "memory");
-    }
-    // in base 2: ln q - ln p(t) = ln 2 * (lg2 q - ((x_t - M) * log2(e)/T - lg2 S))
-    const float M = a.row_max[b * (K + 1) + piece];
-    const float lg2_S = lg2_approx(a.row_sum[b * (K + 1) + piece]);
-    const float scale = 1.4426950408889634f / T;
-    constexpr float LN2 = 0.6931471805599453f;
-    // Sweep 1: g(d) = [d mapped, q(d) > 0] (ln q(d) - ln p(map[d]) + 1), the loss and
-    // sum_d q(d) g(d). The loads of EB ids are issued together (map and q, then the
-    // gathered logits). q(d) g(d) is parked in the gradient row itself (it stays in L2),
-    // so that sweep 2 neither gathers nor takes a logarithm again.
-    const bool park = grad != nullptr;
-    float loss_t = 0.f, qg_t = 0.f;
-    // one id: q (negative = no map), its gathered logit -> the terms of the loss and of sum q g;
-    // returns q(d) g(d)
-    auto term = [&](float qs, float x) -> float {
-        const bool ok = qs >= FLT_MIN;                       // mapped and with (normal) mass
-        const float qa = fabsf(qs);
-        const float f = ok ? LN2 * (lg2_approx(qa) - fmaf(x - M, scale, -lg2_S)) : 0.f;
-        const float g = ok ? f + 1.f : 0.f;
-        loss_t += qa * f;
-        qg_t += qa * g;
-        return qa * g;
+    extern __shared__ __align__(16) unsigned char s_dyn[];   // [chunk] the logit of each mapped id, at its draft id
+    typedef typename Logit<DTYPE>::raw raw_t;
+    raw_t *s_x = (raw_t *)s_dyn;
+    __shared__ double s_red[2][WARPS], s_all[OD_DISTILL_MAX_CHUNKS][2];
+    __shared__ int s_piece[2];
+    const int rank = blockIdx.x, C = gridDim.x, j = blockIdx.y, b = blockIdx.z;
+    const int lo = rank * a.chunk < a.v_q ? rank * a.chunk : a.v_q;
+    const int hi = lo + a.chunk < a.v_q ? lo + a.chunk : a.v_q;
+    const float *q = a.q_rows + ((size_t)b * a.K_max + j) * a.v_q;
+    float *grad = a.grad ? a.grad + ((size_t)b * a.K_max + j) * a.v_q : nullptr;
+    // The chunk's list: groups of 32 entries, one per lane (od_distill_lists). It belongs to the
+    // context: the first entries are requested before the wait, the others a batch ahead.
+    constexpr int EB = 4;                                   // groups per warp and batch
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int2 groups = __ldg((const int2 *)a.list_ofs + rank);
+    const int g_hi = groups.y;
+    int g_at = groups.x + warp;                          // this warp's next group to request
+    uint32_t word[EB];
+    int32_t base[EB];
+    auto load_words = [&]() {
+#pragma unroll
+        for (int e = 0; e < EB; ++e) {
+            const bool in = g_at + e * WARPS < g_hi;
+            word[e] = in ? __ldg(a.list_word + (size_t)(g_at + e * WARPS) * 32 + lane) : 0xFFFFu;
+            base[e] = in ? __ldg(a.list_base + g_at + e * WARPS) : 0;
+        }
+        g_at += EB * WARPS;
     };
+    load_words();
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    const float T = a.temperature[b];
+    int piece, plen;
+    find_piece(a, b, j, s_piece, piece, plen);
+    const bool translated = piece >= 0 && T > 0.f;
+    if (!translated || plen >= 2) {                          // the same for every block of the cluster
+        plain_position<VEC4>(a, b, j, piece, translated, q, grad, lo, hi, rank == 0);
+        return;
+    }
+    cluster_arrive();                                        // this block runs: the others may store to it (waited for below)
+    // ---- a directly mapped token: KL(q' || p_i) over the mapped ids
+    const char *row = (const char *)a.logits + ((size_t)b * a.seq_stride + (size_t)piece * a.row_stride) * sizeof(raw_t);
+    const float M = a.row_max[b * (a.K_max + 1) + piece], S = a.row_sum[b * (a.K_max + 1) + piece];
+    // (the first probabilities travel meanwhile)
+    constexpr int PQ = 2;                                    // vectors of four probabilities in flight per thread
+    float4 qv[PQ];
     if (VEC4) {
-        constexpr int EV = 4;                                // vectors of 4 ids in flight per thread
-        for (int base = threadIdx.x * 4; base < a.v_q; base += THREADS * 4 * EV) {
-            int4 t[EV];
-            float4 qv[EV];
 #pragma unroll
-            for (int e = 0; e < EV; ++e) {
-                const int d = base + e * THREADS * 4;
-                t[e] = d < a.v_q ? __ldg((const int4 *)(a.vocab_map + d)) : make_int4(-1, -1, -1, -1);
-                qv[e] = d < a.v_q ? __ldg((const float4 *)(q + d)) : make_float4(0.f, 0.f, 0.f, 0.f);
-            }
-            float x[EV][4];
+        for (int i = 0; i < PQ; ++i) {
+            const int d = lo + (int)threadIdx.x * 4 + i * THREADS * 4;
+            if (d < hi) qv[i] = __ldg((const float4 *)(q + d));
+        }
+    }
+    // ---- the chunk's logits, gathered in target-id order, to their draft ids in shared memory
+    for (;;) {
+        raw_t x[EB];
+        uint32_t at[EB];
 #pragma unroll
-            for (int e = 0; e < EV; ++e) {
-                x[e][0] = od_load_logit<DTYPE>(row, t[e].x >= 0 ? t[e].x : 0);
-                x[e][1] = od_load_logit<DTYPE>(row, t[e].y >= 0 ? t[e].y : 0);
-                x[e][2] = od_load_logit<DTYPE>(row, t[e].z >= 0 ? t[e].z : 0);
-                x[e][3] = od_load_logit<DTYPE>(row, t[e].w >= 0 ? t[e].w : 0);
+        for (int e = 0; e < EB; ++e) {
+            at[e] = word[e] & 0xFFFFu;
+            if (at[e] != 0xFFFFu) x[e] = __ldg((const raw_t *)row + base[e] + (int)(word[e] >> 16));
+        }
+        const bool more = g_at < g_hi;                       // the same for every lane of a warp
+        if (more) load_words();
+#pragma unroll
+        for (int e = 0; e < EB; ++e)
+            if (at[e] != 0xFFFFu) s_x[at[e]] = x[e];
+        if (!more) break;
+    }
+    KlRow kl;
+    kl.M = M;
+    kl.lg2_S = lg2_approx(S);
+    kl.scale = 1.4426950408889634f / T;
+    __syncthreads();
+    // ---- the loss and sum_e q(e) g(e)
+    float loss_t = 0.f, qg_t = 0.f;
+    // four ids from d: their probabilities with 0 for the ids without a map
+    auto mapped4 = [&](int d, float4 v) {
+        const uint32_t w = __ldg(a.mapped_bits + (d >> 5)) >> (d & 31);
+        return make_float4(w & 1u ? v.x : 0.f, w & 2u ? v.y : 0.f, w & 4u ? v.z : 0.f, w & 8u ? v.w : 0.f);
+    };
+    auto mapped1 = [&](int d, float v) { return __ldg(a.mapped_bits + (d >> 5)) >> (d & 31) & 1u ? v : 0.f; };
+    if (VEC4) {
+        auto sum4 = [&](int d, float4 q4) {
+            const float4 v = mapped4(d, q4);
+            const float4 x = Logit<DTYPE>::load4(s_x + (d - lo));
+            float l = 0.f, g = 0.f;                          // four terms before they meet the running sums
+            kl_term(kl, v.x, x.x, l, g); kl_term(kl, v.y, x.y, l, g);
+            kl_term(kl, v.z, x.z, l, g); kl_term(kl, v.w, x.w, l, g);
+            loss_t += l; qg_t += g;
+        };
+        const int d0 = lo + (int)threadIdx.x * 4;
+        for (int d1 = d0; d1 < hi; d1 += PQ * THREADS * 4) {
+            float4 nx[PQ];
+#pragma unroll
+            for (int i = 0; i < PQ; ++i) {
+                const int d = d1 + (i + PQ) * THREADS * 4;
+                if (d < hi) nx[i] = __ldg((const float4 *)(q + d));
             }
 #pragma unroll
-            for (int e = 0; e < EV; ++e) {
-                const int d = base + e * THREADS * 4;
-                float4 o;
-                o.x = term(t[e].x < 0 ? -qv[e].x : qv[e].x, x[e][0]);
-                o.y = term(t[e].y < 0 ? -qv[e].y : qv[e].y, x[e][1]);
-                o.z = term(t[e].z < 0 ? -qv[e].z : qv[e].z, x[e][2]);
-                o.w = term(t[e].w < 0 ? -qv[e].w : qv[e].w, x[e][3]);
-                if (park && d < a.v_q) *(float4 *)(grad + d) = o;
+            for (int i = 0; i < PQ; ++i) {
+                const int d = d1 + i * THREADS * 4;
+                if (d < hi) sum4(d, qv[i]);
             }
+#pragma unroll
+            for (int i = 0; i < PQ; ++i) qv[i] = nx[i];
         }
     } else {
-        constexpr int EB = 16;
-        for (int base = threadIdx.x; base < a.v_q; base += THREADS * EB) {
-            float qd[EB], x[EB];
-            {
-                int32_t t[EB];
-#pragma unroll
-                for (int e = 0; e < EB; ++e) {
-                    const int d = base + e * THREADS;
-                    t[e] = d < a.v_q ? __ldg(a.vocab_map + d) : -1;
-                    qd[e] = d < a.v_q ? __ldg(q + d) : 0.f;
-                }
-#pragma unroll
-                for (int e = 0; e < EB; ++e)                 // an id without a map: q = 0 drops its term below
-                    if (t[e] < 0) qd[e] = -qd[e];
-#pragma unroll
-                for (int e = 0; e < EB; ++e) x[e] = od_load_logit<DTYPE>(row, t[e] >= 0 ? t[e] : 0);
-            }
-#pragma unroll
-            for (int e = 0; e < EB; ++e) {
-                const int d = base + e * THREADS;
-                const float v = term(qd[e], x[e]);
-                if (park && d < a.v_q) grad[d] = v;
-            }
-        }
+#pragma unroll 4
+        for (int d = lo + (int)threadIdx.x; d < hi; d += THREADS)
+            kl_term(kl, mapped1(d, __ldg(q + d)), Logit<DTYPE>::load(s_x + (d - lo)), loss_t, qg_t);
     }
-    const double loss = block_sum((double)loss_t, s_red);
-    const double qg = block_sum((double)qg_t, s_red);
-    if (threadIdx.x == 0) a.loss[(size_t)b * K + j] = (float)loss;
-    if (grad) {
-        // Sweep 2: grad(d) = q(d) g(d) - q(d) * sum_e q(e) g(e); every thread revisits the
-        // ids it wrote itself, so no barrier is needed for the parked values
-        const float gbar = (float)qg;
-        if (VEC4) {
+    // the block's two sums, to every block of the cluster
+    {
+        double l = loss_t, g = qg_t;
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) {
+            l += __shfl_xor_sync(0xFFFFFFFFu, l, off);
+            g += __shfl_xor_sync(0xFFFFFFFFu, g, off);
+        }
+        if (lane == 0) { s_red[0][warp] = l; s_red[1][warp] = g; }
+        cluster_wait();
+        __syncthreads();
+        if (warp == 0) {
+            const int which = lane >> 4, w = lane & 15;
+            static_assert(WARPS <= 16, "one lane per warp and sum");
+            double v = w < WARPS ? s_red[which][w] : 0.0;
+#pragma unroll
+            for (int off = 8; off > 0; off >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, off);
+            // lanes 0.. store the loss, lanes 16.. the other sum, one block of the cluster each
+            if (w < C) cluster_store(&s_all[rank][which], (uint32_t)w, v);
+        }
+        cluster_arrive();
+        cluster_wait();
+    }
+    double loss = 0.0, qg = 0.0;
+    for (int r = 0; r < C; ++r) { loss += s_all[r][0]; qg += s_all[r][1]; }   // the same order in every block
+    if (rank == 0 && threadIdx.x == 0) a.loss[(size_t)b * a.K_max + j] = (float)loss;
+    if (!grad) return;
+    // ---- the gradient: q(d) (g(d) - sum_e q(e) g(e))
+    const float gbar = (float)qg;
+    if (VEC4) {
 #pragma unroll 4
-            for (int d = threadIdx.x * 4; d < a.v_q; d += THREADS * 4) {
-                const float4 qq = __ldg((const float4 *)(q + d));
-                float4 gv = *(float4 *)(grad + d);
-                gv.x = fmaf(-qq.x, gbar, gv.x); gv.y = fmaf(-qq.y, gbar, gv.y);
-                gv.z = fmaf(-qq.z, gbar, gv.z); gv.w = fmaf(-qq.w, gbar, gv.w);
-                *(float4 *)(grad + d) = gv;
-            }
-        } else {
+        for (int d = lo + (int)threadIdx.x * 4; d < hi; d += THREADS * 4) {
+            const float4 v = __ldg((const float4 *)(q + d)), u = mapped4(d, v);
+            const float4 x = Logit<DTYPE>::load4(s_x + (d - lo));
+            float4 o;
+            o.x = fmaf(-v.x, gbar, v.x * kl_term(kl, u.x, x.x, loss_t, qg_t));
+            o.y = fmaf(-v.y, gbar, v.y * kl_term(kl, u.y, x.y, loss_t, qg_t));
+            o.z = fmaf(-v.z, gbar, v.z * kl_term(kl, u.z, x.z, loss_t, qg_t));
+            o.w = fmaf(-v.w, gbar, v.w * kl_term(kl, u.w, x.w, loss_t, qg_t));
+            __stcs((float4 *)(grad + d), o);
+        }
+    } else {
 #pragma unroll 4
-            for (int d = threadIdx.x; d < a.v_q; d += THREADS) grad[d] = fmaf(-__ldg(q + d), gbar, grad[d]);
+        for (int d = lo + (int)threadIdx.x; d < hi; d += THREADS) {
+            const float v = __ldg(q + d);
+            grad[d] = fmaf(-v, gbar, v * kl_term(kl, mapped1(d, v), Logit<DTYPE>::load(s_x + (d - lo)), loss_t, qg_t));
         }
     }
 }
+
+//XX
+// Draft vocabularies beyond the chunked kernel's shared memory (OD_DISTILL_MAX_CHUNKS chunks of
+// OD_DISTILL_MAX_CHUNK_IDS ids): one block per position, the ids in draft order, each gathering
+// its logit; q(d) g(d) waits in the gradient row for the second sweep.
+template <int DTYPE>
+__global__ void __launch_bounds__(THREADS, 2)
+od_distill_any_kernel(const DistillArgs a)
+{
+    __shared__ double s_red[THREADS / 32];
+    __shared__ int s_piece[2];
+    const int j = blockIdx.y, b = blockIdx.z;
+    const float *q = a.q_rows + ((size_t)b * a.K_max + j) * a.v_q;
+    float *grad = a.grad ? a.grad + ((size_t)b * a.K_max + j) * a.v_q : nullptr;
+    int piece, plen;
+    find_piece(a, b, j, s_piece, piece, plen);
+    const float T = a.temperature[b];
+    const bool translated = piece >= 0 && T > 0.f;
+    if (!translated || plen >= 2) {
+        plain_position<false>(a, b, j, piece, translated, q, grad, 0, a.v_q, true);
+        return;
+    }
+    const size_t esz = DTYPE == OD_BF16 ? 2 : 4;
+    const char *row = (const char *)a.logits + ((size_t)b * a.seq_stride + (size_t)piece * a.row_stride) * esz;
+    KlRow kl;
+    kl.M = a.row_max[b * (a.K_max + 1) + piece];
+    kl.lg2_S = lg2_approx(a.row_sum[b * (a.K_max + 1) + piece]);
+    kl.scale = 1.4426950408889634f / T;
+    float loss_t = 0.f, qg_t = 0.f;
+    constexpr int EB = 16;
+    for (int base = threadIdx.x; base < a.v_q; base += THREADS * EB) {
+        float qd[EB], x[EB];
+        int32_t t[EB];
+#pragma unroll
+        for (int e = 0; e < EB; ++e) {
+            const int d = base + e * THREADS;
+            t[e] = d < a.v_q ? __ldg(a.vocab_map + d) : -1;
+            qd[e] = d < a.v_q ? __ldg(q + d) : 0.f;
+        }
+#pragma unroll
+        for (int e = 0; e < EB; ++e) {
+            x[e] = od_load_logit<DTYPE>(row, t[e] >= 0 ? t[e] : 0);
+            if (t[e] < 0) qd[e] = 0.f;                       // an id without a map has no term
+        }
+#pragma unroll
+        for (int e = 0; e < EB; ++e) {
+            const int d = base + e * THREADS;
+            const float g = kl_term(kl, qd[e], x[e], loss_t, qg_t);
+            if (grad && d < a.v_q) grad[d] = qd[e] * g;
+        }
+    }
+    const double loss = block_sum((double)loss_t, s_red), qg = block_sum((double)qg_t, s_red);
+    if (threadIdx.x == 0) a.loss[(size_t)b * a.K_max + j] = (float)loss;
+    if (grad) {
+        // every thread revisits the ids it wrote itself: no barrier for the parked values
+        const float gbar = (float)qg;
+#pragma unroll 4
+        for (int d = threadIdx.x; d < a.v_q; d += THREADS) grad[d] = fmaf(-__ldg(q + d), gbar, grad[d]);
+    }
+}
+
+template <int DTYPE, bool VEC4>
+cudaError_t launch_chunks(const DistillArgs &a, int C, bool pdl, cudaStream_t s)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)C, (unsigned)a.K_max, (unsigned)a.B);
+    cfg.blockDim = dim3(THREADS);
+    cfg.dynamicSmemBytes = (size_t)a.chunk * (DTYPE == OD_BF16 ? 2 : 4);
+    cfg.stream = s;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = (unsigned)C; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+        cfg.numAttrs = pdl ? 2 : 1;
+    return cudaLaunchKernelEx(&cfg, od_distill_kernel<DTYPE, VEC4>, a);
+}
+
+// draft ids per chunk for a vocabulary cut into C = 1 << level chunks: whole words of the mapped
+// bits, and each a run of the same eighths
+int32_t fine_ids(int32_t v_q) { return ((v_q + 7) / 8 + 31) / 32 * 32; }
+int32_t chunk_ids(int32_t v_q, int level) { return fine_ids(v_q) << (OD_DISTILL_LEVELS - 1 - level); }
+constexpr int CHUNK_BYTES = 36 * 1024;
+static_assert(1 << (OD_DISTILL_LEVELS - 1) == OD_DISTILL_MAX_CHUNKS && OD_DISTILL_MAX_CHUNKS == 8, "the finest level");
 
 }  // namespace
 
@@ -222,20 +438,88 @@ cudaError_t od_launch_distill(od_ctx *c, int32_t B, int32_t K_max, const float *
                               float lambda, int32_t lambda_mode, float *loss, float *grad, cudaStream_t s)
 {
     if (B == 0) return cudaSuccess;
-    DistillArgs a;
+    DistillArgs a = {};
     a.B = B; a.K_max = K_max; a.v_q = c->v_q; a.v_p = c->v_p;
     a.q_rows = q_rows; a.draft_ids = draft_ids; a.tgt_ids = tgt_ids; a.span_start = span_start;
     a.span_len = span_len; a.m = m; a.logits = logits; a.row_stride = row_stride; a.seq_stride = seq_stride;
     a.row_max = row_max; a.row_sum = row_sum; a.p_sel = p_sel; a.temperature = temperature;
     a.vocab_map = c->d_vocab_map; a.lambda = lambda; a.lambda_mode = lambda_mode; a.loss = loss; a.grad = grad;
-    dim3 grid((unsigned)K_max, (unsigned)B);
+    const bool bf = dtype == OD_BF16;
     const bool vec4 = c->v_q % 4 == 0 && ((uintptr_t)q_rows & 15u) == 0 && (!grad || ((uintptr_t)grad & 15u) == 0);
-    if (dtype == OD_BF16) {
-        if (vec4) od_distill_kernel<OD_BF16, true><<<grid, THREADS, 0, s>>>(a);
-        else od_distill_kernel<OD_BF16, false><<<grid, THREADS, 0, s>>>(a);
-    } else {
-        if (vec4) od_distill_kernel<OD_F32, true><<<grid, THREADS, 0, s>>>(a);
-        else od_distill_kernel<OD_F32, false><<<grid, THREADS, 0, s>>>(a);
+    // The number of chunks: the fewest with which a chunk's logits take 36 KB or less (32000 bf16
+    // ids in two chunks of 32 KB: 34.9 us, in one of 64 KB: 44.7, in four: 38 us), more while all
+    // blocks still fit one resident wave (a few positions: 5 x 10 at v_q = 32000 takes 8 chunks).
+    int level = 0;
+    const auto more = [&](int l) { return l + 1 < OD_DISTILL_LEVELS; };
+    while (more(level) && chunk_ids(c->v_q, level) * (bf ? 2 : 4) > CHUNK_BYTES) ++level;
+    while (more(level) && (int64_t)B * K_max * 2 << level <= (int64_t)c->sm_count * 3) ++level;
+    const int C = 1 << level;
+    a.chunk = chunk_ids(c->v_q, level);
+    if (a.chunk > OD_DISTILL_MAX_CHUNK_IDS) {
+        const dim3 grid(1, (unsigned)K_max, (unsigned)B);
+        if (bf) od_distill_any_kernel<OD_BF16><<<grid, THREADS, 0, s>>>(a);
+        else od_distill_any_kernel<OD_F32><<<grid, THREADS, 0, s>>>(a);
+        return cudaGetLastError();
     }
-    return cudaGetLastError();
+    const OdDistillLists l = od_distill_lists(c->d_distill_lists, c->v_q, c->v_p);
+    a.list_word = l.word + (size_t)level * l.groups * 32; a.list_base = l.base + (size_t)level * l.groups;
+    a.list_ofs = l.ofs + level * OD_DISTILL_MAX_CHUNKS * 2; a.mapped_bits = l.bits;
+    const bool pdl = c->opt_pdl != 0;
+    if (vec4) return bf ? launch_chunks<OD_BF16, true>(a, C, pdl, s) : launch_chunks<OD_F32, true>(a, C, pdl, s);
+    return bf ? launch_chunks<OD_BF16, false>(a, C, pdl, s) : launch_chunks<OD_F32, false>(a, C, pdl, s);
+}
+
+// The kernels' dynamic shared memory (a chunk of a draft vocabulary of v_q ids): opt in where it
+// exceeds the default (the device must be current; allocates nothing).
+cudaError_t od_distill_prepare_device(int32_t v_q)
+{
+    const int n = OD_DISTILL_MAX_CHUNK_IDS * 4;
+    if (chunk_ids(v_q, 0) * 4 <= 48 * 1024) return cudaSuccess;
+    cudaError_t e = cudaFuncSetAttribute(od_distill_kernel<OD_BF16, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, n);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(od_distill_kernel<OD_F32, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, n);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(od_distill_kernel<OD_BF16, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, n);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(od_distill_kernel<OD_F32, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, n);
+    return e;
+}
+
+// The gather lists of the distillation kernel, on the host, in the layout of od_distill_lists.
+// `inv` is the inverse map: draft id of each target id, or negative.
+void od_distill_plan(int32_t v_q, int32_t v_p, const int32_t *inv, void *out)
+{
+    const OdDistillLists l = od_distill_lists(out, v_q, v_p);
+    for (int w = 0; w < (v_q + 31) / 32; ++w) l.bits[w] = 0u;
+    struct Open {
+        int32_t n, base;                                     // a chunk's open group: n entries so far, from target `base`
+        int32_t *end;                                        // one past it
+    } open[OD_DISTILL_LEVELS][OD_DISTILL_MAX_CHUNKS];
+    int first = OD_DISTILL_LEVELS - 1;                       // the coarsest level that a launch can ask for
+    while (first > 0 && chunk_ids(v_q, first - 1) * 2 <= CHUNK_BYTES) --first;
+    for (int level = 0; level < OD_DISTILL_LEVELS; ++level)
+        for (int k = 0; k < OD_DISTILL_MAX_CHUNKS; ++k) {
+            int32_t *ofs = l.ofs + (level * OD_DISTILL_MAX_CHUNKS + k) * 2;
+            ofs[0] = ofs[1] = (int32_t)(k * (l.groups >> level));
+            open[level][k] = {32, 0, ofs + 1};
+        }
+    // a chunk's entries in target-id order; a new group of 32 where one is full or the next
+    // target is over 65535 ids on
+    const int32_t fine = fine_ids(v_q);
+    for (int32_t t = 0; t < v_p; ++t) {
+        const int32_t d = inv[t];
+        if (d < 0) continue;
+        const int32_t f = d / fine;
+        l.bits[d >> 5] |= 1u << (d & 31);
+        for (int level = first; level < OD_DISTILL_LEVELS; ++level) {
+            const int32_t shift = OD_DISTILL_LEVELS - 1 - level, k = f >> shift;
+            Open &o = open[level][k];
+            if (o.n == 32 || t - o.base > 0xFFFF) {
+                const size_t g = (size_t)level * l.groups + (*o.end)++;
+                l.base[g] = t;
+                for (int i = 0; i < 32; ++i) l.word[g * 32 + i] = 0xFFFFu;
+                o.n = 0; o.base = t;
+            }
+            // (a chunk of more than OD_DISTILL_MAX_CHUNK_IDS ids is not asked for: the cut does not matter)
+            l.word[((size_t)level * l.groups + *o.end - 1) * 32 + o.n++] =
+                (uint32_t)(t - o.base) << 16 | (uint32_t)((d - (k << shift) * fine) & 0xFFFF);
+        }
+    }
 }

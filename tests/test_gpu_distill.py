@@ -117,3 +117,15 @@ def test_loss_without_a_gradient_buffer(cuda_device, v_q):
             np.testing.assert_allclose(loss[b], want_l, rtol=2e-5, atol=2e-6)
         np.testing.assert_allclose(loss, with_grad.cpu().numpy(), rtol=1e-6, atol=1e-7)
     ctx.close()
+
+
+# one, two, four and eight chunks of draft ids (eight of them for few positions, some empty), chunk
+# edges off the vector width, gaps of over 65535 target ids, and a vocabulary beyond the chunked kernel
+@pytest.mark.parametrize("v_q, v_p, B, k_max", [(600, 1003, 64, 8), (18436, 20011, 120, 2), (36902, 37003, 60, 2),
+                                                (13, 17, 2, 3), (4097, 4099, 3, 2), (40, 400000, 2, 2),
+                                                (450561, 450600, 1, 1)])
+def test_chunks_of_draft_ids(cuda_device, v_q, v_p, B, k_max):
+    """Tolerances as above: fp32 sums of v_q terms, logarithms to 2^-22."""
+    for dtype in ("bf16", "f32"):
+        w = _small(B=B, k_max=k_max, v_q=v_q, v_p=v_p, cache_entries=0, logit_dtype=dtype, gen_seed=0xBEEFF0)
+        _check(w, cuda_device, [0], 0.2, ds.LAMBDA_CONSTANT, positions=sorted({0, B // 3, B - 1}))
