@@ -192,6 +192,8 @@ int32_t od_set_vocab_map(od_ctx *c, const int32_t *host_map)
     std::vector<char> lists(od_distill_lists_bytes(c->v_q, c->v_p));
     od_distill_plan(c->v_q, c->v_p, inv.data(), lists.data());
     OD_CUDA(cudaMemcpy(c->d_distill_lists, lists.data(), lists.size(), cudaMemcpyHostToDevice));
+    c->map_same_ids = true;
+    for (int32_t d = 0; d < c->v_q; ++d) c->map_same_ids = c->map_same_ids && host_map[d] == d;
     c->have_map = true;
     return OD_OK;
     } catch (const std::bad_alloc &) {

@@ -30,6 +30,7 @@ struct od_ctx {
     int32_t *d_inv_map;             // [v_p], -1 outside the image
     void *d_distill_lists;          // gather lists of the distillation kernel (od_distill_lists)
     bool have_map;
+    bool map_same_ids;              // every draft id is mapped to the target id of the same number
 
     // n-gram cache: open addressing over groups of 32 slots
     uint64_t *d_keys;               // [cap], 0 = empty

@@ -77,6 +77,7 @@ struct SampleArgs {
     const uint64_t *seed;
     uint64_t step;
     const int32_t *vocab_map, *inv_map;
+    int32_t same_ids;                   // 1: target id t is draft id t (t < v_q), and the drafter's rows are 16-byte aligned
     int32_t *out_token;
     float *resid_mass;
     uint32_t *flags;
@@ -139,6 +140,17 @@ __device__ __forceinline__ void eq2_ids(const SeqState &q, const SampleArgs &a, 
     }
 }
 
+// The drafter's probabilities of the EPT ids from t0 where target ids are draft ids: two 16-byte
+// loads, nothing looked up. v_q is a multiple of 4; ids >= v_q have none.
+__device__ __forceinline__ void same_id_probs(const SeqState &q, const SampleArgs &a, int t0, float *qq)
+{
+    const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
+    const float4 v0 = t0 < a.v_q ? __ldg((const float4 *)(q.q_row + t0)) : z;
+    const float4 v1 = t0 + 4 < a.v_q ? __ldg((const float4 *)(q.q_row + t0) + 1) : z;
+    qq[0] = v0.x; qq[1] = v0.y; qq[2] = v0.z; qq[3] = v0.w;
+    qq[4] = v1.x; qq[5] = v1.y; qq[6] = v1.z; qq[7] = v1.w;
+}
+
 // r'(t) of the EPT consecutive ids this lane owns in `tile`; ids >= v_p give 0
 template <int DTYPE>
 __device__ __forceinline__ void tile_values(const SeqState &q, const SampleArgs &a, bool residual,
@@ -158,12 +170,16 @@ __device__ __forceinline__ void tile_values(const SeqState &q, const SampleArgs 
             x[4] = v1.x; x[5] = v1.y; x[6] = v1.z; x[7] = v1.w;
         }
         if (residual) {
-            const int4 i0 = __ldg((const int4 *)(a.inv_map + t0));
-            const int4 i1 = __ldg((const int4 *)(a.inv_map + t0) + 1);
-            const int32_t d[EPT] = {i0.x, i0.y, i0.z, i0.w, i1.x, i1.y, i1.z, i1.w};
             float qq[EPT];
+            if (a.same_ids) {
+                same_id_probs(q, a, t0, qq);
+            } else {
+                const int4 i0 = __ldg((const int4 *)(a.inv_map + t0));
+                const int4 i1 = __ldg((const int4 *)(a.inv_map + t0) + 1);
+                const int32_t d[EPT] = {i0.x, i0.y, i0.z, i0.w, i1.x, i1.y, i1.z, i1.w};
 #pragma unroll
-            for (int e = 0; e < EPT; ++e) qq[e] = d[e] >= 0 ? __ldg(q.q_row + d[e]) : 0.f;
+                for (int e = 0; e < EPT; ++e) qq[e] = d[e] >= 0 ? __ldg(q.q_row + d[e]) : 0.f;
+            }
 #pragma unroll
             for (int e = 0; e < EPT; ++e) r[e] = resid_of(q, x[e], qq[e]);
         } else {
@@ -265,6 +281,39 @@ __device__ __forceinline__ void warp_tiles_dense(const SeqState &q, const Sample
     }
 }
 
+// A lane's ids of one whole tile as they are stored, and the tile's residual from them
+template <int DTYPE>
+constexpr int RAW = DTYPE == OD_BF16 ? 1 : 2;               // 16-byte vectors of logits per lane and tile
+template <int DTYPE>
+__device__ __forceinline__ void load_tile(const SeqState &q, int tile, int lane, uint4 *raw)
+{
+    const uint4 *src = (const uint4 *)(q.row + (size_t)(tile * OD_SAMPLE_TILE + lane * EPT) * (DTYPE == OD_BF16 ? 2 : 4));
+    raw[0] = ld_once(src);
+    if (DTYPE != OD_BF16) raw[1] = ld_once(src + 1);
+}
+template <int DTYPE>
+__device__ __forceinline__ float tile_sum(const SeqState &q, const SampleArgs &a, int tile, int lane, const uint4 *raw,
+                                          const float *qq)
+{
+    float x[EPT], r[EPT];
+    if (DTYPE == OD_BF16) {
+        const uint4 v = raw[0];
+        x[0] = od_bf16_lo(v.x); x[1] = od_bf16_hi(v.x); x[2] = od_bf16_lo(v.y); x[3] = od_bf16_hi(v.y);
+        x[4] = od_bf16_lo(v.z); x[5] = od_bf16_hi(v.z); x[6] = od_bf16_lo(v.w); x[7] = od_bf16_hi(v.w);
+    } else {
+        const uint4 v0 = raw[0], v1 = raw[DTYPE == OD_BF16 ? 0 : 1];
+        x[0] = __uint_as_float(v0.x); x[1] = __uint_as_float(v0.y); x[2] = __uint_as_float(v0.z); x[3] = __uint_as_float(v0.w);
+        x[4] = __uint_as_float(v1.x); x[5] = __uint_as_float(v1.y); x[6] = __uint_as_float(v1.z); x[7] = __uint_as_float(v1.w);
+    }
+#pragma unroll
+    for (int e = 0; e < EPT; ++e) r[e] = resid_of(q, x[e], qq[e]);
+    eq2_ids<DTYPE>(q, a, tile * OD_SAMPLE_TILE + lane * EPT, r);
+    float sum = r[0];
+#pragma unroll
+    for (int e = 1; e < EPT; ++e) sum += r[e];
+    return warp_sum_f32(sum);
+}
+
 // Inverse-map entries of a warp's first pair of whole tiles [t_lo, t_hi).
 __device__ __forceinline__ void first_pair_entries(const SampleArgs &a, int t_lo, int t_hi, int lane, int4 (&ni)[2][2])
 {
@@ -285,7 +334,6 @@ template <int DTYPE>
 __device__ __forceinline__ void warp_tiles_dense_piped(const SeqState &q, const SampleArgs &a, int t_lo, int t_hi,
                                                        int lane, double *tile_val, int4 (&ni)[2][2])
 {
-    constexpr int ESZ = DTYPE == OD_BF16 ? 2 : 4;
     for (int t = t_lo; t < t_hi; t += 2) {
         int32_t d[2][EPT];
 #pragma unroll
@@ -302,13 +350,9 @@ __device__ __forceinline__ void warp_tiles_dense_piped(const SeqState &q, const 
             }
         }
         const bool two = t + 1 < t_hi;
-        uint4 raw[2][DTYPE == OD_BF16 ? 1 : 2];
+        uint4 raw[2][RAW<DTYPE>];
 #pragma unroll
-        for (int i = 0; i < 2; ++i) {
-            const uint4 *src = (const uint4 *)(q.row + (size_t)((i == 0 || two ? t + i : t) * OD_SAMPLE_TILE + lane * EPT) * ESZ);
-            raw[i][0] = ld_once(src);
-            if (DTYPE != OD_BF16) raw[i][1] = ld_once(src + 1);
-        }
+        for (int i = 0; i < 2; ++i) load_tile<DTYPE>(q, i == 0 || two ? t + i : t, lane, raw[i]);
         float qq[2][EPT];
 #pragma unroll
         for (int i = 0; i < 2; ++i) {
@@ -318,26 +362,36 @@ __device__ __forceinline__ void warp_tiles_dense_piped(const SeqState &q, const 
         float mine = 0.f;
 #pragma unroll
         for (int i = 0; i < 2; ++i) {
-            float x[EPT], r[EPT];
-            if (DTYPE == OD_BF16) {
-                const uint4 v = raw[i][0];
-                x[0] = od_bf16_lo(v.x); x[1] = od_bf16_hi(v.x); x[2] = od_bf16_lo(v.y); x[3] = od_bf16_hi(v.y);
-                x[4] = od_bf16_lo(v.z); x[5] = od_bf16_hi(v.z); x[6] = od_bf16_lo(v.w); x[7] = od_bf16_hi(v.w);
-            } else {
-                const uint4 v0 = raw[i][0], v1 = raw[i][DTYPE == OD_BF16 ? 0 : 1];
-                x[0] = __uint_as_float(v0.x); x[1] = __uint_as_float(v0.y); x[2] = __uint_as_float(v0.z); x[3] = __uint_as_float(v0.w);
-                x[4] = __uint_as_float(v1.x); x[5] = __uint_as_float(v1.y); x[6] = __uint_as_float(v1.z); x[7] = __uint_as_float(v1.w);
-            }
-#pragma unroll
-            for (int e = 0; e < EPT; ++e) r[e] = resid_of(q, x[e], qq[i][e]);
-            eq2_ids<DTYPE>(q, a, (t + i) * OD_SAMPLE_TILE + lane * EPT, r);
-            float sum = r[0];
-#pragma unroll
-            for (int e = 1; e < EPT; ++e) sum += r[e];
-            sum = warp_sum_f32(sum);
+            const float sum = tile_sum<DTYPE>(q, a, t + i, lane, raw[i], qq[i]);
             if (lane == i) mine = sum;
         }
         if (lane < 2 && t + lane < t_hi) tile_val[t + lane] = (double)mine;
+    }
+}
+
+// The same for target ids that are draft ids: independent 16-byte loads only, the next tile's
+// requested before the current one is worked on.
+template <int DTYPE>
+__device__ __forceinline__ void warp_tiles_same_ids(const SeqState &q, const SampleArgs &a, int t_lo, int t_hi, int lane,
+                                                    double *tile_val)
+{
+    uint4 raw[RAW<DTYPE>];
+    float qq[EPT];
+    load_tile<DTYPE>(q, t_lo, lane, raw);
+    same_id_probs(q, a, t_lo * OD_SAMPLE_TILE + lane * EPT, qq);
+#pragma unroll 1
+    for (int t = t_lo; t < t_hi; ++t) {
+        uint4 nraw[RAW<DTYPE>];
+        float nqq[EPT];
+        const int n = t + 1 < t_hi ? t + 1 : t;
+        load_tile<DTYPE>(q, n, lane, nraw);
+        same_id_probs(q, a, n * OD_SAMPLE_TILE + lane * EPT, nqq);
+        const float sum = tile_sum<DTYPE>(q, a, t, lane, raw, qq);
+        if (lane == 0) tile_val[t] = (double)sum;
+#pragma unroll
+        for (int k = 0; k < RAW<DTYPE>; ++k) raw[k] = nraw[k];
+#pragma unroll
+        for (int e = 0; e < EPT; ++e) qq[e] = nqq[e];
     }
 }
 
@@ -474,7 +528,7 @@ od_sample_kernel(const SampleArgs a)
     if (p_hi > tile_hi) p_hi = tile_hi;
     const int p_hi_w = p_hi < a.v_p / OD_SAMPLE_TILE ? p_hi : a.v_p / OD_SAMPLE_TILE;
     int4 ni[2][2] = {};
-    if (MODE != 2 && p_lo < p_hi_w) first_pair_entries(a, p_lo, p_hi_w, lane, ni);
+    if (MODE != 2 && !a.same_ids && p_lo < p_hi_w) first_pair_entries(a, p_lo, p_hi_w, lane, ni);
 
     // n_accepted and the row statistics come from the verification kernels
     if (a.early) asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -602,7 +656,10 @@ od_sample_kernel(const SampleArgs a)
                 // whole tiles pipelined; the row's ragged last tile (if it is this warp's) on its own
                 const int hi_w = p_hi_w;
                 if (q.residual) {
-                    if (t_lo < hi_w) warp_tiles_dense_piped<DTYPE>(q, a, t_lo, hi_w, lane, tile_val, ni);
+                    if (t_lo < hi_w) {
+                        if (a.same_ids) warp_tiles_same_ids<DTYPE>(q, a, t_lo, hi_w, lane, tile_val);
+                        else warp_tiles_dense_piped<DTYPE>(q, a, t_lo, hi_w, lane, tile_val, ni);
+                    }
                     if (hi_w < t_hi) warp_tiles_dense<DTYPE, 2>(q, a, true, hi_w > t_lo ? hi_w : t_lo, t_hi, lane, tile_val);
                 } else {
                     warp_tiles_dense<DTYPE, 2>(q, a, false, t_lo, t_hi, lane, tile_val);
@@ -890,6 +947,7 @@ static cudaError_t launch_sample(od_ctx *c, int mode, int32_t B, int32_t K_max, 
     a.span_start = span_start; a.span_len = span_len; a.m = m; a.tail_kind = tail_kind;
     a.n_accepted = n_accepted; a.temperature = temperature; a.seed = seed; a.step = step;
     a.vocab_map = c->d_vocab_map; a.inv_map = c->d_inv_map;
+    a.same_ids = c->map_same_ids && c->v_q % 4 == 0 && ((uintptr_t)q_rows & 15u) == 0;
     a.out_token = out_token; a.resid_mass = resid_mass; a.flags = flags;
     a.tile_val = c->d_tile_sums; a.ticket = c->d_samp_ticket;
     a.tile_lo = tile_lo; a.tile_hi = tile_hi; a.col0 = mode == 0 ? 0 : shard_lo;
