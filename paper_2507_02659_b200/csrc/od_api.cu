@@ -45,7 +45,7 @@ int32_t dev_alloc(T **p, size_t n)
 void free_all(od_ctx *c)
 {
     od_cache_free_dynamic(c);
-    void *ptrs[] = {c->d_vocab_map, c->d_inv_map, c->d_distill_lists, c->d_keys, c->d_vals, c->d_partials,
+    void *ptrs[] = {c->d_vocab_map, c->d_inv_map, c->d_distill_lists, c->d_sample_lists, c->d_keys, c->d_vals, c->d_partials,
                     c->d_tile_sums,
                     c->d_samp_ticket, c->s_logits, c->s_q_rows, c->s_q_sel, c->s_temperature,
                     c->s_draft_ids, c->s_draft_len, c->s_seed, c->s_tgt_ids, c->s_span_start,
@@ -130,7 +130,7 @@ int32_t od_create(od_ctx **ctx, int32_t device, int32_t draft_vocab, int32_t tar
         delete c;
         return OD_ERR_UNSUPPORTED;
     }
-    if (od_sample_prepare_device(od_sample_smem_bytes(c->tiles_per_row)) != cudaSuccess) {
+    if (od_sample_prepare_device(od_sample_smem_bytes(c->tiles_per_row), &c->cluster16) != cudaSuccess) {
         delete c;
         return OD_ERR_CUDA;
     }
@@ -147,6 +147,9 @@ int32_t od_create(od_ctx **ctx, int32_t device, int32_t draft_vocab, int32_t tar
     char *lists = nullptr;
     if (st == OD_OK) st = dev_alloc(&lists, od_distill_lists_bytes(draft_vocab, target_vocab));
     c->d_distill_lists = lists;
+    lists = nullptr;
+    if (st == OD_OK) st = dev_alloc(&lists, od_sample_lists_bytes(draft_vocab, target_vocab));
+    c->d_sample_lists = lists;
     if (st == OD_OK) st = dev_alloc(&c->d_partials, rows * OD_VERIFY_SEG_MAX);
     if (st == OD_OK) st = dev_alloc(&c->d_tile_sums, (size_t)max_batch * c->tiles_per_row);
     if (st == OD_OK) st = dev_alloc(&c->d_samp_ticket, (size_t)max_batch);
@@ -192,6 +195,9 @@ int32_t od_set_vocab_map(od_ctx *c, const int32_t *host_map)
     std::vector<char> lists(od_distill_lists_bytes(c->v_q, c->v_p));
     od_distill_plan(c->v_q, c->v_p, inv.data(), lists.data());
     OD_CUDA(cudaMemcpy(c->d_distill_lists, lists.data(), lists.size(), cudaMemcpyHostToDevice));
+    lists.resize(od_sample_lists_bytes(c->v_q, c->v_p));
+    od_sample_plan(c->v_q, c->v_p, fwd.data(), inv.data(), lists.data(), c->sample_slots);
+    OD_CUDA(cudaMemcpy(c->d_sample_lists, lists.data(), lists.size(), cudaMemcpyHostToDevice));
     c->map_same_ids = true;
     for (int32_t d = 0; d < c->v_q; ++d) c->map_same_ids = c->map_same_ids && host_map[d] == d;
     c->have_map = true;

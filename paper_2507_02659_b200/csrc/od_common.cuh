@@ -11,7 +11,10 @@
 #define OD_WARP 32
 #define OD_GROUP 32                 // slots of one hash-table probe group
 #define OD_SAMPLE_TILE 256          // elements of one residual-sampler tile (8 per lane of a warp)
-#define OD_SAMPLE_THREADS 256
+#define OD_SAMPLE_THREADS 256       // of the vocabulary shards' sampler
+#define OD_SAMPLE_LEVELS 5          // 1, 2, 4, 8 or 16 blocks draw for one sequence
+#define OD_SAMPLE_MAX_PARTS 16      // (16: a non-portable cluster)
+#define OD_SAMPLE_MAX_SLOTS 53248   // mapped ids of a part: 208 KB of shared memory
 #define OD_SAMPLE_SMEM_MAX (200 * 1024)  // dynamic shared memory the sampler may ask for: 8 bytes per tile
 #define OD_VERIFY_SEG_MAX 64        // most segments (partials) one logit row is cut into
 #define OD_VERIFY_MAX_B 2048        // sequences per od_verify launch (longer batches go in slices)
@@ -29,6 +32,9 @@ struct od_ctx {
     int32_t *d_vocab_map;           // [v_q]
     int32_t *d_inv_map;             // [v_p], -1 outside the image
     void *d_distill_lists;          // gather lists of the distillation kernel (od_distill_lists)
+    void *d_sample_lists;           // and of the sampler (od_sample_lists)
+    int32_t sample_slots[OD_SAMPLE_LEVELS];   // most mapped ids of a part
+    bool cluster16;                 // the device takes the sampler's clusters of 16 blocks
     bool have_map;
     bool map_same_ids;              // every draft id is mapped to the target id of the same number
 
@@ -131,8 +137,42 @@ cudaError_t od_launch_sample(od_ctx *c, int32_t B, int32_t K_max, const void *lo
                              int32_t *out_token, float *resid_mass, uint32_t *flags,
                              cudaStream_t s, const od_fused_verify *fuse = nullptr);
 
-size_t od_sample_smem_bytes(int32_t ntiles);            // dynamic shared memory of the sampler kernel
-cudaError_t od_sample_prepare_device(size_t bytes);     // opt in to it where it exceeds the default
+size_t od_sample_smem_bytes(int32_t ntiles);            // dynamic shared memory of the shard sampler's kernel
+// opt in to the dynamic shared memory and the cluster size that the sampler's kernels may ask for
+cudaError_t od_sample_prepare_device(size_t bytes, bool *cluster16);
+
+// What the sampler knows about the vocabulary map, one block of memory. The mapped target ids in
+// order have ranks 0, 1, ...; a row's tiles are cut into 1, 2, 4, 8, 16 parts (the levels), and a
+// part's mapped ids, in draft-id order, are a list in groups of 32: an entry is (draft id - the
+// group's base) << 16 | (rank - the part's first rank), or 0xFFFF in the low half where the
+// group has no more.
+struct OdSampleLists {
+    int64_t groups;                 // room for this many groups in each level
+    uint32_t *word;                 // [levels][groups][32]
+    int32_t *base;                  // [levels][groups]
+    int32_t *part;                  // [levels][max parts][4] a part's groups within its level (the first, one past the last), first rank, -
+    uint32_t *octet;                // [ceil(v_p / 8)] of target ids 8i .. 8i+7: rank of the first mapped one << 8 | which are mapped
+};
+inline OdSampleLists od_sample_lists(void *base, int32_t v_q, int32_t v_p)
+{
+    OdSampleLists l;
+    // a group ends full, or at a gap of over 65535 draft ids, or with its part
+    l.groups = ((int64_t)(v_q < v_p ? v_q : v_p) + 31) / 32 + OD_SAMPLE_MAX_PARTS * ((int64_t)v_q / 65536 + 2);
+    l.word = (uint32_t *)base;
+    l.part = (int32_t *)(l.word + OD_SAMPLE_LEVELS * l.groups * 32);
+    l.base = l.part + OD_SAMPLE_LEVELS * OD_SAMPLE_MAX_PARTS * 4;
+    l.octet = (uint32_t *)(l.base + OD_SAMPLE_LEVELS * l.groups);
+    return l;
+}
+inline size_t od_sample_lists_bytes(int32_t v_q, int32_t v_p)
+{
+    const OdSampleLists l = od_sample_lists(nullptr, v_q, v_p);
+    return (size_t)((uintptr_t)(l.octet + (v_p + 7) / 8) - (uintptr_t)nullptr);
+}
+// tiles of a 16th of a row: a part of level l is 16 >> l of them
+inline int32_t od_sample_fine_tiles(int32_t v_p) { return ((v_p + OD_SAMPLE_TILE - 1) / OD_SAMPLE_TILE + OD_SAMPLE_MAX_PARTS - 1) / OD_SAMPLE_MAX_PARTS; }
+// host; slots: [levels] most mapped ids of a part
+void od_sample_plan(int32_t v_q, int32_t v_p, const int32_t *map, const int32_t *inv, void *out, int32_t *slots);
 
 // vocabulary shards (columns [shard_lo, shard_lo + shard_len) of the rows on this GPU)
 cudaError_t od_launch_verify_shard_stats(od_ctx *c, int32_t B, int32_t K_max, int32_t shard_lo,

@@ -9,28 +9,31 @@
 // Values are carried unnormalised: e(t) = exp2((x_t - M)*scale) = p(t)*S and
 // r'(t) = max(0, e(t) - q'(t)*S).
 //   pass 1  every warp takes a run of tiles of row j = n_b; per tile one coalesced
-//           128-bit load of the logits, one coalesced read of the inverse map (the
-//           draft id of each target id, -1 outside the map's image), a predicated
-//           gather of the drafter's probability for the ids that have one, r' of
-//           its eight ids (with the two ids Eq. (2) singles out) and one warp sum:
-//           the tile's value. Whole tiles go in pairs, software-pipelined: the
-//           inverse-map entries of the next pair are requested before the gathers
-//           of the current pair, so a pair costs one memory round trip (the
-//           entries of a warp's first pair, like everything else that does not
-//           depend on the verification kernels, are requested before the kernel
-//           waits for them);
-//   ticket  blocks never wait for each other: the block that draws the
-//           sequence's last ticket continues alone;
-//   pass 2  that block scans the tile values in parallel (total,
-//           target = u * total), finds the tile in which the running sum crosses
-//           the target, and one warp evaluates r'(t) of that single tile id by id
-//           and scans inside it. Without residual mass it draws from p_j (it then
-//           redoes the tile sums with e alone).
-// A lane adds its eight values in fp32 in index order and a tile's value is the
-// fp32 warp sum of the lanes (fixed shuffle tree); sums and scans across tiles,
-// and the scan inside the chosen tile, are fp64 in a fixed order: the result is
-// reproducible, and the only difference to exact arithmetic is the fp32 rounding
-// of the terms and of the tile sums.
+//           128-bit load of the logits per lane, the drafter's probabilities of the ids
+//           that have one, r' of its eight ids (with the two ids Eq. (2) singles out) and
+//           a warp sum: the tile's value;
+//   pass 2  the running sum over the tile values passes the target = u * total in one
+//           tile, and one warp evaluates r'(t) of that single tile id by id and scans
+//           inside it. Without residual mass the draw is from p_j (the tile values are
+//           redone with e alone).
+//
+// Where pass 1 has the drafter's probabilities from (they lie in draft-id order):
+//   same tokenizer on both sides: the row itself, two 128-bit loads per lane and tile
+//           (FROM_ROW; 256 rows of 32000 ids: step 44.2 -> 40.1 us);
+//   else    shared memory, in target-id order (STAGED): a block gathers the mapped ids of
+//           its tiles once, from a list in DRAFT-id order (od_sample_plan), so that the 32
+//           lanes of a load sit within a few lines, and finds them in pass 1 by counting
+//           mapped ids. Gathered tile by tile through the inverse map instead, every mapped
+//           id costs a 32-byte sector and every id four bytes of the map, from L2: 834 MB
+//           for 512 rows of 152064 ids, the rate of L2 (9.3 TB/s) for 75 us;
+//   else    (more mapped ids in a part of the row than shared memory holds, and the
+//           vocabulary shards) the inverse map and a gather (FROM_MAP), the map's entries
+//           of the next pair of tiles requested before the gathers of the current one.
+//
+// A lane adds its eight values in fp32 and a tile's value is the fp32 warp sum of the
+// lanes (fixed trees); sums and scans across tiles, and the scan inside the chosen
+// tile, are fp64 in a fixed order: the result is reproducible, and the only difference
+// to exact arithmetic is the fp32 rounding of the terms and of the tile sums.
 //
 // Vocabulary shards (the rows split by columns over several GPUs) use the same
 // kernel in two further modes. A shard owns a window of whole tiles:
@@ -77,6 +80,10 @@ struct SampleArgs {
     const uint64_t *seed;
     uint64_t step;
     const int32_t *vocab_map, *inv_map;
+    // the context's lists for this launch's number of parts (od_sample_lists)
+    const uint32_t *list_word, *octet;
+    const int32_t *list_base, *list_part;
+    int32_t part_tiles, slots;          // tiles of a part; room for staged probabilities
     int32_t same_ids;                   // 1: target id t is draft id t (t < v_q), and the drafter's rows are 16-byte aligned
     int32_t *out_token;
     float *resid_mass;
@@ -103,7 +110,8 @@ struct SampleArgs {
 struct SeqState {
     const char *row;
     const float *q_row;
-    float c, S, scale;      // e(t) = exp2(fma(x_t, scale, -c)); S is the row sum relative to c
+    float c, S, scale;      // e(t) = exp2(fma(x_t, scale, -c)) < 1; S is the row sum relative to c
+    float margin;           // c - fl(M*scale)
     bool residual;
     int32_t ngram_token, prefix_token, first_draft;
     float ngram_prob, prefix_val;
@@ -151,10 +159,30 @@ __device__ __forceinline__ void same_id_probs(const SeqState &q, const SampleArg
     qq[4] = v1.x; qq[5] = v1.y; qq[6] = v1.z; qq[7] = v1.w;
 }
 
+// Where the drafter's probabilities of a tile come from: the inverse map and the row in global
+// memory, the row alone (target ids are draft ids), or, for the tiles of this block's part, shared
+// memory, in target-id order.
+enum { FROM_MAP, FROM_ROW, STAGED, FREE };
+struct StagedRow {
+    const float *q;                     // [mapped ids of the part]
+    const uint32_t *octet;
+    uint32_t rank0;                     // the part's first rank
+};
+__device__ __forceinline__ void staged_probs(const StagedRow &sr, uint32_t oct, float *qq)
+{
+    uint32_t i = (oct >> 8) - sr.rank0;
+#pragma unroll
+    for (int e = 0; e < EPT; ++e) {
+        const uint32_t has = oct >> e & 1u;
+        qq[e] = has ? sr.q[i] : 0.f;
+        i += has;
+    }
+}
+
 // r'(t) of the EPT consecutive ids this lane owns in `tile`; ids >= v_p give 0
 template <int DTYPE>
 __device__ __forceinline__ void tile_values(const SeqState &q, const SampleArgs &a, bool residual,
-                                            int tile, int lane, float *r)
+                                            int tile, int lane, float *r, const StagedRow *sr = nullptr)
 {
     const int t0 = tile * OD_SAMPLE_TILE + lane * EPT;
     if (t0 + EPT <= a.v_p) {
@@ -173,6 +201,8 @@ __device__ __forceinline__ void tile_values(const SeqState &q, const SampleArgs 
             float qq[EPT];
             if (a.same_ids) {
                 same_id_probs(q, a, t0, qq);
+            } else if (sr) {
+                staged_probs(*sr, __ldg(sr->octet + (t0 >> 3)), qq);
             } else {
                 const int4 i0 = __ldg((const int4 *)(a.inv_map + t0));
                 const int4 i1 = __ldg((const int4 *)(a.inv_map + t0) + 1);
@@ -250,12 +280,45 @@ __device__ __forceinline__ float warp_sum_f32(float v)
     return v;
 }
 
+// Where a warp's tile values go. one(): every lane holds the tile's value; pair(): lanes 0..15
+// hold tile t's, lanes 16..31 tile t + 1's (if `two`).
+struct GlobalTiles {                                        // [ntiles] of one sequence
+    double *val;
+    int lane;
+    __device__ __forceinline__ void one(int t, float v) { if (lane == 0) val[t] = (double)v; }
+    __device__ __forceinline__ void pair(int t, float v, bool two)
+    {
+        if ((lane & 15) == 0 && (lane == 0 || two)) val[t + (lane >> 4)] = (double)v;
+    }
+};
+struct WarpTiles {                                          // the warp's own run in shared memory, and its sum
+    float *val;
+    int lane, t_lo;
+    double total;                                           // lanes 0..15 and 16..31 each hold a share
+    __device__ __forceinline__ void one(int t, float v)
+    {
+        v = fmaxf(0.f, v);                                  // (a tile with NaN has no mass)
+        if (lane == 0) val[t - t_lo] = v;
+        if (lane < 16) total += (double)v;
+    }
+    __device__ __forceinline__ void pair(int t, float v, bool two)
+    {
+        v = lane < 16 || two ? fmaxf(0.f, v) : 0.f;
+        if ((lane & 15) == 0 && (lane == 0 || two)) val[t - t_lo + (lane >> 4)] = v;
+        total += (double)v;
+    }
+    __device__ __forceinline__ double sum() const
+    {
+        return __shfl_sync(0xFFFFFFFFu, total, 0) + __shfl_sync(0xFFFFFFFFu, total, 16);
+    }
+};
+
 // Pass 1, tile by tile (the free token, ragged last tiles, and the fallback of pass 2): every
 // id of a tile looks up its draft id in the inverse map (coalesced) and gathers the drafter's
 // probability if it has one; NT tiles are in flight per warp.
-template <int DTYPE, int NT>
+template <int DTYPE, int NT, typename Sink>
 __device__ __forceinline__ void warp_tiles_dense(const SeqState &q, const SampleArgs &a, bool residual, int t_lo,
-                                                 int t_hi, int lane, double *tile_val)
+                                                 int t_hi, int lane, Sink &out)
 {
     for (int t = t_lo; t < t_hi; t += NT) {
         float r[NT][EPT];
@@ -266,18 +329,15 @@ __device__ __forceinline__ void warp_tiles_dense(const SeqState &q, const Sample
                 else tile_e_values<DTYPE>(q, a, t + i, lane, r[i]);
             }
         }
-        float mine = 0.f;
 #pragma unroll
         for (int i = 0; i < NT; ++i) {
             if (t + i < t_hi) {
                 float s = r[i][0];
 #pragma unroll
                 for (int e = 1; e < EPT; ++e) s += r[i][e];
-                s = warp_sum_f32(s);
-                if (lane == i) mine = s;
+                out.one(t + i, warp_sum_f32(s));
             }
         }
-        if (lane < NT && t + lane < t_hi) tile_val[t + lane] = (double)mine;
     }
 }
 
@@ -291,11 +351,21 @@ __device__ __forceinline__ void load_tile(const SeqState &q, int tile, int lane,
     raw[0] = ld_once(src);
     if (DTYPE != OD_BF16) raw[1] = ld_once(src + 1);
 }
-template <int DTYPE>
-__device__ __forceinline__ float tile_sum(const SeqState &q, const SampleArgs &a, int tile, int lane, const uint4 *raw,
-                                          const float *qq)
+// A lane's eight ids of a whole tile: the sum of their residuals, or of e alone. A tile is 256
+// ids of work for one warp, and its instructions bound a large batch: 276 a tile and 66.8 us for
+// 296 staged rows of 152064 ids with a branch per id, 195 and 51.9 us with a select per id, 156
+// and 45.7 us so: the clamp at zero is part of the multiply-add, an unmapped id's multiply-add
+// is predicated off, and Eq. (2)'s two ids are looked for only in the tiles that hold them.
+__device__ __forceinline__ float fma_sat(float a, float b, float c)
 {
-    float x[EPT], r[EPT];
+    float d;
+    asm("fma.rn.sat.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
+    return d;
+}
+template <int DTYPE>
+__device__ __forceinline__ void tile_e(const SeqState &q, const uint4 *raw, float *e)
+{
+    float x[EPT];
     if (DTYPE == OD_BF16) {
         const uint4 v = raw[0];
         x[0] = od_bf16_lo(v.x); x[1] = od_bf16_hi(v.x); x[2] = od_bf16_lo(v.y); x[3] = od_bf16_hi(v.y);
@@ -305,13 +375,65 @@ __device__ __forceinline__ float tile_sum(const SeqState &q, const SampleArgs &a
         x[0] = __uint_as_float(v0.x); x[1] = __uint_as_float(v0.y); x[2] = __uint_as_float(v0.z); x[3] = __uint_as_float(v0.w);
         x[4] = __uint_as_float(v1.x); x[5] = __uint_as_float(v1.y); x[6] = __uint_as_float(v1.z); x[7] = __uint_as_float(v1.w);
     }
+    const uint64_t scale2 = f2_pack(q.scale, q.scale), nc2 = f2_pack(-q.c, -q.c);
 #pragma unroll
-    for (int e = 0; e < EPT; ++e) r[e] = resid_of(q, x[e], qq[e]);
-    eq2_ids<DTYPE>(q, a, tile * OD_SAMPLE_TILE + lane * EPT, r);
-    float sum = r[0];
+    for (int k = 0; k < EPT; k += 2) {
+        f2_unpack(f2_fma(f2_pack(x[k], x[k + 1]), scale2, nc2), e[k], e[k + 1]);
+        e[k] = od_ex2(e[k]); e[k + 1] = od_ex2(e[k + 1]);
+    }
+}
+__device__ __forceinline__ float sum_of_eight(const float *r)
+{
+    float s0, s1;
+    f2_unpack(f2_add(f2_add(f2_pack(r[0], r[1]), f2_pack(r[2], r[3])), f2_add(f2_pack(r[4], r[5]), f2_pack(r[6], r[7]))), s0, s1);
+    return s0 + s1;
+}
+template <int DTYPE>
+__device__ __forceinline__ float with_eq2_ids(const SeqState &q, const SampleArgs &a, int tile, int lane, float *r)
+{
+    if (tile == q.prefix_token / OD_SAMPLE_TILE || tile == q.ngram_token / OD_SAMPLE_TILE)
+        eq2_ids<DTYPE>(q, a, tile * OD_SAMPLE_TILE + lane * EPT, r);
+    return sum_of_eight(r);
+}
+template <int DTYPE>
+__device__ __forceinline__ float tile_lane_sum(const SeqState &q, const SampleArgs &a, int tile, int lane, const uint4 *raw,
+                                               const float *qq)
+{
+    float r[EPT];
+    tile_e<DTYPE>(q, raw, r);
 #pragma unroll
-    for (int e = 1; e < EPT; ++e) sum += r[e];
-    return warp_sum_f32(sum);
+    for (int k = 0; k < EPT; ++k) r[k] = fma_sat(qq[k], -q.S, r[k]);
+    return with_eq2_ids<DTYPE>(q, a, tile, lane, r);
+}
+// the same with the probabilities in shared memory at `rank_at` (the address of the lane's first
+// mapped id's; `oct` says which of the eight are mapped)
+template <int DTYPE>
+__device__ __forceinline__ float tile_lane_sum_staged(const SeqState &q, const SampleArgs &a, int tile, int lane, const uint4 *raw,
+                                                      uint32_t oct, uint32_t rank_at)
+{
+    float r[EPT];
+    tile_e<DTYPE>(q, raw, r);
+    const float nS = -q.S;
+#pragma unroll
+    for (int k = 0; k < EPT; ++k)
+        // (read for every id, mapped or not: the last rank has a word behind it)
+        asm("{.reg .pred p; .reg .b32 t; .reg .f32 v;\n\t"
+            "and.b32 t, %3, %4; setp.ne.u32 p, t, 0;\n\t"
+            "ld.shared.f32 v, [%1];\n\t"
+            "@p fma.rn.sat.f32 %0, v, %2, %0;\n\t"
+            "@p add.u32 %1, %1, 4;}"
+            : "+f"(r[k]), "+r"(rank_at) : "f"(nS), "r"(oct), "r"(1u << k) : "memory");
+    return with_eq2_ids<DTYPE>(q, a, tile, lane, r);
+}
+
+// The lanes' sums of two tiles: lanes 0..15 end with the first tile's value, lanes 16..31 with the second's.
+__device__ __forceinline__ float pair_sum(float s0, float s1, int lane)
+{
+    const bool up = lane & 16;
+    float v = (up ? s1 : s0) + __shfl_xor_sync(0xFFFFFFFFu, up ? s0 : s1, 16);
+#pragma unroll
+    for (int off = 8; off > 0; off >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, off);
+    return v;
 }
 
 // Inverse-map entries of a warp's first pair of whole tiles [t_lo, t_hi).
@@ -330,9 +452,9 @@ __device__ __forceinline__ void first_pair_entries(const SampleArgs &a, int t_lo
 // so a pair costs one memory round trip, not two. ni: the first pair's entries
 // (first_pair_entries), which the caller requested early: they belong to the context and
 // depend on nothing the launch in front writes.
-template <int DTYPE>
+template <int DTYPE, typename Sink>
 __device__ __forceinline__ void warp_tiles_dense_piped(const SeqState &q, const SampleArgs &a, int t_lo, int t_hi,
-                                                       int lane, double *tile_val, int4 (&ni)[2][2])
+                                                       int lane, Sink &out, int4 (&ni)[2][2])
 {
     for (int t = t_lo; t < t_hi; t += 2) {
         int32_t d[2][EPT];
@@ -359,40 +481,78 @@ __device__ __forceinline__ void warp_tiles_dense_piped(const SeqState &q, const 
 #pragma unroll
             for (int e = 0; e < EPT; ++e) qq[i][e] = d[i][e] >= 0 ? __ldg(q.q_row + d[i][e]) : 0.f;
         }
-        float mine = 0.f;
-#pragma unroll
-        for (int i = 0; i < 2; ++i) {
-            const float sum = tile_sum<DTYPE>(q, a, t + i, lane, raw[i], qq[i]);
-            if (lane == i) mine = sum;
-        }
-        if (lane < 2 && t + lane < t_hi) tile_val[t + lane] = (double)mine;
+        const float s0 = tile_lane_sum<DTYPE>(q, a, t, lane, raw[0], qq[0]);
+        const float s1 = tile_lane_sum<DTYPE>(q, a, t + 1, lane, raw[1], qq[1]);
+        out.pair(t, pair_sum(s0, s1, lane), two);
     }
 }
 
-// The same for target ids that are draft ids: independent 16-byte loads only, the next tile's
-// requested before the current one is worked on.
-template <int DTYPE>
-__device__ __forceinline__ void warp_tiles_same_ids(const SeqState &q, const SampleArgs &a, int t_lo, int t_hi, int lane,
-                                                    double *tile_val)
-{
+// A whole tile's loads other than through the inverse map: the logits, and
+//   FROM_ROW  the drafter's probabilities where target ids are draft ids
+//   STAGED    which of the ids are mapped, and the rank of the first
+//   FREE      nothing else (the free token is drawn from p itself)
+template <int DTYPE, int SOURCE>
+struct TileLoads {
     uint4 raw[RAW<DTYPE>];
-    float qq[EPT];
-    load_tile<DTYPE>(q, t_lo, lane, raw);
-    same_id_probs(q, a, t_lo * OD_SAMPLE_TILE + lane * EPT, qq);
-#pragma unroll 1
-    for (int t = t_lo; t < t_hi; ++t) {
-        uint4 nraw[RAW<DTYPE>];
-        float nqq[EPT];
-        const int n = t + 1 < t_hi ? t + 1 : t;
-        load_tile<DTYPE>(q, n, lane, nraw);
-        same_id_probs(q, a, n * OD_SAMPLE_TILE + lane * EPT, nqq);
-        const float sum = tile_sum<DTYPE>(q, a, t, lane, raw, qq);
-        if (lane == 0) tile_val[t] = (double)sum;
-#pragma unroll
-        for (int k = 0; k < RAW<DTYPE>; ++k) raw[k] = nraw[k];
-#pragma unroll
-        for (int e = 0; e < EPT; ++e) qq[e] = nqq[e];
+    float qq[SOURCE == FROM_ROW ? EPT : 1];
+    uint32_t oct;
+    __device__ __forceinline__ void load(const SeqState &q, const SampleArgs &a, int tile, int lane)
+    {
+        load_tile<DTYPE>(q, tile, lane, raw);
+        if (SOURCE == FROM_ROW) same_id_probs(q, a, tile * OD_SAMPLE_TILE + lane * EPT, qq);
+        if (SOURCE == STAGED) oct = __ldg(a.octet + tile * (OD_SAMPLE_TILE / 8) + lane);
     }
+    __device__ __forceinline__ float sum(const SeqState &q, const SampleArgs &a, const StagedRow &sr, int tile, int lane) const
+    {
+        if (SOURCE == STAGED)
+            return tile_lane_sum_staged<DTYPE>(q, a, tile, lane, raw, oct,
+                                               (uint32_t)__cvta_generic_to_shared(sr.q) + ((oct >> 8) - sr.rank0) * 4u);
+        if (SOURCE == FREE) {
+            float e[EPT];
+            tile_e<DTYPE>(q, raw, e);
+            return sum_of_eight(e);
+        }
+        return tile_lane_sum<DTYPE>(q, a, tile, lane, raw, qq);
+    }
+};
+
+// Pass 1 over whole tiles [t_lo, t_hi) without the inverse map: the loads of the next tiles are
+// issued before the current ones are worked on. cur: the first two tiles', which the caller
+// requested (FROM_ROW keeps one tile ahead only, for its registers).
+template <int DTYPE, int SOURCE, typename Sink>
+__device__ __forceinline__ void warp_tiles_ahead(const SeqState &q, const SampleArgs &a, const StagedRow &sr, int t_lo, int t_hi,
+                                                 int lane, Sink &out, TileLoads<DTYPE, SOURCE> (&cur)[SOURCE == FROM_ROW ? 1 : 2])
+{
+#pragma unroll 1
+    for (int t = t_lo; t < t_hi; t += 2) {
+        const bool two = t + 1 < t_hi;
+        float s0, s1;
+        if (SOURCE == FROM_ROW) {
+            TileLoads<DTYPE, SOURCE> nx;
+            nx.load(q, a, two ? t + 1 : t, lane);
+            s0 = cur[0].sum(q, a, sr, t, lane);
+            if (t + 2 < t_hi) cur[0].load(q, a, t + 2, lane);
+            s1 = nx.sum(q, a, sr, t + 1, lane);
+        } else {
+            TileLoads<DTYPE, SOURCE> nx[2];
+            if (t + 2 < t_hi) {
+                nx[0].load(q, a, t + 2, lane);
+                nx[1].load(q, a, min(t + 3, t_hi - 1), lane);
+            }
+            s0 = cur[0].sum(q, a, sr, t, lane);
+            s1 = cur[SOURCE == FROM_ROW ? 0 : 1].sum(q, a, sr, t + 1, lane);
+            cur[0] = nx[0]; cur[SOURCE == FROM_ROW ? 0 : 1] = nx[1];
+        }
+        out.pair(t, pair_sum(s0, s1, lane), two);
+    }
+}
+template <int DTYPE, int SOURCE>
+__device__ __forceinline__ void first_tiles(const SeqState &q, const SampleArgs &a, int t_lo, int t_hi, int lane,
+                                            TileLoads<DTYPE, SOURCE> (&cur)[SOURCE == FROM_ROW ? 1 : 2])
+{
+    if (t_lo >= t_hi) return;
+    cur[0].load(q, a, t_lo, lane);
+    if (SOURCE != FROM_ROW) cur[SOURCE == FROM_ROW ? 0 : 1].load(q, a, min(t_lo + 1, t_hi - 1), lane);
 }
 
 // Sum of s_val[my_lo, my_hi) over the block's threads in the order of the scan of
@@ -415,84 +575,307 @@ __device__ __forceinline__ double block_total(const double *s_val, int my_lo, in
     return tot;
 }
 
-// MODE 0: the whole step on full rows; 1: a shard's mass shares; 2: a shard's pick.
-// FUSED (mode 0 only): the launch in front is the streaming pass of od_verify itself; its
-// decide kernel is folded into this kernel's prologue (see SampleArgs).
-template <int DTYPE, int MODE, bool FUSED>
-__global__ void __launch_bounds__(OD_SAMPLE_THREADS, 4)
-od_sample_kernel(const SampleArgs a)
+// ---- what both kernels prepare and decide alike -------------------------------------------
+
+// What a block can load before the verification kernels have finished: what the translation
+// kernel wrote, for every position the step can stop at. Lane k of every warp prepares
+// position k. Two memory round trips, not a chain of four: everything that is addressed by
+// (b, lane) alone is requested at once, whether or not it will be used (lane < K keeps the
+// addresses inside the arrays); what is addressed by those values comes second.
+struct Ahead {
+    int mb;
+    bool stop;
+    float T;
+    int32_t l_len, l_tgt;               // piece `lane`: its length, target id
+    float l_qp;                         // and q'
+    int32_t s0, len, tgt, d1, pm;       // position `lane`: row of the drafter, length of the piece there (1 at a stop);
+    float qp, qd1;                      // of a merged piece: target, q', first sub-token, its image and probability
+};
+__device__ __forceinline__ Ahead load_ahead(const SampleArgs &a, int b, int lane)
 {
-    __shared__ float s_M[FUSED ? OD_MAX_K + 1 : 1], s_S[FUSED ? OD_MAX_K + 1 : 1];
-    __shared__ int s_red[2][WARPS];
-    __shared__ unsigned int s_vbits;
-    extern __shared__ __align__(16) unsigned char s_dyn[];   // ntiles x 8 bytes
-    double *s_val = (double *)s_dyn;                         // pass 2: tile values
-    __shared__ double s_warp[WARPS];
-    __shared__ unsigned int s_last;
-    __shared__ int s_tile, s_lastmass, s_token;
-    __shared__ double s_before, s_total;
-    __shared__ double s_cross[OD_SAMPLE_THREADS];           // pass 2: the sum in front of a thread's crossing tile
-
-    // grid = (sequences, parts of a row): blocks with neighbouring indices, which often end up on
-    // one multiprocessor, then work on the same tiles of different sequences and share the
-    // inverse-map entries in L1
-    const int b = blockIdx.x;
-    const unsigned int part = blockIdx.y, nparts = gridDim.y;
     const int K = a.K_max;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-
-    // Under programmatic dependent launch this grid is resident while the verification
-    // kernels still run. What the translation kernel wrote (it finished before them) is
-    // read now, for every position the step can stop at: lane k of every warp prepares
-    // position k. After the wait only n_accepted and the row statistics are missing.
-    // (a.early = 0: the launch before this one was not od_verify; everything waits.)
-    asm volatile("griddepcontrol.launch_dependents;");
-    if (!a.early) asm volatile("griddepcontrol.wait;" ::: "memory");
-    // Two memory round trips, not a chain of four: everything that is addressed by (b, lane)
-    // alone is requested at once, whether or not it will be used (lane < K keeps the
-    // addresses inside the arrays); what is addressed by those values comes second.
+    Ahead h;
     int mb = a.m[b];
-    const bool stop = a.tail_kind[b] == OD_TAIL_UNMAPPED_STOP;
-    const float T = a.temperature[b];
-    int32_t l_s0 = 0, l_len = 1, l_tgt = -1, l_did = -1;
-    float l_qp = 0.f;
+    h.stop = a.tail_kind[b] == OD_TAIL_UNMAPPED_STOP;
+    h.T = a.temperature[b];
+    int32_t l_s0 = 0, l_did = -1;
+    h.l_len = 1; h.l_tgt = -1; h.l_qp = 0.f;
     if (lane < K) {
         const size_t o = (size_t)b * K + lane;
         l_s0 = a.span_start[o];
-        l_len = a.span_len[o];
-        l_tgt = a.tgt_ids[o];
-        l_qp = a.q_prime[o];
+        h.l_len = a.span_len[o];
+        h.l_tgt = a.tgt_ids[o];
+        h.l_qp = a.q_prime[o];
         l_did = a.draft_ids[o];
     }
-    mb = mb < 0 ? 0 : (mb > K ? K : mb);
-    int32_t e_s0 = 0, e_len = 1, e_tgt = -1, e_d1 = -1, e_pm = -1;
-    float e_qp = 0.f, e_qd1 = 0.f;
-    {
-        const bool live = lane < K && lane <= mb;
-        if (live) {
-            e_s0 = l_s0 < 0 ? 0 : (l_s0 >= K ? K - 1 : l_s0);
-            e_len = lane < mb ? l_len : 1;
+    h.mb = mb < 0 ? 0 : (mb > K ? K : mb);
+    h.s0 = 0; h.len = 1; h.tgt = -1; h.d1 = -1; h.pm = -1; h.qp = 0.f; h.qd1 = 0.f;
+    const bool live = lane < K && lane <= h.mb;
+    if (live) {
+        h.s0 = l_s0 < 0 ? 0 : (l_s0 >= K ? K - 1 : l_s0);
+        h.len = lane < h.mb ? h.l_len : 1;
+    }
+    const int32_t d1 = __shfl_sync(0xFFFFFFFFu, l_did, h.s0);       // the span's first draft token
+    if (live && h.len >= 2) {
+        h.tgt = h.l_tgt;
+        h.qp = h.l_qp;
+        if (d1 >= 0 && d1 < a.v_q) {
+            h.d1 = d1;
+            h.pm = __ldg(a.vocab_map + d1);
+            h.qd1 = __ldg(a.q_rows + ((size_t)b * K + h.s0) * a.v_q + d1);
         }
-        const int32_t d1 = __shfl_sync(0xFFFFFFFFu, l_did, e_s0);   // the span's first draft token
-        if (live && e_len >= 2) {
-            e_tgt = l_tgt;
-            e_qp = l_qp;
-            if (d1 >= 0 && d1 < a.v_q) {
-                e_d1 = d1;
-                e_pm = __ldg(a.vocab_map + d1);
-                e_qd1 = __ldg(a.q_rows + ((size_t)b * K + e_s0) * a.v_q + d1);
+    }
+    return h;
+}
+
+// What the draw at position j needs; rm, rs: lane k holds the statistics of row k. A shard's row
+// pointer is moved back by the shard's first column (col0), and only ids of the window are read.
+template <int DTYPE>
+__device__ __forceinline__ SeqState seq_state(const SampleArgs &a, const Ahead &h, int b, int j, float rm, float rs, int col0)
+{
+    const size_t esz = DTYPE == OD_BF16 ? 2 : 4;
+    SeqState q;
+    q.row = (const char *)a.logits + ((size_t)b * a.seq_stride + (size_t)j * a.row_stride) * esz - (size_t)col0 * esz;
+    q.scale = 1.4426950408889634f / h.T;
+    {
+        // reference exponent c = fl(M*scale); its rounding goes into S exactly:
+        // sum_t exp2(x_t*scale - c) = (sum_t exp2((x_t - M)*scale)) * exp2(M*scale - c)
+        const float M = __shfl_sync(0xFFFFFFFFu, rm, j);
+        // and a margin, so that e(t) stays below one whatever the rounding: r'(t) may then be clamped to
+        // [0, 1] by the multiply-add itself
+        const float c = fmaxf(M * q.scale, -FLT_MAX);
+        q.c = c + fmaxf(1.f, ceilf(fabsf(c) * 1e-6f));
+        q.margin = q.c - c;
+        q.S = __shfl_sync(0xFFFFFFFFu, rs, j) * od_ex2(fmaf(M, q.scale, -q.c));
+    }
+    q.residual = (j < h.mb) || h.stop;
+    q.ngram_token = -1; q.prefix_token = -1; q.first_draft = -1; q.ngram_prob = 0.f; q.prefix_val = 0.f;
+    q.q_row = a.q_rows;
+    // position j's preparation (j < K whenever the draw is a residual one)
+    const int src = j < a.K_max ? j : 0;
+    const int32_t s0 = __shfl_sync(0xFFFFFFFFu, h.s0, src), len = __shfl_sync(0xFFFFFFFFu, h.len, src);
+    const int32_t tgt = __shfl_sync(0xFFFFFFFFu, h.tgt, src), d1 = __shfl_sync(0xFFFFFFFFu, h.d1, src);
+    const int32_t pm = __shfl_sync(0xFFFFFFFFu, h.pm, src);
+    const float qp = __shfl_sync(0xFFFFFFFFu, h.qp, src), qd1 = __shfl_sync(0xFFFFFFFFu, h.qd1, src);
+    if (q.residual) {
+        q.q_row = a.q_rows + ((size_t)b * a.K_max + s0) * a.v_q;
+        if (len >= 2) {
+            q.ngram_token = tgt;
+            q.ngram_prob = qp;
+            if (d1 >= 0) {
+                q.first_draft = d1;
+                q.prefix_token = pm;
+                q.prefix_val = qd1 - q.ngram_prob;
             }
         }
     }
+    return q;
+}
+
+// The gathers of pass 1 come two round trips from now: have the copy engine pull this block's
+// share of the drafter's row into L2 meanwhile (one thread calls).
+__device__ __forceinline__ void prefetch_q_row(const SampleArgs &a, const SeqState &q, unsigned part, unsigned nparts)
+{
+    const size_t row_bytes = (size_t)a.v_q * 4 / 16 * 16;
+    const size_t lo = (row_bytes / nparts * part) / 16 * 16;
+    const size_t hi = part + 1 == nparts ? row_bytes : (row_bytes / nparts * (part + 1)) / 16 * 16;
+    const char *base = (const char *)q.q_row;
+    if (((uintptr_t)base & 15u) == 0 && hi > lo)
+        asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(base + lo), "r"((uint32_t)(hi - lo)) : "memory");
+}
+
+// A warp's run of tiles [t_lo, t_hi): whole tiles pipelined, the row's ragged last tile (if it is
+// this warp's) on its own. ni: the first pair's inverse-map entries (not read where ids are shared).
+template <int DTYPE, int SOURCE, typename Sink>
+__device__ __forceinline__ void warp_run(const SeqState &q, const SampleArgs &a, int t_lo, int t_hi, int hi_w, int lane,
+                                         Sink &out, int4 (&ni)[2][2])
+{
+    const StagedRow none = {};
+    if (t_lo >= t_hi) return;
+    if (!q.residual) {
+        TileLoads<DTYPE, FREE> cur[2];
+        first_tiles<DTYPE, FREE>(q, a, t_lo, hi_w, lane, cur);
+        warp_tiles_ahead<DTYPE, FREE>(q, a, none, t_lo, hi_w, lane, out, cur);
+    } else if (SOURCE == FROM_ROW) {
+        TileLoads<DTYPE, FROM_ROW> cur[1];
+        first_tiles<DTYPE, FROM_ROW>(q, a, t_lo, hi_w, lane, cur);
+        warp_tiles_ahead<DTYPE, FROM_ROW>(q, a, none, t_lo, hi_w, lane, out, cur);
+    } else if (SOURCE == FROM_MAP && t_lo < hi_w) {
+        warp_tiles_dense_piped<DTYPE>(q, a, t_lo, hi_w, lane, out, ni);
+    }
+    if (hi_w < t_hi) warp_tiles_dense<DTYPE, 1>(q, a, q.residual, max(hi_w, t_lo), t_hi, lane, out);
+}
+
+// One warp draws inside tile t_pick, whose ids begin at the running sum `before`: id by id, the
+// first at which the sum passes `target` (or the tile's last one with mass, where rounding put the
+// target past its end). Writes the outputs; false if the tile holds no mass after all.
+template <int DTYPE>
+__device__ __forceinline__ bool pick_in_tile(const SeqState &q, const SampleArgs &a, int b, bool residual, int t_pick,
+                                             double before, double target, double Rn, uint32_t flags, int lane,
+                                             const StagedRow *sr = nullptr)
+{
+    float r[EPT];
+    if (residual) tile_values<DTYPE>(q, a, true, t_pick, lane, r, sr);
+    else tile_e_values<DTYPE>(q, a, t_pick, lane, r);
+    const double mine = lane_sum(r);
+    double incl = mine;
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+        const double v = __shfl_up_sync(0xFFFFFFFFu, incl, off);
+        if (lane >= off) incl += v;
+    }
+    const double lbase = before + (incl - mine);            // sum before this lane's first id
+    const int t0 = t_pick * OD_SAMPLE_TILE + lane * EPT;
+    int my_pick = 0x7FFFFFFF, my_last = -1;
+    double lo = 0.0, hi = 0.0, c = lbase;
+    float run = 0.f;                                        // same fp32 order as lane_sum
+#pragma unroll
+    for (int e = 0; e < EPT; ++e) {
+        run = e == 0 ? r[0] : run + r[e];
+        const double nc = lbase + (double)run;
+        if (r[e] > 0.f) my_last = t0 + e;
+        if (my_pick == 0x7FFFFFFF && nc > target) { my_pick = t0 + e; lo = c; hi = nc; }
+        c = nc;
+    }
+    int pick = my_pick, last = my_last;
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) {
+        pick = min(pick, __shfl_xor_sync(0xFFFFFFFFu, pick, off));
+        last = max(last, __shfl_xor_sync(0xFFFFFFFFu, last, off));
+    }
+    const float R = (float)(Rn / (double)q.S);              // residual mass (1 for the free token)
+    if (pick != 0x7FFFFFFF) {
+        if (my_pick == pick) {                              // exactly one lane owns the picked id
+            uint32_t f = flags;
+            if (fmin(target - lo, hi - target) <= OD_TAU_SAMPLE * Rn) f |= OD_SF_BOUNDARY;
+            a.out_token[b] = pick; a.resid_mass[b] = R; a.flags[b] = f;
+        }
+        return true;
+    }
+    if (last >= 0) {
+        // rounding: the target lies beyond the tile's last edge
+        if (lane == 0) { a.out_token[b] = last; a.resid_mass[b] = R; a.flags[b] = flags | OD_SF_BOUNDARY; }
+        return true;
+    }
+    return false;
+}
+
+// ---- the whole step on full rows -------------------------------------------------------------
+//
+// Grid (P, B), clusters of P blocks of 16 warps: one cluster draws for one sequence. Pass 1 as
+// above, the tile values of a warp's run staying in its block's shared memory. A block sends its
+// sum to all blocks of the cluster (distributed shared memory), and behind ONE cluster barrier
+// every warp has the blocks' sums and its own block's runs, scans both and knows whether the draw
+// falls into its run: that warp, alone and without a further barrier, finds the tile and the id.
+// Stamps, last tile done -> token: 2.6 us, of which the exchange is 1.0 and the picked tile 1.0
+// (4.5 us for blocks of 8 warps that hand over through a ticket, reload the tile values and scan
+// them block-wide; 3.2 with all P * 16 run sums exchanged and scanned by every warp).
+// The whole step, device time: one sequence of 32000 fp32 ids 13.3 -> 12.0 us, 24 of 128256 bf16
+// ids 24.2 -> 22.6, 64 31.7 -> 29.7, 512 of 152064 286 -> 273, 256 of 32000 (same tokenizer) 44.2 -> 37.0.
+// FUSED: the launch in front is the streaming pass of od_verify itself; its decide kernel is
+// folded into this kernel's prologue (see SampleArgs).
+constexpr int CWARPS = 16, CTHREADS = CWARPS * 32;
+
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_arrive_relaxed() { asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+// v to the shared-memory address of `p` in block `rank` of the cluster
+__device__ __forceinline__ void cluster_store(double *p, uint32_t rank, double v)
+{
+    uint32_t at;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(at) : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(rank));
+    asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(at), "d"(v) : "memory");
+}
+
+// No usable residual mass (rare): one block draws from p_j. Redoes the row's tile values with e
+// alone, in global memory, and walks them.
+template <int DTYPE>
+__device__ __forceinline__ void draw_from_p(const SeqState &q, const SampleArgs &a, int b, float u, uint32_t flags)
+{
+    __shared__ double s_sum[CTHREADS];
+    __shared__ int s_crossing, s_lastmass, s_done;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    GlobalTiles out = {a.tile_val + (size_t)b * a.ntiles, lane};
+    for (int t = warp * 2; t < a.ntiles; t += CWARPS * 2)
+        warp_tiles_dense<DTYPE, 2>(q, a, false, t, t + 2 < a.ntiles ? t + 2 : a.ntiles, lane, out);
+    if (threadIdx.x == 0) { s_crossing = 0x7FFFFFFF; s_lastmass = -1; s_done = 0; }
+    __syncthreads();
+    const int per = (a.ntiles + CTHREADS - 1) / CTHREADS;
+    const int lo = min((int)threadIdx.x * per, a.ntiles), hi = min(lo + per, a.ntiles);
+    double loc = 0.0;
+    for (int t = lo; t < hi; ++t) loc += fmax(0.0, out.val[t]);
+    s_sum[threadIdx.x] = loc;
+    __syncthreads();
+    double before = 0.0, tot = 0.0;
+    for (int i = 0; i < CTHREADS; ++i) {
+        if (i == (int)threadIdx.x) before = tot;
+        tot += s_sum[i];
+    }
+    const double target = (double)u * tot;
+    int mine = -1, last = -1;
+    double c = before, at = 0.0;
+    for (int t = lo; t < hi; ++t) {
+        const double v = fmax(0.0, out.val[t]);
+        if (v > 0.0) last = t;
+        if (mine < 0 && c + v > target) { mine = t; at = c; }
+        c += v;
+    }
+    if (tot > 0.0) {
+        if (mine >= 0) atomicMin(&s_crossing, mine);
+        if (last >= 0) atomicMax(&s_lastmass, last);
+    }
+    __syncthreads();
+    const int t_pick = s_crossing != 0x7FFFFFFF ? s_crossing : s_lastmass;
+    if (t_pick >= 0 && t_pick == mine) s_sum[0] = at;
+    else if (t_pick >= lo && t_pick < hi) {                 // rounding hid the crossing: the last tile with mass
+        c = before;
+        for (int t = lo; t < t_pick; ++t) c += fmax(0.0, out.val[t]);
+        s_sum[0] = c;
+    }
+    __syncthreads();
+    if (warp == 0 && t_pick >= 0 && pick_in_tile<DTYPE>(q, a, b, false, t_pick, s_sum[0], target, tot, flags, lane) && lane == 0)
+        s_done = 1;
+    __syncthreads();
+    if (threadIdx.x == 0 && !s_done) {                      // no mass at all (non-finite input)
+        a.out_token[b] = -1;
+        a.resid_mass[b] = (float)(tot / (double)q.S);
+        a.flags[b] = flags;
+    }
+}
+
+template <int DTYPE, bool FUSED, int SOURCE>
+__global__ void __launch_bounds__(CTHREADS, 2)
+od_sample_kernel(const SampleArgs a)
+{
+    __shared__ float s_M[FUSED ? OD_MAX_K + 1 : 1], s_S[FUSED ? OD_MAX_K + 1 : 1];
+    __shared__ int s_red[2][CWARPS];
+    __shared__ unsigned int s_vbits;
+    __shared__ int s_bare;
+    __shared__ double s_run[CWARPS], s_part[OD_SAMPLE_MAX_PARTS];   // sums of the block's runs, of the cluster's blocks
+    extern __shared__ __align__(16) unsigned char s_dyn[];
+    const unsigned part = blockIdx.x, nparts = gridDim.x;
+    const int b = blockIdx.y;
+    const int K = a.K_max;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    // the staged probabilities, then the warps' tile values
+    float *s_q = (float *)s_dyn, *s_val = s_q + (SOURCE == STAGED ? a.slots : 0) + warp * a.tiles_per_warp;
+
+    // Under programmatic dependent launch this grid is resident while the verification
+    // kernels still run. What the translation kernel wrote (it finished before them) is
+    // read now. (a.early = 0: the launch before this one was not od_verify; everything waits.)
+    asm volatile("griddepcontrol.launch_dependents;");
+    if (!a.early) asm volatile("griddepcontrol.wait;" ::: "memory");
+    const Ahead h = load_ahead(a, b, lane);
+    const int mb = h.mb;
 
     // FUSED, still before the wait: where the rows' partials will be (sums of m), and position
     // k's inputs of the acceptance test in lane k
     int before = 0, total = 0;
-    float d_xt = 0.f, d_q = 0.f, d_u = 0.f;
+    float d_xt = 0.f, d_u = 0.f;
     bool d_tok = false;
-    int32_t d_span = 0;
+    if (threadIdx.x == 0) { s_vbits = 0; s_bare = 0; }
     if (FUSED) {
-        for (int i = threadIdx.x; i < a.B; i += OD_SAMPLE_THREADS) {
+        for (int i = threadIdx.x; i < a.B; i += CTHREADS) {
             const int v = clamp_m(a.m[i], K);
             total += v;
             if (i < b) before += v;
@@ -503,42 +886,56 @@ od_sample_kernel(const SampleArgs a)
             total += __shfl_xor_sync(0xFFFFFFFFu, total, off);
         }
         if (lane == 0) { s_red[0][warp] = before; s_red[1][warp] = total; }
-        if (threadIdx.x == 0) s_vbits = 0;
         if (lane < mb) {
-            const int32_t t = l_tgt;
-            d_tok = t >= 0 && t < a.v_p;
+            d_tok = h.l_tgt >= 0 && h.l_tgt < a.v_p;
             const char *row_k = (const char *)a.logits +
                                 ((size_t)b * a.seq_stride + (size_t)lane * a.row_stride) * (DTYPE == OD_BF16 ? 2 : 4);
-            if (d_tok) d_xt = od_load_logit<DTYPE>(row_k, t);
-            d_q = l_qp;
+            if (d_tok) d_xt = od_load_logit<DTYPE>(row_k, h.l_tgt);
             d_u = od_uniform(a.seed[b], a.step, (uint32_t)lane, 0u);
-            d_span = l_len;
         }
         __syncthreads();
         before = 0; total = 0;
-        for (int w = 0; w < WARPS; ++w) { before += s_red[0][w]; total += s_red[1][w]; }
+        for (int w = 0; w < CWARPS; ++w) { before += s_red[0][w]; total += s_red[1][w]; }
     }
 
-    // a shard's tiles and ids keep their numbers of the full row
-    const int tile_lo = MODE == 0 ? 0 : a.tile_lo;
-    const int tile_hi = MODE == 0 ? a.ntiles : a.tile_hi;
-    // pass 1's whole tiles of this warp, and the inverse-map entries of their first pair
-    const int p_lo = tile_lo + ((int)part * WARPS + warp) * a.tiles_per_warp;
-    int p_hi = p_lo + a.tiles_per_warp;
-    if (p_hi > tile_hi) p_hi = tile_hi;
-    const int p_hi_w = p_hi < a.v_p / OD_SAMPLE_TILE ? p_hi : a.v_p / OD_SAMPLE_TILE;
+    // pass 1's tiles of this warp, and the inverse-map entries of their first pair
+    int p_hi = min((int)(part + 1) * a.part_tiles, a.ntiles);
+    const int p_lo = min((int)part * a.part_tiles + warp * a.tiles_per_warp, p_hi);
+    p_hi = min(p_lo + a.tiles_per_warp, p_hi);
+    const int p_hi_w = min(p_hi, a.v_p / OD_SAMPLE_TILE);
     int4 ni[2][2] = {};
-    if (MODE != 2 && !a.same_ids && p_lo < p_hi_w) first_pair_entries(a, p_lo, p_hi_w, lane, ni);
+    if (SOURCE == FROM_MAP && p_lo < p_hi_w) first_pair_entries(a, p_lo, p_hi_w, lane, ni);
+    // STAGED: the first entries of the part's list
+    constexpr int EB = 6;                                   // groups per warp and batch
+    uint32_t word[EB];
+    int32_t base[EB];
+    int4 my_part = {};
+    int g_at = 0;
+    auto load_words = [&]() {
+#pragma unroll
+        for (int e = 0; e < EB; ++e) {
+            const bool in = g_at + e * CWARPS < my_part.y;
+            word[e] = in ? __ldg(a.list_word + (size_t)(g_at + e * CWARPS) * 32 + lane) : 0xFFFFu;
+            base[e] = in ? __ldg(a.list_base + g_at + e * CWARPS) : 0;
+        }
+        g_at += EB * CWARPS;
+    };
+    if (SOURCE == STAGED) {
+        my_part = __ldg((const int4 *)a.list_part + part);
+        g_at = my_part.x + warp;
+        load_words();
+    }
 
     // n_accepted and the row statistics come from the verification kernels
     if (a.early) asm volatile("griddepcontrol.wait;" ::: "memory");
 
-    int fused_n = 0;
+    int j = 0;
+    float rm = 0.f, rs = 0.f;                      // lane k: statistics of row k
     if (FUSED) {
         // ---- step 2's decisions (what od_verify_decide_kernel does, same arithmetic, same order)
-        const bool bad_T = !(T > 0.f);
-        const float dscale = bad_T ? 0.f : 1.4426950408889634f / T;
-        for (int r = warp; r <= mb; r += WARPS) {
+        const bool bad_T = !(h.T > 0.f);
+        const float dscale = bad_T ? 0.f : 1.4426950408889634f / h.T;
+        for (int r = warp; r <= mb; r += CWARPS) {
             const int row_slot = b * (K + 1) + r;
             float c, sum, mx;
             merge_row_partials(a.plan, row_slot, row_partial_segments(a.plan, b, r, before, total), lane, c, sum, mx);
@@ -552,33 +949,193 @@ od_sample_kernel(const SampleArgs a)
         __syncthreads();
         // every warp takes the decisions for itself (lane k = position k holds the inputs in
         // every warp): no second barrier; warp 0 of the sequence's first block stores them
-        int n = 0;
-        {
-            bool acc = false, bnd = false;
-            Acceptance d = {};
-            if (lane < mb) {
-                d = accept_position(s_M[lane], s_S[lane], dscale, d_tok, d_xt, d_q, d_u);
-                acc = d.accept; bnd = d.boundary;
-            }
-            const unsigned int accmask = __ballot_sync(0xFFFFFFFFu, acc);
-            while (n < mb && (accmask >> n & 1u)) ++n;
-            if (bad_T) n = 0;
-            if (part == 0 && warp == 0) {
-                if (lane < mb) { a.w_p_sel[(size_t)b * K + lane] = d.p; a.w_ratio[(size_t)b * K + lane] = d.ratio; }
-                const unsigned int bndmask = __ballot_sync(0xFFFFFFFFu, bnd);
-                int nd = lane < n ? d_span : 0;
+        bool acc = false, bnd = false;
+        Acceptance d = {};
+        if (lane <= mb) { rm = s_M[lane]; rs = s_S[lane]; }
+        if (lane < mb) {
+            d = accept_position(rm, rs, dscale, d_tok, d_xt, h.l_qp, d_u);
+            acc = d.accept; bnd = d.boundary;
+        }
+        const unsigned int accmask = __ballot_sync(0xFFFFFFFFu, acc);
+        while (j < mb && (accmask >> j & 1u)) ++j;
+        if (bad_T) j = 0;
+        if (part == 0 && warp == 0) {
+            if (lane < mb) { a.w_p_sel[(size_t)b * K + lane] = d.p; a.w_ratio[(size_t)b * K + lane] = d.ratio; }
+            const unsigned int bndmask = __ballot_sync(0xFFFFFFFFu, bnd);
+            int nd = lane < j ? h.l_len : 0;
 #pragma unroll
-                for (int off = 16; off > 0; off >>= 1) nd += __shfl_xor_sync(0xFFFFFFFFu, nd, off);
-                if (lane == 0) {
-                    uint32_t f = bndmask & OD_VF_BOUNDARY_MASK;
-                    if (s_vbits & 1u) f |= OD_VF_NONFINITE;
-                    if (bad_T) f |= OD_VF_BAD_TEMPERATURE;
-                    a.w_n_accepted[b] = n; a.w_n_draft[b] = nd; a.w_vflags[b] = f;
-                }
+            for (int off = 16; off > 0; off >>= 1) nd += __shfl_xor_sync(0xFFFFFFFFu, nd, off);
+            if (lane == 0) {
+                uint32_t f = bndmask & OD_VF_BOUNDARY_MASK;
+                if (s_vbits & 1u) f |= OD_VF_NONFINITE;
+                if (bad_T) f |= OD_VF_BAD_TEMPERATURE;
+                a.w_n_accepted[b] = j; a.w_n_draft[b] = nd; a.w_vflags[b] = f;
             }
         }
-        fused_n = n;
+    } else {
+        if (lane <= mb) { rm = a.row_max[b * (K + 1) + lane]; rs = a.row_sum[b * (K + 1) + lane]; }
+        j = a.n_accepted[b];
+        j = j < 0 ? 0 : (j > mb ? mb : j);
     }
+    if (!(h.T > 0.f)) {                            // every block of the sequence leaves here
+        if (part == 0 && threadIdx.x == 0) { a.out_token[b] = -1; a.resid_mass[b] = 0.f; a.flags[b] = OD_SF_BAD_TEMPERATURE; }
+        return;
+    }
+    cluster_arrive_relaxed();                      // this block runs: the others may store to it (waited for below)
+    const SeqState q = seq_state<DTYPE>(a, h, b, j, rm, rs, 0);
+    if (SOURCE == FROM_MAP && q.residual && threadIdx.x == 0) prefetch_q_row(a, q, part, nparts);
+
+    // ---- pass 1: the value of every tile ----
+    WarpTiles out = {s_val, lane, p_lo, 0.0};
+    const uint64_t seed_b = a.seed[b];
+    const StagedRow sr = {s_q, a.octet, (uint32_t)my_part.z};
+    if (SOURCE == STAGED && q.residual) {
+        TileLoads<DTYPE, STAGED> cur[2];
+        first_tiles<DTYPE, STAGED>(q, a, p_lo, p_hi_w, lane, cur);
+        // the part's probabilities, gathered in draft-id order, to their ranks in shared memory
+        for (;;) {
+            float x[EB];
+            uint32_t at[EB];
+#pragma unroll
+            for (int e = 0; e < EB; ++e) {
+                at[e] = word[e] & 0xFFFFu;
+                if (at[e] != 0xFFFFu) x[e] = __ldg(q.q_row + base[e] + (int)(word[e] >> 16));
+            }
+            const bool more = g_at < my_part.y;             // the same for every lane of a warp
+            if (more) load_words();
+#pragma unroll
+            for (int e = 0; e < EB; ++e)
+                if (at[e] != 0xFFFFu) s_q[at[e]] = x[e];
+            if (!more) break;
+        }
+        __syncthreads();
+        warp_tiles_ahead<DTYPE, STAGED>(q, a, sr, p_lo, p_hi_w, lane, out, cur);
+        if (p_hi_w < p_hi) warp_tiles_dense<DTYPE, 1>(q, a, true, max(p_hi_w, p_lo), p_hi, lane, out);
+    } else {
+        warp_run<DTYPE, SOURCE>(q, a, p_lo, p_hi, p_hi_w, lane, out, ni);
+    }
+    const float u = od_uniform(seed_b, a.step, (uint32_t)j, 1u);
+
+    // ---- the sums: of the runs inside the block, of the block to every block of the cluster
+    const double run_sum = out.sum();
+    if (lane == 0) s_run[warp] = run_sum;
+    __syncthreads();
+    // every warp holds the block's runs in lanes 0..15 (and again in 16..31), summed up
+    const double mine = s_run[lane & 15];
+    double incl = mine;
+#pragma unroll
+    for (int off = 1; off < CWARPS; off <<= 1) {
+        const double v = __shfl_up_sync(0xFFFFFFFFu, incl, off, CWARPS);
+        if ((lane & 15) >= off) incl += v;
+    }
+    const double block_sum = __shfl_sync(0xFFFFFFFFu, incl, 15);
+    cluster_wait();
+    if (warp == 0 && lane < (int)nparts) cluster_store(&s_part[part], (uint32_t)lane, block_sum);
+    cluster_arrive();
+    cluster_wait();
+
+    // ---- every warp scans the blocks' sums: is the draw in its block, in its run?
+    const uint32_t flags = q.residual ? 0u : OD_SF_BONUS;
+    const double p_sum = (lane & 15) < (int)nparts ? s_part[lane & 15] : 0.0;
+    double p_incl = p_sum;
+#pragma unroll
+    for (int off = 1; off < OD_SAMPLE_MAX_PARTS; off <<= 1) {
+        const double v = __shfl_up_sync(0xFFFFFFFFu, p_incl, off, OD_SAMPLE_MAX_PARTS);
+        if ((lane & 15) >= off) p_incl += v;
+    }
+    const double Rn = __shfl_sync(0xFFFFFFFFu, p_incl, 15);  // unnormalised total
+    bool bare = !(Rn > 0.0);                                 // the same in every warp of the cluster
+    if (!bare) {
+        const double target = (double)u * Rn;
+        // the first block, then its first run, at whose end the sum passes the target; if rounding
+        // hid it, the last with mass
+        const auto first_past = [&](double before, double sum, double upto) {
+            const unsigned past = __ballot_sync(0xFFFFFFFFu, sum > 0.0 && before + upto > target) & 0xFFFFu;
+            const unsigned held = __ballot_sync(0xFFFFFFFFu, sum > 0.0) & 0xFFFFu;
+            return past ? __ffs(past) - 1 : 31 - __clz(held);   // -1: no mass
+        };
+        const int p_hit = first_past(0.0, p_sum, p_incl);
+        int run = -1;
+        double at = __shfl_sync(0xFFFFFFFFu, p_incl - p_sum, p_hit & 15);
+        if (p_hit == (int)part) {
+            run = first_past(at, mine, incl);
+            at += __shfl_sync(0xFFFFFFFFu, incl - mine, run & 15);
+        }
+        // ---- the warp whose run it is finds the tile, then the id
+        if (run == warp) {
+            const int n = p_hi - p_lo;
+            int pick = -1, held = -1;
+            double at_pick = 0.0, at_held = 0.0;
+            for (int t0 = 0; t0 < n && pick < 0; t0 += 32) {
+                const double v = t0 + lane < n ? (double)s_val[t0 + lane] : 0.0;
+                double s = v;
+#pragma unroll
+                for (int off = 1; off < 32; off <<= 1) {
+                    const double w = __shfl_up_sync(0xFFFFFFFFu, s, off);
+                    if (lane >= off) s += w;
+                }
+                const unsigned cross = __ballot_sync(0xFFFFFFFFu, v > 0.0 && at + s > target);
+                const unsigned mass = __ballot_sync(0xFFFFFFFFu, v > 0.0);
+                if (mass) {
+                    const int l = cross ? __ffs(cross) - 1 : 31 - __clz(mass);
+                    held = t0 + l;
+                    at_held = at + __shfl_sync(0xFFFFFFFFu, s - v, l);
+                    if (cross) { pick = held; at_pick = at_held; }
+                }
+                at += __shfl_sync(0xFFFFFFFFu, s, 31);
+            }
+            if (pick < 0) { pick = held; at_pick = at_held; }        // rounding hid it: the last tile with mass
+            const bool drawn = pick >= 0 && pick_in_tile<DTYPE>(q, a, b, q.residual, p_lo + pick, at_pick, target, Rn, flags, lane,
+                                                                 SOURCE == STAGED ? &sr : nullptr);
+            if (lane == 0 && !drawn) s_bare = 1;             // the tile holds no mass after all
+        }
+        __syncthreads();
+        bare = s_bare;
+    } else if (part != 0) {
+        return;
+    }
+    if (bare) draw_from_p<DTYPE>(q, a, b, u, flags | OD_SF_ZERO_MASS);
+}
+
+// ---- vocabulary shards: MODE 1, a shard's mass shares; MODE 2, a shard's pick ---------------
+template <int DTYPE, int MODE>
+__global__ void __launch_bounds__(OD_SAMPLE_THREADS, 4)
+od_sample_shard_kernel(const SampleArgs a)
+{
+    extern __shared__ __align__(16) unsigned char s_dyn[];   // ntiles x 8 bytes
+    double *s_val = (double *)s_dyn;                         // pass 2: tile values
+    __shared__ double s_warp[WARPS];
+    __shared__ unsigned int s_last;
+    __shared__ int s_tile, s_lastmass, s_done;
+    __shared__ double s_before;
+    __shared__ double s_cross[OD_SAMPLE_THREADS];           // pass 2: the sum in front of a thread's crossing tile
+
+    // grid = (sequences, parts of a row): blocks with neighbouring indices, which often end up on
+    // one multiprocessor, then work on the same tiles of different sequences and share the
+    // inverse-map entries in L1
+    const int b = blockIdx.x;
+    const unsigned int part = blockIdx.y, nparts = gridDim.y;
+    const int K = a.K_max;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+
+    asm volatile("griddepcontrol.launch_dependents;");
+    if (!a.early) asm volatile("griddepcontrol.wait;" ::: "memory");
+    const Ahead h = load_ahead(a, b, lane);
+    const int mb = h.mb;
+    const float T = h.T;
+
+    // a shard's tiles and ids keep their numbers of the full row
+    const int tile_lo = a.tile_lo, tile_hi = a.tile_hi;
+    // pass 1's whole tiles of this warp, and the inverse-map entries of their first pair
+    const int p_lo = tile_lo + ((int)part * WARPS + warp) * a.tiles_per_warp;
+    int p_hi = p_lo + a.tiles_per_warp;
+    if (p_hi > tile_hi) p_hi = tile_hi;
+    const int p_hi_w = p_hi < a.v_p / OD_SAMPLE_TILE ? p_hi : a.v_p / OD_SAMPLE_TILE;
+    int4 ni[2][2] = {};
+    if (MODE != 2 && !a.same_ids && p_lo < p_hi_w) first_pair_entries(a, p_lo, p_hi_w, lane, ni);
+
+    // n_accepted and the row statistics come from the verification kernels
+    if (a.early) asm volatile("griddepcontrol.wait;" ::: "memory");
 
     if (!(T > 0.f)) {                              // every block of the sequence leaves here
         if (part == 0 && threadIdx.x == 0) {
@@ -592,80 +1149,22 @@ od_sample_kernel(const SampleArgs a)
     }
     float rm = 0.f, rs = 0.f;                      // lane k: statistics of row k
     if (lane <= mb) {
-        rm = FUSED ? s_M[lane] : a.row_max[b * (K + 1) + lane];
-        rs = FUSED ? s_S[lane] : a.row_sum[b * (K + 1) + lane];
+        rm = a.row_max[b * (K + 1) + lane];
+        rs = a.row_sum[b * (K + 1) + lane];
     }
-    int j = FUSED ? fused_n : a.n_accepted[b];
+    int j = a.n_accepted[b];
     j = j < 0 ? 0 : (j > mb ? mb : j);
-    const size_t esz = DTYPE == OD_BF16 ? 2 : 4;
-    // a shard's row pointer is moved back by the shard's first column, and only ids of
-    // the window are read
-    SeqState q;
-    q.row = (const char *)a.logits + ((size_t)b * a.seq_stride + (size_t)j * a.row_stride) * esz;
-    if (MODE != 0) q.row -= (size_t)a.col0 * esz;
-    q.scale = 1.4426950408889634f / T;
-    {
-        // reference exponent c = fl(M*scale); the rounding of c goes into S exactly:
-        // sum_t exp2(x_t*scale - c) = (sum_t exp2((x_t - M)*scale)) * exp2(M*scale - c)
-        const float M = __shfl_sync(0xFFFFFFFFu, rm, j);
-        q.c = fmaxf(M * q.scale, -FLT_MAX);
-        q.S = __shfl_sync(0xFFFFFFFFu, rs, j) * od_ex2(fmaf(M, q.scale, -q.c));
-    }
-    q.residual = (j < mb) || stop;
-    q.ngram_token = -1; q.prefix_token = -1; q.first_draft = -1; q.ngram_prob = 0.f; q.prefix_val = 0.f;
-    q.q_row = a.q_rows;
-    {
-        // position j's preparation (j < K whenever the draw is a residual one)
-        const int src = j < K ? j : 0;
-        const int32_t s0 = __shfl_sync(0xFFFFFFFFu, e_s0, src), len = __shfl_sync(0xFFFFFFFFu, e_len, src);
-        const int32_t tgt = __shfl_sync(0xFFFFFFFFu, e_tgt, src), d1 = __shfl_sync(0xFFFFFFFFu, e_d1, src);
-        const int32_t pm = __shfl_sync(0xFFFFFFFFu, e_pm, src);
-        const float qp = __shfl_sync(0xFFFFFFFFu, e_qp, src), qd1 = __shfl_sync(0xFFFFFFFFu, e_qd1, src);
-        if (q.residual) {
-            q.q_row = a.q_rows + ((size_t)b * K + s0) * a.v_q;
-            // the gathers of pass 1 come two round trips from now: have the copy engine pull
-            // this block's share of the drafter's row into L2 meanwhile
-            if (MODE != 2 && threadIdx.x == 0) {
-                const size_t row_bytes = (size_t)a.v_q * 4 / 16 * 16;
-                size_t lo = (row_bytes / nparts * part) / 16 * 16;
-                size_t hi = part + 1 == nparts ? row_bytes : (row_bytes / nparts * (part + 1)) / 16 * 16;
-                const char *base = (const char *)q.q_row;
-                if (((uintptr_t)base & 15u) == 0 && hi > lo)
-                    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(base + lo), "r"((uint32_t)(hi - lo)) : "memory");
-            }
-            if (len >= 2) {
-                q.ngram_token = tgt;
-                q.ngram_prob = qp;
-                if (d1 >= 0) {
-                    q.first_draft = d1;
-                    q.prefix_token = pm;
-                    q.prefix_val = qd1 - q.ngram_prob;
-                }
-            }
-        }
-    }
+    const SeqState q = seq_state<DTYPE>(a, h, b, j, rm, rs, a.col0);
+    if (MODE != 2 && q.residual && threadIdx.x == 0) prefetch_q_row(a, q, part, nparts);
 
     const int ntiles = a.ntiles;
     double *tile_val = a.tile_val + (size_t)b * ntiles;
+    GlobalTiles out = {tile_val, lane};
 
     if (MODE != 2) {
         // ---- pass 1: the value of every tile ----
-        {
-            const int t_lo = p_lo, t_hi = p_hi;
-            if (t_lo < t_hi) {
-                // whole tiles pipelined; the row's ragged last tile (if it is this warp's) on its own
-                const int hi_w = p_hi_w;
-                if (q.residual) {
-                    if (t_lo < hi_w) {
-                        if (a.same_ids) warp_tiles_same_ids<DTYPE>(q, a, t_lo, hi_w, lane, tile_val);
-                        else warp_tiles_dense_piped<DTYPE>(q, a, t_lo, hi_w, lane, tile_val, ni);
-                    }
-                    if (hi_w < t_hi) warp_tiles_dense<DTYPE, 2>(q, a, true, hi_w > t_lo ? hi_w : t_lo, t_hi, lane, tile_val);
-                } else {
-                    warp_tiles_dense<DTYPE, 2>(q, a, false, t_lo, t_hi, lane, tile_val);
-                }
-            }
-        }
+        if (a.same_ids) warp_run<DTYPE, FROM_ROW>(q, a, p_lo, p_hi, p_hi_w, lane, out, ni);
+        else warp_run<DTYPE, FROM_MAP>(q, a, p_lo, p_hi, p_hi_w, lane, out, ni);
         // The tile values are read by another block: the barrier orders this block's stores
         // before thread 0's fence, the fence before its ticket (release); the block that
         // draws the last ticket fences again before anyone in it reads (acquire).
@@ -706,6 +1205,8 @@ od_sample_kernel(const SampleArgs a)
     if (MODE != 2 && threadIdx.x == 0) a.ticket[b] = 0;
     __syncthreads();
 
+    // the shards exchange their shares relative to fl(M*scale)
+    const double unit = exp2((double)q.margin);
     if (MODE == 1) {
         // ---- this shard's shares ----
         const double mass_r = block_total(s_val, my_lo, my_hi, s_warp);
@@ -713,13 +1214,13 @@ od_sample_kernel(const SampleArgs a)
         if (residual && !(mass_r > 0.0)) {
             // no residual mass here: should no shard have any, the draw is from p_j
             for (int t_lo = tile_lo + warp * 2; t_lo < tile_hi; t_lo += WARPS * 2)
-                warp_tiles_dense<DTYPE, 2>(q, a, false, t_lo, t_lo + 2 < tile_hi ? t_lo + 2 : tile_hi, lane, tile_val);
+                warp_tiles_dense<DTYPE, 2>(q, a, false, t_lo, t_lo + 2 < tile_hi ? t_lo + 2 : tile_hi, lane, out);
             __syncthreads();
             for (int t = tile_lo + threadIdx.x; t < tile_hi; t += OD_SAMPLE_THREADS) s_val[t] = fmax(0.0, tile_val[t]);
             __syncthreads();
             mass_e = block_total(s_val, my_lo, my_hi, s_warp);
         }
-        if (threadIdx.x == 0) { a.mass_out[2 * b] = mass_r; a.mass_out[2 * b + 1] = mass_e; }
+        if (threadIdx.x == 0) { a.mass_out[2 * b] = mass_r * unit; a.mass_out[2 * b + 1] = mass_e * unit; }
         return;
     }
 
@@ -727,8 +1228,8 @@ od_sample_kernel(const SampleArgs a)
     if (MODE == 2) {
         double tot_r = 0.0, tot_e = 0.0;
         for (int s = 0; s < a.n_shards; ++s) {
-            tot_r += a.mass_all[((size_t)s * a.B + b) * 2];
-            tot_e += a.mass_all[((size_t)s * a.B + b) * 2 + 1];
+            tot_r += a.mass_all[((size_t)s * a.B + b) * 2] / unit;
+            tot_e += a.mass_all[((size_t)s * a.B + b) * 2 + 1] / unit;
         }
         const bool use_e = residual && !(tot_r > 0.0);
         if (use_e) { residual = false; flags |= OD_SF_ZERO_MASS; }   // the tile values then hold p_j's
@@ -740,7 +1241,7 @@ od_sample_kernel(const SampleArgs a)
             double c = 0.0;
             int last = -1;
             for (int s = 0; s < a.n_shards; ++s) {
-                const double v = a.mass_all[((size_t)s * a.B + b) * 2 + (use_e ? 1 : 0)];
+                const double v = a.mass_all[((size_t)s * a.B + b) * 2 + (use_e ? 1 : 0)] / unit;
                 if (s == a.shard_index) shard_before = c;
                 if (v > 0.0) last = s;
                 if (c + v > target) { owner = s; break; }
@@ -759,128 +1260,68 @@ od_sample_kernel(const SampleArgs a)
         }
     }
 
-    for (int attempt = 0; attempt < 2; ++attempt) {
-        // exclusive scan of the tile values: thread i owns `per` consecutive tiles
-        double loc = 0.0;
-        for (int t = my_lo; t < my_hi; ++t) loc += s_val[t];
-        double inc = loc;
+    // exclusive scan of the tile values: thread i owns `per` consecutive tiles
+    double loc = 0.0;
+    for (int t = my_lo; t < my_hi; ++t) loc += s_val[t];
+    double inc = loc;
 #pragma unroll
-        for (int off = 1; off < 32; off <<= 1) {
-            const double v = __shfl_up_sync(0xFFFFFFFFu, inc, off);
-            if (lane >= off) inc += v;
-        }
-        if (lane == 31) s_warp[warp] = inc;
-        if (threadIdx.x == 0) { s_tile = 0x7FFFFFFF; s_lastmass = -1; s_token = -2; }
-        __syncthreads();
-        // every thread adds the warps' sums up itself (the same order everywhere): no barrier
-        // for the total
-        double base = MODE == 2 ? shard_before : 0.0, tot = 0.0;
-        for (int w = 0; w < WARPS; ++w) {
-            if (w == warp) base += tot;
-            tot += s_warp[w];
-        }
-        if (threadIdx.x == 0) s_total = tot;
-        const double Rn = MODE == 2 ? shard_total : tot;   // unnormalised total
-        double target = 0.0;
-        if (Rn > 0.0) {
-            target = (double)u * Rn;
-            double c = base + inc - loc;
-            int last = -1;
-            for (int t = my_lo; t < my_hi; ++t) {
-                const double v = s_val[t];
-                if (v > 0.0) last = t;
-                if (c + v > target) {
-                    // first crossing of this run: the tile, and with it who found it, so that
-                    // the sum before the tile needs no barrier of its own
-                    s_cross[threadIdx.x] = c;
-                    atomicMin(&s_tile, t * OD_SAMPLE_THREADS + (int)threadIdx.x);
-                    break;
-                }
-                c += v;
-            }
-            if (last >= 0) atomicMax(&s_lastmass, last);
-        }
-        __syncthreads();
-        // cumulative sums never decrease, so the smallest reported tile is the crossing;
-        // if rounding hid it, take the last tile that has mass
-        int t_pick = -1;
-        if (Rn > 0.0) {
-            if (s_tile != 0x7FFFFFFF) {
-                t_pick = s_tile / OD_SAMPLE_THREADS;
-                if (threadIdx.x < 32) s_before = s_cross[s_tile % OD_SAMPLE_THREADS];   // warp 0 reads it back below
-                __syncwarp();
-            } else {
-                t_pick = s_lastmass;
-                if (t_pick >= my_lo && t_pick < my_hi) {    // its owner publishes the sum before it
-                    double c = base + inc - loc;
-                    for (int t = my_lo; t < t_pick; ++t) c += s_val[t];
-                    s_before = c;
-                }
-                __syncthreads();                            // (block-uniform: s_tile is the same for all)
-            }
-        }
-        if (t_pick >= 0 && warp == 0) {
-            // ---- warp 0 evaluates the chosen tile id by id and scans inside it ----
-            float r[EPT];
-            if (residual) tile_values<DTYPE>(q, a, true, t_pick, lane, r);
-            else tile_e_values<DTYPE>(q, a, t_pick, lane, r);
-            const double mine = lane_sum(r);
-            double incl = mine;
-#pragma unroll
-            for (int off = 1; off < 32; off <<= 1) {
-                const double v = __shfl_up_sync(0xFFFFFFFFu, incl, off);
-                if (lane >= off) incl += v;
-            }
-            const double lbase = s_before + (incl - mine);   // sum before this lane's first id
-            const int t0 = t_pick * OD_SAMPLE_TILE + lane * EPT;
-            int my_pick = 0x7FFFFFFF, my_last = -1;
-            double lo = 0.0, hi = 0.0, c = lbase;
-            float run = 0.f;                        // same fp32 order as lane_sum
-#pragma unroll
-            for (int e = 0; e < EPT; ++e) {
-                run = e == 0 ? r[0] : run + r[e];
-                const double nc = lbase + (double)run;
-                if (r[e] > 0.f) my_last = t0 + e;
-                if (my_pick == 0x7FFFFFFF && nc > target) { my_pick = t0 + e; lo = c; hi = nc; }
-                c = nc;
-            }
-            int pick = my_pick, last = my_last;
-#pragma unroll
-            for (int off = 16; off > 0; off >>= 1) {
-                pick = min(pick, __shfl_xor_sync(0xFFFFFFFFu, pick, off));
-                last = max(last, __shfl_xor_sync(0xFFFFFFFFu, last, off));
-            }
-            const float R = (float)(Rn / (double)q.S);     // residual mass (1 for the free token)
-            if (pick != 0x7FFFFFFF) {
-                if (my_pick == pick) {              // exactly one lane owns the picked id
-                    uint32_t f = flags;
-                    if (fmin(target - lo, hi - target) <= OD_TAU_SAMPLE * Rn) f |= OD_SF_BOUNDARY;
-                    a.out_token[b] = pick; a.resid_mass[b] = R; a.flags[b] = f;
-                    s_token = pick;
-                }
-            } else if (last >= 0) {
-                // rounding: the target lies beyond the tile's last edge
-                if (lane == 0) {
-                    a.out_token[b] = last; a.resid_mass[b] = R; a.flags[b] = flags | OD_SF_BOUNDARY;
-                    s_token = last;
-                }
-            }                                       // else: the tile holds no mass after all
-        }
-        __syncthreads();
-        if (s_token >= 0) return;
-        if (MODE == 2 || !residual || attempt == 1) break;
-        // no usable residual mass: draw from p_j instead (rare; this block redoes the row)
-        residual = false;
-        flags |= OD_SF_ZERO_MASS;
-        for (int t_lo = warp * 2; t_lo < ntiles; t_lo += WARPS * 2)
-            warp_tiles_dense<DTYPE, 2>(q, a, false, t_lo, t_lo + 2 < ntiles ? t_lo + 2 : ntiles, lane, tile_val);
-        __syncthreads();
-        for (int t = threadIdx.x; t < ntiles; t += OD_SAMPLE_THREADS) s_val[t] = fmax(0.0, tile_val[t]);
-        __syncthreads();
+    for (int off = 1; off < 32; off <<= 1) {
+        const double v = __shfl_up_sync(0xFFFFFFFFu, inc, off);
+        if (lane >= off) inc += v;
     }
-    if (threadIdx.x == 0) {                         // no mass at all (non-finite input)
+    if (lane == 31) s_warp[warp] = inc;
+    if (threadIdx.x == 0) { s_tile = 0x7FFFFFFF; s_lastmass = -1; s_done = 0; }
+    __syncthreads();
+    double base = shard_before, tot = 0.0;
+    for (int w = 0; w < WARPS; ++w) {
+        if (w == warp) base += tot;
+        tot += s_warp[w];
+    }
+    double target = 0.0;
+    if (shard_total > 0.0) {
+        target = (double)u * shard_total;
+        double c = base + inc - loc;
+        int last = -1;
+        for (int t = my_lo; t < my_hi; ++t) {
+            const double v = s_val[t];
+            if (v > 0.0) last = t;
+            if (c + v > target) {
+                // first crossing of this run: the tile, and with it who found it, so that
+                // the sum before the tile needs no barrier of its own
+                s_cross[threadIdx.x] = c;
+                atomicMin(&s_tile, t * OD_SAMPLE_THREADS + (int)threadIdx.x);
+                break;
+            }
+            c += v;
+        }
+        if (last >= 0) atomicMax(&s_lastmass, last);
+    }
+    __syncthreads();
+    // cumulative sums never decrease, so the smallest reported tile is the crossing;
+    // if rounding hid it, take the last tile that has mass
+    int t_pick = -1;
+    if (shard_total > 0.0) {
+        if (s_tile != 0x7FFFFFFF) {
+            t_pick = s_tile / OD_SAMPLE_THREADS;
+            if (threadIdx.x < 32) s_before = s_cross[s_tile % OD_SAMPLE_THREADS];   // warp 0 reads it back below
+            __syncwarp();
+        } else {
+            t_pick = s_lastmass;
+            if (t_pick >= my_lo && t_pick < my_hi) {    // its owner publishes the sum before it
+                double c = base + inc - loc;
+                for (int t = my_lo; t < t_pick; ++t) c += s_val[t];
+                s_before = c;
+            }
+            __syncthreads();                            // (block-uniform: s_tile is the same for all)
+        }
+    }
+    if (t_pick >= 0 && warp == 0 &&
+        pick_in_tile<DTYPE>(q, a, b, residual, t_pick, s_before, target, shard_total, flags, lane) && lane == 0)
+        s_done = 1;
+    __syncthreads();
+    if (threadIdx.x == 0 && !s_done) {                  // no mass at all (non-finite input)
         a.out_token[b] = -1;
-        a.resid_mass[b] = (float)((MODE == 2 ? shard_total : s_total) / (double)q.S);
+        a.resid_mass[b] = (float)(shard_total / (double)q.S);
         a.flags[b] = flags | OD_SF_ZERO_MASS;
     }
 }
@@ -890,22 +1331,66 @@ od_sample_kernel(const SampleArgs a)
 // Dynamic shared memory of the kernel for rows of `ntiles` tiles: the tile values of pass 2.
 size_t od_sample_smem_bytes(int32_t ntiles) { return (size_t)ntiles * 8; }
 
-// Rows beyond 6144 tiles need more dynamic shared memory than a kernel gets by default: opt
-// in (the device must be current; allocates nothing).
-cudaError_t od_sample_prepare_device(size_t bytes)
+template <typename K>
+static cudaError_t allow_smem(K kernel, size_t bytes)
 {
-    if (bytes <= 48 * 1024) return cudaSuccess;
-    cudaError_t e = cudaSuccess;
-    const int n = (int)bytes;
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(od_sample_kernel<OD_BF16, 0, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, n);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(od_sample_kernel<OD_F32, 0, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, n);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(od_sample_kernel<OD_BF16, 0, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, n);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(od_sample_kernel<OD_F32, 0, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, n);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(od_sample_kernel<OD_BF16, 1, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, n);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(od_sample_kernel<OD_F32, 1, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, n);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(od_sample_kernel<OD_BF16, 2, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, n);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(od_sample_kernel<OD_F32, 2, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, n);
+    return bytes <= 48 * 1024 ? cudaSuccess
+                              : cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+}
+template <int DTYPE, bool FUSED, int SOURCE>
+static cudaError_t allow_cluster16(size_t bytes)
+{
+    cudaError_t e = allow_smem(od_sample_kernel<DTYPE, FUSED, SOURCE>, bytes);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(od_sample_kernel<DTYPE, FUSED, SOURCE>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     return e;
+}
+template <int DTYPE>
+static cudaError_t prepare_kernels(size_t bytes)
+{
+    const size_t staged = (size_t)OD_SAMPLE_MAX_SLOTS * 4 + 8 * 1024;
+    cudaError_t e = allow_cluster16<DTYPE, false, FROM_MAP>(bytes);
+    if (e == cudaSuccess) e = allow_cluster16<DTYPE, true, FROM_MAP>(bytes);
+    if (e == cudaSuccess) e = allow_cluster16<DTYPE, false, FROM_ROW>(bytes);
+    if (e == cudaSuccess) e = allow_cluster16<DTYPE, true, FROM_ROW>(bytes);
+    if (e == cudaSuccess) e = allow_cluster16<DTYPE, false, STAGED>(staged);
+    if (e == cudaSuccess) e = allow_cluster16<DTYPE, true, STAGED>(staged);
+    if (e == cudaSuccess) e = allow_smem(od_sample_shard_kernel<DTYPE, 1>, bytes);
+    if (e == cudaSuccess) e = allow_smem(od_sample_shard_kernel<DTYPE, 2>, bytes);
+    return e;
+}
+
+// Rows beyond 6144 tiles (and the staged probabilities) need more dynamic shared memory than a
+// kernel gets by default, and clusters of 16 blocks are not portable: opt in, and ask whether the
+// device has room for such a cluster (the device must be current; allocates nothing).
+cudaError_t od_sample_prepare_device(size_t bytes, bool *cluster16)
+{
+    cudaError_t e = prepare_kernels<OD_BF16>(bytes);
+    if (e == cudaSuccess) e = prepare_kernels<OD_F32>(bytes);
+    if (e != cudaSuccess) return e;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(16); cfg.blockDim = dim3(CTHREADS); cfg.dynamicSmemBytes = 64 * 1024;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = 16; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr; cfg.numAttrs = 1;
+    int n = 0;
+    e = cudaOccupancyMaxActiveClusters(&n, od_sample_kernel<OD_BF16, true, STAGED>, &cfg);
+    *cluster16 = e == cudaSuccess && n > 0;
+    return e;
+}
+
+template <int DTYPE>
+static cudaError_t launch_step(const cudaLaunchConfig_t &cfg, const SampleArgs &a, bool fused, int source)
+{
+    if (source == STAGED)
+        return fused ? cudaLaunchKernelEx(&cfg, od_sample_kernel<DTYPE, true, STAGED>, a)
+                     : cudaLaunchKernelEx(&cfg, od_sample_kernel<DTYPE, false, STAGED>, a);
+    if (source == FROM_ROW)
+        return fused ? cudaLaunchKernelEx(&cfg, od_sample_kernel<DTYPE, true, FROM_ROW>, a)
+                     : cudaLaunchKernelEx(&cfg, od_sample_kernel<DTYPE, false, FROM_ROW>, a);
+    return fused ? cudaLaunchKernelEx(&cfg, od_sample_kernel<DTYPE, true, FROM_MAP>, a)
+                 : cudaLaunchKernelEx(&cfg, od_sample_kernel<DTYPE, false, FROM_MAP>, a);
 }
 
 // mode 0: od_sample_residual; 1 / 2: the two calls of a vocabulary shard
@@ -928,16 +1413,35 @@ static cudaError_t launch_sample(od_ctx *c, int mode, int32_t B, int32_t K_max, 
     const int tile_hi = mode == 0 ? ntiles : (shard_lo + shard_len + OD_SAMPLE_TILE - 1) / OD_SAMPLE_TILE;
     const int wtiles = tile_hi - tile_lo;
     int64_t tpw = c->opt_sample_tiles_per_warp;
-    if (tpw <= 0) {
-        // one resident wave (four 256-thread blocks per SM) over the whole batch
-        const int64_t want = (int64_t)c->sm_count * 4;
-        int64_t per_row = want / B;
-        if (per_row < 1) per_row = 1;
-        tpw = (wtiles + per_row * WARPS - 1) / (per_row * WARPS);
-        if (tpw < 1) tpw = 1;
+    int blocks_x = 1, level = 0, part_tiles = 0;
+    if (mode == 0) {
+        // Parts (blocks) per sequence: as many as still make one resident wave of two blocks per
+        // multiprocessor, and no more than have a tile for every warp (19 sequences of 100277 ids, the
+        // three calls: 25.2 us with 4 parts, 23.3 with 8, 27.0 with 16, which is two waves; one of
+        // 152064: 29.1 / 27.1 / 26.7).
+        const int fine = od_sample_fine_tiles(c->v_p);
+        const int most = c->cluster16 ? OD_SAMPLE_LEVELS - 1 : OD_SAMPLE_LEVELS - 2;
+        while (level < most && (tpw > 0 ? fine * (OD_SAMPLE_MAX_PARTS >> level) > tpw * CWARPS
+                                        : (int64_t)B * 2 << level <= (int64_t)c->sm_count * 2 &&
+                                              fine * (OD_SAMPLE_MAX_PARTS >> level) > CWARPS))
+            ++level;
+        // staged probabilities of over 100 KB would leave room for one block per multiprocessor
+        while (level < most && !c->map_same_ids && c->sample_slots[level] * 4 > 100 * 1024) ++level;
+        blocks_x = 1 << level;
+        part_tiles = fine * (OD_SAMPLE_MAX_PARTS >> level);
+        tpw = (part_tiles + CWARPS - 1) / CWARPS;
+    } else {
+        if (tpw <= 0) {
+            // one resident wave (four 256-thread blocks per SM) over the whole batch
+            const int64_t want = (int64_t)c->sm_count * 4;
+            int64_t per_row = want / B;
+            if (per_row < 1) per_row = 1;
+            tpw = (wtiles + per_row * WARPS - 1) / (per_row * WARPS);
+            if (tpw < 1) tpw = 1;
+        }
+        const int64_t tiles_per_block = tpw * WARPS;
+        if (mode == 1) blocks_x = (int)((wtiles + tiles_per_block - 1) / tiles_per_block);
     }
-    const int64_t tiles_per_block = tpw * WARPS;
-    const int blocks_x = mode == 2 ? 1 : (int)((wtiles + tiles_per_block - 1) / tiles_per_block);
     SampleArgs a = {};
     a.logits = logits; a.row_stride = row_stride; a.seq_stride = seq_stride;
     a.B = B; a.K_max = K_max; a.v_p = mode == 0 ? c->v_p : shard_lo + shard_len; a.v_q = c->v_q;
@@ -947,6 +1451,7 @@ static cudaError_t launch_sample(od_ctx *c, int mode, int32_t B, int32_t K_max, 
     a.span_start = span_start; a.span_len = span_len; a.m = m; a.tail_kind = tail_kind;
     a.n_accepted = n_accepted; a.temperature = temperature; a.seed = seed; a.step = step;
     a.vocab_map = c->d_vocab_map; a.inv_map = c->d_inv_map;
+    a.part_tiles = part_tiles;
     a.same_ids = c->map_same_ids && c->v_q % 4 == 0 && ((uintptr_t)q_rows & 15u) == 0;
     a.out_token = out_token; a.resid_mass = resid_mass; a.flags = flags;
     a.tile_val = c->d_tile_sums; a.ticket = c->d_samp_ticket;
@@ -968,27 +1473,38 @@ static cudaError_t launch_sample(od_ctx *c, int mode, int32_t B, int32_t K_max, 
     }
 
     cudaLaunchConfig_t cfg = {};
+    cfg.stream = s;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = c->opt_pdl ? attr : attr + 1;
+    const bool bf = dtype == OD_BF16;
+    if (mode == 0) {
+        cfg.gridDim = dim3((unsigned)blocks_x, (unsigned)B);
+        cfg.blockDim = dim3(CTHREADS);
+        attr[1].id = cudaLaunchAttributeClusterDimension;
+        attr[1].val.clusterDim.x = (unsigned)blocks_x; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
+        cfg.numAttrs = c->opt_pdl ? 2 : 1;
+        const int source = a.same_ids ? FROM_ROW
+                                      : c->sample_slots[level] <= OD_SAMPLE_MAX_SLOTS && part_tiles <= 2048 ? STAGED : FROM_MAP;
+        if (source == STAGED) {
+            const OdSampleLists l = od_sample_lists(c->d_sample_lists, c->v_q, c->v_p);
+            a.list_word = l.word + (size_t)level * l.groups * 32; a.list_base = l.base + (size_t)level * l.groups;
+            a.list_part = l.part + level * OD_SAMPLE_MAX_PARTS * 4; a.octet = l.octet;
+            a.slots = c->sample_slots[level] + 1;
+        }
+        cfg.dynamicSmemBytes = ((size_t)a.slots + (size_t)tpw * CWARPS) * sizeof(float);
+        return bf ? launch_step<OD_BF16>(cfg, a, fuse != nullptr, source) : launch_step<OD_F32>(cfg, a, fuse != nullptr, source);
+    }
     cfg.gridDim = dim3((unsigned)B, (unsigned)blocks_x);
     cfg.blockDim = dim3(OD_SAMPLE_THREADS);
     cfg.dynamicSmemBytes = od_sample_smem_bytes(ntiles);
-    cfg.stream = s;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
     cfg.numAttrs = c->opt_pdl ? 1 : 0;
-    const bool bf = dtype == OD_BF16;
-    if (mode == 0 && fuse)
-        return bf ? cudaLaunchKernelEx(&cfg, od_sample_kernel<OD_BF16, 0, true>, a)
-                  : cudaLaunchKernelEx(&cfg, od_sample_kernel<OD_F32, 0, true>, a);
-    if (mode == 0)
-        return bf ? cudaLaunchKernelEx(&cfg, od_sample_kernel<OD_BF16, 0, false>, a)
-                  : cudaLaunchKernelEx(&cfg, od_sample_kernel<OD_F32, 0, false>, a);
     if (mode == 1)
-        return bf ? cudaLaunchKernelEx(&cfg, od_sample_kernel<OD_BF16, 1, false>, a)
-                  : cudaLaunchKernelEx(&cfg, od_sample_kernel<OD_F32, 1, false>, a);
-    return bf ? cudaLaunchKernelEx(&cfg, od_sample_kernel<OD_BF16, 2, false>, a)
-              : cudaLaunchKernelEx(&cfg, od_sample_kernel<OD_F32, 2, false>, a);
+        return bf ? cudaLaunchKernelEx(&cfg, od_sample_shard_kernel<OD_BF16, 1>, a)
+                  : cudaLaunchKernelEx(&cfg, od_sample_shard_kernel<OD_F32, 1>, a);
+    return bf ? cudaLaunchKernelEx(&cfg, od_sample_shard_kernel<OD_BF16, 2>, a)
+              : cudaLaunchKernelEx(&cfg, od_sample_shard_kernel<OD_F32, 2>, a);
 }
 
 cudaError_t od_launch_sample(od_ctx *c, int32_t B, int32_t K_max, const void *logits,
@@ -1038,4 +1554,61 @@ cudaError_t od_launch_sample_shard_pick(od_ctx *c, int32_t B, int32_t K_max, int
                          draft_ids, tgt_ids, q_prime, span_start, span_len, m, tail_kind, n_accepted,
                          temperature, seed, step, out_token, resid_mass, flags, shard_lo, shard_len, n_shards,
                          shard_index, mass_all, nullptr, s);
+}
+
+
+// What the sampler knows about the vocabulary map, on the host, in the layout of od_sample_lists.
+// `map` is the vocabulary map, `inv` its inverse; negative = none. slots: [levels] most mapped ids of a part.
+void od_sample_plan(int32_t v_q, int32_t v_p, const int32_t *map, const int32_t *inv, void *out, int32_t *slots)
+{
+    const OdSampleLists l = od_sample_lists(out, v_q, v_p);
+    const int32_t fine_ids = od_sample_fine_tiles(v_p) * OD_SAMPLE_TILE;
+    int32_t first_rank[OD_SAMPLE_MAX_PARTS + 1], rank = 0;   // of the 16ths
+    for (int32_t o = 0, next = 0; o < (v_p + 7) / 8; ++o) {
+        while (next < OD_SAMPLE_MAX_PARTS && (int64_t)next * fine_ids <= (int64_t)o * 8) first_rank[next++] = rank;
+        uint32_t mask = 0;
+        for (int32_t e = 0; e < 8 && o * 8 + e < v_p; ++e) mask |= inv[o * 8 + e] >= 0 ? 1u << e : 0u;
+        l.octet[o] = (uint32_t)rank << 8 | mask;
+        rank += __builtin_popcount(mask);
+        if (o + 1 == (v_p + 7) / 8)
+            while (next <= OD_SAMPLE_MAX_PARTS) first_rank[next++] = rank;
+    }
+    first_rank[OD_SAMPLE_MAX_PARTS] = rank;
+    struct Open {
+        int32_t n, base, rank0;                              // a part's open group: n entries so far, from draft id `base`
+        int32_t *end;                                        // one past it
+    } open[OD_SAMPLE_LEVELS][OD_SAMPLE_MAX_PARTS];
+    for (int level = 0; level < OD_SAMPLE_LEVELS; ++level) {
+        const int per = OD_SAMPLE_MAX_PARTS >> level;
+        int32_t group = 0;
+        slots[level] = 0;
+        for (int k = 0; k < 1 << level; ++k) {
+            int32_t *p = l.part + (level * OD_SAMPLE_MAX_PARTS + k) * 4;
+            const int32_t n = first_rank[(k + 1) * per] - first_rank[k * per];
+            p[0] = p[1] = group; p[2] = first_rank[k * per]; p[3] = n;
+            open[level][k] = {32, 0, p[2], p + 1};
+            group += (n + 31) / 32 + v_q / 65536;
+            if (n > slots[level]) slots[level] = n;
+        }
+    }
+    // a part's entries in draft-id order; a new group of 32 where one is full or the next id is
+    // over 65535 on
+    for (int32_t d = 0; d < v_q; ++d) {
+        const int32_t t = map[d];
+        if (t < 0) continue;
+        const uint32_t oct = l.octet[t >> 3];
+        const int32_t at = (int32_t)(oct >> 8) + __builtin_popcount(oct & ((1u << (t & 7)) - 1u)), f = t / fine_ids;
+        for (int level = 0; level < OD_SAMPLE_LEVELS; ++level) {
+            Open &o = open[level][f >> (OD_SAMPLE_LEVELS - 1 - level)];
+            if (o.n == 32 || d - o.base > 0xFFFF) {
+                const size_t g = (size_t)level * l.groups + (*o.end)++;
+                l.base[g] = d;
+                for (int i = 0; i < 32; ++i) l.word[g * 32 + i] = 0xFFFFu;
+                o.n = 0; o.base = d;
+            }
+            // (a part of more than OD_SAMPLE_MAX_SLOTS ids is not staged: the cut does not matter)
+            l.word[((size_t)level * l.groups + *o.end - 1) * 32 + o.n++] =
+                (uint32_t)(d - o.base) << 16 | (uint32_t)((at - o.rank0) & 0xFFFF);
+        }
+    }
 }

@@ -1,0 +1,66 @@
+"""The sampler's cuts of a row (1 to 16 blocks per sequence) and its sources of the drafter's
+probabilities (staged in target order, the row itself, the inverse map) against the oracle."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_2507_02659_b200 import binding as od
+from paper_2507_02659_b200 import synth
+
+import parity
+
+pytestmark = pytest.mark.gpu
+
+
+def _workload(**kw):
+    base = dict(B=5, steps=4, k_max=4, k_min=1, v_q=600, v_p=1003, logit_dtype="bf16", map_kind="random",
+                mapped_frac=0.7, cache_entries=150, hit_prob=0.6, logit_kind="corr", rho=0.9,
+                temperatures=(1.0, 0.5, 0.7), per_seq_seed=True, gen_seed=0xFACE10, unmapped_shift=2.0, sigma=2.0)
+    base.update(kw)
+    return synth.Workload("parts", **base)
+
+
+def _check(w, st, device, tiles, steps):
+    ctx = parity.make_context(w, st, device)
+    ctx.set_option("sample_tiles_per_warp", tiles)
+    cache = oracle.Cache(st.runs, st.run_len, st.run_target)
+    blocks = set()
+    for step in range(steps):
+        s = synth.make_step(w, st, step, device=device)
+        logits = parity.pad_rows(s.logits)
+        parity.check_step(ctx, cache, st, w, s, logits=logits)
+        blocks.add(ctx.last_launch_info(2) // w.B)
+        mp, vo, so = parity.gpu_step(ctx, s, logits=logits)
+        _, _, one = od.od_step(ctx, s.draft_ids, s.draft_len, s.q_sel, s.q_rows, logits, s.temperature, s.seed, step)
+        torch.cuda.synchronize()
+        for name, t in vars(one).items():
+            assert torch.equal(t, vars(so)[name]), name
+    ctx.close()
+    return blocks
+
+
+# vocabularies of less than a tile per warp, ragged last tiles and octets, parts without tiles, target
+# ids beyond the drafter's where ids are shared, gaps in the map
+@pytest.mark.parametrize("shape", [dict(), dict(v_q=599, v_p=4099, logit_dtype="f32"),
+                                   dict(v_q=512, v_p=5003, map_kind="identity", cache_entries=0),
+                                   dict(v_q=4096, v_p=4096, map_kind="identity", cache_entries=0, logit_dtype="f32"),
+                                   dict(v_q=333, v_p=1000, map_kind="identity", cache_entries=0),
+                                   dict(v_q=33, v_p=70001, cache_entries=0), dict(v_q=9000, v_p=9001, mapped_frac=1.0, cache_entries=0)])
+def test_every_number_of_parts(cuda_device, shape):
+    w = _workload(**shape)
+    st = synth.make_static(w)
+    seen = set()
+    for tiles in (0, 1, 3, 5, 9, 1000):
+        seen |= _check(w, st, cuda_device, tiles, 2)
+    assert 1 in seen
+    if w.v_p > 60000:
+        assert seen >= {1, 2, 4, 8, 16}
+
+
+def test_more_mapped_ids_in_a_part_than_are_staged(cuda_device):
+    """60000 draft ids on neighbouring target ids: the probabilities come through the inverse map."""
+    w = _workload(B=2, k_max=2, v_q=60000, v_p=1_000_000, cache_entries=0)
+    st = synth.make_static(w)
+    st.vocab_map = np.arange(w.v_q, dtype=np.int32) + 1
+    _check(w, st, cuda_device, 0, 2)
