@@ -199,7 +199,11 @@ int32_t od_set_vocab_map(od_ctx *c, const int32_t *host_map)
     od_sample_plan(c->v_q, c->v_p, fwd.data(), inv.data(), lists.data(), c->sample_slots);
     OD_CUDA(cudaMemcpy(c->d_sample_lists, lists.data(), lists.size(), cudaMemcpyHostToDevice));
     c->map_same_ids = true;
-    for (int32_t d = 0; d < c->v_q; ++d) c->map_same_ids = c->map_same_ids && host_map[d] == d;
+    c->n_mapped = 0;
+    for (int32_t d = 0; d < c->v_q; ++d) {
+        c->map_same_ids = c->map_same_ids && host_map[d] == d;
+        c->n_mapped += host_map[d] >= 0 ? 1 : 0;
+    }
     c->have_map = true;
     return OD_OK;
     } catch (const std::bad_alloc &) {

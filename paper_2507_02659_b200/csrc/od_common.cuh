@@ -36,6 +36,7 @@ struct od_ctx {
     int32_t sample_slots[OD_SAMPLE_LEVELS];   // most mapped ids of a part
     bool cluster16;                 // the device takes the sampler's clusters of 16 blocks
     bool have_map;
+    int64_t n_mapped;               // draft ids with a direct map
     bool map_same_ids;              // every draft id is mapped to the target id of the same number
 
     // n-gram cache: open addressing over groups of 32 slots

@@ -163,6 +163,8 @@ struct Logit {
     typedef float raw;
     static __device__ __forceinline__ float load(const float *p) { return *p; }
     static __device__ __forceinline__ float4 load4(const float *p) { return *(const float4 *)p; }
+    static __device__ __forceinline__ float4 load4_global(const float *p) { return __ldg((const float4 *)p); }
+    static __device__ __forceinline__ void store4(float *p, float4 v) { *(float4 *)p = v; }
 };
 template <>
 struct Logit<OD_BF16> {
@@ -173,12 +175,23 @@ struct Logit<OD_BF16> {
         const uint2 v = *(const uint2 *)p;
         return make_float4(od_bf16_lo(v.x), od_bf16_hi(v.x), od_bf16_lo(v.y), od_bf16_hi(v.y));
     }
+    static __device__ __forceinline__ float4 load4_global(const raw *p)
+    {
+        const uint2 v = __ldg((const uint2 *)p);
+        return make_float4(od_bf16_lo(v.x), od_bf16_hi(v.x), od_bf16_lo(v.y), od_bf16_hi(v.y));
+    }
+    static __device__ __forceinline__ void store4(raw *p, float4 v)   // (exact: the values are bf16)
+    {
+        *(uint2 *)p = make_uint2(__float_as_uint(v.x) >> 16 | (__float_as_uint(v.y) & 0xFFFF0000u),
+                                 __float_as_uint(v.z) >> 16 | (__float_as_uint(v.w) & 0xFFFF0000u));
+    }
 };
 
 // Grid (C, K, B), clusters of C blocks. VEC4: the draft vocabulary is a multiple of 4 and the
 // rows are 16-byte aligned, so the coalesced accesses (q, gradient) move four ids per
-// instruction; chunks are multiples of 32 ids.
-template <int DTYPE, bool VEC4>
+// instruction; chunks are multiples of 32 ids. SAME: target ids are draft ids, nothing is
+// gathered; the logits wait in shared memory for the gradient.
+template <int DTYPE, bool VEC4, bool SAME>
 __global__ void __launch_bounds__(THREADS, 3)
 od_distill_kernel(const DistillArgs a)
 {
@@ -196,7 +209,7 @@ od_distill_kernel(const DistillArgs a)
     // context: the first entries are requested before the wait, the others a batch ahead.
     constexpr int EB = 4;                                   // groups per warp and batch
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int2 groups = __ldg((const int2 *)a.list_ofs + rank);
+    const int2 groups = SAME ? make_int2(0, 0) : __ldg((const int2 *)a.list_ofs + rank);
     const int g_hi = groups.y;
     int g_at = groups.x + warp;                          // this warp's next group to request
     uint32_t word[EB];
@@ -210,7 +223,7 @@ od_distill_kernel(const DistillArgs a)
         }
         g_at += EB * WARPS;
     };
-    load_words();
+    if (!SAME) load_words();
     asm volatile("griddepcontrol.wait;" ::: "memory");
     const float T = a.temperature[b];
     int piece, plen;
@@ -224,74 +237,106 @@ od_distill_kernel(const DistillArgs a)
     // ---- a directly mapped token: KL(q' || p_i) over the mapped ids
     const char *row = (const char *)a.logits + ((size_t)b * a.seq_stride + (size_t)piece * a.row_stride) * sizeof(raw_t);
     const float M = a.row_max[b * (a.K_max + 1) + piece], S = a.row_sum[b * (a.K_max + 1) + piece];
-    // (the first probabilities travel meanwhile)
-    constexpr int PQ = 2;                                    // vectors of four probabilities in flight per thread
-    float4 qv[PQ];
-    if (VEC4) {
-#pragma unroll
-        for (int i = 0; i < PQ; ++i) {
-            const int d = lo + (int)threadIdx.x * 4 + i * THREADS * 4;
-            if (d < hi) qv[i] = __ldg((const float4 *)(q + d));
-        }
-    }
-    // ---- the chunk's logits, gathered in target-id order, to their draft ids in shared memory
-    for (;;) {
-        raw_t x[EB];
-        uint32_t at[EB];
-#pragma unroll
-        for (int e = 0; e < EB; ++e) {
-            at[e] = word[e] & 0xFFFFu;
-            if (at[e] != 0xFFFFu) x[e] = __ldg((const raw_t *)row + base[e] + (int)(word[e] >> 16));
-        }
-        const bool more = g_at < g_hi;                       // the same for every lane of a warp
-        if (more) load_words();
-#pragma unroll
-        for (int e = 0; e < EB; ++e)
-            if (at[e] != 0xFFFFu) s_x[at[e]] = x[e];
-        if (!more) break;
-    }
     KlRow kl;
     kl.M = M;
-    kl.lg2_S = lg2_approx(S);
     kl.scale = 1.4426950408889634f / T;
-    __syncthreads();
-    // ---- the loss and sum_e q(e) g(e)
     float loss_t = 0.f, qg_t = 0.f;
     // four ids from d: their probabilities with 0 for the ids without a map
     auto mapped4 = [&](int d, float4 v) {
+        if (SAME) return v;
         const uint32_t w = __ldg(a.mapped_bits + (d >> 5)) >> (d & 31);
         return make_float4(w & 1u ? v.x : 0.f, w & 2u ? v.y : 0.f, w & 4u ? v.z : 0.f, w & 8u ? v.w : 0.f);
     };
-    auto mapped1 = [&](int d, float v) { return __ldg(a.mapped_bits + (d >> 5)) >> (d & 31) & 1u ? v : 0.f; };
-    if (VEC4) {
-        auto sum4 = [&](int d, float4 q4) {
-            const float4 v = mapped4(d, q4);
-            const float4 x = Logit<DTYPE>::load4(s_x + (d - lo));
-            float l = 0.f, g = 0.f;                          // four terms before they meet the running sums
-            kl_term(kl, v.x, x.x, l, g); kl_term(kl, v.y, x.y, l, g);
-            kl_term(kl, v.z, x.z, l, g); kl_term(kl, v.w, x.w, l, g);
-            loss_t += l; qg_t += g;
-        };
-        const int d0 = lo + (int)threadIdx.x * 4;
-        for (int d1 = d0; d1 < hi; d1 += PQ * THREADS * 4) {
-            float4 nx[PQ];
+    auto mapped1 = [&](int d, float v) {
+        return SAME || (__ldg(a.mapped_bits + (d >> 5)) >> (d & 31) & 1u) ? v : 0.f;
+    };
+    // four ids' terms before they meet the running sums
+    auto sum4 = [&](float4 v, float4 x) {
+        float l = 0.f, g = 0.f;
+        kl_term(kl, v.x, x.x, l, g); kl_term(kl, v.y, x.y, l, g);
+        kl_term(kl, v.z, x.z, l, g); kl_term(kl, v.w, x.w, l, g);
+        loss_t += l; qg_t += g;
+    };
+    const raw_t *xrow = (const raw_t *)row;
+    if (!SAME) {
+        // (the first probabilities travel meanwhile)
+        constexpr int PQ = 2;                                // vectors of four probabilities in flight per thread
+        float4 qv[PQ];
+        if (VEC4) {
 #pragma unroll
             for (int i = 0; i < PQ; ++i) {
-                const int d = d1 + (i + PQ) * THREADS * 4;
-                if (d < hi) nx[i] = __ldg((const float4 *)(q + d));
+                const int d = lo + (int)threadIdx.x * 4 + i * THREADS * 4;
+                if (d < hi) qv[i] = __ldg((const float4 *)(q + d));
             }
+        }
+        // ---- the chunk's logits, gathered in target-id order, to their draft ids in shared memory
+        for (;;) {
+            raw_t x[EB];
+            uint32_t at[EB];
 #pragma unroll
-            for (int i = 0; i < PQ; ++i) {
-                const int d = d1 + i * THREADS * 4;
-                if (d < hi) sum4(d, qv[i]);
+            for (int e = 0; e < EB; ++e) {
+                at[e] = word[e] & 0xFFFFu;
+                if (at[e] != 0xFFFFu) x[e] = __ldg((const raw_t *)row + base[e] + (int)(word[e] >> 16));
             }
+            const bool more = g_at < g_hi;                   // the same for every lane of a warp
+            if (more) load_words();
 #pragma unroll
-            for (int i = 0; i < PQ; ++i) qv[i] = nx[i];
+            for (int e = 0; e < EB; ++e)
+                if (at[e] != 0xFFFFu) s_x[at[e]] = x[e];
+            if (!more) break;
+        }
+        kl.lg2_S = lg2_approx(S);
+        __syncthreads();
+        // ---- the loss and sum_e q(e) g(e)
+        if (VEC4) {
+            const int d0 = lo + (int)threadIdx.x * 4;
+            for (int d1 = d0; d1 < hi; d1 += PQ * THREADS * 4) {
+                float4 nx[PQ];
+#pragma unroll
+                for (int i = 0; i < PQ; ++i) {
+                    const int d = d1 + (i + PQ) * THREADS * 4;
+                    if (d < hi) nx[i] = __ldg((const float4 *)(q + d));
+                }
+#pragma unroll
+                for (int i = 0; i < PQ; ++i) {
+                    const int d = d1 + i * THREADS * 4;
+                    if (d < hi) sum4(mapped4(d, qv[i]), Logit<DTYPE>::load4(s_x + (d - lo)));
+                }
+#pragma unroll
+                for (int i = 0; i < PQ; ++i) qv[i] = nx[i];
+            }
+        } else {
+#pragma unroll 4
+            for (int d = lo + (int)threadIdx.x; d < hi; d += THREADS)
+                kl_term(kl, mapped1(d, __ldg(q + d)), Logit<DTYPE>::load(s_x + (d - lo)), loss_t, qg_t);
         }
     } else {
+        kl.lg2_S = lg2_approx(S);
+        if (VEC4) {
+            constexpr int EV = 2;                            // vectors of four ids in flight per thread
+            for (int d1 = lo + (int)threadIdx.x * 4; d1 < hi; d1 += EV * THREADS * 4) {
+                float4 v[EV], x[EV];
+#pragma unroll
+                for (int i = 0; i < EV; ++i) {
+                    const int d = d1 + i * THREADS * 4;
+                    if (d < hi) { v[i] = __ldg((const float4 *)(q + d)); x[i] = Logit<DTYPE>::load4_global(xrow + d); }
+                }
+#pragma unroll
+                for (int i = 0; i < EV; ++i) {
+                    const int d = d1 + i * THREADS * 4;
+                    if (d >= hi) continue;
+                    if (grad) Logit<DTYPE>::store4(s_x + (d - lo), x[i]);
+                    sum4(v[i], x[i]);
+                }
+            }
+        } else {
 #pragma unroll 4
-        for (int d = lo + (int)threadIdx.x; d < hi; d += THREADS)
-            kl_term(kl, mapped1(d, __ldg(q + d)), Logit<DTYPE>::load(s_x + (d - lo)), loss_t, qg_t);
+            for (int d = lo + (int)threadIdx.x; d < hi; d += THREADS) {
+                const raw_t x = __ldg(xrow + d);
+                if (grad) s_x[d - lo] = x;
+                kl_term(kl, __ldg(q + d), Logit<DTYPE>::load(&x), loss_t, qg_t);
+            }
+        }
     }
     // the block's two sums, to every block of the cluster
     {
@@ -337,23 +382,22 @@ od_distill_kernel(const DistillArgs a)
     } else {
 #pragma unroll 4
         for (int d = lo + (int)threadIdx.x; d < hi; d += THREADS) {
-            const float v = __ldg(q + d);
-            grad[d] = fmaf(-v, gbar, v * kl_term(kl, mapped1(d, v), Logit<DTYPE>::load(s_x + (d - lo)), loss_t, qg_t));
+            const float v = __ldg(q + d), x = Logit<DTYPE>::load(s_x + (d - lo));
+            grad[d] = fmaf(-v, gbar, v * kl_term(kl, mapped1(d, v), x, loss_t, qg_t));
         }
     }
 }
 
 //XX
-// Draft vocabularies beyond the chunked kernel's shared memory (OD_DISTILL_MAX_CHUNKS chunks of
-// OD_DISTILL_MAX_CHUNK_IDS ids): one block per position, the ids in draft order, each gathering
-// its logit; q(d) g(d) waits in the gradient row for the second sweep.
-template <int DTYPE>
+// One block per position, the ids in draft order, each gathering its logit; q(d) g(d) waits in
+// the gradient row for the second sweep.
+template <int DTYPE, bool VEC4>
 __global__ void __launch_bounds__(THREADS, 2)
-od_distill_any_kernel(const DistillArgs a)
+od_distill_position_kernel(const DistillArgs a)
 {
     __shared__ double s_red[THREADS / 32];
     __shared__ int s_piece[2];
-    const int j = blockIdx.y, b = blockIdx.z;
+    const int j = blockIdx.x, b = blockIdx.y;
     const float *q = a.q_rows + ((size_t)b * a.K_max + j) * a.v_q;
     float *grad = a.grad ? a.grad + ((size_t)b * a.K_max + j) * a.v_q : nullptr;
     int piece, plen;
@@ -361,55 +405,114 @@ od_distill_any_kernel(const DistillArgs a)
     const float T = a.temperature[b];
     const bool translated = piece >= 0 && T > 0.f;
     if (!translated || plen >= 2) {
-        plain_position<false>(a, b, j, piece, translated, q, grad, 0, a.v_q, true);
+        plain_position<VEC4>(a, b, j, piece, translated, q, grad, 0, a.v_q, true);
         return;
     }
     const size_t esz = DTYPE == OD_BF16 ? 2 : 4;
     const char *row = (const char *)a.logits + ((size_t)b * a.seq_stride + (size_t)piece * a.row_stride) * esz;
+    // the gathers touch practically every sector of the row in no particular order: the copy
+    // engine brings it into L2 as one sequential transfer
+    if (threadIdx.x == 0) {
+        const uint32_t bytes = (uint32_t)((size_t)a.v_p * esz / 16 * 16);
+        if (bytes) asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(row), "r"(bytes) : "memory");
+    }
     KlRow kl;
     kl.M = a.row_max[b * (a.K_max + 1) + piece];
     kl.lg2_S = lg2_approx(a.row_sum[b * (a.K_max + 1) + piece]);
     kl.scale = 1.4426950408889634f / T;
     float loss_t = 0.f, qg_t = 0.f;
-    constexpr int EB = 16;
-    for (int base = threadIdx.x; base < a.v_q; base += THREADS * EB) {
-        float qd[EB], x[EB];
-        int32_t t[EB];
+    // one id: q (negative = no map) and its gathered logit; returns q(d) g(d)
+    auto term = [&](float qs, float x) -> float {
+        const bool ok = qs >= FLT_MIN;
+        const float qa = fabsf(qs);
+        const float f = ok ? 0.6931471805599453f * (lg2_approx(qa) - fmaf(x - kl.M, kl.scale, -kl.lg2_S)) : 0.f;
+        const float g = ok ? f + 1.f : 0.f;
+        loss_t += qa * f;
+        qg_t += qa * g;
+        return qa * g;
+    };
+    if (VEC4) {
+        constexpr int EV = 4;                                // vectors of 4 ids in flight per thread
+        for (int base = threadIdx.x * 4; base < a.v_q; base += THREADS * 4 * EV) {
+            int4 t[EV];
+            float4 qv[EV];
 #pragma unroll
-        for (int e = 0; e < EB; ++e) {
-            const int d = base + e * THREADS;
-            t[e] = d < a.v_q ? __ldg(a.vocab_map + d) : -1;
-            qd[e] = d < a.v_q ? __ldg(q + d) : 0.f;
+            for (int e = 0; e < EV; ++e) {
+                const int d = base + e * THREADS * 4;
+                t[e] = d < a.v_q ? __ldg((const int4 *)(a.vocab_map + d)) : make_int4(-1, -1, -1, -1);
+                qv[e] = d < a.v_q ? __ldg((const float4 *)(q + d)) : make_float4(0.f, 0.f, 0.f, 0.f);
+            }
+            float x[EV][4];
+#pragma unroll
+            for (int e = 0; e < EV; ++e) {
+                x[e][0] = od_load_logit<DTYPE>(row, t[e].x >= 0 ? t[e].x : 0);
+                x[e][1] = od_load_logit<DTYPE>(row, t[e].y >= 0 ? t[e].y : 0);
+                x[e][2] = od_load_logit<DTYPE>(row, t[e].z >= 0 ? t[e].z : 0);
+                x[e][3] = od_load_logit<DTYPE>(row, t[e].w >= 0 ? t[e].w : 0);
+            }
+#pragma unroll
+            for (int e = 0; e < EV; ++e) {
+                const int d = base + e * THREADS * 4;
+                float4 o;
+                o.x = term(t[e].x < 0 ? -qv[e].x : qv[e].x, x[e][0]);
+                o.y = term(t[e].y < 0 ? -qv[e].y : qv[e].y, x[e][1]);
+                o.z = term(t[e].z < 0 ? -qv[e].z : qv[e].z, x[e][2]);
+                o.w = term(t[e].w < 0 ? -qv[e].w : qv[e].w, x[e][3]);
+                if (grad && d < a.v_q) *(float4 *)(grad + d) = o;
+            }
         }
+    } else {
+        constexpr int EB = 16;
+        for (int base = threadIdx.x; base < a.v_q; base += THREADS * EB) {
+            float qd[EB], x[EB];
+            {
+                int32_t t[EB];
 #pragma unroll
-        for (int e = 0; e < EB; ++e) {
-            x[e] = od_load_logit<DTYPE>(row, t[e] >= 0 ? t[e] : 0);
-            if (t[e] < 0) qd[e] = 0.f;                       // an id without a map has no term
-        }
+                for (int e = 0; e < EB; ++e) {
+                    const int d = base + e * THREADS;
+                    t[e] = d < a.v_q ? __ldg(a.vocab_map + d) : -1;
+                    qd[e] = d < a.v_q ? __ldg(q + d) : 0.f;
+                }
 #pragma unroll
-        for (int e = 0; e < EB; ++e) {
-            const int d = base + e * THREADS;
-            const float g = kl_term(kl, qd[e], x[e], loss_t, qg_t);
-            if (grad && d < a.v_q) grad[d] = qd[e] * g;
+                for (int e = 0; e < EB; ++e)
+                    if (t[e] < 0) qd[e] = -qd[e];
+#pragma unroll
+                for (int e = 0; e < EB; ++e) x[e] = od_load_logit<DTYPE>(row, t[e] >= 0 ? t[e] : 0);
+            }
+#pragma unroll
+            for (int e = 0; e < EB; ++e) {
+                const int d = base + e * THREADS;
+                const float v = term(qd[e], x[e]);
+                if (grad && d < a.v_q) grad[d] = v;
+            }
         }
     }
     const double loss = block_sum((double)loss_t, s_red), qg = block_sum((double)qg_t, s_red);
     if (threadIdx.x == 0) a.loss[(size_t)b * a.K_max + j] = (float)loss;
-    if (grad) {
-        // every thread revisits the ids it wrote itself: no barrier for the parked values
-        const float gbar = (float)qg;
+    if (!grad) return;
+    // every thread revisits the ids it wrote itself: no barrier for the parked values
+    const float gbar = (float)qg;
+    if (VEC4) {
+#pragma unroll 4
+        for (int d = threadIdx.x * 4; d < a.v_q; d += THREADS * 4) {
+            const float4 v = __ldg((const float4 *)(q + d));
+            float4 g = *(float4 *)(grad + d);
+            g.x = fmaf(-v.x, gbar, g.x); g.y = fmaf(-v.y, gbar, g.y); g.z = fmaf(-v.z, gbar, g.z); g.w = fmaf(-v.w, gbar, g.w);
+            *(float4 *)(grad + d) = g;
+        }
+    } else {
 #pragma unroll 4
         for (int d = threadIdx.x; d < a.v_q; d += THREADS) grad[d] = fmaf(-__ldg(q + d), gbar, grad[d]);
     }
 }
 
-template <int DTYPE, bool VEC4>
+template <int DTYPE, bool VEC4, bool SAME>
 cudaError_t launch_chunks(const DistillArgs &a, int C, bool pdl, cudaStream_t s)
 {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)C, (unsigned)a.K_max, (unsigned)a.B);
     cfg.blockDim = dim3(THREADS);
-    cfg.dynamicSmemBytes = (size_t)a.chunk * (DTYPE == OD_BF16 ? 2 : 4);
+    cfg.dynamicSmemBytes = SAME && !a.grad ? 0 : (size_t)a.chunk * (DTYPE == OD_BF16 ? 2 : 4);
     cfg.stream = s;
     cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -417,8 +520,17 @@ cudaError_t launch_chunks(const DistillArgs &a, int C, bool pdl, cudaStream_t s)
     attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-        cfg.numAttrs = pdl ? 2 : 1;
-    return cudaLaunchKernelEx(&cfg, od_distill_kernel<DTYPE, VEC4>, a);
+    cfg.numAttrs = pdl ? 2 : 1;
+    return cudaLaunchKernelEx(&cfg, od_distill_kernel<DTYPE, VEC4, SAME>, a);
+}
+template <int DTYPE, bool VEC4>
+cudaError_t launch(const DistillArgs &a, int C, bool same, bool pdl, cudaStream_t s)
+{
+    if (C == 0) {
+        od_distill_position_kernel<DTYPE, VEC4><<<dim3((unsigned)a.K_max, (unsigned)a.B), THREADS, 0, s>>>(a);
+        return cudaGetLastError();
+    }
+    return same ? launch_chunks<DTYPE, VEC4, true>(a, C, pdl, s) : launch_chunks<DTYPE, VEC4, false>(a, C, pdl, s);
 }
 
 // draft ids per chunk for a vocabulary cut into C = 1 << level chunks: whole words of the mapped
@@ -444,29 +556,33 @@ cudaError_t od_launch_distill(od_ctx *c, int32_t B, int32_t K_max, const float *
     a.span_len = span_len; a.m = m; a.logits = logits; a.row_stride = row_stride; a.seq_stride = seq_stride;
     a.row_max = row_max; a.row_sum = row_sum; a.p_sel = p_sel; a.temperature = temperature;
     a.vocab_map = c->d_vocab_map; a.lambda = lambda; a.lambda_mode = lambda_mode; a.loss = loss; a.grad = grad;
-    const bool bf = dtype == OD_BF16;
+    const bool bf = dtype == OD_BF16, same = c->map_same_ids, pdl = c->opt_pdl != 0;
     const bool vec4 = c->v_q % 4 == 0 && ((uintptr_t)q_rows & 15u) == 0 && (!grad || ((uintptr_t)grad & 15u) == 0);
-    // The number of chunks: the fewest with which a chunk's logits take 36 KB or less (32000 bf16
-    // ids in two chunks of 32 KB: 34.9 us, in one of 64 KB: 44.7, in four: 38 us), more while all
-    // blocks still fit one resident wave (a few positions: 5 x 10 at v_q = 32000 takes 8 chunks).
+    // The number of chunks: the fewest with which a chunk's logits take 36 KB or less (what is left of
+    // a multiprocessor's memory is the L1 that the gather lives on: 32000 bf16 ids in two chunks of
+    // 32 KB 34.9 us, in one of 64 KB 44.7, in four 38), more while all blocks still fit one resident
+    // wave (a few positions: 5 x 10 at v_q = 32000 takes 8 chunks).
     int level = 0;
     const auto more = [&](int l) { return l + 1 < OD_DISTILL_LEVELS; };
-    while (more(level) && chunk_ids(c->v_q, level) * (bf ? 2 : 4) > CHUNK_BYTES) ++level;
-    while (more(level) && (int64_t)B * K_max * 2 << level <= (int64_t)c->sm_count * 3) ++level;
-    const int C = 1 << level;
+    const int64_t positions = (int64_t)B * K_max, wave = (int64_t)c->sm_count * 3;
+    while (more(level) && !(same && !grad) && chunk_ids(c->v_q, level) * (bf ? 2 : 4) > (same ? 2 : 1) * CHUNK_BYTES) ++level;
+    while (more(level) && positions * 2 << level <= wave) ++level;
     a.chunk = chunk_ids(c->v_q, level);
-    if (a.chunk > OD_DISTILL_MAX_CHUNK_IDS) {
-        const dim3 grid(1, (unsigned)K_max, (unsigned)B);
-        if (bf) od_distill_any_kernel<OD_BF16><<<grid, THREADS, 0, s>>>(a);
-        else od_distill_any_kernel<OD_F32><<<grid, THREADS, 0, s>>>(a);
-        return cudaGetLastError();
-    }
+    // One block per position instead where the chunks would not fit, or where the target row is so
+    // short that the gather in draft order finds its lines in L1 and there are positions enough
+    // (128 x 10, v_q = 32000, 22400 ids mapped, v_p = 34330 / 45000 / 64000 / 128000: without a gradient
+    // 43 / 32 / 34 / 45 us against 55 / 36 / 36 / 40, with one 80 / 59 / 65 us against 81 / 53 / 54),
+    // or where target ids are draft ids, so that the gather is coalesced as it stands (64 x 6 at 32000:
+    // 27.8 us against 28.2, without a gradient 16.6 against 19.0; 5 x 6: 12.4 against 5.5).
+    const int64_t short_row = c->n_mapped * (grad ? 9 : 16) / 5;
+    int C = 1 << level;
+    if ((a.chunk > OD_DISTILL_MAX_CHUNK_IDS && !(same && !grad)) ||
+        (!same && c->v_p < short_row && positions >= wave) || (same && vec4 && positions >= c->sm_count * 2)) C = 0;
     const OdDistillLists l = od_distill_lists(c->d_distill_lists, c->v_q, c->v_p);
     a.list_word = l.word + (size_t)level * l.groups * 32; a.list_base = l.base + (size_t)level * l.groups;
     a.list_ofs = l.ofs + level * OD_DISTILL_MAX_CHUNKS * 2; a.mapped_bits = l.bits;
-    const bool pdl = c->opt_pdl != 0;
-    if (vec4) return bf ? launch_chunks<OD_BF16, true>(a, C, pdl, s) : launch_chunks<OD_F32, true>(a, C, pdl, s);
-    return bf ? launch_chunks<OD_BF16, false>(a, C, pdl, s) : launch_chunks<OD_F32, false>(a, C, pdl, s);
+    if (vec4) return bf ? launch<OD_BF16, true>(a, C, same, pdl, s) : launch<OD_F32, true>(a, C, same, pdl, s);
+    return bf ? launch<OD_BF16, false>(a, C, same, pdl, s) : launch<OD_F32, false>(a, C, same, pdl, s);
 }
 
 // The kernels' dynamic shared memory (a chunk of a draft vocabulary of v_q ids): opt in where it
@@ -475,10 +591,14 @@ cudaError_t od_distill_prepare_device(int32_t v_q)
 {
     const int n = OD_DISTILL_MAX_CHUNK_IDS * 4;
     if (chunk_ids(v_q, 0) * 4 <= 48 * 1024) return cudaSuccess;
-    cudaError_t e = cudaFuncSetAttribute(od_distill_kernel<OD_BF16, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, n);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(od_distill_kernel<OD_F32, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, n);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(od_distill_kernel<OD_BF16, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, n);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(od_distill_kernel<OD_F32, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, n);
+    cudaError_t e = cudaFuncSetAttribute(od_distill_kernel<OD_BF16, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, n);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(od_distill_kernel<OD_F32, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, n);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(od_distill_kernel<OD_BF16, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, n);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(od_distill_kernel<OD_F32, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, n);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(od_distill_kernel<OD_BF16, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, n);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(od_distill_kernel<OD_F32, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, n);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(od_distill_kernel<OD_BF16, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, n);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(od_distill_kernel<OD_F32, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, n);
     return e;
 }
 
