@@ -53,8 +53,12 @@ struct TrimState {
     unsigned int k;             // entries to drop in this trim
     unsigned int invalid;       // malformed candidates seen by od_cache_insert
     unsigned int dropped;       // candidates that found no free slot on their whole probe sequence
-    unsigned int n_live;        // entries of the dense list
-    unsigned long long hi_and, hi_or;   // AND / OR of (new?, score) over the live entries: bits that never vary
+    // what the pass over the table finds out; two, used in turn: a trim resets the next one's
+    struct Live {
+        unsigned int n;         // entries of the dense list
+        unsigned long long hi_and, hi_or;   // AND / OR of (new?, score) over the live entries: bits that never vary
+    } live[2];
+    unsigned long long thr_hi, thr_lo;      // trim_select_kernel: the k-th order key
     SelState sel[PASSES + 1];   // sel[p]: written by block 0 of pass p (sel[PASSES]: by the rebuild)
     unsigned int n_out[PASSES]; // entries pass p copied into its output list
     unsigned int hist[PASSES][256];
@@ -158,11 +162,19 @@ __global__ void insert_claim_kernel(int32_t N, int32_t v_q, int32_t v_p, const i
             if (head[h] == 0ull || head[h] == key) s0 = h;
         for (int s = s0; s < OD_GROUP; ++s) {
             const int64_t slot = (int64_t)(g * OD_GROUP + s);
-            unsigned long long cur = keys[slot];
-            if (cur == 0ull) cur = atomicCAS(keys + slot, 0ull, key);   // 0 again: the slot is ours
+            // the slot as it was read with its group: empty, or the candidate's run (then its value tells
+            // whether it is an entry or another candidate's claim); a slot that was empty has no value
+            unsigned long long seen = 0ull;
+            if (s < HEAD) {
+#pragma unroll
+                for (int h = 0; h < HEAD; ++h) seen = h == s ? head[h] : seen;
+            } else {
+                seen = keys[slot];
+            }
+            const unsigned long long cur = seen == 0ull ? atomicCAS(keys + slot, 0ull, key) : seen;
             if (cur == 0ull || cur == key) {
                 // an entry with a value was there before this batch: nothing to add
-                if (((volatile const int32_t *)vals)[slot] < 0) {
+                if (seen == 0ull || ((volatile const int32_t *)vals)[slot] < 0) {
                     atomicMin(owner + slot, (unsigned int)i);
                     cand_slot[i] = (int32_t)slot;
                 }
@@ -191,14 +203,14 @@ __global__ void insert_commit_kernel(int32_t N, const int32_t *__restrict__ targ
     atomicAdd(&st->size, 1u);
 }
 
+__device__ __forceinline__ void reset_live(TrimState::Live &l) { l.n = 0u; l.hi_and = ~0ull; l.hi_or = 0ull; }
+
 __global__ void trim_begin_kernel(TrimState *st, unsigned int max_entries)
 {
     chain_wait();
     const unsigned int k = st->size > max_entries ? st->size - max_entries : 0u;
     if (threadIdx.x == 0) {
         st->k = k;
-        st->n_live = 0u;
-        st->hi_and = ~0ull; st->hi_or = 0ull;
         SelState z = {};
         z.k_rem = k;
         st->sel[0] = z;
@@ -230,12 +242,14 @@ __device__ __forceinline__ unsigned int block_offsets(unsigned int n, unsigned i
 }
 
 // One pass over the table: every live entry goes into the dense list (in no particular
-// order: one append per block and iteration), and the spare table is cleared.
+// order: one append per block and iteration), and the spare table is cleared: its keys and values,
+// which say whether a slot is taken and set (stamp, freq and born of a free slot are never read,
+// and written with the entry). Bound by L2 traffic, of which the empty slots were most: four
+// slots without a key cost no more than their keys.
 __global__ void trim_compact_kernel(int policy, unsigned int clock, const unsigned long long *keys,
                                     const int32_t *vals, const unsigned int *stamp, const unsigned int *freq,
                                     const unsigned int *born, unsigned long long *nkeys, int32_t *nvals,
-                                    unsigned int *nstamp, unsigned int *nfreq, unsigned int *nborn,
-                                    int64_t cap, void *lists, TrimState *st)
+                                    int64_t cap, void *lists, TrimState *st, int which)
 {
     __shared__ unsigned int s_warp[32];
     __shared__ unsigned int s_base;
@@ -244,49 +258,61 @@ __global__ void trim_compact_kernel(int policy, unsigned int clock, const unsign
     const TrimLists L = trim_lists(lists, cap);
     if (threadIdx.x == 0) { s_and = ~0ull; s_or = 0ull; }
     unsigned long long t_and = ~0ull, t_or = 0ull;
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x * 4;
-    for (int64_t slot0 = (int64_t)blockIdx.x * blockDim.x * 4; slot0 < cap; slot0 += stride) {
-        const int64_t slot = slot0 + (int64_t)threadIdx.x * 4;
-        unsigned long long kk[4] = {0ull, 0ull, 0ull, 0ull};
-        int vv[4] = {-1, -1, -1, -1};
-        unsigned int ss[4] = {0, 0, 0, 0}, ff[4] = {0, 0, 0, 0}, bb[4] = {0, 0, 0, 0};
-        if (slot < cap) {                                   // cap is a multiple of 64
-            const ulonglong2 k01 = __ldg((const ulonglong2 *)(keys + slot));
-            const ulonglong2 k23 = __ldg((const ulonglong2 *)(keys + slot) + 1);
-            const int4 v4 = __ldg((const int4 *)(vals + slot));
-            const uint4 s4 = __ldg((const uint4 *)(stamp + slot));
-            const uint4 f4 = __ldg((const uint4 *)(freq + slot));
-            const uint4 b4 = __ldg((const uint4 *)(born + slot));
-            kk[0] = k01.x; kk[1] = k01.y; kk[2] = k23.x; kk[3] = k23.y;
-            vv[0] = v4.x; vv[1] = v4.y; vv[2] = v4.z; vv[3] = v4.w;
-            ss[0] = s4.x; ss[1] = s4.y; ss[2] = s4.z; ss[3] = s4.w;
-            ff[0] = f4.x; ff[1] = f4.y; ff[2] = f4.z; ff[3] = f4.w;
-            bb[0] = b4.x; bb[1] = b4.y; bb[2] = b4.z; bb[3] = b4.w;
-            *(ulonglong2 *)(nkeys + slot) = make_ulonglong2(0ull, 0ull);
-            *((ulonglong2 *)(nkeys + slot) + 1) = make_ulonglong2(0ull, 0ull);
-            *(int4 *)(nvals + slot) = make_int4(-1, -1, -1, -1);
-            *(uint4 *)(nstamp + slot) = make_uint4(0, 0, 0, 0);
-            *(uint4 *)(nfreq + slot) = make_uint4(0, 0, 0, 0);
-            *(uint4 *)(nborn + slot) = make_uint4(0, 0, 0, 0);
-            if ((slot & (OD_GROUP - 1)) == 0) L.grp_fill[slot / OD_GROUP] = 0u;
+    // two vectors of four slots per thread and iteration, one append for both
+    constexpr int NV = 1;
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x * 4 * NV;
+    for (int64_t slot0 = (int64_t)blockIdx.x * blockDim.x * 4 * NV; slot0 < cap; slot0 += stride) {
+        unsigned long long kk[NV][4];
+        int vv[NV][4];
+        uint4 ss[NV], ff[NV], bb[NV];
+#pragma unroll
+        for (int v = 0; v < NV; ++v) {
+            const int64_t slot = slot0 + ((int64_t)v * blockDim.x + threadIdx.x) * 4;
+            kk[v][0] = kk[v][1] = kk[v][2] = kk[v][3] = 0ull;
+            if (slot < cap) {                               // cap is a multiple of 64
+                const ulonglong2 k01 = __ldg((const ulonglong2 *)(keys + slot));
+                const ulonglong2 k23 = __ldg((const ulonglong2 *)(keys + slot) + 1);
+                kk[v][0] = k01.x; kk[v][1] = k01.y; kk[v][2] = k23.x; kk[v][3] = k23.y;
+                *(ulonglong2 *)(nkeys + slot) = make_ulonglong2(0ull, 0ull);
+                *((ulonglong2 *)(nkeys + slot) + 1) = make_ulonglong2(0ull, 0ull);
+                *(int4 *)(nvals + slot) = make_int4(-1, -1, -1, -1);
+                if ((slot & (OD_GROUP - 1)) == 0) L.grp_fill[slot / OD_GROUP] = 0u;
+            }
         }
         unsigned int n = 0;
 #pragma unroll
-        for (int e = 0; e < 4; ++e) n += (kk[e] != 0ull && vv[e] >= 0) ? 1u : 0u;
+        for (int v = 0; v < NV; ++v) {
+            const int64_t slot = slot0 + ((int64_t)v * blockDim.x + threadIdx.x) * 4;
+            vv[v][0] = vv[v][1] = vv[v][2] = vv[v][3] = -1;
+            if ((kk[v][0] | kk[v][1] | kk[v][2] | kk[v][3]) != 0ull) {
+                const int4 v4 = __ldg((const int4 *)(vals + slot));
+                ss[v] = __ldg((const uint4 *)(stamp + slot));
+                ff[v] = __ldg((const uint4 *)(freq + slot));
+                bb[v] = __ldg((const uint4 *)(born + slot));
+                vv[v][0] = v4.x; vv[v][1] = v4.y; vv[v][2] = v4.z; vv[v][3] = v4.w;
+            }
+#pragma unroll
+            for (int e = 0; e < 4; ++e) n += (kk[v][e] != 0ull && vv[v][e] >= 0) ? 1u : 0u;
+        }
         unsigned int total;
         unsigned int at = block_offsets(n, s_warp, total);
-        if (threadIdx.x == 0) s_base = total ? atomicAdd(&st->n_live, total) : 0u;
+        if (threadIdx.x == 0) s_base = total ? atomicAdd(&st->live[which].n, total) : 0u;
         __syncthreads();
         at += s_base;
 #pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            if (kk[e] == 0ull || vv[e] < 0) continue;
-            unsigned long long hi, lo;
-            order_key(policy, clock, kk[e], ss[e], ff[e], bb[e], hi, lo);
-            t_and &= hi; t_or |= hi;
-            L.r_hi[at] = hi; L.r_key[at] = lo;
-            L.r_val[at] = vv[e]; L.r_stamp[at] = ss[e]; L.r_freq[at] = ff[e]; L.r_born[at] = bb[e];
-            ++at;
+        for (int v = 0; v < NV; ++v) {
+            const unsigned int s4[4] = {ss[v].x, ss[v].y, ss[v].z, ss[v].w}, f4[4] = {ff[v].x, ff[v].y, ff[v].z, ff[v].w};
+            const unsigned int b4[4] = {bb[v].x, bb[v].y, bb[v].z, bb[v].w};
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                if (kk[v][e] == 0ull || vv[v][e] < 0) continue;
+                unsigned long long hi, lo;
+                order_key(policy, clock, kk[v][e], s4[e], f4[e], b4[e], hi, lo);
+                t_and &= hi; t_or |= hi;
+                L.r_hi[at] = hi; L.r_key[at] = lo;
+                L.r_val[at] = vv[v][e]; L.r_stamp[at] = s4[e]; L.r_freq[at] = f4[e]; L.r_born[at] = b4[e];
+                ++at;
+            }
         }
     }
     // which bits of (new?, score) vary at all: AND and OR over the live entries
@@ -297,8 +323,181 @@ __global__ void trim_compact_kernel(int policy, unsigned int clock, const unsign
     }
     if ((threadIdx.x & 31) == 0) { atomicAnd(&s_and, t_and); atomicOr(&s_or, t_or); }
     __syncthreads();
-    if (threadIdx.x == 0) { atomicAnd(&st->hi_and, s_and); atomicOr(&st->hi_or, s_or); }
+    if (threadIdx.x == 0) { atomicAnd(&st->live[which].hi_and, s_and); atomicOr(&st->live[which].hi_or, s_or); }
 }
+
+// ---- the k-th order key in one launch ------------------------------------------------------
+//
+// One cluster of P blocks, each with a slice of the dense list: a most-significant-digit radix
+// select in which a pass is a histogram in shared memory, ONE cluster barrier and the sum of the
+// P histograms over distributed shared memory, by every block alike. The digits of (new?, score)
+// that vary are settled first, over the slices; the keys of the entries that tie at that score
+// then stay in shared memory for the eight bytes of the run key, and the select ends as soon as
+// every candidate that is left is among the k (usually two bytes into the run's ids). As a chain
+// of 13 launches of the whole grid, two dependent round trips and a launch each, the passes were
+// 52 of the 107 us of an insertion, a trim and a translation (262144 entries, 16384 new ones).
+constexpr int SELECT_THREADS = 1024, SELECT_MAX_BLOCKS = 16;
+
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+__device__ __forceinline__ unsigned int cluster_load(const unsigned int *p, uint32_t rank)
+{
+    uint32_t at;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(at) : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(rank));
+    unsigned int v;
+    asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(at) : "memory");
+    return v;
+}
+
+// Count digit `d` of the lanes with `ok` into hist: digits are heavily tied (scores, the upper
+// bytes of short runs), so lanes that agree count as one add.
+__device__ __forceinline__ void count_digit(unsigned int *hist, unsigned int d, bool ok)
+{
+    const unsigned int same = __match_any_sync(0xFFFFFFFFu, ok ? d : 256u);
+    if (ok && __ffs(same) - 1 == (int)(threadIdx.x & 31)) atomicAdd(hist + d, (unsigned int)__popc(same));
+}
+
+__global__ void __launch_bounds__(SELECT_THREADS, 1)
+trim_select_kernel(unsigned int max_entries, unsigned int room, int64_t cap, void *lists, TrimState *st, int which)
+{
+    extern __shared__ __align__(16) unsigned long long s_keys[];   // [room]
+    __shared__ unsigned int s_hist[2][256], s_sum[256];
+    __shared__ unsigned int s_n, s_digit, s_run, s_in;
+    const unsigned int P = gridDim.x, rank = blockIdx.x, lane = threadIdx.x & 31u;
+    chain_wait();
+    const unsigned int size = __ldcg(&st->size), k = size > max_entries ? size - max_entries : 0u;
+    const unsigned int n = __ldcg(&st->live[which].n);
+    const unsigned long long hi_and = __ldcg(&st->live[which].hi_and), hi_or = __ldcg(&st->live[which].hi_or);
+    if (k == 0u) {                                          // nothing to drop: every block leaves
+        if (rank == 0 && threadIdx.x == 0) { st->k = 0u; reset_live(st->live[which ^ 1]); }
+        return;
+    }
+    const TrimLists L = trim_lists(lists, cap);
+    const unsigned int per = (n + P - 1) / P, lo = min(rank * per, n), hi_end = min(lo + per, n);
+    for (int i = threadIdx.x; i < 512; i += SELECT_THREADS) s_hist[i >> 8][i & 255] = 0u;
+    if (threadIdx.x == 0) s_n = 0u;
+    __syncthreads();
+
+    unsigned int k_rem = k, n_match = n, buf = 0;
+    // the first digit at which the running count over all blocks reaches k_rem
+    auto settle = [&]() -> unsigned int {
+        cluster_arrive(); cluster_wait();                   // every block's histogram is complete
+        if (threadIdx.x < 256) {
+            unsigned int h[SELECT_MAX_BLOCKS], t = 0;       // all loads before the first use: one trip, not P
+#pragma unroll
+            for (unsigned int r = 0; r < SELECT_MAX_BLOCKS; ++r) h[r] = r < P ? cluster_load(&s_hist[buf][threadIdx.x], r) : 0u;
+#pragma unroll
+            for (unsigned int r = 0; r < SELECT_MAX_BLOCKS; ++r) t += h[r];
+            s_sum[threadIdx.x] = t;
+            s_hist[buf ^ 1][threadIdx.x] = 0u;              // (read by the others before the barrier above)
+        }
+        __syncthreads();
+        if (threadIdx.x < 32) {
+            unsigned int mine = 0;
+#pragma unroll
+            for (int i = 0; i < 8; ++i) mine += s_sum[lane * 8 + i];
+            unsigned int inc = mine;
+#pragma unroll
+            for (int off = 1; off < 32; off <<= 1) {
+                const unsigned int v = __shfl_up_sync(0xFFFFFFFFu, inc, off);
+                if (lane >= (unsigned)off) inc += v;
+            }
+            const unsigned int reach = __ballot_sync(0xFFFFFFFFu, inc >= k_rem);
+            const unsigned int owner = reach ? __ffs(reach) - 1 : 31;
+            if (lane == owner) {
+                unsigned int run = inc - mine, d = lane * 8;
+                for (; d < lane * 8 + 7 && run + s_sum[d] < k_rem; ++d) run += s_sum[d];
+                s_digit = d; s_run = run; s_in = s_sum[d];
+            }
+        }
+        __syncthreads();
+        buf ^= 1u;
+        k_rem -= s_run; n_match = s_in;
+        return s_digit;
+    };
+
+    // ---- (new?, score): the bits that vary, over the slice
+    const unsigned long long vary = hi_or & ~hi_and;
+    unsigned long long thr_hi = hi_and, known = ~vary;
+    for (int byte = 4; byte >= 0; --byte) {
+        if ((vary >> (8 * byte) & 0xFFull) == 0ull) continue;
+        constexpr int U = 9;
+        for (unsigned int i0 = lo; i0 < hi_end; i0 += SELECT_THREADS * U) {
+            unsigned long long h[U];
+#pragma unroll
+            for (int e = 0; e < U; ++e) {
+                const unsigned int i = i0 + e * SELECT_THREADS + threadIdx.x;
+                h[e] = i < hi_end ? __ldcg(L.r_hi + i) : 0ull;
+            }
+#pragma unroll
+            for (int e = 0; e < U; ++e)
+                count_digit(s_hist[buf], (unsigned int)(h[e] >> (8 * byte)) & 0xFFu,
+                            i0 + e * SELECT_THREADS + threadIdx.x < hi_end && (h[e] & known) == (thr_hi & known));
+        }
+        const unsigned int d = settle();
+        thr_hi = (thr_hi & ~(0xFFull << (8 * byte))) | (unsigned long long)d << (8 * byte);
+        known |= 0xFFull << (8 * byte);
+    }
+    // ---- the run keys of the entries that tie at that score
+    unsigned long long thr_lo = 0ull, decided = 0ull;
+    if (n_match > k_rem) {
+        constexpr int U = 9;
+        for (unsigned int i0 = lo; i0 < hi_end; i0 += SELECT_THREADS * U) {
+            unsigned long long h[U], key[U];
+#pragma unroll
+            for (int e = 0; e < U; ++e) {
+                const unsigned int i = i0 + e * SELECT_THREADS + threadIdx.x;
+                h[e] = i < hi_end ? __ldcg(L.r_hi + i) : ~thr_hi;
+            }
+#pragma unroll
+            for (int e = 0; e < U; ++e)
+                if (h[e] == thr_hi) key[e] = __ldcg(L.r_key + i0 + e * SELECT_THREADS + threadIdx.x);
+            unsigned int mine = 0;
+#pragma unroll
+            for (int e = 0; e < U; ++e) mine += h[e] == thr_hi ? 1u : 0u;
+            // one append per warp, its lanes in order
+            unsigned int inc = mine;
+#pragma unroll
+            for (int off = 1; off < 32; off <<= 1) {
+                const unsigned int v = __shfl_up_sync(0xFFFFFFFFu, inc, off);
+                if (lane >= (unsigned)off) inc += v;
+            }
+            unsigned int at = 0;
+            if (lane == 31 && inc) at = atomicAdd(&s_n, inc);
+            at = __shfl_sync(0xFFFFFFFFu, at, 31) + inc - mine;
+#pragma unroll
+            for (int e = 0; e < U; ++e)
+                if (h[e] == thr_hi) { if (at < room) s_keys[at] = key[e]; ++at; }
+        }
+        __syncthreads();
+        const bool held = s_n <= room;                      // else the slice is read again (a table trimmed late)
+        const unsigned int c_end = held ? s_n : hi_end - lo;
+        for (int byte = 7; byte >= 0 && n_match > k_rem; --byte) {
+            for (unsigned int i0 = 0; i0 < c_end; i0 += SELECT_THREADS) {
+                const unsigned int i = i0 + threadIdx.x;
+                bool ok = i < c_end;
+                unsigned long long key = 0ull;
+                if (ok) {
+                    key = held ? s_keys[i] : __ldcg(L.r_key + lo + i);
+                    ok = (key & decided) == thr_lo && (held || __ldcg(L.r_hi + lo + i) == thr_hi);
+                }
+                count_digit(s_hist[buf], (unsigned int)(key >> (8 * byte)) & 0xFFu, ok);
+            }
+            const unsigned int d = settle();
+            thr_lo |= (unsigned long long)d << (8 * byte);
+            decided |= 0xFFull << (8 * byte);
+        }
+    }
+    thr_lo |= ~decided;                                     // every candidate left is among the k
+    cluster_arrive(); cluster_wait();                       // nobody leaves while its histogram may still be read
+    if (rank == 0 && threadIdx.x == 0) {
+        st->k = k; st->size = size - k;
+        st->thr_hi = thr_hi; st->thr_lo = thr_lo;
+        reset_live(st->live[which ^ 1]);
+    }
+}
+
+// ---- the same as a chain of launches, for tables too large for one cluster -----------------
 
 // Is digit `pass` the same in every live entry? Only asked for the five bytes of (new?, score).
 __device__ __forceinline__ bool digit_is_constant(int pass, unsigned long long hi_and, unsigned long long hi_or)
@@ -309,11 +508,12 @@ __device__ __forceinline__ bool digit_is_constant(int pass, unsigned long long h
 // The state at the start of pass `pass` (0..PASSES), worked out from the state at the start of
 // the pass before it and that pass's histogram: by every block alike, the same arithmetic on the
 // same numbers. All threads of the block call; s_hist (256 words) and s_sel are its scratch.
-__device__ __forceinline__ SelState select_state(int pass, const TrimState *st, unsigned int *s_hist, SelState *s_sel)
+__device__ __forceinline__ SelState select_state(int pass, const TrimState *st, int which, unsigned int *s_hist, SelState *s_sel)
 {
+    const TrimState::Live &live = st->live[which];
     if (pass == 0) {
         SelState z = st->sel[0];
-        z.n_in = z.n_match = __ldcg(&st->n_live);
+        z.n_in = z.n_match = __ldcg(&live.n);
         return z;
     }
     const int q = pass - 1;                                  // the digit to settle
@@ -325,10 +525,10 @@ __device__ __forceinline__ SelState select_state(int pass, const TrimState *st, 
         t.mask_hi = __ldcg(&g->mask_hi); t.mask_lo = __ldcg(&g->mask_lo);
         t.k_rem = __ldcg(&g->k_rem); t.n_in = __ldcg(&g->n_in);
         t.n_match = __ldcg(&g->n_match); t.cur = __ldcg(&g->cur);
-        if (q == 0) t.n_in = t.n_match = __ldcg(&st->n_live);
+        if (q == 0) t.n_in = t.n_match = __ldcg(&live.n);
         *s_sel = t;
     }
-    const unsigned long long hi_and = __ldcg(&st->hi_and), hi_or = __ldcg(&st->hi_or);
+    const unsigned long long hi_and = __ldcg(&live.hi_and), hi_or = __ldcg(&live.hi_or);
     const unsigned int n_out = __ldcg(&st->n_out[q]);
     __syncthreads();
     if (threadIdx.x < 32) {
@@ -385,7 +585,7 @@ __device__ __forceinline__ SelState select_state(int pass, const TrimState *st, 
 // Pass `pass` of the radix select over the current candidate list: histogram of digit `pass`
 // over the candidates that match the digits decided so far. If those are at most half of the
 // list, they are copied into the other scratch list on the way (the next pass reads that one).
-__global__ void trim_hist_kernel(int pass, int64_t cap, void *lists, TrimState *st)
+__global__ void trim_hist_kernel(int pass, int64_t cap, void *lists, TrimState *st, int which)
 {
     __shared__ unsigned int s_hist[256];
     __shared__ unsigned int s_warp[32];
@@ -393,9 +593,9 @@ __global__ void trim_hist_kernel(int pass, int64_t cap, void *lists, TrimState *
     __shared__ SelState s_sel;
     chain_wait();
     if (st->k == 0u) return;                                 // nothing to drop: every block leaves
-    const SelState S = select_state(pass, st, s_hist, &s_sel);
+    const SelState S = select_state(pass, st, which, s_hist, &s_sel);
     if (blockIdx.x == 0 && threadIdx.x == 0) st->sel[pass] = S;
-    if (digit_is_constant(pass, __ldcg(&st->hi_and), __ldcg(&st->hi_or))) return;   // the next pass fills it in
+    if (digit_is_constant(pass, __ldcg(&st->live[which].hi_and), __ldcg(&st->live[which].hi_or))) return;   // the next pass fills it in
     __syncthreads();
     s_hist[threadIdx.x] = 0u;
     __syncthreads();
@@ -446,17 +646,21 @@ __global__ void trim_hist_kernel(int pass, int64_t cap, void *lists, TrimState *
 // entry gets depends on timing, the set of entries does not
 __global__ void trim_rebuild_kernel(unsigned long long *nkeys, int32_t *nvals, unsigned int *nstamp,
                                     unsigned int *nfreq, unsigned int *nborn, int64_t cap, void *lists,
-                                    const TrimState *st)
+                                    const TrimState *st, int which, int selected)
 {
     __shared__ unsigned int s_hist[256];
     __shared__ SelState s_sel;
     chain_wait();
     const TrimLists L = trim_lists(lists, cap);
-    const unsigned int n = __ldcg(&st->n_live), k = st->k;
+    const unsigned int n = __ldcg(&st->live[which].n), k = st->k;
     unsigned long long thr_hi = 0ull, thr_lo = 0ull;
     if (k > 0u) {                                           // block-uniform
-        const SelState S = select_state(PASSES, st, s_hist, &s_sel);
-        thr_hi = S.pre_hi; thr_lo = S.pre_lo;
+        if (selected) {
+            thr_hi = st->thr_hi; thr_lo = st->thr_lo;
+        } else {
+            const SelState S = select_state(PASSES, st, which, s_hist, &s_sel);
+            thr_hi = S.pre_hi; thr_lo = S.pre_lo;
+        }
     }
     const uint64_t ngroups = (uint64_t)cap / OD_GROUP;
     for (unsigned int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
@@ -482,10 +686,11 @@ __global__ void trim_rebuild_kernel(unsigned long long *nkeys, int32_t *nvals, u
     }
 }
 
-__global__ void trim_end_kernel(TrimState *st)
+__global__ void trim_end_kernel(TrimState *st, int which)
 {
     chain_wait();
     st->size -= st->k; st->k = 0u;
+    reset_live(st->live[which ^ 1]);
 }
 
 #define OD_CUDA(call)                                  \
@@ -508,6 +713,46 @@ int32_t alloc_zero(T **p, size_t n)
     if (e == cudaErrorMemoryAllocation) return OD_ERR_NOMEM;
     if (e != cudaSuccess) return OD_ERR_CUDA;
     return cudaMemset(*p, 0, (n ? n : 1) * sizeof(T)) == cudaSuccess ? OD_OK : OD_ERR_CUDA;
+}
+
+// Room for the tying keys in a block's shared memory: a slice of the entries that one insertion
+// leaves over the bound.
+unsigned int select_room(const od_ctx *c, int blocks)
+{
+    return (unsigned int)((c->dyn_max + c->dyn_max_insert + blocks - 1) / blocks);
+}
+constexpr unsigned int SELECT_ROOM_MAX = 24 * 1024;         // 192 KB
+
+void select_config(cudaLaunchConfig_t &cfg, cudaLaunchAttribute *attr, const od_ctx *c, int blocks)
+{
+    cfg.gridDim = dim3((unsigned)blocks); cfg.blockDim = dim3(SELECT_THREADS);
+    cfg.dynamicSmemBytes = (size_t)select_room(c, blocks) * 8;
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = (unsigned)blocks; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr; cfg.numAttrs = 1;
+}
+
+// Blocks of the one-launch select: a cluster of 16, or of the portable 8, whose shared memory holds
+// the tying keys (393216 / 196608 entries); 0 = the table is too large for it.
+int select_blocks(const od_ctx *c)
+{
+    if (cudaFuncSetAttribute(trim_select_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||
+        cudaFuncSetAttribute(trim_select_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SELECT_ROOM_MAX * 8) != cudaSuccess) {
+        cudaGetLastError();
+        return 0;
+    }
+    for (int blocks = SELECT_MAX_BLOCKS; blocks >= 8; blocks /= 2) {
+        if (select_room(c, blocks) > SELECT_ROOM_MAX) continue;
+        cudaLaunchConfig_t cfg = {};
+        cudaLaunchAttribute attr[2];
+        select_config(cfg, attr, c, blocks);
+        int n = 0;
+        if (cudaOccupancyMaxActiveClusters(&n, trim_select_kernel, &cfg) == cudaSuccess && n > 0) return blocks;
+        cudaGetLastError();
+    }
+    return 0;
 }
 
 }  // namespace
@@ -565,8 +810,14 @@ int32_t od_cache_configure(od_ctx *c, int64_t max_entries, int32_t policy, int32
     OD_CUDA(cudaMemset(c->d_owner, 0xFF, (size_t)cap * sizeof(uint32_t)));
     c->cap = cap;
     c->table_written = true;
+    TrimState *dst = (TrimState *)c->d_trim;
+    const TrimState::Live empty = {0u, ~0ull, 0ull};
+    OD_CUDA(cudaMemcpy(&dst->live[0], &empty, sizeof(empty), cudaMemcpyHostToDevice));
+    OD_CUDA(cudaMemcpy(&dst->live[1], &empty, sizeof(empty), cudaMemcpyHostToDevice));
+    c->trim_turn = 0;
     c->dyn = true; c->dyn_policy = policy; c->dyn_max = max_entries; c->dyn_max_insert = max_insert;
     c->clock = 0;
+    c->trim_blocks = select_blocks(c);
     return OD_OK;
 }
 
@@ -613,21 +864,33 @@ int32_t od_cache_trim(od_ctx *c, void *stream)
     c->last_was_map = false;
     c->table_written = true;
     TrimState *st = (TrimState *)c->d_trim;
-    const int grid = c->sm_count * 4;
+    const int grid = c->sm_count * 4, which = c->trim_turn;
     const bool pdl = c->opt_pdl != 0;
-    OD_CUDA(chain_launch(trim_begin_kernel, 1u, 256u, s, pdl, st, (unsigned int)c->dyn_max));
+    const int blocks = c->trim_blocks;                      // 0: the select is a chain of launches
+    if (!blocks) OD_CUDA(chain_launch(trim_begin_kernel, 1u, 256u, s, pdl, st, (unsigned int)c->dyn_max));
     OD_CUDA(chain_launch(trim_compact_kernel, (unsigned)grid, 256u, s, pdl, c->dyn_policy, c->clock,
                          (const unsigned long long *)c->d_keys, (const int32_t *)c->d_vals,
                          (const unsigned int *)c->d_stamp, (const unsigned int *)c->d_freq,
                          (const unsigned int *)c->d_born, (unsigned long long *)c->d_keys2, c->d_vals2,
-                         c->d_stamp2, c->d_freq2, c->d_born2, c->cap, c->d_trim_lists, st));
-    for (int pass = 0; pass < PASSES; ++pass)
-        OD_CUDA(chain_launch(trim_hist_kernel, (unsigned)c->sm_count, 256u, s, pdl, pass, c->cap,
-                             c->d_trim_lists, st));
+                         c->cap, c->d_trim_lists, st, which));
+    if (blocks) {
+        cudaLaunchConfig_t cfg = {};
+        cudaLaunchAttribute attr[2];
+        select_config(cfg, attr, c, blocks);
+        cfg.stream = s;
+        cfg.numAttrs = pdl ? 2 : 1;
+        OD_CUDA(cudaLaunchKernelEx(&cfg, trim_select_kernel, (unsigned int)c->dyn_max, select_room(c, blocks), c->cap,
+                                   c->d_trim_lists, st, which));
+    } else {
+        for (int pass = 0; pass < PASSES; ++pass)
+            OD_CUDA(chain_launch(trim_hist_kernel, (unsigned)c->sm_count, 256u, s, pdl, pass, c->cap,
+                                 c->d_trim_lists, st, which));
+    }
     OD_CUDA(chain_launch(trim_rebuild_kernel, (unsigned)grid, 256u, s, pdl, (unsigned long long *)c->d_keys2,
                          c->d_vals2, c->d_stamp2, c->d_freq2, c->d_born2, c->cap, c->d_trim_lists,
-                         (const TrimState *)st));
-    OD_CUDA(chain_launch(trim_end_kernel, 1u, 1u, s, pdl, st));
+                         (const TrimState *)st, which, blocks ? 1 : 0));
+    if (!blocks) OD_CUDA(chain_launch(trim_end_kernel, 1u, 1u, s, pdl, st, which));
+    c->trim_turn ^= 1;
     // the rebuilt table is the table for every call enqueued from now on
     std::swap(c->d_keys, c->d_keys2); std::swap(c->d_vals, c->d_vals2);
     std::swap(c->d_stamp, c->d_stamp2); std::swap(c->d_freq, c->d_freq2); std::swap(c->d_born, c->d_born2);

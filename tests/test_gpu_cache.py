@@ -127,6 +127,36 @@ def test_full_size_cache_fills_and_trims_to_its_bound(cuda_device):
     ctx.close()
 
 
+# a table of a few entries (blocks of the select without any), ties that overflow the select's shared
+# memory because the trim comes late, ties that fill it, and a table too large for one cluster
+@pytest.mark.parametrize("bound, batch, batches", [(5, 8, 2), (1000, 512, 5), (20000, 8000, 2), (400000, 65536, 8)])
+@pytest.mark.parametrize("policy", [cp.LRU, cp.LFU])
+def test_trim_over_ties(cuda_device, policy, bound, batch, batches):
+    """All scores equal but for the last batch's: the run keys decide."""
+    rng = np.random.default_rng(50)
+    v_q, v_p, dev = 32000, 128256, cuda_device
+    ctx = od.Context(cuda_device, v_q, v_p, 4, 4)
+    ctx.set_vocab_map(np.full(v_q, -1, np.int32))
+    ctx.cache_configure(bound, policy, batch)
+    ref = cp.DynamicCache(bound, policy, v_q, v_p)
+    for turn in range(2):
+        for i in range(batches):
+            clock = 10 * turn + (2 if i == batches - 1 else 1)
+            ctx.cache_set_clock(clock); ref.set_clock(clock)
+            runs, lens = _universe(rng, batch, v_q)
+            tg = rng.integers(0, v_p, size=batch).astype(np.int32)
+            ctx.cache_insert(torch.from_numpy(runs).to(dev), torch.from_numpy(lens).to(dev), torch.from_numpy(tg).to(dev))
+            ref.insert_batch(runs, lens, tg)
+        ctx.cache_trim(); ref.trim()
+        assert len(ref) <= bound and ctx.cache_stats()[0] == len(ref)
+        _compare(ctx, ref)
+        if bound == 400000:
+            break
+    ctx.cache_trim()                                        # nothing to drop
+    _compare(ctx, ref)
+    ctx.close()
+
+
 def test_online_cache_argument_checks(cuda_device):
     ctx = od.Context(cuda_device, 100, 100, 4, 4)
     with pytest.raises(od.OdError) as e:
