@@ -242,7 +242,8 @@ int32_t od_cache_dump(od_ctx *ctx, int64_t max_out, int32_t *runs, int32_t *len,
  * conventions above; default 0),
  * "verify_grid" (thread blocks of od_verify's streaming kernel, 0 = one per
  * multiprocessor, the default), "sample_tiles_per_warp" (256-id tiles one warp of
- * od_sample_residual sums, 0 = automatic). Unknown name: INVALID_ARG. */
+ * od_sample_residual sums, at most: it takes the fewest of 1, 2, 4, 8, 16 blocks per
+ * sequence that keep to it; 0 = automatic). Unknown name: INVALID_ARG. */
 int32_t od_set_option(od_ctx *ctx, const char *name, int64_t value);
 
 /* ---- the step ----------------------------------------------------------- */

@@ -16,16 +16,13 @@
 //           are dropped, score = last-access clock (LRU) or frequency (LFU). One
 //           pass over the table packs the live entries into a dense list (and clears
 //           the spare table); the k-th smallest is found by a most-significant-digit
-//           radix select over the 104-bit order key, 13 passes of a histogram kernel
-//           over the CANDIDATES only: a pass copies the entries that still match the
-//           decided prefix into the next list whenever that at least halves it, so
-//           after the first digit that tells entries apart the passes are a few
-//           hundred entries long. A pass is two dependent memory round trips: every
-//           block works out the digit the pass before it decided from that pass's
-//           256-bin histogram (redundantly, the same arithmetic everywhere), then
-//           histograms its share of the next digit; no tickets, no fences, and a
-//           digit of (new?, score) that is the same in every live entry costs no
-//           histogram at all. Then the survivors are re-inserted from the dense list
+//           radix select over the 104-bit order key, by one cluster of blocks
+//           (trim_select_kernel). Tables too large for that take a chain of 13 histogram
+//           launches over the CANDIDATES only: a pass copies the entries that still match
+//           the decided prefix into the next list whenever that at least halves it, every
+//           block works out the digit the pass before it decided from that pass's 256-bin
+//           histogram, and a digit of (new?, score) that is the same in every live entry
+//           costs no histogram. Then the survivors are re-inserted from the dense list
 //           into the spare table, which becomes the table. No kernel waits for another.
 #include <stddef.h>
 #include <string.h>
