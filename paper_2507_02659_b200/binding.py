@@ -4,6 +4,10 @@ Only argument marshalling lives here: tensors become raw device pointers, the
 current torch stream becomes the `stream` argument, status codes become
 exceptions. Every step of the path runs inside the CUDA library; there is no
 CPU fallback: if the library is missing or a call fails, this module raises.
+
+The calls of a decode loop go through `_marshal` (csrc/marshal.cpp), which looks at the
+tensors natively; where it finds an argument that the call does not take as it stands, it calls
+nothing, and the checks here say what is wrong.
 """
 from __future__ import annotations
 
@@ -45,11 +49,12 @@ class OdError(RuntimeError):
 
 
 _lib = None
+_native = None              # the _marshal extension, loaded with the library
 
 
 def lib():
     """The loaded library. Raises if it has not been built."""
-    global _lib
+    global _lib, _native
     if _lib is None:
         if not os.path.exists(_LIB_PATH):
             raise RuntimeError(
@@ -91,6 +96,8 @@ def lib():
         for name in EXPORTS:
             if name not in ("od_status_string", "od_last_launch_info"):
                 getattr(L, name).restype = i32
+        from . import _marshal
+        _native = _marshal
         _lib = L
     return _lib
 
@@ -141,6 +148,7 @@ class Context:
         h = C.c_void_p()
         _check(lib().od_create(C.byref(h), idx, draft_vocab, target_vocab, max_batch, max_k), "od_create")
         self.handle = h
+        self.address, self.index = h.value, idx     # what _marshal takes
         self.draft_vocab, self.target_vocab = draft_vocab, target_vocab
         self.max_batch, self.max_k = max_batch, max_k
 
@@ -148,6 +156,7 @@ class Context:
         if getattr(self, "handle", None):
             lib().od_destroy(self.handle)
             self.handle = None
+            self.address = 0
 
     def __del__(self):
         try:
@@ -184,10 +193,16 @@ class Context:
         N = int(run_len.shape[0])
         if tuple(runs.shape) != (N, 4) or run_target.shape[0] != N:
             raise ValueError("candidates must be runs [N, 4], len [N], target [N]")
+        status = _native.cache_insert(self.address, self.index, N, runs, run_len, run_target)
+        if status is not None:
+            return _check(status, "od_cache_insert")
         _check(lib().od_cache_insert(self.handle, N, _dp(runs, i32, d), _dp(run_len, i32, d),
                                      _dp(run_target, i32, d), _stream(d)), "od_cache_insert")
 
     def cache_trim(self):
+        status = _native.cache_trim(self.address, self.index)
+        if status is not None:
+            return _check(status, "od_cache_trim")
         _check(lib().od_cache_trim(self.handle, _stream(self.device)), "od_cache_trim")
 
     def cache_stats(self):
@@ -278,6 +293,11 @@ def _strides(logits: torch.Tensor, B: int, K: int, v_p: int):
 def od_map_proposals(ctx: Context, draft_ids, draft_len, q_sel, out: Optional[MapOut] = None) -> MapOut:
     B, K = draft_ids.shape
     out = out or alloc_map_out(ctx, B, K)
+    status = _native.map_proposals(ctx.address, ctx.index, B, K, draft_ids, draft_len, q_sel, out.tgt_ids, out.q_prime,
+                                   out.span_start, out.span_len, out.m, out.tail_kind, out.counters)
+    if status is not None:
+        _check(status, "od_map_proposals")
+        return out
     d, i32, f32 = ctx.device, torch.int32, torch.float32
     _check(lib().od_map_proposals(
         ctx.handle, B, K, _dp(draft_ids, i32, d), _dp(draft_len, i32, d), _dp(q_sel, f32, d),
@@ -291,6 +311,12 @@ def od_verify(ctx: Context, logits, mp: MapOut, temperature, seed, step: int,
               out: Optional[VerifyOut] = None) -> VerifyOut:
     B, K = mp.tgt_ids.shape
     out = out or alloc_verify_out(ctx, B, K)
+    status = _native.verify(ctx.address, ctx.index, B, K, ctx.target_vocab, logits, mp.tgt_ids, mp.q_prime, mp.span_len,
+                            mp.m, temperature, seed, step, out.row_max, out.row_sum, out.p_sel, out.ratio,
+                            out.n_accepted, out.n_draft_accepted, out.flags)
+    if status is not None:
+        _check(status, "od_verify")
+        return out
     d, i32, f32 = ctx.device, torch.int32, torch.float32
     rs, ss = _strides(logits, B, K, ctx.target_vocab)
     if logits.device != d:
@@ -331,11 +357,17 @@ def od_distill_loss(ctx: Context, q_rows, draft_ids, mp: MapOut, logits, vo: Ver
     """Eq. (3) per draft position: (loss f32 [B, K], grad f32 [B, K, V_q] or None)."""
     B, K = mp.tgt_ids.shape
     d, i32, f32 = ctx.device, torch.int32, torch.float32
-    rs, ss = _strides(logits, B, K, ctx.target_vocab)
     if loss is None:
         loss = torch.zeros(B, K, dtype=f32, device=d)
     if grad is None and want_grad:
         grad = torch.empty(B, K, ctx.draft_vocab, dtype=f32, device=d)
+    status = _native.distill_loss(ctx.address, ctx.index, B, K, ctx.target_vocab, q_rows, draft_ids, mp.tgt_ids,
+                                  mp.span_start, mp.span_len, mp.m, logits, vo.row_max, vo.row_sum, vo.p_sel, temperature,
+                                  lam, lambda_mode, loss, grad)
+    if status is not None:
+        _check(status, "od_distill_loss")
+        return loss, grad
+    rs, ss = _strides(logits, B, K, ctx.target_vocab)
     _check(lib().od_distill_loss(
         ctx.handle, B, K, _dp(q_rows, f32, d), _dp(draft_ids, i32, d), _dp(mp.tgt_ids, i32, d),
         _dp(mp.span_start, i32, d), _dp(mp.span_len, i32, d), _dp(mp.m, i32, d),
@@ -349,9 +381,14 @@ def od_exit_rule(ctx: Context, head_logits, avail_len, gamma: float):
     """Eq. (4)-(6): (draft_len int32 [B], reject_prob f32 [B, K], exit_flags int32 [B])."""
     B, K = head_logits.shape
     d, i32, f32 = ctx.device, torch.int32, torch.float32
-    draft_len = torch.zeros(B, dtype=i32, device=d)
-    reject = torch.zeros(B, K, dtype=f32, device=d)
-    flags = torch.zeros(B, dtype=i32, device=d)
+    # (the kernel writes every element)
+    draft_len = torch.empty(B, dtype=i32, device=d)
+    reject = torch.empty(B, K, dtype=f32, device=d)
+    flags = torch.empty(B, dtype=i32, device=d)
+    status = _native.exit_rule(ctx.address, ctx.index, B, K, head_logits, avail_len, gamma, draft_len, reject, flags)
+    if status is not None:
+        _check(status, "od_exit_rule")
+        return draft_len, reject, flags
     _check(lib().od_exit_rule(ctx.handle, B, K, _dp(head_logits, f32, d), _dp(avail_len, i32, d),
                               C.c_float(gamma), _dp(draft_len, i32, d), _dp(reject, f32, d),
                               _dp(flags, i32, d), _stream(d)), "od_exit_rule")
@@ -362,6 +399,13 @@ def od_sample_residual(ctx: Context, logits, vo: VerifyOut, q_rows, draft_ids, m
                        temperature, seed, step: int, out: Optional[SampleOut] = None) -> SampleOut:
     B, K = mp.tgt_ids.shape
     out = out or alloc_sample_out(ctx, B)
+    status = _native.sample_residual(ctx.address, ctx.index, B, K, ctx.draft_vocab, ctx.target_vocab, logits, vo.row_max,
+                                     vo.row_sum, q_rows, draft_ids, mp.tgt_ids, mp.q_prime, mp.span_start, mp.span_len, mp.m,
+                                     mp.tail_kind, vo.n_accepted, temperature, seed, step, out.out_token, out.resid_mass,
+                                     out.flags)
+    if status is not None:
+        _check(status, "od_sample_residual")
+        return out
     d, i32, f32 = ctx.device, torch.int32, torch.float32
     rs, ss = _strides(logits, B, K, ctx.target_vocab)
     if logits.device != d:
@@ -387,6 +431,13 @@ def od_step(ctx: Context, s_draft_ids, s_draft_len, s_q_sel, s_q_rows, logits, t
     mp = mp or alloc_map_out(ctx, B, K)
     vo = vo or alloc_verify_out(ctx, B, K)
     so = so or alloc_sample_out(ctx, B)
+    status = _native.step(ctx.address, ctx.index, B, K, ctx.draft_vocab, ctx.target_vocab, s_draft_ids, s_draft_len, s_q_sel,
+                          s_q_rows, logits, temperature, seed, step, mp.tgt_ids, mp.q_prime, mp.span_start, mp.span_len,
+                          mp.m, mp.tail_kind, mp.counters, vo.row_max, vo.row_sum, vo.p_sel, vo.ratio, vo.n_accepted,
+                          vo.n_draft_accepted, vo.flags, so.out_token, so.resid_mass, so.flags)
+    if status is not None:
+        _check(status, "od_step")
+        return mp, vo, so
     d, i32, f32 = ctx.device, torch.int32, torch.float32
     rs, ss = _strides(logits, B, K, ctx.target_vocab)
     if logits.device != d:
@@ -424,6 +475,11 @@ def od_verify_shard_stats(ctx: Context, shard_lo: int, logits, mp: MapOut, tempe
     rs, ss = _shard_strides(logits, B, K, shard_len)
     if out is None:
         out = torch.zeros(B, K + 1, 4, dtype=f32, device=d)
+    status = _native.verify_shard_stats(ctx.address, ctx.index, B, K, shard_lo, shard_len, logits, mp.tgt_ids, mp.m,
+                                        temperature, out)
+    if status is not None:
+        _check(status, "od_verify_shard_stats")
+        return out
     _check(lib().od_verify_shard_stats(
         ctx.handle, B, K, shard_lo, shard_len, C.c_void_p(logits.data_ptr()), logit_dtype_code(logits),
         rs, ss, _dp(mp.tgt_ids, i32, d), _dp(mp.m, i32, d), _dp(temperature, f32, d), _dp(out, f32, d),
@@ -438,6 +494,12 @@ def od_verify_shard_finish(ctx: Context, stats_all: torch.Tensor, mp: MapOut, te
     if stats_all.dim() != 4 or tuple(stats_all.shape[1:]) != (B, K + 1, 4):
         raise ValueError("stats_all must be [n_shards, B, K+1, 4]")
     out = out or alloc_verify_out(ctx, B, K)
+    status = _native.verify_shard_finish(ctx.address, ctx.index, B, K, stats_all.shape[0], stats_all, mp.tgt_ids, mp.q_prime,
+                                         mp.span_len, mp.m, temperature, seed, step, out.row_max, out.row_sum, out.p_sel,
+                                         out.ratio, out.n_accepted, out.n_draft_accepted, out.flags)
+    if status is not None:
+        _check(status, "od_verify_shard_finish")
+        return out
     d, i32, f32 = ctx.device, torch.int32, torch.float32
     _check(lib().od_verify_shard_finish(
         ctx.handle, B, K, int(stats_all.shape[0]), _dp(stats_all, f32, d),
@@ -460,6 +522,12 @@ def od_sample_shard_mass(ctx: Context, shard_lo: int, logits, vo: VerifyOut, q_r
         raise ValueError("q_rows must be [B, K, V_q]")
     if out is None:
         out = torch.zeros(B, 2, dtype=torch.float64, device=d)
+    status = _native.sample_shard_mass(ctx.address, ctx.index, B, K, ctx.draft_vocab, shard_lo, shard_len, logits, vo.row_max,
+                                       vo.row_sum, q_rows, draft_ids, mp.tgt_ids, mp.q_prime, mp.span_start, mp.span_len,
+                                       mp.m, mp.tail_kind, vo.n_accepted, temperature, out)
+    if status is not None:
+        _check(status, "od_sample_shard_mass")
+        return out
     _check(lib().od_sample_shard_mass(
         ctx.handle, B, K, shard_lo, shard_len, C.c_void_p(logits.data_ptr()), logit_dtype_code(logits),
         rs, ss, _dp(vo.row_max, f32, d), _dp(vo.row_sum, f32, d), _dp(q_rows, f32, d),
@@ -481,6 +549,13 @@ def od_sample_shard_pick(ctx: Context, shard_index: int, shard_lo: int, mass_all
     out = out or alloc_sample_out(ctx, B)
     d, i32, f32 = ctx.device, torch.int32, torch.float32
     shard_len = int(logits.shape[2])
+    status = _native.sample_shard_pick(ctx.address, ctx.index, B, K, mass_all.shape[0], shard_index, shard_lo, shard_len,
+                                       mass_all, logits, vo.row_max, vo.row_sum, q_rows, draft_ids, mp.tgt_ids, mp.q_prime,
+                                       mp.span_start, mp.span_len, mp.m, mp.tail_kind, vo.n_accepted, temperature, seed, step,
+                                       out.out_token, out.resid_mass, out.flags)
+    if status is not None:
+        _check(status, "od_sample_shard_pick")
+        return out
     rs, ss = _shard_strides(logits, B, K, shard_len)
     _check(lib().od_sample_shard_pick(
         ctx.handle, B, K, int(mass_all.shape[0]), shard_index, shard_lo, shard_len,

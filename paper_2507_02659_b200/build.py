@@ -1,4 +1,5 @@
-"""Builds libomnidraft.so (the C-ABI CUDA library) in-tree with nvcc for sm_100a."""
+"""Builds libomnidraft.so (the C-ABI CUDA library, nvcc for sm_100a) and _marshal.so (the
+binding's argument marshalling, a Python extension) in-tree."""
 from __future__ import annotations
 
 import os
@@ -9,6 +10,7 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libomnidraft.so")
+EXT = os.path.join(HERE, "_marshal.so")
 SOURCES = ["od_api.cu", "od_map.cu", "od_verify.cu", "od_sample.cu", "od_noalloc.cu", "od_exit.cu", "od_cache.cu", "od_distill.cu"]
 
 
@@ -19,12 +21,40 @@ def _newest_source() -> float:
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
+    if force or not os.path.exists(EXT) or os.path.getmtime(EXT) < _newest_source():
+        _build_lib(force, verbose)
+        _build_marshal(verbose)
+    return LIB
+
+
+def _build_marshal(verbose: bool) -> None:
+    import sysconfig
+    import torch
+    root = os.path.dirname(torch.__file__)
+    inc = os.path.join(root, "include")
+    cuda = os.environ.get("CUDA_HOME", "/usr/local/cuda")
+    tmp = EXT + f".{os.getpid()}.tmp"
+    cmd = ["g++", "-O2", "-std=c++17", "-shared", "-fPIC", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch.compiled_with_cxx11_abi())}",
+           "-I", os.path.join(ROOT, "include"), "-I", inc, "-I", os.path.join(inc, "torch", "csrc", "api", "include"),
+           "-I", os.path.join(cuda, "include"), "-I", sysconfig.get_paths()["include"], "-o", tmp,
+           os.path.join(CSRC, "marshal.cpp"), "-L", HERE, "-l:libomnidraft.so", "-L", os.path.join(root, "lib"),
+           "-ltorch_python", "-ltorch_cpu", "-lc10", "-lc10_cuda",
+           "-Wl,-rpath,$ORIGIN:" + os.path.join(root, "lib")]
+    res = subprocess.run(cmd, capture_output=True, text=True)
+    if verbose or res.returncode != 0:
+        sys.stderr.write(res.stdout + res.stderr)
+    if res.returncode != 0:
+        raise RuntimeError("g++ failed building _marshal.so")
+    os.replace(tmp, EXT)
+
+
+def _build_lib(force: bool = False, verbose: bool = False) -> str:
     if not force and os.path.exists(LIB) and os.path.getmtime(LIB) >= _newest_source():
         return LIB
     nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
     tmp = LIB + f".{os.getpid()}.tmp"
     cmd = [nvcc, "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3",
-           "-std=c++17", "-shared", "-Xcompiler", "-fPIC", "-Xptxas", "-v",
+           "-std=c++17", "-shared", "-Xcompiler", "-fPIC", "-Xlinker", "-soname=libomnidraft.so", "-Xptxas", "-v",
            "-I", os.path.join(ROOT, "include"), "-I", CSRC, "-o", tmp]
     cmd += [os.path.join(CSRC, s) for s in SOURCES]
     res = subprocess.run(cmd, capture_output=True, text=True)
