@@ -34,7 +34,7 @@ struct od_ctx {
     void *d_distill_lists;          // gather lists of the distillation kernel (od_distill_lists)
     void *d_sample_lists;           // and of the sampler (od_sample_lists)
     int32_t sample_slots[OD_SAMPLE_LEVELS];   // most mapped ids of a part
-    bool cluster16;                 // the device takes the sampler's clusters of 16 blocks
+    int32_t sample_clusters[OD_SAMPLE_LEVELS];   // clusters of the sampler that are resident at a time
     bool have_map;
     int64_t n_mapped;               // draft ids with a direct map
     bool map_same_ids;              // every draft id is mapped to the target id of the same number
@@ -142,7 +142,7 @@ cudaError_t od_launch_sample(od_ctx *c, int32_t B, int32_t K_max, const void *lo
 
 size_t od_sample_smem_bytes(int32_t ntiles);            // dynamic shared memory of the shard sampler's kernel
 // opt in to the dynamic shared memory and the cluster size that the sampler's kernels may ask for
-cudaError_t od_sample_prepare_device(size_t bytes, bool *cluster16);
+cudaError_t od_sample_prepare_device(size_t bytes, int32_t *clusters);   // clusters: [levels] resident at a time
 
 // What the sampler knows about the vocabulary map, one block of memory. The mapped target ids in
 // order have ranks 0, 1, ...; a row's tiles are cut into 1, 2, 4, 8, 16 parts (the levels), and a

@@ -644,7 +644,7 @@ __device__ __forceinline__ SeqState seq_state(const SampleArgs &a, const Ahead &
         // and a margin, so that e(t) stays below one whatever the rounding: r'(t) may then be clamped to
         // [0, 1] by the multiply-add itself
         const float c = fmaxf(M * q.scale, -FLT_MAX);
-        q.c = c + fmaxf(1.f, ceilf(fabsf(c) * 1e-6f));
+        q.c = c + fmaf(fabsf(c), 1e-6f, 1e-6f);
         q.margin = q.c - c;
         q.S = __shfl_sync(0xFFFFFFFFu, rs, j) * od_ex2(fmaf(M, q.scale, -q.c));
     }
@@ -1361,23 +1361,29 @@ static cudaError_t prepare_kernels(size_t bytes)
 }
 
 // Rows beyond 6144 tiles (and the staged probabilities) need more dynamic shared memory than a
-// kernel gets by default, and clusters of 16 blocks are not portable: opt in, and ask whether the
-// device has room for such a cluster (the device must be current; allocates nothing).
-cudaError_t od_sample_prepare_device(size_t bytes, bool *cluster16)
+// kernel gets by default, and clusters of 16 blocks are not portable: opt in, and ask how many
+// clusters of each size are resident at a time (0: the device has no room for one; the device must be
+// current; allocates nothing).
+cudaError_t od_sample_prepare_device(size_t bytes, int32_t *clusters)
 {
     cudaError_t e = prepare_kernels<OD_BF16>(bytes);
     if (e == cudaSuccess) e = prepare_kernels<OD_F32>(bytes);
     if (e != cudaSuccess) return e;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(16); cfg.blockDim = dim3(CTHREADS); cfg.dynamicSmemBytes = 64 * 1024;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = 16; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr; cfg.numAttrs = 1;
-    int n = 0;
-    e = cudaOccupancyMaxActiveClusters(&n, od_sample_kernel<OD_BF16, true, STAGED>, &cfg);
-    *cluster16 = e == cudaSuccess && n > 0;
-    return e;
+    for (int level = 0; level < OD_SAMPLE_LEVELS; ++level) {
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(1u << level); cfg.blockDim = dim3(CTHREADS); cfg.dynamicSmemBytes = 64 * 1024;
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = 1u << level; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+        cfg.attrs = attr; cfg.numAttrs = 1;
+        int n = 0;
+        if (cudaOccupancyMaxActiveClusters(&n, od_sample_kernel<OD_BF16, true, STAGED>, &cfg) != cudaSuccess) {
+            cudaGetLastError();
+            n = 0;
+        }
+        clusters[level] = n;
+    }
+    return cudaSuccess;
 }
 
 template <int DTYPE>
@@ -1415,14 +1421,14 @@ static cudaError_t launch_sample(od_ctx *c, int mode, int32_t B, int32_t K_max, 
     int64_t tpw = c->opt_sample_tiles_per_warp;
     int blocks_x = 1, level = 0, part_tiles = 0;
     if (mode == 0) {
-        // Parts (blocks) per sequence: as many as still make one resident wave of two blocks per
-        // multiprocessor, and no more than have a tile for every warp (19 sequences of 100277 ids, the
+        // Parts (blocks) per sequence: as many as still make one resident wave (73 sequences of four blocks
+        // have 296 places, but not as resident clusters: 32.3 us, of two blocks each 29.9), and no more than have a tile for every warp (19 sequences of 100277 ids, the
         // three calls: 25.2 us with 4 parts, 23.3 with 8, 27.0 with 16, which is two waves; one of
         // 152064: 29.1 / 27.1 / 26.7).
         const int fine = od_sample_fine_tiles(c->v_p);
-        const int most = c->cluster16 ? OD_SAMPLE_LEVELS - 1 : OD_SAMPLE_LEVELS - 2;
+        const int most = c->sample_clusters[OD_SAMPLE_LEVELS - 1] > 0 ? OD_SAMPLE_LEVELS - 1 : OD_SAMPLE_LEVELS - 2;
         while (level < most && (tpw > 0 ? fine * (OD_SAMPLE_MAX_PARTS >> level) > tpw * CWARPS
-                                        : (int64_t)B * 2 << level <= (int64_t)c->sm_count * 2 &&
+                                        : B <= c->sample_clusters[level + 1] &&
                                               fine * (OD_SAMPLE_MAX_PARTS >> level) > CWARPS))
             ++level;
         // staged probabilities of over 100 KB would leave room for one block per multiprocessor
