@@ -110,9 +110,9 @@ struct SampleArgs {
 struct SeqState {
     const char *row;
     const float *q_row;
-    float c, S, scale;      // e(t) = exp2(fma(x_t, scale, -c)) < 1; S is the row sum relative to c
-    float margin;           // c - fl(M*scale)
-    bool residual;
+    float c, S, scale;      // e(t) = exp2(fma(x_t, scale, -c)); S is the row sum relative to c
+    float above;            // c - fl(M*scale)
+    bool residual, bounded;  // bounded: e(t) <= 2
     int32_t ngram_token, prefix_token, first_draft;
     float ngram_prob, prefix_val;
 };
@@ -133,16 +133,16 @@ __device__ __forceinline__ float resid_of(const SeqState &q, float x, float qq)
 // an id (its ids are t0 .. t0 + EPT - 1) redoes it: prefix sub-token first, the n-gram
 // token last.
 template <int DTYPE>
-__device__ __forceinline__ void eq2_ids(const SeqState &q, const SampleArgs &a, int t0, float *r)
+__device__ __forceinline__ void eq2_ids(const SeqState &q, const SampleArgs &a, int t0, float *r, float unit = 1.f)
 {
     const int dp = q.prefix_token - t0, dn = q.ngram_token - t0;
     if ((unsigned)dp < (unsigned)EPT && q.prefix_token < a.v_p) {
-        const float v = resid_of(q, od_load_logit<DTYPE>(q.row, q.prefix_token), q.prefix_val);
+        const float v = resid_of(q, od_load_logit<DTYPE>(q.row, q.prefix_token), q.prefix_val) * unit;
 #pragma unroll
         for (int e = 0; e < EPT; ++e) r[e] = e == dp ? v : r[e];
     }
     if ((unsigned)dn < (unsigned)EPT && q.ngram_token < a.v_p) {
-        const float v = resid_of(q, od_load_logit<DTYPE>(q.row, q.ngram_token), q.ngram_prob);
+        const float v = resid_of(q, od_load_logit<DTYPE>(q.row, q.ngram_token), q.ngram_prob) * unit;
 #pragma unroll
         for (int e = 0; e < EPT; ++e) r[e] = e == dn ? v : r[e];
     }
@@ -356,6 +356,8 @@ __device__ __forceinline__ void load_tile(const SeqState &q, int tile, int lane,
 // 296 staged rows of 152064 ids with a branch per id, 195 and 51.9 us with a select per id, 156
 // and 45.7 us so: the clamp at zero is part of the multiply-add, an unmapped id's multiply-add
 // is predicated off, and Eq. (2)'s two ids are looked for only in the tiles that hold them.
+// The multiply-add clamps to [0, 1] and e(t) may be up to 2 (SeqState::bounded): the residuals are
+// formed as halves, which is exact.
 __device__ __forceinline__ float fma_sat(float a, float b, float c)
 {
     float d;
@@ -382,18 +384,24 @@ __device__ __forceinline__ void tile_e(const SeqState &q, const uint4 *raw, floa
         e[k] = od_ex2(e[k]); e[k + 1] = od_ex2(e[k + 1]);
     }
 }
+__device__ __forceinline__ void halve(float *r)
+{
+#pragma unroll
+    for (int k = 0; k < EPT; k += 2) f2_unpack(f2_mul(f2_pack(r[k], r[k + 1]), f2_pack(0.5f, 0.5f)), r[k], r[k + 1]);
+}
 __device__ __forceinline__ float sum_of_eight(const float *r)
 {
     float s0, s1;
     f2_unpack(f2_add(f2_add(f2_pack(r[0], r[1]), f2_pack(r[2], r[3])), f2_add(f2_pack(r[4], r[5]), f2_pack(r[6], r[7]))), s0, s1);
     return s0 + s1;
 }
+// r: halves of the residuals
 template <int DTYPE>
 __device__ __forceinline__ float with_eq2_ids(const SeqState &q, const SampleArgs &a, int tile, int lane, float *r)
 {
     if (tile == q.prefix_token / OD_SAMPLE_TILE || tile == q.ngram_token / OD_SAMPLE_TILE)
-        eq2_ids<DTYPE>(q, a, tile * OD_SAMPLE_TILE + lane * EPT, r);
-    return sum_of_eight(r);
+        eq2_ids<DTYPE>(q, a, tile * OD_SAMPLE_TILE + lane * EPT, r, 0.5f);
+    return 2.f * sum_of_eight(r);
 }
 template <int DTYPE>
 __device__ __forceinline__ float tile_lane_sum(const SeqState &q, const SampleArgs &a, int tile, int lane, const uint4 *raw,
@@ -401,8 +409,10 @@ __device__ __forceinline__ float tile_lane_sum(const SeqState &q, const SampleAr
 {
     float r[EPT];
     tile_e<DTYPE>(q, raw, r);
+    halve(r);
+    const float nS = -0.5f * q.S;
 #pragma unroll
-    for (int k = 0; k < EPT; ++k) r[k] = fma_sat(qq[k], -q.S, r[k]);
+    for (int k = 0; k < EPT; ++k) r[k] = fma_sat(qq[k], nS, r[k]);
     return with_eq2_ids<DTYPE>(q, a, tile, lane, r);
 }
 // the same with the probabilities in shared memory at `rank_at` (the address of the lane's first
@@ -413,7 +423,8 @@ __device__ __forceinline__ float tile_lane_sum_staged(const SeqState &q, const S
 {
     float r[EPT];
     tile_e<DTYPE>(q, raw, r);
-    const float nS = -q.S;
+    halve(r);
+    const float nS = -0.5f * q.S;
 #pragma unroll
     for (int k = 0; k < EPT; ++k)
         // (read for every id, mapped or not: the last rank has a word behind it)
@@ -638,14 +649,16 @@ __device__ __forceinline__ SeqState seq_state(const SampleArgs &a, const Ahead &
     q.row = (const char *)a.logits + ((size_t)b * a.seq_stride + (size_t)j * a.row_stride) * esz - (size_t)col0 * esz;
     q.scale = 1.4426950408889634f / h.T;
     {
-        // reference exponent c = fl(M*scale); its rounding goes into S exactly:
+        // reference exponent c = fl(M*scale), od_verify's own, so that the errors of e(t) are those of the
+        // row sum; its rounding goes into S exactly:
         // sum_t exp2(x_t*scale - c) = (sum_t exp2((x_t - M)*scale)) * exp2(M*scale - c)
-        const float M = __shfl_sync(0xFFFFFFFFu, rm, j);
-        // and a margin, so that e(t) stays below one whatever the rounding: r'(t) may then be clamped to
-        // [0, 1] by the multiply-add itself
-        const float c = fmaxf(M * q.scale, -FLT_MAX);
-        q.c = c + fmaf(fabsf(c), 1e-6f, 1e-6f);
-        q.margin = q.c - c;
+        const float M = __shfl_sync(0xFFFFFFFFu, rm, j), c = fmaxf(M * q.scale, -FLT_MAX);
+        // e(M) is exp2 of c's rounding: up to 2 while |c| < 2^24. Above (M = 20, T = 1e-6: near-greedy
+        // draws) c is rounded up, so that e(M) lies between exp2(-32) and 1 up to |c| = 2^29; beyond that the
+        // tiles are worked on without an upper clamp.
+        q.c = fabsf(c) < 0x1p23f ? c : fabsf(c) < 0x1p29f ? __fmul_ru(M, q.scale) : c;
+        q.above = q.c - c;
+        q.bounded = fabsf(c) < 0x1p29f;
         q.S = __shfl_sync(0xFFFFFFFFu, rs, j) * od_ex2(fmaf(M, q.scale, -q.c));
     }
     q.residual = (j < h.mb) || h.stop;
@@ -985,13 +998,14 @@ od_sample_kernel(const SampleArgs a)
     const SeqState q = seq_state<DTYPE>(a, h, b, j, rm, rs, 0);
     if (SOURCE == FROM_MAP && q.residual && threadIdx.x == 0) prefetch_q_row(a, q, part, nparts);
 
-    // ---- pass 1: the value of every tile ----
+    // ---- pass 1: the value of every tile; the ragged last one (all of them, if e is not bounded) one by one ----
     WarpTiles out = {s_val, lane, p_lo, 0.0};
+    const int hi_w = q.bounded ? p_hi_w : p_lo;
     const uint64_t seed_b = a.seed[b];
     const StagedRow sr = {s_q, a.octet, (uint32_t)my_part.z};
     if (SOURCE == STAGED && q.residual) {
         TileLoads<DTYPE, STAGED> cur[2];
-        first_tiles<DTYPE, STAGED>(q, a, p_lo, p_hi_w, lane, cur);
+        first_tiles<DTYPE, STAGED>(q, a, p_lo, hi_w, lane, cur);
         // the part's probabilities, gathered in draft-id order, to their ranks in shared memory
         for (;;) {
             float x[EB];
@@ -1009,10 +1023,10 @@ od_sample_kernel(const SampleArgs a)
             if (!more) break;
         }
         __syncthreads();
-        warp_tiles_ahead<DTYPE, STAGED>(q, a, sr, p_lo, p_hi_w, lane, out, cur);
-        if (p_hi_w < p_hi) warp_tiles_dense<DTYPE, 1>(q, a, true, max(p_hi_w, p_lo), p_hi, lane, out);
+        warp_tiles_ahead<DTYPE, STAGED>(q, a, sr, p_lo, hi_w, lane, out, cur);
+        if (hi_w < p_hi) warp_tiles_dense<DTYPE, 1>(q, a, true, max(hi_w, p_lo), p_hi, lane, out);
     } else {
-        warp_run<DTYPE, SOURCE>(q, a, p_lo, p_hi, p_hi_w, lane, out, ni);
+        warp_run<DTYPE, SOURCE>(q, a, p_lo, p_hi, hi_w, lane, out, ni);
     }
     const float u = od_uniform(seed_b, a.step, (uint32_t)j, 1u);
 
@@ -1163,8 +1177,9 @@ od_sample_shard_kernel(const SampleArgs a)
 
     if (MODE != 2) {
         // ---- pass 1: the value of every tile ----
-        if (a.same_ids) warp_run<DTYPE, FROM_ROW>(q, a, p_lo, p_hi, p_hi_w, lane, out, ni);
-        else warp_run<DTYPE, FROM_MAP>(q, a, p_lo, p_hi, p_hi_w, lane, out, ni);
+        const int hi_w = q.bounded ? p_hi_w : p_lo;
+        if (a.same_ids) warp_run<DTYPE, FROM_ROW>(q, a, p_lo, p_hi, hi_w, lane, out, ni);
+        else warp_run<DTYPE, FROM_MAP>(q, a, p_lo, p_hi, hi_w, lane, out, ni);
         // The tile values are read by another block: the barrier orders this block's stores
         // before thread 0's fence, the fence before its ticket (release); the block that
         // draws the last ticket fences again before anyone in it reads (acquire).
@@ -1206,7 +1221,7 @@ od_sample_shard_kernel(const SampleArgs a)
     __syncthreads();
 
     // the shards exchange their shares relative to fl(M*scale)
-    const double unit = exp2((double)q.margin);
+    const double unit = exp2((double)q.above);
     if (MODE == 1) {
         // ---- this shard's shares ----
         const double mass_r = block_total(s_val, my_lo, my_hi, s_warp);
