@@ -50,12 +50,14 @@ struct TrimState {
     unsigned int k;             // entries to drop in this trim
     unsigned int invalid;       // malformed candidates seen by od_cache_insert
     unsigned int dropped;       // candidates that found no free slot on their whole probe sequence
-    // what the pass over the table finds out; two, used in turn: a trim resets the next one's
+    // what the pass over the table finds out; empty again when a trim has read it, so that a
+    // trim that is replayed from a CUDA graph starts like the one that was captured
     struct Live {
         unsigned int n;         // entries of the dense list
         unsigned long long hi_and, hi_or;   // AND / OR of (new?, score) over the live entries: bits that never vary
-    } live[2];
-    unsigned long long thr_hi, thr_lo;      // trim_select_kernel: the k-th order key
+    } live;
+    unsigned int n_list;        // trim_select_kernel: live.n as it was, for the rebuild,
+    unsigned long long thr_hi, thr_lo;      // and the k-th order key
     SelState sel[PASSES + 1];   // sel[p]: written by block 0 of pass p (sel[PASSES]: by the rebuild)
     unsigned int n_out[PASSES]; // entries pass p copied into its output list
     unsigned int hist[PASSES][256];
@@ -208,6 +210,7 @@ __global__ void trim_begin_kernel(TrimState *st, unsigned int max_entries)
     const unsigned int k = st->size > max_entries ? st->size - max_entries : 0u;
     if (threadIdx.x == 0) {
         st->k = k;
+        reset_live(st->live);
         SelState z = {};
         z.k_rem = k;
         st->sel[0] = z;
@@ -246,7 +249,7 @@ __device__ __forceinline__ unsigned int block_offsets(unsigned int n, unsigned i
 __global__ void trim_compact_kernel(int policy, unsigned int clock, const unsigned long long *keys,
                                     const int32_t *vals, const unsigned int *stamp, const unsigned int *freq,
                                     const unsigned int *born, unsigned long long *nkeys, int32_t *nvals,
-                                    int64_t cap, void *lists, TrimState *st, int which)
+                                    int64_t cap, void *lists, TrimState *st)
 {
     __shared__ unsigned int s_warp[32];
     __shared__ unsigned int s_base;
@@ -293,7 +296,7 @@ __global__ void trim_compact_kernel(int policy, unsigned int clock, const unsign
         }
         unsigned int total;
         unsigned int at = block_offsets(n, s_warp, total);
-        if (threadIdx.x == 0) s_base = total ? atomicAdd(&st->live[which].n, total) : 0u;
+        if (threadIdx.x == 0) s_base = total ? atomicAdd(&st->live.n, total) : 0u;
         __syncthreads();
         at += s_base;
 #pragma unroll
@@ -302,7 +305,7 @@ __global__ void trim_compact_kernel(int policy, unsigned int clock, const unsign
             const unsigned int b4[4] = {bb[v].x, bb[v].y, bb[v].z, bb[v].w};
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
-                if (kk[v][e] == 0ull || vv[v][e] < 0) continue;
+                if (kk[v][e] == 0ull || vv[v][e] < 0 || at >= cap) continue;   // (never beyond the list)
                 unsigned long long hi, lo;
                 order_key(policy, clock, kk[v][e], s4[e], f4[e], b4[e], hi, lo);
                 t_and &= hi; t_or |= hi;
@@ -320,7 +323,7 @@ __global__ void trim_compact_kernel(int policy, unsigned int clock, const unsign
     }
     if ((threadIdx.x & 31) == 0) { atomicAnd(&s_and, t_and); atomicOr(&s_or, t_or); }
     __syncthreads();
-    if (threadIdx.x == 0) { atomicAnd(&st->live[which].hi_and, s_and); atomicOr(&st->live[which].hi_or, s_or); }
+    if (threadIdx.x == 0) { atomicAnd(&st->live.hi_and, s_and); atomicOr(&st->live.hi_or, s_or); }
 }
 
 // ---- the k-th order key in one launch ------------------------------------------------------
@@ -355,7 +358,7 @@ __device__ __forceinline__ void count_digit(unsigned int *hist, unsigned int d, 
 }
 
 __global__ void __launch_bounds__(SELECT_THREADS, 1)
-trim_select_kernel(unsigned int max_entries, unsigned int room, int64_t cap, void *lists, TrimState *st, int which)
+trim_select_kernel(unsigned int max_entries, unsigned int room, int64_t cap, void *lists, TrimState *st)
 {
     extern __shared__ __align__(16) unsigned long long s_keys[];   // [room]
     __shared__ unsigned int s_hist[2][256], s_sum[256];
@@ -363,10 +366,10 @@ trim_select_kernel(unsigned int max_entries, unsigned int room, int64_t cap, voi
     const unsigned int P = gridDim.x, rank = blockIdx.x, lane = threadIdx.x & 31u;
     chain_wait();
     const unsigned int size = __ldcg(&st->size), k = size > max_entries ? size - max_entries : 0u;
-    const unsigned int n = __ldcg(&st->live[which].n);
-    const unsigned long long hi_and = __ldcg(&st->live[which].hi_and), hi_or = __ldcg(&st->live[which].hi_or);
-    if (k == 0u) {                                          // nothing to drop: every block leaves
-        if (rank == 0 && threadIdx.x == 0) { st->k = 0u; reset_live(st->live[which ^ 1]); }
+    const unsigned int n = (unsigned int)min((int64_t)__ldcg(&st->live.n), cap);
+    const unsigned long long hi_and = __ldcg(&st->live.hi_and), hi_or = __ldcg(&st->live.hi_or);
+    if (k == 0u) {                                          // nothing to drop: every block leaves (the others use none of what block 0 resets)
+        if (rank == 0 && threadIdx.x == 0) { st->k = 0u; st->n_list = n; reset_live(st->live); }
         return;
     }
     const TrimLists L = trim_lists(lists, cap);
@@ -490,7 +493,8 @@ trim_select_kernel(unsigned int max_entries, unsigned int room, int64_t cap, voi
     if (rank == 0 && threadIdx.x == 0) {
         st->k = k; st->size = size - k;
         st->thr_hi = thr_hi; st->thr_lo = thr_lo;
-        reset_live(st->live[which ^ 1]);
+        st->n_list = n;
+        reset_live(st->live);                               // (read by every block before its first barrier)
     }
 }
 
@@ -505,9 +509,9 @@ __device__ __forceinline__ bool digit_is_constant(int pass, unsigned long long h
 // The state at the start of pass `pass` (0..PASSES), worked out from the state at the start of
 // the pass before it and that pass's histogram: by every block alike, the same arithmetic on the
 // same numbers. All threads of the block call; s_hist (256 words) and s_sel are its scratch.
-__device__ __forceinline__ SelState select_state(int pass, const TrimState *st, int which, unsigned int *s_hist, SelState *s_sel)
+__device__ __forceinline__ SelState select_state(int pass, const TrimState *st, unsigned int *s_hist, SelState *s_sel)
 {
-    const TrimState::Live &live = st->live[which];
+    const TrimState::Live &live = st->live;
     if (pass == 0) {
         SelState z = st->sel[0];
         z.n_in = z.n_match = __ldcg(&live.n);
@@ -582,7 +586,7 @@ __device__ __forceinline__ SelState select_state(int pass, const TrimState *st, 
 // Pass `pass` of the radix select over the current candidate list: histogram of digit `pass`
 // over the candidates that match the digits decided so far. If those are at most half of the
 // list, they are copied into the other scratch list on the way (the next pass reads that one).
-__global__ void trim_hist_kernel(int pass, int64_t cap, void *lists, TrimState *st, int which)
+__global__ void trim_hist_kernel(int pass, int64_t cap, void *lists, TrimState *st)
 {
     __shared__ unsigned int s_hist[256];
     __shared__ unsigned int s_warp[32];
@@ -590,9 +594,9 @@ __global__ void trim_hist_kernel(int pass, int64_t cap, void *lists, TrimState *
     __shared__ SelState s_sel;
     chain_wait();
     if (st->k == 0u) return;                                 // nothing to drop: every block leaves
-    const SelState S = select_state(pass, st, which, s_hist, &s_sel);
+    const SelState S = select_state(pass, st, s_hist, &s_sel);
     if (blockIdx.x == 0 && threadIdx.x == 0) st->sel[pass] = S;
-    if (digit_is_constant(pass, __ldcg(&st->live[which].hi_and), __ldcg(&st->live[which].hi_or))) return;   // the next pass fills it in
+    if (digit_is_constant(pass, __ldcg(&st->live.hi_and), __ldcg(&st->live.hi_or))) return;   // the next pass fills it in
     __syncthreads();
     s_hist[threadIdx.x] = 0u;
     __syncthreads();
@@ -643,19 +647,19 @@ __global__ void trim_hist_kernel(int pass, int64_t cap, void *lists, TrimState *
 // entry gets depends on timing, the set of entries does not
 __global__ void trim_rebuild_kernel(unsigned long long *nkeys, int32_t *nvals, unsigned int *nstamp,
                                     unsigned int *nfreq, unsigned int *nborn, int64_t cap, void *lists,
-                                    const TrimState *st, int which, int selected)
+                                    const TrimState *st, int selected)
 {
     __shared__ unsigned int s_hist[256];
     __shared__ SelState s_sel;
     chain_wait();
     const TrimLists L = trim_lists(lists, cap);
-    const unsigned int n = __ldcg(&st->live[which].n), k = st->k;
+    const unsigned int n = __ldcg(selected ? &st->n_list : &st->live.n), k = st->k;
     unsigned long long thr_hi = 0ull, thr_lo = 0ull;
     if (k > 0u) {                                           // block-uniform
         if (selected) {
             thr_hi = st->thr_hi; thr_lo = st->thr_lo;
         } else {
-            const SelState S = select_state(PASSES, st, which, s_hist, &s_sel);
+            const SelState S = select_state(PASSES, st, s_hist, &s_sel);
             thr_hi = S.pre_hi; thr_lo = S.pre_lo;
         }
     }
@@ -683,11 +687,10 @@ __global__ void trim_rebuild_kernel(unsigned long long *nkeys, int32_t *nvals, u
     }
 }
 
-__global__ void trim_end_kernel(TrimState *st, int which)
+__global__ void trim_end_kernel(TrimState *st)
 {
     chain_wait();
     st->size -= st->k; st->k = 0u;
-    reset_live(st->live[which ^ 1]);
 }
 
 #define OD_CUDA(call)                                  \
@@ -809,9 +812,7 @@ int32_t od_cache_configure(od_ctx *c, int64_t max_entries, int32_t policy, int32
     c->table_written = true;
     TrimState *dst = (TrimState *)c->d_trim;
     const TrimState::Live empty = {0u, ~0ull, 0ull};
-    OD_CUDA(cudaMemcpy(&dst->live[0], &empty, sizeof(empty), cudaMemcpyHostToDevice));
-    OD_CUDA(cudaMemcpy(&dst->live[1], &empty, sizeof(empty), cudaMemcpyHostToDevice));
-    c->trim_turn = 0;
+    OD_CUDA(cudaMemcpy(&dst->live, &empty, sizeof(empty), cudaMemcpyHostToDevice));
     c->dyn = true; c->dyn_policy = policy; c->dyn_max = max_entries; c->dyn_max_insert = max_insert;
     c->clock = 0;
     c->trim_blocks = select_blocks(c);
@@ -861,7 +862,7 @@ int32_t od_cache_trim(od_ctx *c, void *stream)
     c->last_was_map = false;
     c->table_written = true;
     TrimState *st = (TrimState *)c->d_trim;
-    const int grid = c->sm_count * 4, which = c->trim_turn;
+    const int grid = c->sm_count * 4;
     const bool pdl = c->opt_pdl != 0;
     const int blocks = c->trim_blocks;                      // 0: the select is a chain of launches
     if (!blocks) OD_CUDA(chain_launch(trim_begin_kernel, 1u, 256u, s, pdl, st, (unsigned int)c->dyn_max));
@@ -869,7 +870,7 @@ int32_t od_cache_trim(od_ctx *c, void *stream)
                          (const unsigned long long *)c->d_keys, (const int32_t *)c->d_vals,
                          (const unsigned int *)c->d_stamp, (const unsigned int *)c->d_freq,
                          (const unsigned int *)c->d_born, (unsigned long long *)c->d_keys2, c->d_vals2,
-                         c->cap, c->d_trim_lists, st, which));
+                         c->cap, c->d_trim_lists, st));
     if (blocks) {
         cudaLaunchConfig_t cfg = {};
         cudaLaunchAttribute attr[2];
@@ -877,17 +878,16 @@ int32_t od_cache_trim(od_ctx *c, void *stream)
         cfg.stream = s;
         cfg.numAttrs = pdl ? 2 : 1;
         OD_CUDA(cudaLaunchKernelEx(&cfg, trim_select_kernel, (unsigned int)c->dyn_max, select_room(c, blocks), c->cap,
-                                   c->d_trim_lists, st, which));
+                                   c->d_trim_lists, st));
     } else {
         for (int pass = 0; pass < PASSES; ++pass)
             OD_CUDA(chain_launch(trim_hist_kernel, (unsigned)c->sm_count, 256u, s, pdl, pass, c->cap,
-                                 c->d_trim_lists, st, which));
+                                 c->d_trim_lists, st));
     }
     OD_CUDA(chain_launch(trim_rebuild_kernel, (unsigned)grid, 256u, s, pdl, (unsigned long long *)c->d_keys2,
                          c->d_vals2, c->d_stamp2, c->d_freq2, c->d_born2, c->cap, c->d_trim_lists,
-                         (const TrimState *)st, which, blocks ? 1 : 0));
-    if (!blocks) OD_CUDA(chain_launch(trim_end_kernel, 1u, 1u, s, pdl, st, which));
-    c->trim_turn ^= 1;
+                         (const TrimState *)st, blocks ? 1 : 0));
+    if (!blocks) OD_CUDA(chain_launch(trim_end_kernel, 1u, 1u, s, pdl, st));
     // the rebuilt table is the table for every call enqueued from now on
     std::swap(c->d_keys, c->d_keys2); std::swap(c->d_vals, c->d_vals2);
     std::swap(c->d_stamp, c->d_stamp2); std::swap(c->d_freq, c->d_freq2); std::swap(c->d_born, c->d_born2);

@@ -57,7 +57,6 @@ struct od_ctx {
     uint32_t *d_owner;              // [cap] first-wins claims of a batch (0xFFFFFFFF = none)
     int32_t *d_cand_slot;           // [dyn_max_insert]
     void *d_trim;                   // trim / size state (device)
-    int32_t trim_turn;              // which of the two TrimState::live the next trim uses
     int32_t trim_blocks;            // blocks of the one-launch select, 0 = the table is too large for it
     void *d_trim_lists;             // trim scratch: the live entries' records and two candidate lists, 64 bytes per slot
 

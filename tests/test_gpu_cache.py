@@ -157,6 +157,37 @@ def test_trim_over_ties(cuda_device, policy, bound, batch, batches):
     ctx.close()
 
 
+# the select in one launch, and the chain of launches for a table too large for it
+@pytest.mark.parametrize("bound", [100, 400000])
+@pytest.mark.parametrize("trims", [1, 2])
+def test_a_trim_replayed_from_a_graph(cuda_device, bound, trims):
+    """A captured trim leaves nothing behind that its next replay adds to: the same entries every
+    time. (One trim per graph reads the same table at every replay; two end on the one they began with.)"""
+    rng = np.random.default_rng(60)
+    v_q, v_p, dev = 32000, 128256, cuda_device
+    ctx = od.Context(dev, v_q, v_p, 4, 4)
+    ctx.set_vocab_map(np.full(v_q, -1, np.int32))
+    ctx.cache_configure(bound, cp.LRU, 64)
+    ctx.cache_set_clock(1)
+    runs, lens = _universe(rng, 50, v_q)
+    insert = lambda: ctx.cache_insert(*(torch.from_numpy(a).to(dev) for a in (runs, lens, np.arange(50, dtype=np.int32))))
+    insert()
+    ctx.cache_trim()
+    want = ctx.cache_dump()
+    assert len(want) == 50
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        for _ in range(trims):
+            ctx.cache_trim()
+    for _ in range(8):
+        graph.replay()
+        assert ctx.cache_dump() == want
+    insert()                                                # the same runs: nothing new
+    ctx.cache_trim()
+    assert ctx.cache_dump() == want and ctx.cache_stats()[0] == 50
+    ctx.close()
+
+
 def test_online_cache_argument_checks(cuda_device):
     ctx = od.Context(cuda_device, 100, 100, 4, 4)
     with pytest.raises(od.OdError) as e:
