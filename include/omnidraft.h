@@ -152,7 +152,9 @@ int32_t od_destroy(od_ctx *ctx);
  * (Eq. (1), first case). host_map: int32[draft_vocab], target id or -1.
  * Builds the inverse map, uploads both (synchronous). Rejects target ids
  * outside [0, target_vocab) (INVALID_ARG) and maps that send two draft ids to
- * one target id (MAP_NOT_INJECTIVE). */
+ * one target id (MAP_NOT_INJECTIVE). Calls are laid out for the map of their time:
+ * a CUDA graph captured under an earlier map computes with the present one, but
+ * more slowly than one captured again. */
 int32_t od_set_vocab_map(od_ctx *ctx, const int32_t *host_map);
 
 /* n-gram cache C = {(t, [d_1..d_n])} (Section 3.1). host_runs: int32[E,4],

@@ -45,7 +45,7 @@ int32_t dev_alloc(T **p, size_t n)
 void free_all(od_ctx *c)
 {
     od_cache_free_dynamic(c);
-    void *ptrs[] = {c->d_vocab_map, c->d_inv_map, c->d_distill_lists, c->d_sample_lists, c->d_keys, c->d_vals, c->d_partials,
+    void *ptrs[] = {c->d_vocab_map, c->d_inv_map, c->d_map_serial, c->d_distill_lists, c->d_sample_lists, c->d_keys, c->d_vals, c->d_partials,
                     c->d_tile_sums,
                     c->d_samp_ticket, c->s_logits, c->s_q_rows, c->s_q_sel, c->s_temperature,
                     c->s_draft_ids, c->s_draft_len, c->s_seed, c->s_tgt_ids, c->s_span_start,
@@ -144,6 +144,7 @@ int32_t od_create(od_ctx **ctx, int32_t device, int32_t draft_vocab, int32_t tar
     int32_t st = OD_OK;
     if (st == OD_OK) st = dev_alloc(&c->d_vocab_map, (size_t)draft_vocab);
     if (st == OD_OK) st = dev_alloc(&c->d_inv_map, (size_t)target_vocab + 8);
+    if (st == OD_OK) st = dev_alloc(&c->d_map_serial, 1);
     char *lists = nullptr;
     if (st == OD_OK) st = dev_alloc(&lists, od_distill_lists_bytes(draft_vocab, target_vocab));
     c->d_distill_lists = lists;
@@ -196,7 +197,7 @@ int32_t od_set_vocab_map(od_ctx *c, const int32_t *host_map)
     od_distill_plan(c->v_q, c->v_p, inv.data(), lists.data());
     OD_CUDA(cudaMemcpy(c->d_distill_lists, lists.data(), lists.size(), cudaMemcpyHostToDevice));
     lists.resize(od_sample_lists_bytes(c->v_q, c->v_p));
-    od_sample_plan(c->v_q, c->v_p, fwd.data(), inv.data(), lists.data(), c->sample_slots);
+    od_sample_plan(c->v_q, c->v_p, fwd.data(), inv.data(), ++c->map_serial, lists.data(), c->sample_slots);
     OD_CUDA(cudaMemcpy(c->d_sample_lists, lists.data(), lists.size(), cudaMemcpyHostToDevice));
     c->map_same_ids = true;
     c->n_mapped = 0;
@@ -204,6 +205,8 @@ int32_t od_set_vocab_map(od_ctx *c, const int32_t *host_map)
         c->map_same_ids = c->map_same_ids && host_map[d] == d;
         c->n_mapped += host_map[d] >= 0 ? 1 : 0;
     }
+    OD_CUDA(cudaMemcpy(c->d_map_serial, &c->map_serial, sizeof(int32_t), cudaMemcpyHostToDevice));
+    OD_CUDA(cudaDeviceSynchronize());       // kernels read the maps and lists before they wait for their stream
     c->have_map = true;
     return OD_OK;
     } catch (const std::bad_alloc &) {

@@ -36,6 +36,10 @@ struct od_ctx {
     int32_t sample_slots[OD_SAMPLE_LEVELS];   // most mapped ids of a part
     int32_t sample_clusters[OD_SAMPLE_LEVELS];   // clusters of the sampler that are resident at a time
     bool have_map;
+    // The map's serial number. A launch is laid out for the map of its time (where ids are shared, how many
+    // are staged); a kernel that finds another number on the device was replayed from a CUDA graph
+    // captured before od_set_vocab_map, and looks every id up in the maps instead.
+    int32_t map_serial, *d_map_serial;
     int64_t n_mapped;               // draft ids with a direct map
     bool map_same_ids;              // every draft id is mapped to the target id of the same number
 
@@ -152,7 +156,7 @@ struct OdSampleLists {
     int64_t groups;                 // room for this many groups in each level
     uint32_t *word;                 // [levels][groups][32]
     int32_t *base;                  // [levels][groups]
-    int32_t *part;                  // [levels][max parts][4] a part's groups within its level (the first, one past the last), first rank, -
+    int32_t *part;                  // [levels][max parts][4] a part's groups within its level (the first, one past the last), first rank, the map's serial number
     uint32_t *octet;                // [ceil(v_p / 8)] of target ids 8i .. 8i+7: rank of the first mapped one << 8 | which are mapped
 };
 inline OdSampleLists od_sample_lists(void *base, int32_t v_q, int32_t v_p)
@@ -174,7 +178,7 @@ inline size_t od_sample_lists_bytes(int32_t v_q, int32_t v_p)
 // tiles of a 16th of a row: a part of level l is 16 >> l of them
 inline int32_t od_sample_fine_tiles(int32_t v_p) { return ((v_p + OD_SAMPLE_TILE - 1) / OD_SAMPLE_TILE + OD_SAMPLE_MAX_PARTS - 1) / OD_SAMPLE_MAX_PARTS; }
 // host; slots: [levels] most mapped ids of a part
-void od_sample_plan(int32_t v_q, int32_t v_p, const int32_t *map, const int32_t *inv, void *out, int32_t *slots);
+void od_sample_plan(int32_t v_q, int32_t v_p, const int32_t *map, const int32_t *inv, int32_t serial, void *out, int32_t *slots);
 
 // vocabulary shards (columns [shard_lo, shard_lo + shard_len) of the rows on this GPU)
 cudaError_t od_launch_verify_shard_stats(od_ctx *c, int32_t B, int32_t K_max, int32_t shard_lo,

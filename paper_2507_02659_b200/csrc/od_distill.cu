@@ -53,6 +53,8 @@ struct DistillArgs {
     const int32_t *list_base, *list_ofs;
     const uint32_t *list_word, *mapped_bits;
     int32_t chunk;
+    int32_t map_serial;                                      // of the map this launch was laid out for
+    const int32_t *map_serial_now;
     float lambda;
     int32_t lambda_mode;
     float *loss, *grad;
@@ -224,6 +226,8 @@ od_distill_kernel(const DistillArgs a)
         g_at += EB * WARPS;
     };
     if (!SAME) load_words();
+    // the map is the one this launch was laid out for (else every id is looked up in it)
+    const bool planned = __ldg(a.map_serial_now) == a.map_serial;
     asm volatile("griddepcontrol.wait;" ::: "memory");
     const float T = a.temperature[b];
     int piece, plen;
@@ -258,7 +262,16 @@ od_distill_kernel(const DistillArgs a)
         loss_t += l; qg_t += g;
     };
     const raw_t *xrow = (const raw_t *)row;
-    if (!SAME) {
+    const auto looked_up = [&](int d, float v, float &l, float &g) {
+        const int32_t t = __ldg(a.vocab_map + d);
+        const raw_t x = t >= 0 ? __ldg(xrow + t) : raw_t();
+        return kl_term(kl, t >= 0 ? v : 0.f, Logit<DTYPE>::load(&x), l, g);
+    };
+    if (!planned) {
+        kl.lg2_S = lg2_approx(S);
+#pragma unroll 1
+        for (int d = lo + (int)threadIdx.x; d < hi; d += THREADS) looked_up(d, __ldg(q + d), loss_t, qg_t);
+    } else if (!SAME) {
         // (the first probabilities travel meanwhile)
         constexpr int PQ = 2;                                // vectors of four probabilities in flight per thread
         float4 qv[PQ];
@@ -367,7 +380,13 @@ od_distill_kernel(const DistillArgs a)
     if (!grad) return;
     // ---- the gradient: q(d) (g(d) - sum_e q(e) g(e))
     const float gbar = (float)qg;
-    if (VEC4) {
+    if (!planned) {
+#pragma unroll 1
+        for (int d = lo + (int)threadIdx.x; d < hi; d += THREADS) {
+            const float v = __ldg(q + d);
+            grad[d] = fmaf(-v, gbar, v * looked_up(d, v, loss_t, qg_t));
+        }
+    } else if (VEC4) {
 #pragma unroll 4
         for (int d = lo + (int)threadIdx.x * 4; d < hi; d += THREADS * 4) {
             const float4 v = __ldg((const float4 *)(q + d)), u = mapped4(d, v);
@@ -555,7 +574,7 @@ cudaError_t od_launch_distill(od_ctx *c, int32_t B, int32_t K_max, const float *
     a.q_rows = q_rows; a.draft_ids = draft_ids; a.tgt_ids = tgt_ids; a.span_start = span_start;
     a.span_len = span_len; a.m = m; a.logits = logits; a.row_stride = row_stride; a.seq_stride = seq_stride;
     a.row_max = row_max; a.row_sum = row_sum; a.p_sel = p_sel; a.temperature = temperature;
-    a.vocab_map = c->d_vocab_map; a.lambda = lambda; a.lambda_mode = lambda_mode; a.loss = loss; a.grad = grad;
+    a.vocab_map = c->d_vocab_map; a.map_serial = c->map_serial; a.map_serial_now = c->d_map_serial; a.lambda = lambda; a.lambda_mode = lambda_mode; a.loss = loss; a.grad = grad;
     const bool bf = dtype == OD_BF16, same = c->map_same_ids, pdl = c->opt_pdl != 0;
     const bool vec4 = c->v_q % 4 == 0 && ((uintptr_t)q_rows & 15u) == 0 && (!grad || ((uintptr_t)grad & 15u) == 0);
     // The number of chunks: the fewest with which a chunk's logits take 36 KB or less (what is left of

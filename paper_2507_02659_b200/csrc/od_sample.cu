@@ -85,6 +85,8 @@ struct SampleArgs {
     const int32_t *list_base, *list_part;
     int32_t part_tiles, slots;          // tiles of a part; room for staged probabilities
     int32_t same_ids;                   // 1: target id t is draft id t (t < v_q), and the drafter's rows are 16-byte aligned
+    int32_t map_serial;                 // of the map this launch was laid out for
+    const int32_t *map_serial_now;
     int32_t *out_token;
     float *resid_mass;
     uint32_t *flags;
@@ -113,6 +115,7 @@ struct SeqState {
     float c, S, scale;      // e(t) = exp2(fma(x_t, scale, -c)); S is the row sum relative to c
     float above;            // c - fl(M*scale)
     bool residual, bounded;  // bounded: e(t) <= 2
+    bool from_row;          // the drafter's probabilities are read at the target ids
     int32_t ngram_token, prefix_token, first_draft;
     float ngram_prob, prefix_val;
 };
@@ -199,7 +202,7 @@ __device__ __forceinline__ void tile_values(const SeqState &q, const SampleArgs 
         }
         if (residual) {
             float qq[EPT];
-            if (a.same_ids) {
+            if (q.from_row) {
                 same_id_probs(q, a, t0, qq);
             } else if (sr) {
                 staged_probs(*sr, __ldg(sr->octet + (t0 >> 3)), qq);
@@ -642,7 +645,8 @@ __device__ __forceinline__ Ahead load_ahead(const SampleArgs &a, int b, int lane
 // What the draw at position j needs; rm, rs: lane k holds the statistics of row k. A shard's row
 // pointer is moved back by the shard's first column (col0), and only ids of the window are read.
 template <int DTYPE>
-__device__ __forceinline__ SeqState seq_state(const SampleArgs &a, const Ahead &h, int b, int j, float rm, float rs, int col0)
+__device__ __forceinline__ SeqState seq_state(const SampleArgs &a, const Ahead &h, int b, int j, float rm, float rs, int col0,
+                                              bool planned)
 {
     const size_t esz = DTYPE == OD_BF16 ? 2 : 4;
     SeqState q;
@@ -662,6 +666,7 @@ __device__ __forceinline__ SeqState seq_state(const SampleArgs &a, const Ahead &
         q.S = __shfl_sync(0xFFFFFFFFu, rs, j) * od_ex2(fmaf(M, q.scale, -q.c));
     }
     q.residual = (j < h.mb) || h.stop;
+    q.from_row = a.same_ids && planned;
     q.ngram_token = -1; q.prefix_token = -1; q.first_draft = -1; q.ngram_prob = 0.f; q.prefix_val = 0.f;
     q.q_row = a.q_rows;
     // position j's preparation (j < K whenever the draw is a residual one)
@@ -878,6 +883,7 @@ od_sample_kernel(const SampleArgs a)
     // read now. (a.early = 0: the launch before this one was not od_verify; everything waits.)
     asm volatile("griddepcontrol.launch_dependents;");
     if (!a.early) asm volatile("griddepcontrol.wait;" ::: "memory");
+    const int32_t map_serial = SOURCE == FROM_ROW ? __ldg(a.map_serial_now) : a.map_serial;
     const Ahead h = load_ahead(a, b, lane);
     const int mb = h.mb;
 
@@ -915,7 +921,7 @@ od_sample_kernel(const SampleArgs a)
     int p_hi = min((int)(part + 1) * a.part_tiles, a.ntiles);
     const int p_lo = min((int)part * a.part_tiles + warp * a.tiles_per_warp, p_hi);
     p_hi = min(p_lo + a.tiles_per_warp, p_hi);
-    const int p_hi_w = min(p_hi, a.v_p / OD_SAMPLE_TILE);
+    int p_hi_w = min(p_hi, a.v_p / OD_SAMPLE_TILE);
     int4 ni[2][2] = {};
     if (SOURCE == FROM_MAP && p_lo < p_hi_w) first_pair_entries(a, p_lo, p_hi_w, lane, ni);
     // STAGED: the first entries of the part's list
@@ -935,6 +941,7 @@ od_sample_kernel(const SampleArgs a)
     };
     if (SOURCE == STAGED) {
         my_part = __ldg((const int4 *)a.list_part + part);
+        if (my_part.w != a.map_serial) { my_part.y = 0; p_hi_w = p_lo; }   // another map: nothing is staged, all is looked up
         g_at = my_part.x + warp;
         load_words();
     }
@@ -994,13 +1001,16 @@ od_sample_kernel(const SampleArgs a)
         if (part == 0 && threadIdx.x == 0) { a.out_token[b] = -1; a.resid_mass[b] = 0.f; a.flags[b] = OD_SF_BAD_TEMPERATURE; }
         return;
     }
+    // FROM_ROW: the map is still the one this launch was laid out for
+    const bool planned = map_serial == a.map_serial;
     cluster_arrive_relaxed();                      // this block runs: the others may store to it (waited for below)
-    const SeqState q = seq_state<DTYPE>(a, h, b, j, rm, rs, 0);
+    const SeqState q = seq_state<DTYPE>(a, h, b, j, rm, rs, 0, planned);
     if (SOURCE == FROM_MAP && q.residual && threadIdx.x == 0) prefetch_q_row(a, q, part, nparts);
 
-    // ---- pass 1: the value of every tile; the ragged last one (all of them, if e is not bounded) one by one ----
+    // ---- pass 1: the value of every tile; the ragged last one (all of them, if e is not bounded or
+    // the map is another) one by one ----
     WarpTiles out = {s_val, lane, p_lo, 0.0};
-    const int hi_w = q.bounded ? p_hi_w : p_lo;
+    const int hi_w = q.bounded && planned ? p_hi_w : p_lo;
     const uint64_t seed_b = a.seed[b];
     const StagedRow sr = {s_q, a.octet, (uint32_t)my_part.z};
     if (SOURCE == STAGED && q.residual) {
@@ -1100,7 +1110,7 @@ od_sample_kernel(const SampleArgs a)
             }
             if (pick < 0) { pick = held; at_pick = at_held; }        // rounding hid it: the last tile with mass
             const bool drawn = pick >= 0 && pick_in_tile<DTYPE>(q, a, b, q.residual, p_lo + pick, at_pick, target, Rn, flags, lane,
-                                                                 SOURCE == STAGED ? &sr : nullptr);
+                                                                 SOURCE == STAGED && my_part.y ? &sr : nullptr);
             if (lane == 0 && !drawn) s_bare = 1;             // the tile holds no mass after all
         }
         __syncthreads();
@@ -1137,6 +1147,7 @@ od_sample_shard_kernel(const SampleArgs a)
     const Ahead h = load_ahead(a, b, lane);
     const int mb = h.mb;
     const float T = h.T;
+    const bool planned = __ldg(a.map_serial_now) == a.map_serial;   // (as in od_sample_kernel)
 
     // a shard's tiles and ids keep their numbers of the full row
     const int tile_lo = a.tile_lo, tile_hi = a.tile_hi;
@@ -1168,7 +1179,7 @@ od_sample_shard_kernel(const SampleArgs a)
     }
     int j = a.n_accepted[b];
     j = j < 0 ? 0 : (j > mb ? mb : j);
-    const SeqState q = seq_state<DTYPE>(a, h, b, j, rm, rs, a.col0);
+    const SeqState q = seq_state<DTYPE>(a, h, b, j, rm, rs, a.col0, planned);
     if (MODE != 2 && q.residual && threadIdx.x == 0) prefetch_q_row(a, q, part, nparts);
 
     const int ntiles = a.ntiles;
@@ -1177,7 +1188,7 @@ od_sample_shard_kernel(const SampleArgs a)
 
     if (MODE != 2) {
         // ---- pass 1: the value of every tile ----
-        const int hi_w = q.bounded ? p_hi_w : p_lo;
+        const int hi_w = q.bounded && (planned || !a.same_ids) ? p_hi_w : p_lo;
         if (a.same_ids) warp_run<DTYPE, FROM_ROW>(q, a, p_lo, p_hi, hi_w, lane, out, ni);
         else warp_run<DTYPE, FROM_MAP>(q, a, p_lo, p_hi, hi_w, lane, out, ni);
         // The tile values are read by another block: the barrier orders this block's stores
@@ -1473,6 +1484,7 @@ static cudaError_t launch_sample(od_ctx *c, int mode, int32_t B, int32_t K_max, 
     a.n_accepted = n_accepted; a.temperature = temperature; a.seed = seed; a.step = step;
     a.vocab_map = c->d_vocab_map; a.inv_map = c->d_inv_map;
     a.part_tiles = part_tiles;
+    a.map_serial = c->map_serial; a.map_serial_now = c->d_map_serial;
     a.same_ids = c->map_same_ids && c->v_q % 4 == 0 && ((uintptr_t)q_rows & 15u) == 0;
     a.out_token = out_token; a.resid_mass = resid_mass; a.flags = flags;
     a.tile_val = c->d_tile_sums; a.ticket = c->d_samp_ticket;
@@ -1580,7 +1592,7 @@ cudaError_t od_launch_sample_shard_pick(od_ctx *c, int32_t B, int32_t K_max, int
 
 // What the sampler knows about the vocabulary map, on the host, in the layout of od_sample_lists.
 // `map` is the vocabulary map, `inv` its inverse; negative = none. slots: [levels] most mapped ids of a part.
-void od_sample_plan(int32_t v_q, int32_t v_p, const int32_t *map, const int32_t *inv, void *out, int32_t *slots)
+void od_sample_plan(int32_t v_q, int32_t v_p, const int32_t *map, const int32_t *inv, int32_t serial, void *out, int32_t *slots)
 {
     const OdSampleLists l = od_sample_lists(out, v_q, v_p);
     const int32_t fine_ids = od_sample_fine_tiles(v_p) * OD_SAMPLE_TILE;
@@ -1606,7 +1618,7 @@ void od_sample_plan(int32_t v_q, int32_t v_p, const int32_t *map, const int32_t 
         for (int k = 0; k < 1 << level; ++k) {
             int32_t *p = l.part + (level * OD_SAMPLE_MAX_PARTS + k) * 4;
             const int32_t n = first_rank[(k + 1) * per] - first_rank[k * per];
-            p[0] = p[1] = group; p[2] = first_rank[k * per]; p[3] = n;
+            p[0] = p[1] = group; p[2] = first_rank[k * per]; p[3] = serial;
             open[level][k] = {32, 0, p[2], p + 1};
             group += (n + 31) / 32 + v_q / 65536;
             if (n > slots[level]) slots[level] = n;
