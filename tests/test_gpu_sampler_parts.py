@@ -1,5 +1,7 @@
 """The sampler's cuts of a row (1 to 16 blocks per sequence) and its sources of the drafter's
 probabilities (staged in target order, the row itself, the inverse map) against the oracle."""
+import dataclasses
+
 import numpy as np
 import pytest
 import torch
@@ -64,3 +66,27 @@ def test_more_mapped_ids_in_a_part_than_are_staged(cuda_device):
     st = synth.make_static(w)
     st.vocab_map = np.arange(w.v_q, dtype=np.int32) + 1
     _check(w, st, cuda_device, 0, 2)
+
+
+# where ids are shared: an odd vocabulary, and rows that begin off a 16-byte boundary; a few sequences, and
+# more than are resident at a time; vocabularies that staged would fill a block's shared memory or not fit it
+@pytest.mark.parametrize("v_q, v_p, B, offset", [(333, 1000, 5, 0), (512, 1003, 5, 1), (50001, 50001, 4, 0), (50001, 50001, 300, 0),
+                                                 (60001, 60100, 300, 0), (4096, 4096, 300, 3)])
+def test_shared_ids_off_the_vector_width(cuda_device, v_q, v_p, B, offset):
+    w = _workload(B=B, k_max=2, v_q=v_q, v_p=v_p, map_kind="identity", cache_entries=0)
+    st = synth.make_static(w)
+    ctx = parity.make_context(w, st, cuda_device)
+    cache = oracle.Cache(st.runs, st.run_len, st.run_target)
+    s = synth.make_step(w, st, 0, device=cuda_device)
+    rows = torch.empty(s.q_rows.numel() + offset, device=cuda_device)[offset:].view(s.q_rows.shape).copy_(s.q_rows)
+    s = dataclasses.replace(s, q_rows=rows)
+    assert rows.data_ptr() % 16 == 4 * offset
+    logits = parity.pad_rows(s.logits)
+    stats = parity.check_step(ctx, cache, st, w, s, logits=logits, sel=list(range(min(B, 12))))
+    assert stats.sample_compared > 0
+    mp, vo, so = parity.gpu_step(ctx, s, logits=logits)
+    _, _, one = od.od_step(ctx, s.draft_ids, s.draft_len, s.q_sel, s.q_rows, logits, s.temperature, s.seed, 0)
+    torch.cuda.synchronize()
+    for name, t in vars(one).items():
+        assert torch.equal(t, vars(so)[name]), name
+    ctx.close()
