@@ -177,38 +177,49 @@ int32_t od_set_vocab_map(od_ctx *c, const int32_t *host_map)
 {
     if (!c || !host_map) return OD_ERR_INVALID_ARG;
     try {
-    std::vector<int32_t> inv((size_t)c->v_p, -1);
-    for (int32_t d = 0; d < c->v_q; ++d) {
-        const int32_t t = host_map[d];
-        if (t < 0) continue;
-        if (t >= c->v_p) return OD_ERR_INVALID_ARG;
-        if (inv[t] >= 0) return OD_ERR_MAP_NOT_INJECTIVE;
-        inv[t] = d;
-    }
-    DeviceGuard g(c->device);
-    if (!g.ok) return OD_ERR_CUDA;
-    OD_CUDA(cudaDeviceSynchronize());
-    // store -1 for every unmapped id, whatever negative value the caller used
-    std::vector<int32_t> fwd((size_t)c->v_q);
-    for (int32_t d = 0; d < c->v_q; ++d) fwd[d] = host_map[d] < 0 ? -1 : host_map[d];
-    OD_CUDA(cudaMemcpy(c->d_vocab_map, fwd.data(), fwd.size() * sizeof(int32_t), cudaMemcpyHostToDevice));
-    OD_CUDA(cudaMemcpy(c->d_inv_map, inv.data(), inv.size() * sizeof(int32_t), cudaMemcpyHostToDevice));
-    std::vector<char> lists(od_distill_lists_bytes(c->v_q, c->v_p));
-    od_distill_plan(c->v_q, c->v_p, inv.data(), lists.data());
-    OD_CUDA(cudaMemcpy(c->d_distill_lists, lists.data(), lists.size(), cudaMemcpyHostToDevice));
-    lists.resize(od_sample_lists_bytes(c->v_q, c->v_p));
-    od_sample_plan(c->v_q, c->v_p, fwd.data(), inv.data(), ++c->map_serial, lists.data(), c->sample_slots);
-    OD_CUDA(cudaMemcpy(c->d_sample_lists, lists.data(), lists.size(), cudaMemcpyHostToDevice));
-    c->map_same_ids = true;
-    c->n_mapped = 0;
-    for (int32_t d = 0; d < c->v_q; ++d) {
-        c->map_same_ids = c->map_same_ids && host_map[d] == d;
-        c->n_mapped += host_map[d] >= 0 ? 1 : 0;
-    }
-    OD_CUDA(cudaMemcpy(c->d_map_serial, &c->map_serial, sizeof(int32_t), cudaMemcpyHostToDevice));
-    OD_CUDA(cudaDeviceSynchronize());       // kernels read the maps and lists before they wait for their stream
-    c->have_map = true;
-    return OD_OK;
+        std::vector<int32_t> inv((size_t)c->v_p, -1), fwd((size_t)c->v_q);
+        bool same_ids = true;
+        int64_t n_mapped = 0;
+        for (int32_t d = 0; d < c->v_q; ++d) {
+            const int32_t t = host_map[d];
+            fwd[d] = t < 0 ? -1 : t;            // -1 for every unmapped id, whatever negative value the caller used
+            same_ids = same_ids && t == d;
+            if (t < 0) continue;
+            if (t >= c->v_p) return OD_ERR_INVALID_ARG;
+            if (inv[t] >= 0) return OD_ERR_MAP_NOT_INJECTIVE;
+            inv[t] = d;
+            ++n_mapped;
+        }
+        // where every target id is the draft id, nothing is gathered: no lists
+        std::vector<char> distill, sample;
+        int32_t slots[OD_SAMPLE_LEVELS] = {};
+        if (!same_ids) {
+            distill.resize(od_distill_lists_bytes(c->v_q, c->v_p));
+            od_distill_plan(c->v_q, c->v_p, inv.data(), distill.data());
+            sample.resize(od_sample_lists_bytes(c->v_q, c->v_p));
+            od_sample_plan(c->v_q, c->v_p, fwd.data(), inv.data(), c->map_serial + 1, sample.data(), slots);
+        }
+        DeviceGuard g(c->device);
+        if (!g.ok) return OD_ERR_CUDA;
+        OD_CUDA(cudaDeviceSynchronize());
+        c->have_map = false;                    // until all of it is there
+        OD_CUDA(cudaMemcpy(c->d_vocab_map, fwd.data(), fwd.size() * sizeof(int32_t), cudaMemcpyHostToDevice));
+        OD_CUDA(cudaMemcpy(c->d_inv_map, inv.data(), inv.size() * sizeof(int32_t), cudaMemcpyHostToDevice));
+        if (!same_ids) {
+            OD_CUDA(cudaMemcpy(c->d_distill_lists, distill.data(), distill.size(), cudaMemcpyHostToDevice));
+            OD_CUDA(cudaMemcpy(c->d_sample_lists, sample.data(), sample.size(), cudaMemcpyHostToDevice));
+        } else {                                // lists of an earlier map: of no serial number any more
+            const OdSampleLists l = od_sample_lists(c->d_sample_lists, c->v_q, c->v_p);
+            OD_CUDA(cudaMemset(l.part, 0, (size_t)((char *)l.base - (char *)l.part)));
+        }
+        ++c->map_serial;
+        OD_CUDA(cudaMemcpy(c->d_map_serial, &c->map_serial, sizeof(int32_t), cudaMemcpyHostToDevice));
+        OD_CUDA(cudaDeviceSynchronize());       // kernels read the maps and lists before they wait for their stream
+        memcpy(c->sample_slots, slots, sizeof(slots));
+        c->map_same_ids = same_ids;
+        c->n_mapped = n_mapped;
+        c->have_map = true;
+        return OD_OK;
     } catch (const std::bad_alloc &) {
         return OD_ERR_NOMEM;
     }
