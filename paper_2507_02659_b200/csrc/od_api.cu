@@ -194,10 +194,19 @@ int32_t od_set_vocab_map(od_ctx *c, const int32_t *host_map)
         std::vector<char> distill, sample;
         int32_t slots[OD_SAMPLE_LEVELS] = {};
         if (!same_ids) {
+            OdMappedIds mapped;
+            mapped.target.resize((size_t)c->v_p + 1);
+            for (int32_t t = 0, n = 0; t < c->v_p; ++t) {
+                mapped.target[n] = t;
+                n += inv[t] >= 0 ? 1 : 0;
+            }
+            mapped.target.resize((size_t)n_mapped);
+            mapped.draft.resize((size_t)n_mapped);
+            for (int64_t i = 0; i < n_mapped; ++i) mapped.draft[i] = inv[mapped.target[i]];
             distill.resize(od_distill_lists_bytes(c->v_q, c->v_p));
-            od_distill_plan(c->v_q, c->v_p, inv.data(), distill.data());
+            od_distill_plan(c->v_q, c->v_p, mapped, distill.data());
             sample.resize(od_sample_lists_bytes(c->v_q, c->v_p));
-            od_sample_plan(c->v_q, c->v_p, fwd.data(), inv.data(), c->map_serial + 1, sample.data(), slots);
+            od_sample_plan(c->v_q, c->v_p, mapped, c->map_serial + 1, sample.data(), slots);
         }
         DeviceGuard g(c->device);
         if (!g.ok) return OD_ERR_CUDA;

@@ -6,14 +6,16 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <vector>
+
 #include "omnidraft.h"
 
 #define OD_WARP 32
 #define OD_GROUP 32                 // slots of one hash-table probe group
 #define OD_SAMPLE_TILE 256          // elements of one residual-sampler tile (8 per lane of a warp)
 #define OD_SAMPLE_THREADS 256       // of the vocabulary shards' sampler
-#define OD_SAMPLE_LEVELS 5          // 1, 2, 4, 8 or 16 blocks draw for one sequence
-#define OD_SAMPLE_MAX_PARTS 16      // (16: a non-portable cluster)
+#define OD_SAMPLE_LEVELS 7          // 1, 2, 3, 4, 6, 8 or 16 blocks draw for one sequence
+#define OD_SAMPLE_MAX_PARTS 16      // (over 8: a non-portable cluster)
 #define OD_SAMPLE_MAX_SLOTS 53248   // mapped ids of a part: 208 KB of shared memory
 #define OD_SAMPLE_SMEM_MAX (200 * 1024)  // dynamic shared memory the sampler may ask for: 8 bytes per tile
 #define OD_VERIFY_SEG_MAX 64        // most segments (partials) one logit row is cut into
@@ -147,8 +149,20 @@ size_t od_sample_smem_bytes(int32_t ntiles);            // dynamic shared memory
 // opt in to the dynamic shared memory and the cluster size that the sampler's kernels may ask for
 cudaError_t od_sample_prepare_device(size_t bytes, int32_t *clusters);   // clusters: [levels] resident at a time
 
+// The pairs of a vocabulary map in target-id order (host).
+struct OdMappedIds {
+    std::vector<int32_t> target, draft;
+};
+
+// The lists below: pads the open group of 32 words at `next` and gives the groups from `end` on their base.
+inline void od_end_group(uint32_t *words, uint32_t *&next, int32_t *bases, int32_t base, int32_t &end)
+{
+    while ((next - words) % 32) *next++ = 0xFFFFu;
+    for (; end < (next - words) / 32; ++end) bases[end] = base;
+}
+
 // What the sampler knows about the vocabulary map, one block of memory. The mapped target ids in
-// order have ranks 0, 1, ...; a row's tiles are cut into 1, 2, 4, 8, 16 parts (the levels), and a
+// order have ranks 0, 1, ...; a row's tiles are cut into 1, 2, 3, ... parts (the levels), and a
 // part's mapped ids, in draft-id order, are a list in groups of 32: an entry is (draft id - the
 // group's base) << 16 | (rank - the part's first rank), or 0xFFFF in the low half where the
 // group has no more.
@@ -162,7 +176,7 @@ struct OdSampleLists {
 inline OdSampleLists od_sample_lists(void *base, int32_t v_q, int32_t v_p)
 {
     OdSampleLists l;
-    // a group ends full, or at a gap of over 65535 draft ids, or with its part
+    // a group ends full, or with 65536 draft ids, or with its part
     l.groups = ((int64_t)(v_q < v_p ? v_q : v_p) + 31) / 32 + OD_SAMPLE_MAX_PARTS * ((int64_t)v_q / 65536 + 2);
     l.word = (uint32_t *)base;
     l.part = (int32_t *)(l.word + OD_SAMPLE_LEVELS * l.groups * 32);
@@ -175,10 +189,19 @@ inline size_t od_sample_lists_bytes(int32_t v_q, int32_t v_p)
     const OdSampleLists l = od_sample_lists(nullptr, v_q, v_p);
     return (size_t)((uintptr_t)(l.octet + (v_p + 7) / 8) - (uintptr_t)nullptr);
 }
-// tiles of a 16th of a row: a part of level l is 16 >> l of them
-inline int32_t od_sample_fine_tiles(int32_t v_p) { return ((v_p + OD_SAMPLE_TILE - 1) / OD_SAMPLE_TILE + OD_SAMPLE_MAX_PARTS - 1) / OD_SAMPLE_MAX_PARTS; }
+// parts of a level, and the tiles of one
+inline int32_t od_sample_parts(int level)
+{
+    const int32_t parts[OD_SAMPLE_LEVELS] = {1, 2, 3, 4, 6, 8, 16};
+    return parts[level];
+}
+inline int32_t od_sample_part_tiles(int32_t v_p, int level)
+{
+    const int32_t n = od_sample_parts(level);
+    return ((v_p + OD_SAMPLE_TILE - 1) / OD_SAMPLE_TILE + n - 1) / n;
+}
 // host; slots: [levels] most mapped ids of a part
-void od_sample_plan(int32_t v_q, int32_t v_p, const int32_t *map, const int32_t *inv, int32_t serial, void *out, int32_t *slots);
+void od_sample_plan(int32_t v_q, int32_t v_p, const OdMappedIds &mapped, int32_t serial, void *out, int32_t *slots);
 
 // vocabulary shards (columns [shard_lo, shard_lo + shard_len) of the rows on this GPU)
 cudaError_t od_launch_verify_shard_stats(od_ctx *c, int32_t B, int32_t K_max, int32_t shard_lo,
@@ -233,7 +256,7 @@ struct OdDistillLists {
 inline OdDistillLists od_distill_lists(void *base, int32_t v_q, int32_t v_p)
 {
     OdDistillLists l;
-    // a group ends full, or at a gap of over 65535 target ids, or with its chunk; a chunk is whole
+    // a group ends full, or with 65536 target ids, or with its chunk; a chunk is whole
     // multiples of 32 ids
     l.groups = OD_DISTILL_MAX_CHUNKS * (((int64_t)v_q + 255) / 256 + (int64_t)v_p / 65536 + 1);
     l.word = (uint32_t *)base;
@@ -247,7 +270,7 @@ inline size_t od_distill_lists_bytes(int32_t v_q, int32_t v_p)
     const OdDistillLists l = od_distill_lists(nullptr, v_q, v_p);
     return (size_t)((uintptr_t)(l.bits + (v_q + 31) / 32) - (uintptr_t)nullptr);
 }
-void od_distill_plan(int32_t v_q, int32_t v_p, const int32_t *inv, void *out);   // host
+void od_distill_plan(int32_t v_q, int32_t v_p, const OdMappedIds &mapped, void *out);   // host
 cudaError_t od_distill_prepare_device(int32_t v_q);
 
 void od_cache_free_dynamic(od_ctx *c);   // frees what od_cache_configure allocated beyond keys / vals

@@ -34,6 +34,8 @@
 // threads (39 to 59 us), bulk prefetches of the rows into L2 (no change), one chunk at 64 KB (45 us).
 #include <float.h>
 
+#include <vector>
+
 #include "od_common.cuh"
 
 namespace {
@@ -622,43 +624,34 @@ cudaError_t od_distill_prepare_device(int32_t v_q)
 }
 
 // The gather lists of the distillation kernel, on the host, in the layout of od_distill_lists.
-// `inv` is the inverse map: draft id of each target id, or negative.
-void od_distill_plan(int32_t v_q, int32_t v_p, const int32_t *inv, void *out)
+void od_distill_plan(int32_t v_q, int32_t v_p, const OdMappedIds &mapped, void *out)
 {
     const OdDistillLists l = od_distill_lists(out, v_q, v_p);
     for (int w = 0; w < (v_q + 31) / 32; ++w) l.bits[w] = 0u;
-    struct Open {
-        int32_t n, base;                                     // a chunk's open group: n entries so far, from target `base`
-        int32_t *end;                                        // one past it
-    } open[OD_DISTILL_LEVELS][OD_DISTILL_MAX_CHUNKS];
+    for (int32_t d : mapped.draft) l.bits[d >> 5] |= 1u << (d & 31);
+    const int32_t fine = fine_ids(v_q);
+    std::vector<uint8_t> eighth((size_t)(v_q + 31) / 32);    // of 32 ids
+    for (size_t w = 0; w < eighth.size(); ++w) eighth[w] = (uint8_t)((int32_t)w * 32 / fine);
     int first = OD_DISTILL_LEVELS - 1;                       // the coarsest level that a launch can ask for
     while (first > 0 && chunk_ids(v_q, first - 1) * 2 <= CHUNK_BYTES) --first;
-    for (int level = 0; level < OD_DISTILL_LEVELS; ++level)
+    for (int level = 0; level < OD_DISTILL_LEVELS; ++level) {
+        uint32_t *words = l.word + (size_t)level * l.groups * 32, *next[OD_DISTILL_MAX_CHUNKS];   // a chunk's next entry
+        int32_t *bases = l.base + (size_t)level * l.groups, *ofs = l.ofs + level * OD_DISTILL_MAX_CHUNKS * 2;
         for (int k = 0; k < OD_DISTILL_MAX_CHUNKS; ++k) {
-            int32_t *ofs = l.ofs + (level * OD_DISTILL_MAX_CHUNKS + k) * 2;
-            ofs[0] = ofs[1] = (int32_t)(k * (l.groups >> level));
-            open[level][k] = {32, 0, ofs + 1};
+            ofs[k * 2] = ofs[k * 2 + 1] = (int32_t)(k * (l.groups >> level));
+            next[k] = words + (size_t)ofs[k * 2] * 32;
         }
-    // a chunk's entries in target-id order; a new group of 32 where one is full or the next
-    // target is over 65535 ids on
-    const int32_t fine = fine_ids(v_q);
-    for (int32_t t = 0; t < v_p; ++t) {
-        const int32_t d = inv[t];
-        if (d < 0) continue;
-        const int32_t f = d / fine;
-        l.bits[d >> 5] |= 1u << (d & 31);
-        for (int level = first; level < OD_DISTILL_LEVELS; ++level) {
-            const int32_t shift = OD_DISTILL_LEVELS - 1 - level, k = f >> shift;
-            Open &o = open[level][k];
-            if (o.n == 32 || t - o.base > 0xFFFF) {
-                const size_t g = (size_t)level * l.groups + (*o.end)++;
-                l.base[g] = t;
-                for (int i = 0; i < 32; ++i) l.word[g * 32 + i] = 0xFFFFu;
-                o.n = 0; o.base = t;
-            }
+        if (level < first) continue;
+        const int32_t shift = OD_DISTILL_LEVELS - 1 - level;
+        // a chunk's entries in target-id order; groups end with 65536 target ids, of which the first is their base
+        size_t i = 0;
+        for (int32_t page = 0; page < v_p; page += 65536) {
             // (a chunk of more than OD_DISTILL_MAX_CHUNK_IDS ids is not asked for: the cut does not matter)
-            l.word[((size_t)level * l.groups + *o.end - 1) * 32 + o.n++] =
-                (uint32_t)(t - o.base) << 16 | (uint32_t)((d - (k << shift) * fine) & 0xFFFF);
+            for (; i < mapped.target.size() && mapped.target[i] - page < 65536; ++i) {
+                const int32_t d = mapped.draft[i], k = eighth[d >> 5] >> shift;
+                *next[k]++ = (uint32_t)(mapped.target[i] - page) << 16 | (uint32_t)((d - (k << shift) * fine) & 0xFFFF);
+            }
+            for (int k = 0; k < 1 << level; ++k) od_end_group(words, next[k], bases, page, ofs[k * 2 + 1]);
         }
     }
 }

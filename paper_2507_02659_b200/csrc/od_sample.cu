@@ -46,6 +46,8 @@
 //           window (offset by the shares before it) as in pass 2.
 #include <float.h>
 
+#include <vector>
+
 #include "od_common.cuh"
 #include "od_decide.cuh"
 
@@ -788,7 +790,7 @@ __device__ __forceinline__ bool pick_in_tile(const SeqState &q, const SampleArgs
 
 // ---- the whole step on full rows -------------------------------------------------------------
 //
-// Grid (P, B), clusters of P blocks of 16 warps: one cluster draws for one sequence. Pass 1 as
+// Grid (P, B), clusters of P blocks (od_sample_parts) of 16 warps: one cluster draws for one sequence. Pass 1 as
 // above, the tile values of a warp's run staying in its block's shared memory. A block sends its
 // sum to all blocks of the cluster (distributed shared memory), and behind ONE cluster barrier
 // every warp has the blocks' sums and its own block's runs, scans both and knows whether the draw
@@ -1382,7 +1384,7 @@ static cudaError_t allow_cluster16(size_t bytes)
 template <int DTYPE>
 static cudaError_t prepare_kernels(size_t bytes)
 {
-    const size_t staged = (size_t)OD_SAMPLE_MAX_SLOTS * 4 + 8 * 1024;
+    const size_t staged = (size_t)(OD_SAMPLE_MAX_SLOTS + 1) * 4 + 8 * 1024;
     cudaError_t e = allow_cluster16<DTYPE, false, FROM_MAP>(bytes);
     if (e == cudaSuccess) e = allow_cluster16<DTYPE, true, FROM_MAP>(bytes);
     if (e == cudaSuccess) e = allow_cluster16<DTYPE, false, FROM_ROW>(bytes);
@@ -1405,10 +1407,11 @@ cudaError_t od_sample_prepare_device(size_t bytes, int32_t *clusters)
     if (e != cudaSuccess) return e;
     for (int level = 0; level < OD_SAMPLE_LEVELS; ++level) {
         cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3(1u << level); cfg.blockDim = dim3(CTHREADS); cfg.dynamicSmemBytes = 64 * 1024;
+        const unsigned parts = (unsigned)od_sample_parts(level);
+        cfg.gridDim = dim3(parts); cfg.blockDim = dim3(CTHREADS); cfg.dynamicSmemBytes = 64 * 1024;
         cudaLaunchAttribute attr[1];
         attr[0].id = cudaLaunchAttributeClusterDimension;
-        attr[0].val.clusterDim.x = 1u << level; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+        attr[0].val.clusterDim.x = parts; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
         cfg.attrs = attr; cfg.numAttrs = 1;
         int n = 0;
         if (cudaOccupancyMaxActiveClusters(&n, od_sample_kernel<OD_BF16, true, STAGED>, &cfg) != cudaSuccess) {
@@ -1455,20 +1458,30 @@ static cudaError_t launch_sample(od_ctx *c, int mode, int32_t B, int32_t K_max, 
     int64_t tpw = c->opt_sample_tiles_per_warp;
     int blocks_x = 1, level = 0, part_tiles = 0;
     if (mode == 0) {
-        // Parts (blocks) per sequence: as many as still make one resident wave (73 sequences of four blocks
-        // have 296 places, but not as resident clusters: 32.3 us, of two blocks each 29.9), and no more than have a tile for every warp (19 sequences of 100277 ids, the
-        // three calls: 25.2 us with 4 parts, 23.3 with 8, 27.0 with 16, which is two waves; one of
-        // 152064: 29.1 / 27.1 / 26.7).
-        const int fine = od_sample_fine_tiles(c->v_p);
-        const int most = c->sample_clusters[OD_SAMPLE_LEVELS - 1] > 0 ? OD_SAMPLE_LEVELS - 1 : OD_SAMPLE_LEVELS - 2;
-        while (level < most && (tpw > 0 ? fine * (OD_SAMPLE_MAX_PARTS >> level) > tpw * CWARPS
-                                        : B <= c->sample_clusters[level + 1] &&
-                                              fine * (OD_SAMPLE_MAX_PARTS >> level) > CWARPS))
-            ++level;
+        // Parts (blocks) per sequence: as many as still make one resident wave of clusters, and no more
+        // than have a tile for every warp (19 sequences of 100277 ids, the three calls: 25.2 us with 4 parts, 23.3
+        // with 8, 27.0 with 16, which is two waves); under the option, the fewest of a power of two that
+        // keep to it. 3 and 6 are for batches that just miss 4 and 8 (device time of the step, 37 and 73
+        // sequences of 128256 bf16 ids: 23.7 -> 23.0 and 35.1 -> 32.9 us, of 152064 fp32 ids 35.6 -> 33.8 and 58.5
+        // -> 52.9), where they save a warp two tiles (else they only add blocks: 37 of 32000 ids 14.4 us with 6,
+        // 14.1 with 4). 12 was slower than 8 (19 sequences: 20.9 us, 18.4): a large cluster waits long for its place.
+        int most = OD_SAMPLE_LEVELS - 1;
+        while (most > 0 && c->sample_clusters[most] <= 0) --most;
+        for (int next = 1; next <= most; ++next) {
+            const int32_t tiles = od_sample_part_tiles(c->v_p, level), parts = od_sample_parts(next);
+            const bool doubling = (parts & (parts - 1)) == 0;
+            if (tpw > 0) {
+                if (doubling && tiles > tpw * CWARPS) level = next;
+            } else {
+                if (B > c->sample_clusters[next]) break;
+                const int32_t then = od_sample_part_tiles(c->v_p, next);
+                if (doubling ? tiles > CWARPS : (tiles + CWARPS - 1) / CWARPS >= (then + CWARPS - 1) / CWARPS + 2) level = next;
+            }
+        }
         // staged probabilities of over 100 KB would leave room for one block per multiprocessor
         while (level < most && !c->map_same_ids && c->sample_slots[level] * 4 > 100 * 1024) ++level;
-        blocks_x = 1 << level;
-        part_tiles = fine * (OD_SAMPLE_MAX_PARTS >> level);
+        blocks_x = od_sample_parts(level);
+        part_tiles = od_sample_part_tiles(c->v_p, level);
         tpw = (part_tiles + CWARPS - 1) / CWARPS;
     } else {
         if (tpw <= 0) {
@@ -1600,57 +1613,57 @@ cudaError_t od_launch_sample_shard_pick(od_ctx *c, int32_t B, int32_t K_max, int
 
 
 // What the sampler knows about the vocabulary map, on the host, in the layout of od_sample_lists.
-// `map` is the vocabulary map, `inv` its inverse; negative = none. slots: [levels] most mapped ids of a part.
-void od_sample_plan(int32_t v_q, int32_t v_p, const int32_t *map, const int32_t *inv, int32_t serial, void *out, int32_t *slots)
+// slots: [levels] most mapped ids of a part.
+void od_sample_plan(int32_t v_q, int32_t v_p, const OdMappedIds &mapped, int32_t serial, void *out, int32_t *slots)
 {
     const OdSampleLists l = od_sample_lists(out, v_q, v_p);
-    const int32_t fine_ids = od_sample_fine_tiles(v_p) * OD_SAMPLE_TILE;
-    int32_t first_rank[OD_SAMPLE_MAX_PARTS + 1], rank = 0;   // of the 16ths
-    for (int32_t o = 0, next = 0; o < (v_p + 7) / 8; ++o) {
-        while (next < OD_SAMPLE_MAX_PARTS && (int64_t)next * fine_ids <= (int64_t)o * 8) first_rank[next++] = rank;
-        uint32_t mask = 0;
-        for (int32_t e = 0; e < 8 && o * 8 + e < v_p; ++e) mask |= inv[o * 8 + e] >= 0 ? 1u << e : 0u;
+    const int32_t total = (int32_t)mapped.target.size(), octets = (v_p + 7) / 8;
+    for (int32_t o = 0; o < octets; ++o) l.octet[o] = 0u;
+    for (int32_t t : mapped.target) l.octet[t >> 3] |= 1u << (t & 7);
+    for (int32_t o = 0, rank = 0; o < octets; ++o) {
+        const uint32_t mask = l.octet[o];
         l.octet[o] = (uint32_t)rank << 8 | mask;
         rank += __builtin_popcount(mask);
-        if (o + 1 == (v_p + 7) / 8)
-            while (next <= OD_SAMPLE_MAX_PARTS) first_rank[next++] = rank;
     }
-    first_rank[OD_SAMPLE_MAX_PARTS] = rank;
-    struct Open {
-        int32_t n, base, rank0;                              // a part's open group: n entries so far, from draft id `base`
-        int32_t *end;                                        // one past it
-    } open[OD_SAMPLE_LEVELS][OD_SAMPLE_MAX_PARTS];
+    // the mapped ids in draft-id order
+    std::vector<int32_t> rank_of((size_t)v_q, -1), draft((size_t)v_q + 1);
+    for (int32_t r = 0; r < total; ++r) rank_of[mapped.draft[r]] = r;
+    for (int32_t d = 0, n = 0; d < v_q; ++d) {
+        draft[n] = d;
+        n += rank_of[d] >= 0 ? 1 : 0;
+    }
+    std::vector<int32_t> rank((size_t)total), tile((size_t)total);
+    for (int32_t i = 0; i < total; ++i) {
+        rank[i] = rank_of[draft[i]];
+        tile[i] = mapped.target[rank[i]] / OD_SAMPLE_TILE;
+    }
+    std::vector<uint8_t> part_of((size_t)(v_p + OD_SAMPLE_TILE - 1) / OD_SAMPLE_TILE);
     for (int level = 0; level < OD_SAMPLE_LEVELS; ++level) {
-        const int per = OD_SAMPLE_MAX_PARTS >> level;
-        int32_t group = 0;
+        const int32_t parts = od_sample_parts(level), tiles = od_sample_part_tiles(v_p, level);
+        for (size_t t = 0; t < part_of.size(); ++t) part_of[t] = (uint8_t)((int32_t)t / tiles);
+        const auto rank_at = [&](int32_t part) {             // of the first mapped id of a part
+            const int64_t t = (int64_t)part * tiles * OD_SAMPLE_TILE;
+            return t < v_p ? (int32_t)(l.octet[t >> 3] >> 8) : total;
+        };
+        uint32_t *words = l.word + (size_t)level * l.groups * 32, *next[OD_SAMPLE_MAX_PARTS];   // a part's next entry
+        int32_t *bases = l.base + (size_t)level * l.groups, rank0[OD_SAMPLE_MAX_PARTS], group = 0;
         slots[level] = 0;
-        for (int k = 0; k < 1 << level; ++k) {
+        for (int32_t k = 0; k < parts; ++k) {
+            const int32_t n = rank_at(k + 1) - (rank0[k] = rank_at(k));
             int32_t *p = l.part + (level * OD_SAMPLE_MAX_PARTS + k) * 4;
-            const int32_t n = first_rank[(k + 1) * per] - first_rank[k * per];
-            p[0] = p[1] = group; p[2] = first_rank[k * per]; p[3] = serial;
-            open[level][k] = {32, 0, p[2], p + 1};
+            p[0] = p[1] = group; p[2] = rank0[k]; p[3] = serial;
+            next[k] = words + (size_t)group * 32;
             group += (n + 31) / 32 + v_q / 65536;
             if (n > slots[level]) slots[level] = n;
         }
-    }
-    // a part's entries in draft-id order; a new group of 32 where one is full or the next id is
-    // over 65535 on
-    for (int32_t d = 0; d < v_q; ++d) {
-        const int32_t t = map[d];
-        if (t < 0) continue;
-        const uint32_t oct = l.octet[t >> 3];
-        const int32_t at = (int32_t)(oct >> 8) + __builtin_popcount(oct & ((1u << (t & 7)) - 1u)), f = t / fine_ids;
-        for (int level = 0; level < OD_SAMPLE_LEVELS; ++level) {
-            Open &o = open[level][f >> (OD_SAMPLE_LEVELS - 1 - level)];
-            if (o.n == 32 || d - o.base > 0xFFFF) {
-                const size_t g = (size_t)level * l.groups + (*o.end)++;
-                l.base[g] = d;
-                for (int i = 0; i < 32; ++i) l.word[g * 32 + i] = 0xFFFFu;
-                o.n = 0; o.base = d;
+        // a part's entries in draft-id order; groups end with 65536 draft ids, of which the first is their base
+        for (int32_t i = 0, page = 0; page < v_q; page += 65536) {
+            // (a part of more than OD_SAMPLE_MAX_SLOTS ids is not staged: the cut of its ranks does not matter)
+            for (; i < total && draft[i] - page < 65536; ++i) {
+                const int32_t k = part_of[tile[i]];
+                *next[k]++ = (uint32_t)(draft[i] - page) << 16 | (uint32_t)((rank[i] - rank0[k]) & 0xFFFF);
             }
-            // (a part of more than OD_SAMPLE_MAX_SLOTS ids is not staged: the cut does not matter)
-            l.word[((size_t)level * l.groups + *o.end - 1) * 32 + o.n++] =
-                (uint32_t)(d - o.base) << 16 | (uint32_t)((at - o.rank0) & 0xFFFF);
+            for (int32_t k = 0; k < parts; ++k) od_end_group(words, next[k], bases, page, l.part[(level * OD_SAMPLE_MAX_PARTS + k) * 4 + 1]);
         }
     }
 }

@@ -90,3 +90,24 @@ def test_shared_ids_off_the_vector_width(cuda_device, v_q, v_p, B, offset):
     for name, t in vars(one).items():
         assert torch.equal(t, vars(so)[name]), name
     ctx.close()
+
+
+def test_parts_between_the_powers_of_two(cuda_device):
+    """From one sequence to more than fill the chip: every number of parts that the batch can choose."""
+    seen = set()
+    for B in (1, 13, 24, 30, 37, 48, 60, 73, 90, 148, 300):
+        w = _workload(B=B, k_max=2, v_q=1500, v_p=70001, cache_entries=0, mapped_frac=0.9, gen_seed=0xFACE50 + B)
+        st = synth.make_static(w)
+        ctx = parity.make_context(w, st, cuda_device)
+        cache = oracle.Cache(st.runs, st.run_len, st.run_target)
+        s = synth.make_step(w, st, 0, device=cuda_device)
+        logits = parity.pad_rows(s.logits)
+        stats = parity.check_step(ctx, cache, st, w, s, logits=logits, sel=sorted({0, B // 2, B - 1}))
+        seen.add(ctx.last_launch_info(2) // B)
+        mp, vo, so = parity.gpu_step(ctx, s, logits=logits)
+        _, _, one = od.od_step(ctx, s.draft_ids, s.draft_len, s.q_sel, s.q_rows, logits, s.temperature, s.seed, 0)
+        torch.cuda.synchronize()
+        for name, t in vars(one).items():
+            assert torch.equal(t, vars(so)[name]), name
+        ctx.close()
+    assert seen == {1, 2, 3, 4, 6, 8, 16}, seen
