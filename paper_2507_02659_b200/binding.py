@@ -7,12 +7,15 @@ CPU fallback: if the library is missing or a call fails, this module raises.
 
 The calls of a decode loop go through `_marshal` (csrc/marshal.cpp), which looks at the
 tensors natively; where it finds an argument that the call does not take as it stands, it calls
-nothing, and the checks here say what is wrong.
+nothing, and the checks here say what is wrong. Where the extension is not usable (not built, or
+for another Python or torch) the checks here do it all. od_step_host, which takes a millisecond, and
+od_verify_noalloc, which has no context, always go through them.
 """
 from __future__ import annotations
 
 import ctypes as C
 import os
+import warnings
 from dataclasses import dataclass
 from typing import Optional
 
@@ -96,10 +99,29 @@ def lib():
         for name in EXPORTS:
             if name not in ("od_status_string", "od_last_launch_info"):
                 getattr(L, name).restype = i32
-        from . import _marshal
-        _native = _marshal
+        _native = _load_marshal()
         _lib = L
     return _lib
+
+
+class _InPython:
+    """In the place of _marshal: takes no call, so that the wrappers go on to their own checks."""
+
+    def __getattr__(self, name):
+        return lambda *args: None
+
+
+def _load_marshal():
+    from . import build
+    try:
+        from . import _marshal
+        if _marshal.built_for != build.built_for():
+            raise ImportError(f"built for {_marshal.built_for}, this is {build.built_for()}")
+    except ImportError as e:
+        warnings.warn(f"_marshal is not usable ({e}): calls look at their arguments in Python, 15 to 20 us a step "
+                      "(`python -m paper_2507_02659_b200.build` builds it)", RuntimeWarning)
+        return _InPython()
+    return _marshal
 
 
 def _check(status: int, where: str):

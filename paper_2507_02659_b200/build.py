@@ -11,6 +11,7 @@ ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libomnidraft.so")
 EXT = os.path.join(HERE, "_marshal.so")
+EXT_FOR = os.path.join(HERE, "_build", "marshal_built_for")
 SOURCES = ["od_api.cu", "od_map.cu", "od_verify.cu", "od_sample.cu", "od_noalloc.cu", "od_exit.cu", "od_cache.cu", "od_distill.cu"]
 
 
@@ -21,31 +22,52 @@ def _newest_source() -> float:
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
-    if force or not os.path.exists(EXT) or os.path.getmtime(EXT) < _newest_source():
-        _build_lib(force, verbose)
-        _build_marshal(verbose)
+    _build_lib(force, verbose)
+    _build_marshal(force, verbose)
     return LIB
 
 
-def _build_marshal(verbose: bool) -> None:
+def built_for() -> str:
+    """What _marshal.so depends on besides its sources."""
+    import platform
+    import torch
+    return f"python {platform.python_version()}, torch {torch.__version__}"
+
+
+def _build_marshal(force: bool = False, verbose: bool = False) -> None:
+    """The extension is optional: without it (no g++, no torch headers) the binding marshals in Python."""
     import sysconfig
     import torch
+    fresh = os.path.exists(EXT) and os.path.getmtime(EXT) >= _newest_source()
+    if not force and fresh and os.path.exists(EXT_FOR) and open(EXT_FOR).read() == built_for():
+        return
     root = os.path.dirname(torch.__file__)
     inc = os.path.join(root, "include")
     cuda = os.environ.get("CUDA_HOME", "/usr/local/cuda")
     tmp = EXT + f".{os.getpid()}.tmp"
     cmd = ["g++", "-O2", "-std=c++17", "-shared", "-fPIC", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch.compiled_with_cxx11_abi())}",
+           f'-DOD_BUILT_FOR="{built_for()}"',
            "-I", os.path.join(ROOT, "include"), "-I", inc, "-I", os.path.join(inc, "torch", "csrc", "api", "include"),
            "-I", os.path.join(cuda, "include"), "-I", sysconfig.get_paths()["include"], "-o", tmp,
            os.path.join(CSRC, "marshal.cpp"), "-L", HERE, "-l:libomnidraft.so", "-L", os.path.join(root, "lib"),
            "-ltorch_python", "-ltorch_cpu", "-lc10", "-lc10_cuda",
            "-Wl,-rpath,$ORIGIN:" + os.path.join(root, "lib")]
-    res = subprocess.run(cmd, capture_output=True, text=True)
-    if verbose or res.returncode != 0:
-        sys.stderr.write(res.stdout + res.stderr)
-    if res.returncode != 0:
-        raise RuntimeError("g++ failed building _marshal.so")
+    try:
+        res = subprocess.run(cmd, capture_output=True, text=True)
+        failed, said = res.returncode != 0, res.stdout + res.stderr
+    except OSError as e:
+        failed, said = True, f"{e}\n"
+    if verbose or failed:
+        sys.stderr.write(said)
+    if failed:
+        sys.stderr.write("_marshal.so could not be built: the binding will look at its arguments in Python\n")
+        if os.path.exists(EXT):                             # of other sources, or for another torch
+            os.remove(EXT)
+        return
     os.replace(tmp, EXT)
+    os.makedirs(os.path.dirname(EXT_FOR), exist_ok=True)
+    with open(EXT_FOR, "w") as f:
+        f.write(built_for())
 
 
 def _build_lib(force: bool = False, verbose: bool = False) -> str:

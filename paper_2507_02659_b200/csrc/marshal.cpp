@@ -127,14 +127,15 @@ struct Logits {
     }
 };
 
-// calls fn with the tuple's elements (a braced tuple evaluates its elements in order)
+// calls fn with the tuple's elements (a braced tuple evaluates its elements in order) and the current stream
 template <typename F, typename T>
 PyObject *call(const Args &x, F fn, const T &args)
 {
     if (!x.ok || x.at != x.n) Py_RETURN_NONE;
+    void *stream = x.stream();
     int32_t status;
     Py_BEGIN_ALLOW_THREADS
-    status = std::apply(fn, args);
+    status = std::apply([&](auto... v) { return fn(v..., stream); }, args);
     Py_END_ALLOW_THREADS
     return PyLong_FromLong(status);
 }
@@ -145,7 +146,7 @@ PyObject *map_proposals(PyObject *, PyObject *const *a, Py_ssize_t n)
     od_ctx *c = x.ctx();
     const int32_t B = x.i32(), K = x.i32();
     std::tuple args{c, B, K, x.pi(), x.pi(), x.pf(), x.pi(), x.pf(), x.pi(), x.pi(), x.pi(), x.pb(), x.pu()};
-    return call(x, [&](auto... v) { return od_map_proposals(v..., x.stream()); }, args);
+    return call(x, od_map_proposals, args);
 }
 
 PyObject *verify(PyObject *, PyObject *const *a, Py_ssize_t n)
@@ -156,7 +157,7 @@ PyObject *verify(PyObject *, PyObject *const *a, Py_ssize_t n)
     const Logits l(x, B, K, v_p);
     std::tuple args{c, B, K, l.p, l.dtype, l.row_stride, l.seq_stride, x.pi(), x.pf(), x.pi(), x.pi(), x.pf(), x.pl(),
                     x.u64(), x.pf(), x.pf(), x.pf(), x.pf(), x.pi(), x.pi(), x.pu()};
-    return call(x, [&](auto... v) { return od_verify(v..., x.stream()); }, args);
+    return call(x, od_verify, args);
 }
 
 PyObject *sample_residual(PyObject *, PyObject *const *a, Py_ssize_t n)
@@ -167,7 +168,7 @@ PyObject *sample_residual(PyObject *, PyObject *const *a, Py_ssize_t n)
     const Logits l(x, B, K, v_p);
     std::tuple args{c, B, K, l.p, l.dtype, l.row_stride, l.seq_stride, x.pf(), x.pf(), x.q_rows(B, K, v_q), x.pi(), x.pi(),
                     x.pf(), x.pi(), x.pi(), x.pi(), x.pb(), x.pi(), x.pf(), x.pl(), x.u64(), x.pi(), x.pf(), x.pu()};
-    return call(x, [&](auto... v) { return od_sample_residual(v..., x.stream()); }, args);
+    return call(x, od_sample_residual, args);
 }
 
 PyObject *step(PyObject *, PyObject *const *a, Py_ssize_t n)
@@ -181,7 +182,7 @@ PyObject *step(PyObject *, PyObject *const *a, Py_ssize_t n)
     std::tuple args{c, B, K, ids, len, q_sel, q, l.p, l.dtype, l.row_stride, l.seq_stride, x.pf(), x.pl(), x.u64(),
                     x.pi(), x.pf(), x.pi(), x.pi(), x.pi(), x.pb(), x.pu(),
                     x.pf(), x.pf(), x.pf(), x.pf(), x.pi(), x.pi(), x.pu(), x.pi(), x.pf(), x.pu()};
-    return call(x, [&](auto... v) { return od_step(v..., x.stream()); }, args);
+    return call(x, od_step, args);
 }
 
 PyObject *exit_rule(PyObject *, PyObject *const *a, Py_ssize_t n)
@@ -190,7 +191,7 @@ PyObject *exit_rule(PyObject *, PyObject *const *a, Py_ssize_t n)
     od_ctx *c = x.ctx();
     const int32_t B = x.i32(), K = x.i32();
     std::tuple args{c, B, K, x.pf(), x.pi(true), x.f32(), x.pi(), x.pf(), x.pu()};
-    return call(x, [&](auto... v) { return od_exit_rule(v..., x.stream()); }, args);
+    return call(x, od_exit_rule, args);
 }
 
 PyObject *distill_loss(PyObject *, PyObject *const *a, Py_ssize_t n)
@@ -203,7 +204,7 @@ PyObject *distill_loss(PyObject *, PyObject *const *a, Py_ssize_t n)
     const Logits l(x, B, K, v_p);
     std::tuple args{c, B, K, q, ids, tgt, s0, sl, m, l.p, l.dtype, l.row_stride, l.seq_stride, x.pf(), x.pf(), x.pf(),
                     x.pf(), x.f32(), x.i32(), x.pf(), x.pf(true)};
-    return call(x, [&](auto... v) { return od_distill_loss(v..., x.stream()); }, args);
+    return call(x, od_distill_loss, args);
 }
 
 PyObject *verify_shard_stats(PyObject *, PyObject *const *a, Py_ssize_t n)
@@ -213,7 +214,7 @@ PyObject *verify_shard_stats(PyObject *, PyObject *const *a, Py_ssize_t n)
     const int32_t B = x.i32(), K = x.i32(), lo = x.i32(), len = x.i32();
     const Logits l(x, B, K, len);
     std::tuple args{c, B, K, lo, len, l.p, l.dtype, l.row_stride, l.seq_stride, x.pi(), x.pi(), x.pf(), x.pf()};
-    return call(x, [&](auto... v) { return od_verify_shard_stats(v..., x.stream()); }, args);
+    return call(x, od_verify_shard_stats, args);
 }
 
 PyObject *verify_shard_finish(PyObject *, PyObject *const *a, Py_ssize_t n)
@@ -223,7 +224,7 @@ PyObject *verify_shard_finish(PyObject *, PyObject *const *a, Py_ssize_t n)
     const int32_t B = x.i32(), K = x.i32(), shards = x.i32();
     std::tuple args{c, B, K, shards, x.pf(), x.pi(), x.pf(), x.pi(), x.pi(), x.pf(), x.pl(), x.u64(),
                     x.pf(), x.pf(), x.pf(), x.pf(), x.pi(), x.pi(), x.pu()};
-    return call(x, [&](auto... v) { return od_verify_shard_finish(v..., x.stream()); }, args);
+    return call(x, od_verify_shard_finish, args);
 }
 
 PyObject *sample_shard_mass(PyObject *, PyObject *const *a, Py_ssize_t n)
@@ -234,7 +235,7 @@ PyObject *sample_shard_mass(PyObject *, PyObject *const *a, Py_ssize_t n)
     const Logits l(x, B, K, len);
     std::tuple args{c, B, K, lo, len, l.p, l.dtype, l.row_stride, l.seq_stride, x.pf(), x.pf(), x.q_rows(B, K, v_q), x.pi(),
                     x.pi(), x.pf(), x.pi(), x.pi(), x.pi(), x.pb(), x.pi(), x.pf(), x.pd()};
-    return call(x, [&](auto... v) { return od_sample_shard_mass(v..., x.stream()); }, args);
+    return call(x, od_sample_shard_mass, args);
 }
 
 PyObject *sample_shard_pick(PyObject *, PyObject *const *a, Py_ssize_t n)
@@ -247,7 +248,7 @@ PyObject *sample_shard_pick(PyObject *, PyObject *const *a, Py_ssize_t n)
     std::tuple args{c, B, K, shards, index, lo, len, mass, l.p, l.dtype, l.row_stride, l.seq_stride, x.pf(), x.pf(), x.pf(),
                     x.pi(), x.pi(), x.pf(), x.pi(), x.pi(), x.pi(), x.pb(), x.pi(), x.pf(), x.pl(), x.u64(), x.pi(), x.pf(),
                     x.pu()};
-    return call(x, [&](auto... v) { return od_sample_shard_pick(v..., x.stream()); }, args);
+    return call(x, od_sample_shard_pick, args);
 }
 
 PyObject *cache_insert(PyObject *, PyObject *const *a, Py_ssize_t n)
@@ -256,14 +257,14 @@ PyObject *cache_insert(PyObject *, PyObject *const *a, Py_ssize_t n)
     od_ctx *c = x.ctx();
     const int32_t N = x.i32();
     std::tuple args{c, N, x.pi(), x.pi(), x.pi()};
-    return call(x, [&](auto... v) { return od_cache_insert(v..., x.stream()); }, args);
+    return call(x, od_cache_insert, args);
 }
 
 PyObject *cache_trim(PyObject *, PyObject *const *a, Py_ssize_t n)
 {
     Args x(a, n, 2);
     std::tuple args{x.ctx()};
-    return call(x, [&](auto... v) { return od_cache_trim(v..., x.stream()); }, args);
+    return call(x, od_cache_trim, args);
 }
 
 // a tensor without memory of its own (one that is being traced or mapped over) throws when asked
@@ -288,4 +289,10 @@ PyModuleDef module = {PyModuleDef_HEAD_INIT, "_marshal", nullptr, -1, methods, n
 
 }  // namespace
 
-PyMODINIT_FUNC PyInit__marshal(void) { return PyModule_Create(&module); }
+PyMODINIT_FUNC PyInit__marshal(void)
+{
+    PyObject *m = PyModule_Create(&module);
+    // it reads tensors by the layout of the torch that it was compiled against: the binding compares
+    if (m && PyModule_AddStringConstant(m, "built_for", OD_BUILT_FOR) != 0) Py_CLEAR(m);
+    return m;
+}
