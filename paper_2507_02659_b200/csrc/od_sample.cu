@@ -116,8 +116,7 @@ struct SeqState {
     const char *row;
     const float *q_row;
     float c, S, scale;      // e(t) = exp2(fma(x_t, scale, -c)); S is the row sum relative to c
-    float above;            // c - fl(M*scale)
-    bool residual, bounded;  // bounded: e(t) <= 2
+    bool residual;
     bool from_row;          // the drafter's probabilities are read at the target ids
     int32_t ngram_token, prefix_token, first_draft;
     float ngram_prob, prefix_val;
@@ -139,16 +138,16 @@ __device__ __forceinline__ float resid_of(const SeqState &q, float x, float qq)
 // an id (its ids are t0 .. t0 + EPT - 1) redoes it: prefix sub-token first, the n-gram
 // token last.
 template <int DTYPE>
-__device__ __forceinline__ void eq2_ids(const SeqState &q, const SampleArgs &a, int t0, float *r, float unit = 1.f)
+__device__ __forceinline__ void eq2_ids(const SeqState &q, const SampleArgs &a, int t0, float *r)
 {
     const int dp = q.prefix_token - t0, dn = q.ngram_token - t0;
     if ((unsigned)dp < (unsigned)EPT && q.prefix_token < a.v_p) {
-        const float v = resid_of(q, od_load_logit<DTYPE>(q.row, q.prefix_token), q.prefix_val) * unit;
+        const float v = resid_of(q, od_load_logit<DTYPE>(q.row, q.prefix_token), q.prefix_val);
 #pragma unroll
         for (int e = 0; e < EPT; ++e) r[e] = e == dp ? v : r[e];
     }
     if ((unsigned)dn < (unsigned)EPT && q.ngram_token < a.v_p) {
-        const float v = resid_of(q, od_load_logit<DTYPE>(q.row, q.ngram_token), q.ngram_prob) * unit;
+        const float v = resid_of(q, od_load_logit<DTYPE>(q.row, q.ngram_token), q.ngram_prob);
 #pragma unroll
         for (int e = 0; e < EPT; ++e) r[e] = e == dn ? v : r[e];
     }
@@ -366,17 +365,11 @@ __device__ __forceinline__ void load_tile(const SeqState &q, int tile, int lane,
 }
 // A lane's eight ids of a whole tile: the sum of their residuals, or of e alone. A tile is 256
 // ids of work for one warp, and its instructions bound a large batch: 276 a tile and 66.8 us for
-// 296 staged rows of 152064 ids with a branch per id, 195 and 51.9 us with a select per id, 156
-// and 45.7 us so: the clamp at zero is part of the multiply-add, an unmapped id's multiply-add
-// is predicated off, and Eq. (2)'s two ids are looked for only in the tiles that hold them.
-// The multiply-add clamps to [0, 1] and e(t) may be up to 2 (SeqState::bounded): the residuals are
-// formed as halves, which is exact.
-__device__ __forceinline__ float fma_sat(float a, float b, float c)
-{
-    float d;
-    asm("fma.rn.sat.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
-    return d;
-}
+// 296 staged rows of 152064 ids with a branch per id, 195 and 51.9 us with a select per id,
+// 154 and 44.8 us so: an unmapped id's multiply-add is predicated off, and Eq. (2)'s two ids are
+// looked for only in the tiles that hold them. (The clamp at zero as the multiply-add's own .sat is 0.8 % of
+// the step faster, but clamps at one too, which e(M) may exceed by c's rounding; with the residuals as
+// halves, to allow for that, it is no faster than the maximum.)
 template <int DTYPE>
 __device__ __forceinline__ void tile_e(const SeqState &q, const uint4 *raw, float *e)
 {
@@ -397,24 +390,18 @@ __device__ __forceinline__ void tile_e(const SeqState &q, const uint4 *raw, floa
         e[k] = od_ex2(e[k]); e[k + 1] = od_ex2(e[k + 1]);
     }
 }
-__device__ __forceinline__ void halve(float *r)
-{
-#pragma unroll
-    for (int k = 0; k < EPT; k += 2) f2_unpack(f2_mul(f2_pack(r[k], r[k + 1]), f2_pack(0.5f, 0.5f)), r[k], r[k + 1]);
-}
 __device__ __forceinline__ float sum_of_eight(const float *r)
 {
     float s0, s1;
     f2_unpack(f2_add(f2_add(f2_pack(r[0], r[1]), f2_pack(r[2], r[3])), f2_add(f2_pack(r[4], r[5]), f2_pack(r[6], r[7]))), s0, s1);
     return s0 + s1;
 }
-// r: halves of the residuals
 template <int DTYPE>
 __device__ __forceinline__ float with_eq2_ids(const SeqState &q, const SampleArgs &a, int tile, int lane, float *r)
 {
     if (tile == q.prefix_token / OD_SAMPLE_TILE || tile == q.ngram_token / OD_SAMPLE_TILE)
-        eq2_ids<DTYPE>(q, a, tile * OD_SAMPLE_TILE + lane * EPT, r, 0.5f);
-    return 2.f * sum_of_eight(r);
+        eq2_ids<DTYPE>(q, a, tile * OD_SAMPLE_TILE + lane * EPT, r);
+    return sum_of_eight(r);
 }
 template <int DTYPE>
 __device__ __forceinline__ float tile_lane_sum(const SeqState &q, const SampleArgs &a, int tile, int lane, const uint4 *raw,
@@ -422,10 +409,8 @@ __device__ __forceinline__ float tile_lane_sum(const SeqState &q, const SampleAr
 {
     float r[EPT];
     tile_e<DTYPE>(q, raw, r);
-    halve(r);
-    const float nS = -0.5f * q.S;
 #pragma unroll
-    for (int k = 0; k < EPT; ++k) r[k] = fma_sat(qq[k], nS, r[k]);
+    for (int k = 0; k < EPT; ++k) r[k] = fmaxf(0.f, fmaf(-qq[k], q.S, r[k]));
     return with_eq2_ids<DTYPE>(q, a, tile, lane, r);
 }
 // the same with the probabilities in shared memory at `rank_at` (the address of the lane's first
@@ -436,16 +421,15 @@ __device__ __forceinline__ float tile_lane_sum_staged(const SeqState &q, const S
 {
     float r[EPT];
     tile_e<DTYPE>(q, raw, r);
-    halve(r);
-    const float nS = -0.5f * q.S;
+    const float nS = -q.S;
 #pragma unroll
     for (int k = 0; k < EPT; ++k)
         // (read for every id, mapped or not: the last rank has a word behind it)
         asm("{.reg .pred p; .reg .b32 t; .reg .f32 v;\n\t"
             "and.b32 t, %3, %4; setp.ne.u32 p, t, 0;\n\t"
             "ld.shared.f32 v, [%1];\n\t"
-            "@p fma.rn.sat.f32 %0, v, %2, %0;\n\t"
-            "@p add.u32 %1, %1, 4;}"
+            "@p fma.rn.f32 %0, v, %2, %0;\n\t"
+            "@p add.u32 %1, %1, 4; max.f32 %0, %0, 0f00000000;}"
             : "+f"(r[k]), "+r"(rank_at) : "f"(nS), "r"(oct), "r"(1u << k) : "memory");
     return with_eq2_ids<DTYPE>(q, a, tile, lane, r);
 }
@@ -664,15 +648,11 @@ __device__ __forceinline__ SeqState seq_state(const SampleArgs &a, const Ahead &
     q.scale = 1.4426950408889634f / h.T;
     {
         // reference exponent c = fl(M*scale), od_verify's own, so that the errors of e(t) are those of the
-        // row sum; its rounding goes into S exactly:
+        // row sum (a margin on it, to keep e(t) below one, made the residual mass's mean error 5 to 10 %
+        // larger, and at |M|/T > 8.8e7 zero of everything); its rounding goes into S exactly:
         // sum_t exp2(x_t*scale - c) = (sum_t exp2((x_t - M)*scale)) * exp2(M*scale - c)
-        const float M = __shfl_sync(0xFFFFFFFFu, rm, j), c = fmaxf(M * q.scale, -FLT_MAX);
-        // e(M) is exp2 of c's rounding: up to 2 while |c| < 2^24. Above (M = 20, T = 1e-6: near-greedy
-        // draws) c is rounded up, so that e(M) lies between exp2(-32) and 1 up to |c| = 2^29; beyond that the
-        // tiles are worked on without an upper clamp.
-        q.c = fabsf(c) < 0x1p23f ? c : fabsf(c) < 0x1p29f ? __fmul_ru(M, q.scale) : c;
-        q.above = q.c - c;
-        q.bounded = fabsf(c) < 0x1p29f;
+        const float M = __shfl_sync(0xFFFFFFFFu, rm, j);
+        q.c = fmaxf(M * q.scale, -FLT_MAX);
         q.S = __shfl_sync(0xFFFFFFFFu, rs, j) * od_ex2(fmaf(M, q.scale, -q.c));
     }
     q.residual = (j < h.mb) || h.stop;
@@ -1017,10 +997,9 @@ od_sample_kernel(const SampleArgs a)
     const SeqState q = seq_state<DTYPE>(a, h, b, j, rm, rs, 0, planned);
     if (SOURCE == FROM_MAP && q.residual && threadIdx.x == 0) prefetch_q_row(a, q, part, nparts);
 
-    // ---- pass 1: the value of every tile; the ragged last one (all of them, if e is not bounded or
-    // the map is another) one by one ----
+    // ---- pass 1: the value of every tile; the ragged last one (all of them, if the map is another) one by one ----
     WarpTiles out = {s_val, lane, p_lo, 0.0};
-    const int hi_w = q.bounded && planned ? p_hi_w : p_lo;
+    const int hi_w = planned ? p_hi_w : p_lo;
     const uint64_t seed_b = a.seed[b];
     const StagedRow sr = {s_q, a.octet, (uint32_t)my_part.z};
     if (SOURCE == STAGED && q.residual) {
@@ -1198,7 +1177,7 @@ od_sample_shard_kernel(const SampleArgs a)
 
     if (MODE != 2) {
         // ---- pass 1: the value of every tile ----
-        const int hi_w = q.bounded && (planned || !a.same_ids) ? p_hi_w : p_lo;
+        const int hi_w = planned || !a.same_ids ? p_hi_w : p_lo;
         if (a.same_ids) warp_run<DTYPE, FROM_ROW>(q, a, p_lo, p_hi, hi_w, lane, out, ni);
         else warp_run<DTYPE, FROM_MAP>(q, a, p_lo, p_hi, hi_w, lane, out, ni);
         // The tile values are read by another block: the barrier orders this block's stores
@@ -1241,8 +1220,6 @@ od_sample_shard_kernel(const SampleArgs a)
     if (MODE != 2 && threadIdx.x == 0) a.ticket[b] = 0;
     __syncthreads();
 
-    // the shards exchange their shares relative to fl(M*scale)
-    const double unit = exp2((double)q.above);
     if (MODE == 1) {
         // ---- this shard's shares ----
         const double mass_r = block_total(s_val, my_lo, my_hi, s_warp);
@@ -1256,7 +1233,7 @@ od_sample_shard_kernel(const SampleArgs a)
             __syncthreads();
             mass_e = block_total(s_val, my_lo, my_hi, s_warp);
         }
-        if (threadIdx.x == 0) { a.mass_out[2 * b] = mass_r * unit; a.mass_out[2 * b + 1] = mass_e * unit; }
+        if (threadIdx.x == 0) { a.mass_out[2 * b] = mass_r; a.mass_out[2 * b + 1] = mass_e; }
         return;
     }
 
@@ -1264,8 +1241,8 @@ od_sample_shard_kernel(const SampleArgs a)
     if (MODE == 2) {
         double tot_r = 0.0, tot_e = 0.0;
         for (int s = 0; s < a.n_shards; ++s) {
-            tot_r += a.mass_all[((size_t)s * a.B + b) * 2] / unit;
-            tot_e += a.mass_all[((size_t)s * a.B + b) * 2 + 1] / unit;
+            tot_r += a.mass_all[((size_t)s * a.B + b) * 2];
+            tot_e += a.mass_all[((size_t)s * a.B + b) * 2 + 1];
         }
         const bool use_e = residual && !(tot_r > 0.0);
         if (use_e) { residual = false; flags |= OD_SF_ZERO_MASS; }   // the tile values then hold p_j's
@@ -1277,7 +1254,7 @@ od_sample_shard_kernel(const SampleArgs a)
             double c = 0.0;
             int last = -1;
             for (int s = 0; s < a.n_shards; ++s) {
-                const double v = a.mass_all[((size_t)s * a.B + b) * 2 + (use_e ? 1 : 0)] / unit;
+                const double v = a.mass_all[((size_t)s * a.B + b) * 2 + (use_e ? 1 : 0)];
                 if (s == a.shard_index) shard_before = c;
                 if (v > 0.0) last = s;
                 if (c + v > target) { owner = s; break; }
