@@ -190,10 +190,11 @@ int32_t od_set_vocab_map(od_ctx *c, const int32_t *host_map)
             inv[t] = d;
             ++n_mapped;
         }
-        // where every target id is the draft id, nothing is gathered: no lists
+        // Where every target id is the draft id, nothing is gathered: no lists. (But a graph captured under
+        // an earlier map with lists reads the distillation kernel's from the place where it found them.)
         std::vector<char> distill, sample;
         int32_t slots[OD_SAMPLE_LEVELS] = {};
-        if (!same_ids) {
+        if (!same_ids || c->distill_lists) {
             OdMappedIds mapped;
             mapped.target.resize((size_t)c->v_p + 1);
             for (int32_t t = 0, n = 0; t < c->v_p; ++t) {
@@ -205,8 +206,10 @@ int32_t od_set_vocab_map(od_ctx *c, const int32_t *host_map)
             for (int64_t i = 0; i < n_mapped; ++i) mapped.draft[i] = inv[mapped.target[i]];
             distill.resize(od_distill_lists_bytes(c->v_q, c->v_p));
             od_distill_plan(c->v_q, c->v_p, mapped, distill.data());
-            sample.resize(od_sample_lists_bytes(c->v_q, c->v_p));
-            od_sample_plan(c->v_q, c->v_p, mapped, c->map_serial + 1, sample.data(), slots);
+            if (!same_ids) {
+                sample.resize(od_sample_lists_bytes(c->v_q, c->v_p));
+                od_sample_plan(c->v_q, c->v_p, mapped, c->map_serial + 1, sample.data(), slots);
+            }
         }
         DeviceGuard g(c->device);
         if (!g.ok) return OD_ERR_CUDA;
@@ -214,8 +217,11 @@ int32_t od_set_vocab_map(od_ctx *c, const int32_t *host_map)
         c->have_map = false;                    // until all of it is there
         OD_CUDA(cudaMemcpy(c->d_vocab_map, fwd.data(), fwd.size() * sizeof(int32_t), cudaMemcpyHostToDevice));
         OD_CUDA(cudaMemcpy(c->d_inv_map, inv.data(), inv.size() * sizeof(int32_t), cudaMemcpyHostToDevice));
-        if (!same_ids) {
+        if (!distill.empty()) {
             OD_CUDA(cudaMemcpy(c->d_distill_lists, distill.data(), distill.size(), cudaMemcpyHostToDevice));
+            c->distill_lists = true;
+        }
+        if (!same_ids) {
             OD_CUDA(cudaMemcpy(c->d_sample_lists, sample.data(), sample.size(), cudaMemcpyHostToDevice));
         } else {                                // lists of an earlier map: of no serial number any more
             const OdSampleLists l = od_sample_lists(c->d_sample_lists, c->v_q, c->v_p);

@@ -38,6 +38,7 @@ struct od_ctx {
     int32_t sample_slots[OD_SAMPLE_LEVELS];   // most mapped ids of a part
     int32_t sample_clusters[OD_SAMPLE_LEVELS];   // clusters of the sampler that are resident at a time
     bool have_map;
+    bool distill_lists;             // some map had gather lists: every later one has the distillation kernel's
     // The map's serial number. A launch is laid out for the map of its time (where ids are shared, how many
     // are staged); a kernel that finds another number on the device was replayed from a CUDA graph
     // captured before od_set_vocab_map, and looks every id up in the maps instead.

@@ -191,13 +191,51 @@ struct Logit<OD_BF16> {
     }
 };
 
+// One position by one block, every id looked up in the map: a launch for shared ids under another map (the
+// other kernels read lists that are the present map's whenever they were laid out). Out of line: loops in the
+// kernel below, in all its forms, cost 0.15 us of 5 to 13 although they are not run.
+template <int DTYPE>
+__device__ __noinline__ void looked_up_position(const DistillArgs &a, int b, int j, int *s_piece, double *s_red)
+{
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    int piece, plen;
+    find_piece(a, b, j, s_piece, piece, plen);
+    const float T = a.temperature[b];
+    const bool translated = piece >= 0 && T > 0.f;
+    const size_t o = (size_t)b * a.K_max + j, row_of = (size_t)b * (a.K_max + 1) + piece;
+    const char *row = (const char *)a.logits + ((size_t)b * a.seq_stride + (size_t)piece * a.row_stride) * (DTYPE == OD_BF16 ? 2 : 4);
+    const float *q = a.q_rows + o * a.v_q;
+    float *grad = a.grad ? a.grad + o * a.v_q : nullptr;
+    if (!translated || plen >= 2) {
+        plain_position<false>(a, b, j, piece, translated, q, grad, 0, a.v_q, true);
+        return;
+    }
+    KlRow kl;
+    kl.M = a.row_max[row_of];
+    kl.scale = 1.4426950408889634f / T;
+    kl.lg2_S = lg2_approx(a.row_sum[row_of]);
+    float loss_t = 0.f, qg_t = 0.f;
+    const auto g_of = [&](int d, float v) {
+        const int32_t t = __ldg(a.vocab_map + d);
+        return kl_term(kl, t >= 0 ? v : 0.f, od_load_logit<DTYPE>(row, t >= 0 ? t : 0), loss_t, qg_t);
+    };
+    for (int d = threadIdx.x; d < a.v_q; d += THREADS) g_of(d, __ldg(q + d));
+    const double l = block_sum((double)loss_t, s_red), qg = block_sum((double)qg_t, s_red);
+    if (threadIdx.x == 0) a.loss[o] = (float)l;
+    if (!grad) return;
+    for (int d = threadIdx.x; d < a.v_q; d += THREADS) {
+        const float v = __ldg(q + d);
+        grad[d] = fmaf(-v, (float)qg, v * g_of(d, v));
+    }
+}
+
 // Grid (C, K, B), clusters of C blocks. VEC4: the draft vocabulary is a multiple of 4 and the
 // rows are 16-byte aligned, so the coalesced accesses (q, gradient) move four ids per
 // instruction; chunks are multiples of 32 ids. SAME: target ids are draft ids, nothing is
 // gathered; the logits wait in shared memory for the gradient.
 template <int DTYPE, bool VEC4, bool SAME>
 __global__ void __launch_bounds__(THREADS, 3)
-od_distill_kernel(const DistillArgs a)
+od_distill_kernel(const __grid_constant__ DistillArgs a)
 {
     extern __shared__ __align__(16) unsigned char s_dyn[];   // [chunk] the logit of each mapped id, at its draft id
     typedef typename Logit<DTYPE>::raw raw_t;
@@ -228,13 +266,16 @@ od_distill_kernel(const DistillArgs a)
         g_at += EB * WARPS;
     };
     if (!SAME) load_words();
-    // the map is the one this launch was laid out for (else every id is looked up in it)
-    const bool planned = __ldg(a.map_serial_now) == a.map_serial;
+    const int32_t map_serial = SAME ? __ldg(a.map_serial_now) : a.map_serial;
     asm volatile("griddepcontrol.wait;" ::: "memory");
     const float T = a.temperature[b];
     int piece, plen;
     find_piece(a, b, j, s_piece, piece, plen);
     const bool translated = piece >= 0 && T > 0.f;
+    if (SAME && map_serial != a.map_serial) {                // ids are not shared any more (asked here, where the answer has arrived)
+        if (rank == 0) looked_up_position<DTYPE>(a, b, j, s_piece, s_red[0]);
+        return;
+    }
     if (!translated || plen >= 2) {                          // the same for every block of the cluster
         plain_position<VEC4>(a, b, j, piece, translated, q, grad, lo, hi, rank == 0);
         return;
@@ -264,16 +305,7 @@ od_distill_kernel(const DistillArgs a)
         loss_t += l; qg_t += g;
     };
     const raw_t *xrow = (const raw_t *)row;
-    const auto looked_up = [&](int d, float v, float &l, float &g) {
-        const int32_t t = __ldg(a.vocab_map + d);
-        const raw_t x = t >= 0 ? __ldg(xrow + t) : raw_t();
-        return kl_term(kl, t >= 0 ? v : 0.f, Logit<DTYPE>::load(&x), l, g);
-    };
-    if (!planned) {
-        kl.lg2_S = lg2_approx(S);
-#pragma unroll 1
-        for (int d = lo + (int)threadIdx.x; d < hi; d += THREADS) looked_up(d, __ldg(q + d), loss_t, qg_t);
-    } else if (!SAME) {
+    if (!SAME) {
         // (the first probabilities travel meanwhile)
         constexpr int PQ = 2;                                // vectors of four probabilities in flight per thread
         float4 qv[PQ];
@@ -382,13 +414,7 @@ od_distill_kernel(const DistillArgs a)
     if (!grad) return;
     // ---- the gradient: q(d) (g(d) - sum_e q(e) g(e))
     const float gbar = (float)qg;
-    if (!planned) {
-#pragma unroll 1
-        for (int d = lo + (int)threadIdx.x; d < hi; d += THREADS) {
-            const float v = __ldg(q + d);
-            grad[d] = fmaf(-v, gbar, v * looked_up(d, v, loss_t, qg_t));
-        }
-    } else if (VEC4) {
+    if (VEC4) {
 #pragma unroll 4
         for (int d = lo + (int)threadIdx.x * 4; d < hi; d += THREADS * 4) {
             const float4 v = __ldg((const float4 *)(q + d)), u = mapped4(d, v);
