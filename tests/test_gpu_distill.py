@@ -129,3 +129,30 @@ def test_chunks_of_draft_ids(cuda_device, v_q, v_p, B, k_max):
     for dtype in ("bf16", "f32"):
         w = _small(B=B, k_max=k_max, v_q=v_q, v_p=v_p, cache_entries=0, logit_dtype=dtype, gen_seed=0xBEEFF0)
         _check(w, cuda_device, [0], 0.2, ds.LAMBDA_CONSTANT, positions=sorted({0, B // 3, B - 1}))
+
+
+# the kernels behind the dispatch: ids shared with the target (chunks read along the rows; from two positions
+# per multiprocessor on, one block per position where rows are whole vectors), and a target row that is short for
+# the mapped ids with many positions (one block per position, gathered in draft order); on and off the vector width
+@pytest.mark.parametrize("dtype", ["bf16", "f32"])
+@pytest.mark.parametrize("kind, v_q, v_p, B, k_max", [("identity", 600, 1003, 6, 5), ("identity", 333, 1003, 6, 5),
+                                                      ("identity", 600, 600, 64, 8), ("identity", 333, 1003, 64, 8),
+                                                      ("random", 600, 700, 64, 8), ("random", 601, 700, 64, 8)])
+def test_shared_ids_and_short_target_rows(cuda_device, kind, v_q, v_p, B, k_max, dtype):
+    """Tolerances as above."""
+    w = _small(B=B, k_max=k_max, v_q=v_q, v_p=v_p, map_kind=kind, cache_entries=0, logit_dtype=dtype, gen_seed=0xBEEFF8)
+    some = sorted({0, 1, B // 2, B - 1})
+    assert _check(w, cuda_device, [0], 0.2, ds.LAMBDA_CONSTANT, positions=some)["kl"] > 0
+    st = synth.make_static(w)
+    ctx = parity.make_context(w, st, cuda_device)
+    s = synth.make_step(w, st, 0, device=cuda_device)
+    logits = parity.pad_rows(s.logits)
+    mp = od.od_map_proposals(ctx, s.draft_ids, s.draft_len, s.q_sel)
+    vo = od.od_verify(ctx, logits, mp, s.temperature, s.seed, 0)
+    a = (ctx, s.q_rows, s.draft_ids, mp, logits, vo, s.temperature, 0.2, ds.LAMBDA_CONSTANT)
+    lone, none = od.od_distill_loss(*a, want_grad=False)
+    loss, _ = od.od_distill_loss(*a)
+    assert none is None and (loss != 0).any()
+    # the same terms, in another order where the two take different kernels
+    torch.testing.assert_close(lone, loss, rtol=2e-5, atol=2e-6)
+    ctx.close()

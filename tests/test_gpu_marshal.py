@@ -90,3 +90,35 @@ def test_the_same_errors(cuda_device):
         call(logits=torch.empty(w.B, w.k_max + 1, w.v_p + 1, dtype=torch.bfloat16, device=cuda_device)[:, :, :w.v_p])
     call(step=2 ** 64 + 3)
     ctx.close()
+
+
+class _Recorder:
+    """Passes calls on to _marshal and keeps what each returned."""
+
+    def __init__(self, native):
+        self.native, self.calls = native, []
+
+    def __getattr__(self, name):
+        def call(*a):
+            status = getattr(self.native, name)(*a)
+            self.calls.append((name, status))
+            return status
+        return call
+
+
+def test_every_well_formed_call_is_made_natively(cuda_device, monkeypatch):
+    w, ctx, s, logits = _inputs(cuda_device, "bf16")
+    assert not isinstance(od._native, od._InPython)
+    rec = _Recorder(od._native)
+    monkeypatch.setattr(od, "_native", rec)
+    _run(w, ctx, s, logits)
+    assert {n for n, _ in rec.calls} == {"map_proposals", "verify", "sample_residual", "step", "exit_rule", "distill_loss",
+                                         "verify_shard_stats", "verify_shard_finish", "sample_shard_mass", "sample_shard_pick",
+                                         "cache_insert", "cache_trim"}
+    assert all(status == 0 for _, status in rec.calls), rec.calls
+    # and one that does not take its arguments as they stand is not
+    del rec.calls[:]
+    with pytest.raises(TypeError):
+        od.od_map_proposals(ctx, s.draft_ids.long(), s.draft_len, s.q_sel)
+    assert rec.calls == [("map_proposals", None)]
+    ctx.close()
