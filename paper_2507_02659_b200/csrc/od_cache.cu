@@ -258,61 +258,47 @@ __global__ void trim_compact_kernel(int policy, unsigned int clock, const unsign
     const TrimLists L = trim_lists(lists, cap);
     if (threadIdx.x == 0) { s_and = ~0ull; s_or = 0ull; }
     unsigned long long t_and = ~0ull, t_or = 0ull;
-    // two vectors of four slots per thread and iteration, one append for both
-    constexpr int NV = 1;
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x * 4 * NV;
-    for (int64_t slot0 = (int64_t)blockIdx.x * blockDim.x * 4 * NV; slot0 < cap; slot0 += stride) {
-        unsigned long long kk[NV][4];
-        int vv[NV][4];
-        uint4 ss[NV], ff[NV], bb[NV];
-#pragma unroll
-        for (int v = 0; v < NV; ++v) {
-            const int64_t slot = slot0 + ((int64_t)v * blockDim.x + threadIdx.x) * 4;
-            kk[v][0] = kk[v][1] = kk[v][2] = kk[v][3] = 0ull;
-            if (slot < cap) {                               // cap is a multiple of 64
-                const ulonglong2 k01 = __ldg((const ulonglong2 *)(keys + slot));
-                const ulonglong2 k23 = __ldg((const ulonglong2 *)(keys + slot) + 1);
-                kk[v][0] = k01.x; kk[v][1] = k01.y; kk[v][2] = k23.x; kk[v][3] = k23.y;
-                *(ulonglong2 *)(nkeys + slot) = make_ulonglong2(0ull, 0ull);
-                *((ulonglong2 *)(nkeys + slot) + 1) = make_ulonglong2(0ull, 0ull);
-                *(int4 *)(nvals + slot) = make_int4(-1, -1, -1, -1);
-                if ((slot & (OD_GROUP - 1)) == 0) L.grp_fill[slot / OD_GROUP] = 0u;
-            }
+    // four slots per thread and iteration
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x * 4;
+    for (int64_t slot0 = (int64_t)blockIdx.x * blockDim.x * 4; slot0 < cap; slot0 += stride) {
+        const int64_t slot = slot0 + (int64_t)threadIdx.x * 4;
+        unsigned long long kk[4] = {0ull, 0ull, 0ull, 0ull};
+        int vv[4] = {-1, -1, -1, -1};
+        uint4 ss, ff, bb;
+        if (slot < cap) {                                   // cap is a multiple of 64
+            const ulonglong2 k01 = __ldg((const ulonglong2 *)(keys + slot));
+            const ulonglong2 k23 = __ldg((const ulonglong2 *)(keys + slot) + 1);
+            kk[0] = k01.x; kk[1] = k01.y; kk[2] = k23.x; kk[3] = k23.y;
+            *(ulonglong2 *)(nkeys + slot) = make_ulonglong2(0ull, 0ull);
+            *((ulonglong2 *)(nkeys + slot) + 1) = make_ulonglong2(0ull, 0ull);
+            *(int4 *)(nvals + slot) = make_int4(-1, -1, -1, -1);
+            if ((slot & (OD_GROUP - 1)) == 0) L.grp_fill[slot / OD_GROUP] = 0u;
+        }
+        if ((kk[0] | kk[1] | kk[2] | kk[3]) != 0ull) {
+            const int4 v4 = __ldg((const int4 *)(vals + slot));
+            ss = __ldg((const uint4 *)(stamp + slot));
+            ff = __ldg((const uint4 *)(freq + slot));
+            bb = __ldg((const uint4 *)(born + slot));
+            vv[0] = v4.x; vv[1] = v4.y; vv[2] = v4.z; vv[3] = v4.w;
         }
         unsigned int n = 0;
 #pragma unroll
-        for (int v = 0; v < NV; ++v) {
-            const int64_t slot = slot0 + ((int64_t)v * blockDim.x + threadIdx.x) * 4;
-            vv[v][0] = vv[v][1] = vv[v][2] = vv[v][3] = -1;
-            if ((kk[v][0] | kk[v][1] | kk[v][2] | kk[v][3]) != 0ull) {
-                const int4 v4 = __ldg((const int4 *)(vals + slot));
-                ss[v] = __ldg((const uint4 *)(stamp + slot));
-                ff[v] = __ldg((const uint4 *)(freq + slot));
-                bb[v] = __ldg((const uint4 *)(born + slot));
-                vv[v][0] = v4.x; vv[v][1] = v4.y; vv[v][2] = v4.z; vv[v][3] = v4.w;
-            }
-#pragma unroll
-            for (int e = 0; e < 4; ++e) n += (kk[v][e] != 0ull && vv[v][e] >= 0) ? 1u : 0u;
-        }
+        for (int e = 0; e < 4; ++e) n += (kk[e] != 0ull && vv[e] >= 0) ? 1u : 0u;
         unsigned int total;
         unsigned int at = block_offsets(n, s_warp, total);
         if (threadIdx.x == 0) s_base = total ? atomicAdd(&st->live.n, total) : 0u;
         __syncthreads();
         at += s_base;
+        const unsigned int s4[4] = {ss.x, ss.y, ss.z, ss.w}, f4[4] = {ff.x, ff.y, ff.z, ff.w}, b4[4] = {bb.x, bb.y, bb.z, bb.w};
 #pragma unroll
-        for (int v = 0; v < NV; ++v) {
-            const unsigned int s4[4] = {ss[v].x, ss[v].y, ss[v].z, ss[v].w}, f4[4] = {ff[v].x, ff[v].y, ff[v].z, ff[v].w};
-            const unsigned int b4[4] = {bb[v].x, bb[v].y, bb[v].z, bb[v].w};
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                if (kk[v][e] == 0ull || vv[v][e] < 0 || at >= cap) continue;   // (never beyond the list)
-                unsigned long long hi, lo;
-                order_key(policy, clock, kk[v][e], s4[e], f4[e], b4[e], hi, lo);
-                t_and &= hi; t_or |= hi;
-                L.r_hi[at] = hi; L.r_key[at] = lo;
-                L.r_val[at] = vv[v][e]; L.r_stamp[at] = s4[e]; L.r_freq[at] = f4[e]; L.r_born[at] = b4[e];
-                ++at;
-            }
+        for (int e = 0; e < 4; ++e) {
+            if (kk[e] == 0ull || vv[e] < 0 || at >= cap) continue;   // (never beyond the list)
+            unsigned long long hi, lo;
+            order_key(policy, clock, kk[e], s4[e], f4[e], b4[e], hi, lo);
+            t_and &= hi; t_or |= hi;
+            L.r_hi[at] = hi; L.r_key[at] = lo;
+            L.r_val[at] = vv[e]; L.r_stamp[at] = s4[e]; L.r_freq[at] = f4[e]; L.r_born[at] = b4[e];
+            ++at;
         }
     }
     // which bits of (new?, score) vary at all: AND and OR over the live entries
@@ -337,17 +323,6 @@ __global__ void trim_compact_kernel(int policy, unsigned int clock, const unsign
 // of 13 launches of the whole grid, two dependent round trips and a launch each, the passes were
 // 52 of the 107 us of an insertion, a trim and a translation (262144 entries, 16384 new ones).
 constexpr int SELECT_THREADS = 1024, SELECT_MAX_BLOCKS = 16;
-
-__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
-__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
-__device__ __forceinline__ unsigned int cluster_load(const unsigned int *p, uint32_t rank)
-{
-    uint32_t at;
-    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(at) : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(rank));
-    unsigned int v;
-    asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(at) : "memory");
-    return v;
-}
 
 // Count digit `d` of the lanes with `ok` into hist: digits are heavily tied (scores, the upper
 // bytes of short runs), so lanes that agree count as one add.
@@ -381,11 +356,11 @@ trim_select_kernel(unsigned int max_entries, unsigned int room, int64_t cap, voi
     unsigned int k_rem = k, n_match = n, buf = 0;
     // the first digit at which the running count over all blocks reaches k_rem
     auto settle = [&]() -> unsigned int {
-        cluster_arrive(); cluster_wait();                   // every block's histogram is complete
+        od_cluster_arrive(); od_cluster_wait();             // every block's histogram is complete
         if (threadIdx.x < 256) {
             unsigned int h[SELECT_MAX_BLOCKS], t = 0;       // all loads before the first use: one trip, not P
 #pragma unroll
-            for (unsigned int r = 0; r < SELECT_MAX_BLOCKS; ++r) h[r] = r < P ? cluster_load(&s_hist[buf][threadIdx.x], r) : 0u;
+            for (unsigned int r = 0; r < SELECT_MAX_BLOCKS; ++r) h[r] = r < P ? od_cluster_load(&s_hist[buf][threadIdx.x], r) : 0u;
 #pragma unroll
             for (unsigned int r = 0; r < SELECT_MAX_BLOCKS; ++r) t += h[r];
             s_sum[threadIdx.x] = t;
@@ -489,7 +464,7 @@ trim_select_kernel(unsigned int max_entries, unsigned int room, int64_t cap, voi
         }
     }
     thr_lo |= ~decided;                                     // every candidate left is among the k
-    cluster_arrive(); cluster_wait();                       // nobody leaves while its histogram may still be read
+    od_cluster_arrive(); od_cluster_wait();                 // nobody leaves while its histogram may still be read
     if (rank == 0 && threadIdx.x == 0) {
         st->k = k; st->size = size - k;
         st->thr_hi = thr_hi; st->thr_lo = thr_lo;

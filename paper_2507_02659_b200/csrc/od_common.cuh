@@ -332,6 +332,28 @@ __device__ __forceinline__ float od_ex2(float x)
     return y;
 }
 
+// Thread-block clusters: the barrier in its two halves, and a word of block `rank`'s shared memory, at the
+// address of `p` in this block.
+__device__ __forceinline__ void od_cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void od_cluster_arrive_relaxed() { asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory"); }
+__device__ __forceinline__ void od_cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+__device__ __forceinline__ uint32_t od_cluster_address(const void *p, uint32_t rank)
+{
+    uint32_t at;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(at) : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(rank));
+    return at;
+}
+__device__ __forceinline__ void od_cluster_store(double *p, uint32_t rank, double v)
+{
+    asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(od_cluster_address(p, rank)), "d"(v) : "memory");
+}
+__device__ __forceinline__ unsigned int od_cluster_load(const unsigned int *p, uint32_t rank)
+{
+    unsigned int v;
+    asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(od_cluster_address(p, rank)) : "memory");
+    return v;
+}
+
 // Packed fp32 pairs (one instruction for two lanes of arithmetic on sm_100).
 __device__ __forceinline__ uint64_t f2_pack(float lo, float hi)
 {

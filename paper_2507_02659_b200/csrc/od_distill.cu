@@ -152,15 +152,6 @@ __device__ __forceinline__ double block_sum(double v, double *s_red)
     return t;
 }
 
-__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
-__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
-// v to the shared-memory address of `p` in block `rank` of the cluster
-__device__ __forceinline__ void cluster_store(double *p, uint32_t rank, double v)
-{
-    uint32_t at;
-    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(at) : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(rank));
-    asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(at), "d"(v) : "memory");
-}
 // A logit as it is stored
 template <int DTYPE>
 struct Logit {
@@ -280,7 +271,7 @@ od_distill_kernel(const __grid_constant__ DistillArgs a)
         plain_position<VEC4>(a, b, j, piece, translated, q, grad, lo, hi, rank == 0);
         return;
     }
-    cluster_arrive();                                        // this block runs: the others may store to it (waited for below)
+    od_cluster_arrive();                                     // this block runs: the others may store to it (waited for below)
     // ---- a directly mapped token: KL(q' || p_i) over the mapped ids
     const char *row = (const char *)a.logits + ((size_t)b * a.seq_stride + (size_t)piece * a.row_stride) * sizeof(raw_t);
     const float M = a.row_max[b * (a.K_max + 1) + piece], S = a.row_sum[b * (a.K_max + 1) + piece];
@@ -394,7 +385,7 @@ od_distill_kernel(const __grid_constant__ DistillArgs a)
             g += __shfl_xor_sync(0xFFFFFFFFu, g, off);
         }
         if (lane == 0) { s_red[0][warp] = l; s_red[1][warp] = g; }
-        cluster_wait();
+        od_cluster_wait();
         __syncthreads();
         if (warp == 0) {
             const int which = lane >> 4, w = lane & 15;
@@ -403,10 +394,10 @@ od_distill_kernel(const __grid_constant__ DistillArgs a)
 #pragma unroll
             for (int off = 8; off > 0; off >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, off);
             // lanes 0.. store the loss, lanes 16.. the other sum, one block of the cluster each
-            if (w < C) cluster_store(&s_all[rank][which], (uint32_t)w, v);
+            if (w < C) od_cluster_store(&s_all[rank][which], (uint32_t)w, v);
         }
-        cluster_arrive();
-        cluster_wait();
+        od_cluster_arrive();
+        od_cluster_wait();
     }
     double loss = 0.0, qg = 0.0;
     for (int r = 0; r < C; ++r) { loss += s_all[r][0]; qg += s_all[r][1]; }   // the same order in every block
@@ -435,7 +426,6 @@ od_distill_kernel(const __grid_constant__ DistillArgs a)
     }
 }
 
-//XX
 // One block per position, the ids in draft order, each gathering its logit; q(d) g(d) waits in
 // the gradient row for the second sweep.
 template <int DTYPE, bool VEC4>

@@ -118,7 +118,7 @@ struct SeqState {
     float c, S, scale;      // e(t) = exp2(fma(x_t, scale, -c)); S is the row sum relative to c
     bool residual;
     bool from_row;          // the drafter's probabilities are read at the target ids
-    int32_t ngram_token, prefix_token, first_draft;
+    int32_t ngram_token, prefix_token;
     float ngram_prob, prefix_val;
 };
 
@@ -247,8 +247,8 @@ __device__ __forceinline__ void tile_values(const SeqState &q, const SampleArgs 
     if (residual) eq2_ids<DTYPE>(q, a, t0, r);
 }
 
-// a lane's eight values are added in fp32 in index order (both passes do exactly
-// this); everything across lanes and tiles is fp64
+// inside the picked tile a lane's eight values are added in fp32 in index order (pass 1 adds a tile in
+// pairs); everything across lanes and tiles is fp64
 __device__ __forceinline__ double lane_sum(const float *r)
 {
     float s = r[0];
@@ -657,7 +657,7 @@ __device__ __forceinline__ SeqState seq_state(const SampleArgs &a, const Ahead &
     }
     q.residual = (j < h.mb) || h.stop;
     q.from_row = a.same_ids && planned;
-    q.ngram_token = -1; q.prefix_token = -1; q.first_draft = -1; q.ngram_prob = 0.f; q.prefix_val = 0.f;
+    q.ngram_token = -1; q.prefix_token = -1; q.ngram_prob = 0.f; q.prefix_val = 0.f;
     q.q_row = a.q_rows;
     // position j's preparation (j < K whenever the draw is a residual one)
     const int src = j < a.K_max ? j : 0;
@@ -671,7 +671,6 @@ __device__ __forceinline__ SeqState seq_state(const SampleArgs &a, const Ahead &
             q.ngram_token = tgt;
             q.ngram_prob = qp;
             if (d1 >= 0) {
-                q.first_draft = d1;
                 q.prefix_token = pm;
                 q.prefix_val = qd1 - q.ngram_prob;
             }
@@ -783,17 +782,6 @@ __device__ __forceinline__ bool pick_in_tile(const SeqState &q, const SampleArgs
 // FUSED: the launch in front is the streaming pass of od_verify itself; its decide kernel is
 // folded into this kernel's prologue (see SampleArgs).
 constexpr int CWARPS = 16, CTHREADS = CWARPS * 32;
-
-__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
-__device__ __forceinline__ void cluster_arrive_relaxed() { asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory"); }
-__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
-// v to the shared-memory address of `p` in block `rank` of the cluster
-__device__ __forceinline__ void cluster_store(double *p, uint32_t rank, double v)
-{
-    uint32_t at;
-    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(at) : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(rank));
-    asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(at), "d"(v) : "memory");
-}
 
 // No usable residual mass (rare): one block draws from p_j. Redoes the row's tile values with e
 // alone, in global memory, and walks them.
@@ -993,7 +981,7 @@ od_sample_kernel(const SampleArgs a)
     }
     // FROM_ROW: the map is still the one this launch was laid out for
     const bool planned = map_serial == a.map_serial;
-    cluster_arrive_relaxed();                      // this block runs: the others may store to it (waited for below)
+    od_cluster_arrive_relaxed();                   // this block runs: the others may store to it (waited for below)
     const SeqState q = seq_state<DTYPE>(a, h, b, j, rm, rs, 0, planned);
     if (SOURCE == FROM_MAP && q.residual && threadIdx.x == 0) prefetch_q_row(a, q, part, nparts);
 
@@ -1042,10 +1030,10 @@ od_sample_kernel(const SampleArgs a)
         if ((lane & 15) >= off) incl += v;
     }
     const double block_sum = __shfl_sync(0xFFFFFFFFu, incl, 15);
-    cluster_wait();
-    if (warp == 0 && lane < (int)nparts) cluster_store(&s_part[part], (uint32_t)lane, block_sum);
-    cluster_arrive();
-    cluster_wait();
+    od_cluster_wait();
+    if (warp == 0 && lane < (int)nparts) od_cluster_store(&s_part[part], (uint32_t)lane, block_sum);
+    od_cluster_arrive();
+    od_cluster_wait();
 
     // ---- every warp scans the blocks' sums: is the draw in its block, in its run?
     const uint32_t flags = q.residual ? 0u : OD_SF_BONUS;
