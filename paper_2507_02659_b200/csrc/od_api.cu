@@ -130,7 +130,7 @@ int32_t od_create(od_ctx **ctx, int32_t device, int32_t draft_vocab, int32_t tar
         delete c;
         return OD_ERR_UNSUPPORTED;
     }
-    if (od_sample_prepare_device(od_sample_smem_bytes(c->tiles_per_row), c->sample_clusters) != cudaSuccess) {
+    if (od_sample_prepare_device(c->sample_clusters) != cudaSuccess) {
         delete c;
         return OD_ERR_CUDA;
     }

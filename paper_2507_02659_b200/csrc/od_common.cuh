@@ -148,7 +148,7 @@ cudaError_t od_launch_sample(od_ctx *c, int32_t B, int32_t K_max, const void *lo
 
 size_t od_sample_smem_bytes(int32_t ntiles);            // dynamic shared memory of the shard sampler's kernel
 // opt in to the dynamic shared memory and the cluster size that the sampler's kernels may ask for
-cudaError_t od_sample_prepare_device(size_t bytes, int32_t *clusters);   // clusters: [levels] resident at a time
+cudaError_t od_sample_prepare_device(int32_t *clusters);   // clusters: [levels] resident at a time
 
 // The pairs of a vocabulary map in target-id order (host).
 struct OdMappedIds {

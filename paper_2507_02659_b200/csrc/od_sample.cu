@@ -1335,8 +1335,7 @@ size_t od_sample_smem_bytes(int32_t ntiles) { return (size_t)ntiles * 8; }
 template <typename K>
 static cudaError_t allow_smem(K kernel, size_t bytes)
 {
-    return bytes <= 48 * 1024 ? cudaSuccess
-                              : cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
 }
 template <int DTYPE, bool FUSED, int SOURCE>
 static cudaError_t allow_cluster16(size_t bytes)
@@ -1347,8 +1346,9 @@ static cudaError_t allow_cluster16(size_t bytes)
     return e;
 }
 template <int DTYPE>
-static cudaError_t prepare_kernels(size_t bytes)
+static cudaError_t prepare_kernels()
 {
+    const size_t bytes = OD_SAMPLE_SMEM_MAX;
     const size_t staged = (size_t)(OD_SAMPLE_MAX_SLOTS + 1) * 4 + 8 * 1024;
     cudaError_t e = allow_cluster16<DTYPE, false, FROM_MAP>(bytes);
     if (e == cudaSuccess) e = allow_cluster16<DTYPE, true, FROM_MAP>(bytes);
@@ -1362,13 +1362,14 @@ static cudaError_t prepare_kernels(size_t bytes)
 }
 
 // Rows beyond 6144 tiles (and the staged probabilities) need more dynamic shared memory than a
-// kernel gets by default, and clusters of 16 blocks are not portable: opt in, and ask how many
+// kernel gets by default, and clusters of 16 blocks are not portable: opt in, to the same limit in every
+// context (it is the kernel's: a smaller one would take it from a context made earlier), and ask how many
 // clusters of each size are resident at a time (0: the device has no room for one; the device must be
 // current; allocates nothing).
-cudaError_t od_sample_prepare_device(size_t bytes, int32_t *clusters)
+cudaError_t od_sample_prepare_device(int32_t *clusters)
 {
-    cudaError_t e = prepare_kernels<OD_BF16>(bytes);
-    if (e == cudaSuccess) e = prepare_kernels<OD_F32>(bytes);
+    cudaError_t e = prepare_kernels<OD_BF16>();
+    if (e == cudaSuccess) e = prepare_kernels<OD_F32>();
     if (e != cudaSuccess) return e;
     for (int level = 0; level < OD_SAMPLE_LEVELS; ++level) {
         cudaLaunchConfig_t cfg = {};

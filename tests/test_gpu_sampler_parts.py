@@ -8,7 +8,7 @@ import torch
 
 import oracle
 from paper_2507_02659_b200 import binding as od
-from paper_2507_02659_b200 import synth
+from paper_2507_02659_b200 import synth, vshard
 
 import parity
 
@@ -111,3 +111,21 @@ def test_parts_between_the_powers_of_two(cuda_device):
             assert torch.equal(t, vars(so)[name]), name
         ctx.close()
     assert seen == {1, 2, 3, 4, 6, 8, 16}, seen
+
+
+def test_a_smaller_context_made_after_a_larger_one(cuda_device):
+    """The limit of dynamic shared memory belongs to the kernels, not to a context: a shard of the larger one
+    keeps the tile values of its rows (8 bytes per 256 ids, over 48 KB in both) as before."""
+    w = _workload(B=1, k_max=1, v_q=300, v_p=4_000_000, cache_entries=0)
+    st = synth.make_static(w)
+    ctx = parity.make_context(w, st, cuda_device)
+    other = od.Context(cuda_device, 300, 2_000_000, 1, 1)
+    s = synth.make_step(w, st, 0, device=cuda_device)
+    cache = oracle.Cache(st.runs, st.run_len, st.run_target)
+    parity.check_step(ctx, cache, st, w, s)
+    mp, vo, so = parity.gpu_step(ctx, s)
+    _, sh, _ = vshard.emulate_step(ctx, s.logits, 2, mp, s.q_rows, s.draft_ids, s.temperature, s.seed, 0)
+    torch.cuda.synchronize()
+    assert int((so.flags | sh.flags)[0]) & od.OD_SF_BOUNDARY or torch.equal(sh.out_token, so.out_token)
+    other.close()
+    ctx.close()
