@@ -18,8 +18,8 @@
 //           redone with e alone).
 //
 // Where pass 1 has the drafter's probabilities from (they lie in draft-id order):
-//   same tokenizer on both sides: the row itself, two 128-bit loads per lane and tile
-//           (FROM_ROW; 256 rows of 32000 ids: step 44.2 -> 40.1 us);
+//   same tokenizer on both sides: the row itself, two 128-bit loads per lane and tile, or id by id
+//           where rows are not whole vectors (FROM_ROW; 256 rows of 32000 ids: step 44.2 -> 40.1 us);
 //   else    shared memory, in target-id order (STAGED): a block gathers the mapped ids of
 //           its tiles once, from a list in DRAFT-id order (od_sample_plan), so that the 32
 //           lanes of a load sit within a few lines, and finds them in pass 1 by counting
