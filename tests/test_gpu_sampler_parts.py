@@ -86,9 +86,12 @@ def test_shared_ids_off_the_vector_width(cuda_device, v_q, v_p, B, offset):
     assert stats.sample_compared > 0
     mp, vo, so = parity.gpu_step(ctx, s, logits=logits)
     _, _, one = od.od_step(ctx, s.draft_ids, s.draft_len, s.q_sel, s.q_rows, logits, s.temperature, s.seed, 0)
+    _, sh, _ = vshard.emulate_step(ctx, logits, 2, mp, s.q_rows, s.draft_ids, s.temperature, s.seed, 0)
     torch.cuda.synchronize()
     for name, t in vars(one).items():
         assert torch.equal(t, vars(so)[name]), name
+    settled = ((so.flags | sh.flags) & od.OD_SF_BOUNDARY) == 0
+    assert settled.any() and torch.equal(sh.out_token[settled], so.out_token[settled])
     ctx.close()
 
 
