@@ -41,7 +41,8 @@
  *     wait in two cases only: inside od_step / od_step_host, where the
  *     translation kernel is the launch in front of the streaming kernel and has
  *     itself waited for everything earlier in the stream before letting it
- *     start (logits and temperatures, by the streaming kernel); and when the
+ *     start (logits and temperatures, by the streaming kernel; where od_step is
+ *     one launch it reads nothing of the caller's early); and when the
  *     caller has set option "early_inputs" = 1, which is the caller's promise
  *     that the inputs of a call were complete before the launch that precedes
  *     the call was enqueued (a producer two launches back, or data resident
@@ -51,8 +52,9 @@
  *     q_sel) early and, unless od_cache_insert or od_cache_trim was called on
  *     the context since its last translation, probe the n-gram table early
  *     (the table belongs to the context; the library keeps track of who writes
- *     it); and od_step lets its streaming kernel start on logit rows 0 while the
- *     launch in front of the step still runs. What the library keeps track of
+ *     it); and od_step lets its streaming kernel start on logit rows 0 (where it is
+ *     one launch: reads all its inputs) while the launch in front of the step still
+ *     runs. What the library keeps track of
  *     it knows at the time of the call: a CUDA graph that captured
  *     od_map_proposals or od_step under "early_inputs" = 1 must not be launched
  *     directly behind od_cache_insert or od_cache_trim (any launch in between
@@ -330,11 +332,13 @@ int32_t od_sample_residual(od_ctx *ctx, int32_t B, int32_t K_max,
                            uint32_t *sample_flags, void *stream);
 
 /* Steps 1-3 in one call (Algorithm 1 from the translation line to the free-token
- * line): exactly od_map_proposals, od_verify and od_sample_residual on the same
- * arguments, enqueued back to back on `stream`. Besides saving two calls, this is
+ * line): od_map_proposals, od_verify and od_sample_residual on the same
+ * arguments. Besides saving two calls, this is
  * the form in which the library knows its own launch order, so the streaming
  * kernel may start on rows 0 of the logits while the translation kernel still
  * runs, with no promise needed from the caller (see "pdl" in the conventions).
+ * Small batches are one launch, which may add a row's terms in another
+ * order than od_verify does (the row sums' last bits).
  * All pointers are device pointers owned by the caller; inputs and outputs as
  * documented for the three calls (counters may be NULL). Asynchronous; allocates
  * nothing; errors as for the three calls, checked before the first launch. */

@@ -2,6 +2,7 @@
 // host-side builds of the vocabulary map and of the n-gram cache table,
 // argument validation, and the whole-step entry point for host buffers.
 #include <algorithm>
+#include <mutex>
 #include <new>
 #include <string.h>
 #include <vector>
@@ -96,6 +97,42 @@ int32_t check_shard(const od_ctx *c, int32_t shard_lo, int32_t shard_len)
     return OD_OK;
 }
 
+// The kernels' limits, set for every context (they are lost with the device's primary context), and how many
+// clusters of each size are resident at a time, asked for once per device (sixteen occupancy questions, most of what a context cost).
+bool prepare_kernels(od_ctx *c)
+{
+    struct Resident { bool known; int32_t sample[OD_SAMPLE_LEVELS], step[OD_SAMPLE_LEVELS]; };
+    constexpr int DEVICES = 64;
+    static std::mutex mutex;
+    static Resident of[DEVICES];
+    std::lock_guard<std::mutex> lock(mutex);
+    Resident here = {};
+    Resident &r = c->device < DEVICES ? of[c->device] : here;
+    if (od_sample_prepare_device(r.known ? nullptr : r.sample) != cudaSuccess ||
+        od_step_prepare_device(r.known ? nullptr : r.step) != cudaSuccess)
+        return false;
+    r.known = true;
+    memcpy(c->sample_clusters, r.sample, sizeof(r.sample));
+    memcpy(c->step_clusters, r.step, sizeof(r.step));
+    return true;
+}
+
+// step 2, in one launch where the batch allows it; early: rows 0 may be read before the launch in front is done
+cudaError_t verify(od_ctx *c, int32_t B, int32_t K_max, const void *logits, int32_t dtype, int64_t row_stride, int64_t seq_stride,
+                   const int32_t *tgt_ids, const float *q_prime, const int32_t *span_len, const int32_t *m, const float *temperature,
+                   const uint64_t *seed, uint64_t step, float *row_max, float *row_sum, float *p_sel, float *ratio,
+                   int32_t *n_accepted, int32_t *n_draft_accepted, uint32_t *flags, bool early, cudaStream_t s)
+{
+    if (od_verify_one_launch(c, B, K_max, c->v_p, dtype)) {
+        const od_fused_verify out = {0, 0, 0, 0, 0, row_max, row_sum, p_sel, ratio, n_accepted, n_draft_accepted, flags};
+        return od_launch_verify_rows(c, B, K_max, logits, dtype, row_stride, seq_stride, tgt_ids, q_prime, span_len, m, temperature,
+                                     seed, step, &out, early, s);
+    }
+    c->verify_early = early;
+    return od_launch_verify(c, B, K_max, logits, dtype, row_stride, seq_stride, tgt_ids, q_prime, span_len, m, temperature, seed,
+                            step, row_max, row_sum, p_sel, ratio, n_accepted, n_draft_accepted, flags, s);
+}
+
 }  // namespace
 
 extern "C" {
@@ -130,11 +167,7 @@ int32_t od_create(od_ctx **ctx, int32_t device, int32_t draft_vocab, int32_t tar
         delete c;
         return OD_ERR_UNSUPPORTED;
     }
-    if (od_sample_prepare_device(c->sample_clusters) != cudaSuccess) {
-        delete c;
-        return OD_ERR_CUDA;
-    }
-    if (od_distill_prepare_device(draft_vocab) != cudaSuccess) {
+    if (!prepare_kernels(c) || od_distill_prepare_device(draft_vocab) != cudaSuccess) {
         delete c;
         return OD_ERR_CUDA;
     }
@@ -344,11 +377,9 @@ int32_t od_verify(od_ctx *c, int32_t B, int32_t K_max, const void *logits, int32
         return OD_ERR_INVALID_ARG;
     DeviceGuard g(c->device);
     if (!g.ok) return OD_ERR_CUDA;
-    c->verify_early = c->opt_early_inputs != 0;
-    OD_CUDA(od_launch_verify(c, B, K_max, logits, logit_dtype, row_stride, seq_stride, tgt_ids,
-                             q_prime, span_len, m, temperature, seed, step, row_max, row_sum,
-                             p_sel, ratio, n_accepted, n_draft_accepted, verify_flags,
-                             (cudaStream_t)stream));
+    OD_CUDA(verify(c, B, K_max, logits, logit_dtype, row_stride, seq_stride, tgt_ids, q_prime, span_len, m, temperature, seed,
+                   step, row_max, row_sum, p_sel, ratio, n_accepted, n_draft_accepted, verify_flags,
+                   c->opt_early_inputs != 0, (cudaStream_t)stream));
     return OD_OK;
 }
 
@@ -399,6 +430,13 @@ int32_t od_step(od_ctx *c, int32_t B, int32_t K_max, const int32_t *draft_ids, c
     DeviceGuard g(c->device);
     if (!g.ok) return OD_ERR_CUDA;
     cudaStream_t s = (cudaStream_t)stream;
+    if (od_step_one_launch(c, B, K_max, logit_dtype)) {
+        const od_fused_verify out = {0, 0, 0, 0, 0, row_max, row_sum, p_sel, ratio, n_accepted, n_draft_accepted, verify_flags};
+        OD_CUDA(od_launch_step(c, B, K_max, draft_ids, draft_len, q_sel, q_rows, logits, logit_dtype, row_stride, seq_stride,
+                               temperature, seed, step, tgt_ids, q_prime, span_start, span_len, m, tail_kind, counters, &out,
+                               out_token, resid_mass, sample_flags, c->opt_early_inputs != 0, s));
+        return OD_OK;
+    }
     OD_CUDA(od_launch_map(c, B, K_max, draft_ids, draft_len, q_sel, tgt_ids, q_prime, span_start, span_len, m,
                           tail_kind, counters, c->opt_early_inputs != 0, c->opt_early_inputs != 0, s));
     // The translation kernel waits for everything in front of it before it lets the next
@@ -444,6 +482,11 @@ int32_t od_verify_shard_stats(od_ctx *c, int32_t B, int32_t K_max, int32_t shard
     if (!aligned16(stats)) return OD_ERR_ALIGNMENT;
     DeviceGuard g(c->device);
     if (!g.ok) return OD_ERR_CUDA;
+    if (od_verify_one_launch(c, B, K_max, shard_len, logit_dtype)) {
+        OD_CUDA(od_launch_shard_rows(c, B, K_max, shard_lo, shard_len, logits, logit_dtype, row_stride, seq_stride, tgt_ids, m,
+                                     temperature, stats, c->opt_early_inputs != 0, (cudaStream_t)stream));
+        return OD_OK;
+    }
     c->verify_early = c->opt_early_inputs != 0;
     OD_CUDA(od_launch_verify_shard_stats(c, B, K_max, shard_lo, shard_len, logits, logit_dtype, row_stride,
                                          seq_stride, tgt_ids, m, temperature, stats, (cudaStream_t)stream));
@@ -663,11 +706,10 @@ int32_t od_step_host(od_ctx *c, int32_t B, int32_t K_max, const int32_t *draft_i
     OD_CUDA(od_launch_map(c, B, K_max, c->s_draft_ids, c->s_draft_len, c->s_q_sel, c->s_tgt_ids,
                           c->s_q_prime, c->s_span_start, c->s_span_len, c->s_m, c->s_tail, nullptr,
                           false /* the copies above are the launches in front */, false, s));
-    c->verify_early = true;     // the translation kernel is the launch in front: see od_step
-    OD_CUDA(od_launch_verify(c, B, K_max, c->s_logits, logit_dtype, row_stride, seq_stride,
-                             c->s_tgt_ids, c->s_q_prime, c->s_span_len, c->s_m, c->s_temperature,
-                             c->s_seed, step, c->s_row_max, c->s_row_sum, c->s_p_sel, c->s_ratio,
-                             c->s_n_acc, c->s_n_draft, c->s_vflags, s));
+    // (early: the translation kernel is the launch in front, and has waited for what was in front of it)
+    OD_CUDA(verify(c, B, K_max, c->s_logits, logit_dtype, row_stride, seq_stride, c->s_tgt_ids, c->s_q_prime, c->s_span_len,
+                   c->s_m, c->s_temperature, c->s_seed, step, c->s_row_max, c->s_row_sum, c->s_p_sel, c->s_ratio,
+                   c->s_n_acc, c->s_n_draft, c->s_vflags, true, s));
     OD_CUDA(od_launch_sample(c, B, K_max, c->s_logits, logit_dtype, row_stride, seq_stride,
                              c->s_row_max, c->s_row_sum, c->s_q_rows, c->s_draft_ids, c->s_tgt_ids,
                              c->s_q_prime, c->s_span_start, c->s_span_len, c->s_m, c->s_tail,

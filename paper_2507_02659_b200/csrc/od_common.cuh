@@ -14,7 +14,7 @@
 #define OD_GROUP 32                 // slots of one hash-table probe group
 #define OD_SAMPLE_TILE 256          // elements of one residual-sampler tile (8 per lane of a warp)
 #define OD_SAMPLE_THREADS 256       // of the vocabulary shards' sampler
-#define OD_SAMPLE_LEVELS 7          // 1, 2, 3, 4, 6, 8 or 16 blocks draw for one sequence
+#define OD_SAMPLE_LEVELS 8          // 1, 2, 3, 4, 5, 6, 8 or 16 blocks draw for one sequence
 #define OD_SAMPLE_MAX_PARTS 16      // (over 8: a non-portable cluster)
 #define OD_SAMPLE_MAX_SLOTS 53248   // mapped ids of a part: 208 KB of shared memory
 #define OD_SAMPLE_SMEM_MAX (200 * 1024)  // dynamic shared memory the sampler may ask for: 8 bytes per tile
@@ -37,6 +37,7 @@ struct od_ctx {
     void *d_sample_lists;           // and of the sampler (od_sample_lists)
     int32_t sample_slots[OD_SAMPLE_LEVELS];   // most mapped ids of a part
     int32_t sample_clusters[OD_SAMPLE_LEVELS];   // clusters of the sampler that are resident at a time
+    int32_t step_clusters[OD_SAMPLE_LEVELS];     // of the whole step in one launch: a multiprocessor to each block
     bool have_map;
     bool distill_lists;             // some map had gather lists: every later one has the distillation kernel's
     // The map's serial number. A launch is laid out for the map of its time (where ids are shared, how many
@@ -130,6 +131,23 @@ struct od_fused_verify {
     int32_t *n_accepted, *n_draft_accepted;
     uint32_t *flags;
 };
+// od_step and od_verify in one launch (od_step.cu), where a batch's clusters are all resident at a time
+bool od_step_one_launch(const od_ctx *c, int32_t B, int32_t K_max, int32_t dtype);
+bool od_verify_one_launch(const od_ctx *c, int32_t B, int32_t K_max, int32_t v_len, int32_t dtype);
+cudaError_t od_step_prepare_device(int32_t *clusters);
+cudaError_t od_launch_step(od_ctx *c, int32_t B, int32_t K_max, const int32_t *draft_ids, const int32_t *draft_len,
+                           const float *q_sel, const float *q_rows, const void *logits, int32_t dtype, int64_t row_stride,
+                           int64_t seq_stride, const float *temperature, const uint64_t *seed, uint64_t step, int32_t *tgt_ids,
+                           float *q_prime, int32_t *span_start, int32_t *span_len, int32_t *m, uint8_t *tail_kind,
+                           uint32_t *counters, const od_fused_verify *fuse, int32_t *out_token, float *resid_mass, uint32_t *flags,
+                           bool early, cudaStream_t s);
+cudaError_t od_launch_verify_rows(od_ctx *c, int32_t B, int32_t K_max, const void *logits, int32_t dtype, int64_t row_stride,
+                                  int64_t seq_stride, const int32_t *tgt_ids, const float *q_prime, const int32_t *span_len,
+                                  const int32_t *m, const float *temperature, const uint64_t *seed, uint64_t step,
+                                  const od_fused_verify *out, bool early, cudaStream_t s);
+cudaError_t od_launch_shard_rows(od_ctx *c, int32_t B, int32_t K_max, int32_t shard_lo, int32_t shard_len, const void *logits,
+                                 int32_t dtype, int64_t row_stride, int64_t seq_stride, const int32_t *tgt_ids, const int32_t *m,
+                                 const float *temperature, float *stats, bool early, cudaStream_t s);
 int32_t od_verify_slice(int32_t K_max, int32_t v_len, int32_t dtype);   // sequences one stream launch takes
 cudaError_t od_launch_verify_stream(od_ctx *c, int32_t B, int32_t K_max, const void *logits, int32_t dtype,
                                     int64_t row_stride, int64_t seq_stride, const int32_t *m,
@@ -193,7 +211,7 @@ inline size_t od_sample_lists_bytes(int32_t v_q, int32_t v_p)
 // parts of a level, and the tiles of one
 inline int32_t od_sample_parts(int level)
 {
-    const int32_t parts[OD_SAMPLE_LEVELS] = {1, 2, 3, 4, 6, 8, 16};
+    const int32_t parts[OD_SAMPLE_LEVELS] = {1, 2, 3, 4, 5, 6, 8, 16};
     return parts[level];
 }
 inline int32_t od_sample_part_tiles(int32_t v_p, int level)

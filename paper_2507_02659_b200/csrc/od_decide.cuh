@@ -40,15 +40,19 @@ __device__ __forceinline__ void pair_merge(float &c, float &s, float c2, float s
     c = cm;
 }
 
+// the warp's maximum in one instruction (NaN is passed over, as by fmaxf)
+__device__ __forceinline__ float warp_max(float v)
+{
+    float m;
+    asm volatile("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(m) : "f"(v));
+    return m;
+}
+
 // all lanes end with the merged (c, s, mx): one rescale per lane, then plain reductions
 __device__ __forceinline__ void warp_merge(float &c, float &s, float &mx)
 {
-    float cm = c;
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
-        cm = fmaxf(cm, __shfl_xor_sync(0xFFFFFFFFu, cm, off));
-        mx = fmaxf(mx, __shfl_xor_sync(0xFFFFFFFFu, mx, off));
-    }
+    const float cm = warp_max(c);
+    mx = warp_max(mx);
     s *= od_ex2(c - cm);
     c = cm;
 #pragma unroll

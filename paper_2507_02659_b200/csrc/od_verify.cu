@@ -49,6 +49,7 @@
 
 #include "od_common.cuh"
 #include "od_decide.cuh"
+#include "od_stream.cuh"
 
 namespace {
 
@@ -61,7 +62,6 @@ namespace {
 constexpr int NARROW_WARPS = 8, WIDE_WARPS = 16;
 constexpr int WIDE_MIN_UNITS = 256;
 static_assert(OD_VERIFY_SEG_MAX % WIDE_WARPS == 0 && OD_VERIFY_SEG_MAX / WIDE_WARPS >= 3, "segments per row");
-constexpr int U = 4;                            // 16-byte loads in flight per thread
 constexpr int A_PARK = 8;                       // partials of space A a block can hold back
 #ifndef OD_VERIFY_MAXNREG
 #define OD_VERIFY_MAXNREG 56
@@ -102,176 +102,25 @@ struct VerifyArgs {
     int64_t stats_rows;
 };
 
-__device__ __forceinline__ uint4 ld_stream(const uint4 *p)
-{
-    uint4 v;
-    asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];"
-                 : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
-                 : "l"(p));
-    return v;
-}
-
-__device__ __forceinline__ uint32_t bf16x2_max(uint32_t a, uint32_t b)
-{
-    uint32_t d;
-    asm("max.bf16x2 %0, %1, %2;" : "=r"(d) : "r"(a), "r"(b));
-    return d;
-}
-
-// Running state of one thread inside a segment.
-template <int DTYPE>
-struct Lane {
-    float c, s;             // reference exponent (scaled domain), sum of exp2(x*scale - c)
-    float mx;               // fp32 rows: running maximum
-    uint32_t pm;            // bf16 rows: packed running maxima (exact)
-    __device__ __forceinline__ void reset()
-    {
-        c = -FLT_MAX; s = 0.f; mx = -INFINITY; pm = 0xFF80FF80u;
-    }
-    // make c >= gm*scale (branch-free: one rescale per group of vectors)
-    __device__ __forceinline__ void raise(float gm, float scale)
-    {
-        const float cn = fmaxf(fmaxf(gm * scale, -FLT_MAX), c);
-        s *= od_ex2(c - cn);
-        c = cn;
-    }
-    __device__ __forceinline__ float max_seen() const
-    {
-        if (DTYPE == OD_BF16) return fmaxf(od_bf16_lo(pm), od_bf16_hi(pm));
-        return mx;
-    }
-};
-
-// absorb N 16-byte vectors held in registers
-template <int DTYPE, int N>
-__device__ __forceinline__ void absorb(Lane<DTYPE> &L, const uint4 *v, float scale)
-{
-    if (DTYPE == OD_BF16) {
-        uint32_t g = L.pm;
-#pragma unroll
-        for (int u = 0; u < N; ++u) {
-            g = bf16x2_max(g, v[u].x); g = bf16x2_max(g, v[u].y);
-            g = bf16x2_max(g, v[u].z); g = bf16x2_max(g, v[u].w);
-        }
-        L.pm = g;
-        L.raise(fmaxf(od_bf16_lo(g), od_bf16_hi(g)), scale);
-    } else {
-        float gm = -INFINITY;
-#pragma unroll
-        for (int u = 0; u < N; ++u) {
-            gm = fmaxf(gm, fmaxf(fmaxf(__uint_as_float(v[u].x), __uint_as_float(v[u].y)),
-                                 fmaxf(__uint_as_float(v[u].z), __uint_as_float(v[u].w))));
-        }
-        L.mx = fmaxf(L.mx, gm);
-        L.raise(gm, scale);
-    }
-    const uint64_t scale2 = f2_pack(scale, scale), nc2 = f2_pack(-L.c, -L.c);
-    uint64_t a0 = 0ull, a1 = 0ull;                          // two pairs of zeros
-#pragma unroll
-    for (int u = 0; u < N; ++u) {
-        if (DTYPE == OD_BF16) {
-            a0 = f2_exp_acc(a0, od_bf16_lo(v[u].x), od_bf16_hi(v[u].x), scale2, nc2);
-            a1 = f2_exp_acc(a1, od_bf16_lo(v[u].y), od_bf16_hi(v[u].y), scale2, nc2);
-            a0 = f2_exp_acc(a0, od_bf16_lo(v[u].z), od_bf16_hi(v[u].z), scale2, nc2);
-            a1 = f2_exp_acc(a1, od_bf16_lo(v[u].w), od_bf16_hi(v[u].w), scale2, nc2);
-        } else {
-            a0 = f2_exp_acc(a0, __uint_as_float(v[u].x), __uint_as_float(v[u].y), scale2, nc2);
-            a1 = f2_exp_acc(a1, __uint_as_float(v[u].z), __uint_as_float(v[u].w), scale2, nc2);
-        }
-    }
-    float s0, s1;
-    f2_unpack(f2_add(a0, a1), s0, s1);
-    L.s += s0 + s1;
-}
-
-template <int DTYPE>
-__device__ __forceinline__ void absorb_one(Lane<DTYPE> &L, float x, float scale)
-{
-    if (DTYPE == OD_BF16) {
-        // x is a bf16 value: keep the packed maximum exact
-        L.pm = bf16x2_max(L.pm, __float_as_uint(x) >> 16 | 0xFF800000u);
-    } else {
-        L.mx = fmaxf(L.mx, x);
-    }
-    L.raise(x, scale);
-    L.s += od_ex2(fmaf(x, scale, -L.c));
-}
-
-// the first n (1..U, the same for the whole warp) loads of a group
-template <int TW>
-__device__ __forceinline__ void load_group(uint4 (&x)[U], const uint4 *p, int n)
-{
-#pragma unroll
-    for (int u = 0; u < U; ++u)
-        if (u < n) x[u] = ld_stream(p + u * TW * 32);
-}
-
-template <int DTYPE>
-__device__ __forceinline__ void absorb_group(Lane<DTYPE> &L, const uint4 (&x)[U], int n, float scale)
-{
-    static_assert(U == 4, "one case per group size");
-    if (n == 4) absorb<DTYPE, 4>(L, x, scale);
-    else if (n == 3) absorb<DTYPE, 3>(L, x, scale);
-    else if (n == 2) absorb<DTYPE, 2>(L, x, scale);
-    else absorb<DTYPE, 1>(L, x, scale);
-}
-
 // Units [v0, v1) of row (b, r) by the whole block; warp w stores its partial to dst[w]
 // (global or shared memory).
 template <int DTYPE, int TW>
 __device__ __forceinline__ void block_segment(const VerifyArgs &a, int b, int r, int v0, int v1, float4 *dst)
 {
-    constexpr int VEC = DTYPE == OD_BF16 ? 8 : 4;          // elements per 16 bytes
     constexpr size_t ESZ = DTYPE == OD_BF16 ? 2 : 4;
     const float T = a.temperature[b];
     const float scale = (T > 0.f) ? 1.4426950408889634f / T : 0.f;   // log2(e)/T
     const char *row = (const char *)a.logits + ((size_t)b * a.seq_stride + (size_t)r * a.row_stride) * ESZ;
     Lane<DTYPE> L;
     L.reset();
-    // A warp owns whole units (512 bytes, 16 per lane): units v0 + warp, + TW, ...
+    // a warp owns whole units: units v0 + warp, + TW, ...
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int full_vecs = a.v_p / VEC;                     // whole 16-byte vectors in the row
-    const int full_units = full_vecs >> 5;                 // units whose 32 lanes are all inside
-    const int v1f = v1 < full_units ? v1 : full_units;
-    const int v = v0 + warp;
-    const uint4 *p = (const uint4 *)row + (size_t)v * 32 + lane;
-    // Software pipeline over groups of U units: the loads of the next group are
-    // issued before the current group is folded in, so a warp always has loads in
-    // flight while it keeps the exp pipe busy (warps of a block move in lockstep,
-    // they cannot hide one another's latency). The last group holds what is left
-    // (1..U units) and is requested like any other, one group ahead; no lane ever
-    // computes on padding. Only the row's last unit can be ragged (lanes past the
-    // end of the row, or a final piece under 16 bytes).
-    int cnt = v < v1f ? (v1f - v + TW - 1) / TW : 0;   // this warp's whole units
-    if (cnt > 0) {
-        uint4 xa[U], xb[U];
-        int na = cnt < U ? cnt : U, nb = 0;
-        load_group<TW>(xa, p, na);
-        cnt -= na; p += U * TW * 32;
-        for (;;) {
-            if (cnt == 0) { absorb_group<DTYPE>(L, xa, na, scale); break; }
-            nb = cnt < U ? cnt : U;
-            load_group<TW>(xb, p, nb);
-            cnt -= nb; p += U * TW * 32;
-            absorb<DTYPE, U>(L, xa, scale);
-            if (cnt == 0) { absorb_group<DTYPE>(L, xb, nb, scale); break; }
-            na = cnt < U ? cnt : U;
-            load_group<TW>(xa, p, na);
-            cnt -= na; p += U * TW * 32;
-            absorb<DTYPE, U>(L, xb, scale);
-        }
-    }
-    if (v1 > full_units && warp == ((full_units - v0) & (TW - 1))) {
-        // the row's ragged last unit (v1 == W here): whole vectors, then single elements
-        const int i = full_units * 32 + lane;
-        if (i < full_vecs) {
-            uint4 x[1];
-            x[0] = ld_stream((const uint4 *)row + i);
-            absorb<DTYPE, 1>(L, x, scale);
-        }
-        const int e = full_vecs * VEC + lane;
-        if (e < a.v_p) absorb_one<DTYPE>(L, od_load_logit<DTYPE>(row, e), scale);
-    }
+    const int full_units = full_units_of<DTYPE>(a.v_p);
+    UnitRun<DTYPE, TW> run;
+    run.begin(row, v0 + warp, v1 < full_units ? v1 : full_units, lane);
+    run.finish(L, scale);
+    if (v1 > full_units && warp == ((full_units - v0) & (TW - 1)))
+        absorb_ragged<DTYPE>(L, row, a.v_p, lane, scale);   // (v1 == W here)
     // every warp publishes its own partial: no block barrier anywhere in the stream
     float c = L.c, s = L.s, mx = L.max_seen();
     warp_merge(c, s, mx);

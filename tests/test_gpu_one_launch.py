@@ -1,0 +1,119 @@
+"""The whole step in one launch (small batches): every number of blocks per sequence, both sources of the
+drafter's probabilities and the inverse map, against the oracle and against the same step in three launches."""
+import dataclasses
+
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_2507_02659_b200 import binding as od
+from paper_2507_02659_b200 import synth
+
+import parity
+
+pytestmark = pytest.mark.gpu
+
+
+def _workload(**kw):
+    base = dict(B=1, steps=4, k_max=4, k_min=1, v_q=3000, v_p=40000, logit_dtype="bf16", map_kind="random",
+                mapped_frac=0.7, cache_entries=600, hit_prob=0.6, logit_kind="corr", rho=0.9,
+                temperatures=(1.0, 0.5, 0.7), per_seq_seed=True, gen_seed=0x0E51A0, unmapped_shift=2.0, sigma=2.0)
+    base.update(kw)
+    return synth.Workload("onelaunch", **base)
+
+
+def _step(ctx, s, logits):
+    out = od.od_step(ctx, s.draft_ids, s.draft_len, s.q_sel, s.q_rows, logits, s.temperature, s.seed, s.step)
+    torch.cuda.synchronize()
+    return out
+
+
+# batches at which the number of blocks changes; row ends inside a unit, a tile and a vector; a part without tiles
+# (33 tiles in 16 parts of 3); the longest proposals; more mapped ids in a part than are staged
+@pytest.mark.parametrize("kw", [dict(B=B) for B in (1, 7, 8, 15, 16, 22, 23, 30, 36, 40)] +
+                         [dict(B=1, v_q=600, v_p=1003), dict(B=40, v_q=600, v_p=4096, logit_dtype="f32"), dict(B=120, v_q=64, v_p=300),
+                          dict(B=3, v_p=8449, logit_dtype="f32"), dict(B=4, v_p=50001, k_max=16), dict(B=2, v_p=50003, k_max=16, logit_dtype="f32"),
+                          dict(B=5, v_q=5003, v_p=5003, map_kind="identity", cache_entries=0),
+                          dict(B=18, v_q=4096, v_p=4096, map_kind="identity", cache_entries=0, logit_dtype="f32"),
+                          dict(B=1, v_q=60000, v_p=900_000, k_max=1, cache_entries=0)])
+def test_one_launch_against_the_oracle_and_three_launches(cuda_device, kw):
+    w = _workload(**kw)
+    st = synth.make_static(w)
+    if w.v_p >= 900_000:
+        st.vocab_map = np.arange(w.v_q, dtype=np.int32) + 1
+    ctx = parity.make_context(w, st, cuda_device)
+    cache = oracle.Cache(st.runs, st.run_len, st.run_target)
+    for step in range(2):
+        s = synth.make_step(w, st, step, device=cuda_device)
+        lg = parity.pad_rows(s.logits)
+        mp, vo, so = _step(ctx, s, lg)
+        if w.B <= 14 and w.v_p < 900_000:                                   # (how many larger clusters are resident differs from chip to chip)
+            assert ctx.last_launch_info(0) == ctx.last_launch_info(2)      # one grid
+        sel = sorted({0, w.B // 3, w.B // 2, w.B - 1})
+        ref = parity.oracle_step(cache, st, w, dataclasses.replace(
+            s.to("cpu"), **{k: getattr(s, k).cpu()[sel] for k in ("draft_ids", "draft_len", "q_sel", "q_rows", "logits", "temperature", "seed")}),
+            probe=so.out_token.cpu().numpy()[sel])
+        stats = parity.compare(mp, vo, so, ref, s.draft_len.cpu().numpy()[sel], step, s.seed.cpu().numpy().astype(np.uint64)[sel],
+                               bf16=w.logit_dtype == "bf16", sel=np.asarray(sel))
+        assert stats.sequences == len(sel)
+        ctx.set_option("verify_grid", 100)                                  # three launches
+        mp3, vo3, so3 = _step(ctx, s, lg)
+        ctx.set_option("verify_grid", 0)
+        for name in ("m", "tail_kind", "counters"):
+            assert torch.equal(getattr(mp, name), getattr(mp3, name)), name
+        pos = torch.arange(w.k_max, device=cuda_device)[None, :] < mp.m[:, None]
+        for name in ("tgt_ids", "q_prime", "span_start", "span_len"):
+            assert torch.equal(getattr(mp, name)[pos], getattr(mp3, name)[pos]), name
+        rows = torch.arange(w.k_max + 1, device=cuda_device)[None, :] <= mp.m[:, None]
+        assert torch.equal(vo.row_max[rows], vo3.row_max[rows])
+        # two sums of up to 9e5 positive fp32 terms, each within 2e-5 / 2 of exact (the parity bound)
+        torch.testing.assert_close(vo.row_sum[rows], vo3.row_sum[rows], rtol=2e-5, atol=0)
+        settled = ((vo.flags | vo3.flags) == 0) & ((so.flags | so3.flags) & od.OD_SF_BOUNDARY == 0)
+        assert torch.equal(vo.n_accepted[settled], vo3.n_accepted[settled])
+        assert torch.equal(vo.n_draft_accepted[settled], vo3.n_draft_accepted[settled])
+        assert torch.equal(so.out_token[settled], so3.out_token[settled])
+    ctx.close()
+
+
+def test_one_launch_with_nothing_to_translate_and_bad_temperatures(cuda_device):
+    """Empty proposals, ids outside the vocabulary, a temperature of zero: flags and outputs as in three launches."""
+    w = _workload(B=6, k_max=3)
+    st = synth.make_static(w)
+    ctx = parity.make_context(w, st, cuda_device)
+    s = synth.make_step(w, st, 0, device=cuda_device)
+    s.draft_len[:3] = torch.tensor([0, -5, 99], dtype=torch.int32)
+    s.draft_ids[3, 0] = w.v_q + 7
+    s.temperature[4] = 0.0
+    lg = parity.pad_rows(s.logits)
+    one = _step(ctx, s, lg)
+    ctx.set_option("verify_grid", 100)
+    three = _step(ctx, s, lg)
+    for a, b in zip(one, three):
+        for name in ("m", "tail_kind", "counters", "n_accepted", "n_draft_accepted", "flags", "out_token"):
+            if hasattr(a, name):
+                assert torch.equal(getattr(a, name), getattr(b, name)), name
+    assert int(one[0].counters[od.OD_CNT_INVALID_IDS]) >= 1
+    assert int(one[2].out_token[4]) == -1
+    ctx.close()
+
+
+def test_one_launch_stamps_the_online_cache_once(cuda_device):
+    """Several blocks look a run up; its access counts once."""
+    freq = []
+    for grid in (0, 100):
+        w = _workload(B=4, k_max=4, cache_entries=64, hit_prob=1.0)
+        st = synth.make_static(w)
+        ctx = parity.make_context(w, st, cuda_device)
+        ctx.cache_configure(256, 1, 64)
+        dev = lambda x: torch.as_tensor(np.ascontiguousarray(x), dtype=torch.int32, device=cuda_device)
+        ctx.cache_set_clock(1)
+        ctx.cache_insert(dev(st.runs), dev(st.run_len), dev(st.run_target))
+        ctx.set_option("verify_grid", grid)
+        for step in range(3):
+            s = synth.make_step(w, st, step, device=cuda_device)
+            ctx.cache_set_clock(2 + step)
+            _step(ctx, s, parity.pad_rows(s.logits))
+        freq.append(ctx.cache_dump())
+        ctx.close()
+    assert freq[0] == freq[1] and max(f for _, _, f in freq[0].values()) > 1
