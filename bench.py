@@ -165,14 +165,12 @@ def step_bytes(s):
     return sum(x.numel() * x.element_size() for x in t)
 
 
-def host_step_bytes(s, w):
-    """Bytes od_step_host copies to the device for step `s`: the small per-sequence arrays, and of
-    the logits and the drafter's distributions only the rows the step can read (rows 0..K_b and
-    0..K_b-1 of sequence b)."""
+def host_step_bytes(s, w, out, bonus_flag):
+    """Bytes of step `s` that cross the bus in od_step_host from page-locked buffers: the small per-sequence
+    arrays, the logit rows 0..m_b, and the drafter's row of each draw that needs one (`out`: the step's results)."""
     small = sum(x.numel() * x.element_size() for x in (s.draft_ids, s.draft_len, s.q_sel, s.temperature, s.seed))
-    kb = s.draft_len.clamp(0, w.k_max).long()
-    rows_l = int((kb + 1).sum())
-    rows_q = int(kb.sum())
+    rows_l = int((out.m.long() + 1).sum())
+    rows_q = int(((out.sample_flags & bonus_flag) == 0).sum())
     return small + rows_l * w.v_p * s.logits.element_size() + rows_q * w.v_q * 4
 
 
@@ -668,12 +666,13 @@ def main():
         torch.cuda.synchronize(dev)
         ms_e = e0.elapsed_time(e1)
         tok_e = sum(int(hosts[k % hp].draft_len.sum()) for k in range(n_e))
+        h2d = host_step_bytes(hosts[(n_e - 1) % hp], w, hout, od.OD_SF_BONUS)
         ms_e_max, tok_e_all = shard.reduce_timing(ms_e, tok_e, dev)
         d2h = sum(t.numel() * t.element_size() for t in
                   (hout.n_accepted, hout.n_draft_accepted, hout.out_token, hout.tgt_ids, hout.m,
                    hout.verify_flags, hout.sample_flags))
         e2e = {"value": tok_e_all / (ms_e_max * 1e-3), "unit": UNIT, "steps": n_e,
-               "ms_per_step": ms_e_max / n_e, "h2d_bytes_per_step": host_step_bytes(hosts[0], w),
+               "ms_per_step": ms_e_max / n_e, "h2d_bytes_per_step": h2d,
                "d2h_bytes_per_step": d2h, "api": "od_step_host (pinned host buffers)"}
 
     cpu = None

@@ -456,11 +456,14 @@ int32_t od_verify_noalloc(int32_t target_vocab, int32_t B, int32_t K_max,
  * max_batch x max_k, logits of `logit_dtype` stored densely. Synchronous. */
 int32_t od_host_step_reserve(od_ctx *ctx, int32_t logit_dtype);
 
-/* Steps 1-3 on HOST buffers (pinned memory recommended): copies the inputs to
- * the staging area, runs the three kernels, copies the results back, all on
+/* Steps 1-3 on HOST buffers (pinned memory recommended): brings the inputs to
+ * the staging area, runs the three steps, copies the results back, all on
  * `stream`, and synchronises that stream before returning. Host layouts are
- * the dense ones above (logits [B, K_max+1, target_vocab]); of the logits and
- * of q_rows only the rows the step can read are copied (rows 0..K_b and
+ * the dense ones above (logits [B, K_max+1, target_vocab]). Where logits and
+ * q_rows are page-locked (16-byte aligned, each inside one page-locked range) the
+ * device reads the rows that the step needs from them: rows 0..m_b of the logits
+ * and the one drafter row of a sequence's draw. Of other buffers the rows that the
+ * step can read are copied (rows 0..K_b and
  * 0..K_b-1 of sequence b, K_b = draft_len[b] read on the host). Outputs: host
  * int32[B] each for n_accepted, n_draft_accepted, out_token; int32[B,K_max]
  * tgt_ids; int32[B] m; uint32[B] verify_flags and sample_flags (any output may

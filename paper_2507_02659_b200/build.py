@@ -12,7 +12,7 @@ CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libomnidraft.so")
 EXT = os.path.join(HERE, "_marshal.so")
 EXT_FOR = os.path.join(HERE, "_build", "marshal_built_for")
-SOURCES = ["od_api.cu", "od_map.cu", "od_verify.cu", "od_sample.cu", "od_step.cu", "od_noalloc.cu", "od_exit.cu", "od_cache.cu", "od_distill.cu"]
+SOURCES = ["od_api.cu", "od_map.cu", "od_verify.cu", "od_sample.cu", "od_step.cu", "od_host.cu", "od_noalloc.cu", "od_exit.cu", "od_cache.cu", "od_distill.cu"]
 
 
 def _newest_source() -> float:

@@ -679,12 +679,15 @@ int32_t od_step_host(od_ctx *c, int32_t B, int32_t K_max, const int32_t *draft_i
     OD_CUDA(cudaMemcpyAsync(c->s_q_sel, q_sel, nB * K * 4, H2D, s));
     OD_CUDA(cudaMemcpyAsync(c->s_temperature, temperature, nB * 4, H2D, s));
     OD_CUDA(cudaMemcpyAsync(c->s_seed, seed, nB * 8, H2D, s));
-    // Only the rows the step can read cross the bus: logit rows 0..K_b and drafter rows
-    // 0..K_b-1 of sequence b (m_b <= K_b). Neighbouring sequences with full proposals
+    // Only the rows the step can read cross the bus. Page-locked buffers are read by the device, row by row as the
+    // step finds out which ones it needs (od_host.cu). Of others logit rows 0..K_b and drafter rows
+    // 0..K_b-1 of sequence b are copied (m_b <= K_b): neighbouring sequences with full proposals
     // merge into one copy; the rest of the staging buffers keeps earlier contents, which
     // no kernel looks at.
-    {
-        const size_t lrow = (size_t)c->v_p * esz, qrow = (size_t)c->v_q * 4;
+    const size_t lrow = (size_t)c->v_p * esz, qrow = (size_t)c->v_q * 4;
+    const char *d_logits, *d_q_rows;
+    const bool fetched = od_host_rows_readable(logits, nB * (K + 1) * lrow, q_rows, nB * K * qrow, &d_logits, &d_q_rows);
+    if (!fetched) {
         size_t l_from = 0, l_bytes = 0, q_from = 0, q_bytes = 0;   // pending runs (byte offsets)
         for (size_t b = 0; b <= nB; ++b) {
             int32_t kb = 0;
@@ -706,10 +709,12 @@ int32_t od_step_host(od_ctx *c, int32_t B, int32_t K_max, const int32_t *draft_i
     OD_CUDA(od_launch_map(c, B, K_max, c->s_draft_ids, c->s_draft_len, c->s_q_sel, c->s_tgt_ids,
                           c->s_q_prime, c->s_span_start, c->s_span_len, c->s_m, c->s_tail, nullptr,
                           false /* the copies above are the launches in front */, false, s));
+    if (fetched) OD_CUDA(od_launch_fetch_logits(c, B, K_max, d_logits, lrow, s));
     // (early: the translation kernel is the launch in front, and has waited for what was in front of it)
     OD_CUDA(verify(c, B, K_max, c->s_logits, logit_dtype, row_stride, seq_stride, c->s_tgt_ids, c->s_q_prime, c->s_span_len,
                    c->s_m, c->s_temperature, c->s_seed, step, c->s_row_max, c->s_row_sum, c->s_p_sel, c->s_ratio,
-                   c->s_n_acc, c->s_n_draft, c->s_vflags, true, s));
+                   c->s_n_acc, c->s_n_draft, c->s_vflags, !fetched, s));
+    if (fetched) OD_CUDA(od_launch_fetch_drafter(c, B, K_max, d_q_rows, s));
     OD_CUDA(od_launch_sample(c, B, K_max, c->s_logits, logit_dtype, row_stride, seq_stride,
                              c->s_row_max, c->s_row_sum, c->s_q_rows, c->s_draft_ids, c->s_tgt_ids,
                              c->s_q_prime, c->s_span_start, c->s_span_len, c->s_m, c->s_tail,

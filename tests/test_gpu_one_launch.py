@@ -1,5 +1,6 @@
 """The whole step in one launch (small batches): every number of blocks per sequence, both sources of the
-drafter's probabilities and the inverse map, against the oracle and against the same step in three launches."""
+drafter's probabilities and the inverse map, against the oracle and against the same step in three launches; and
+the page-locked form of the step on host buffers."""
 import dataclasses
 
 import numpy as np
@@ -117,3 +118,31 @@ def test_one_launch_stamps_the_online_cache_once(cuda_device):
         freq.append(ctx.cache_dump())
         ctx.close()
     assert freq[0] == freq[1] and max(f for _, _, f in freq[0].values()) > 1
+
+
+# page-locked buffers, which the device fetches itself (drafter rows of whole vectors, and not), parts of a larger
+# page-locked block, a base off 16 bytes and pageable memory, which are copied
+@pytest.mark.parametrize("v_q", [2000, 2001])
+@pytest.mark.parametrize("where", ["pinned", "inside", "offset", "pageable"])
+def test_host_buffers(cuda_device, v_q, where):
+    w = _workload(B=9, v_q=v_q, v_p=30000, k_max=5)
+    st = synth.make_static(w)
+    ctx = parity.make_context(w, st, cuda_device)
+    ctx.host_step_reserve(od.OD_BF16)
+    for step in range(2):
+        s = synth.make_step(w, st, step, device=cuda_device)
+        mp, vo, so = parity.gpu_step(ctx, s)
+        h = s.to("cpu")
+
+        def put(t):
+            if where == "pageable":
+                return t.contiguous()
+            pad = {"pinned": 0, "inside": 64, "offset": 2}[where] if t.dtype in (torch.bfloat16, torch.float32) else 0
+            big = torch.empty(t.numel() + 2 * pad, dtype=t.dtype, pin_memory=True)
+            return big[pad:pad + t.numel()].view(t.shape).copy_(t)
+        out = od.od_step_host(ctx, put(h.draft_ids), put(h.draft_len), put(h.q_sel), put(h.q_rows), put(h.logits),
+                              put(h.temperature), put(h.seed), s.step)
+        for name, ref in (("n_accepted", vo.n_accepted), ("n_draft_accepted", vo.n_draft_accepted), ("out_token", so.out_token),
+                          ("m", mp.m), ("verify_flags", vo.flags), ("sample_flags", so.flags)):
+            assert torch.equal(getattr(out, name), ref.cpu()), name
+    ctx.close()
