@@ -316,10 +316,12 @@ __global__ void trim_compact_kernel(int policy, unsigned int clock, const unsign
 //
 // One cluster of P blocks, each with a slice of the dense list: a most-significant-digit radix
 // select in which a pass is a histogram in shared memory, ONE cluster barrier and the sum of the
-// P histograms over distributed shared memory, by every block alike. The digits of (new?, score)
+// P histograms over distributed shared memory, by every block alike. The bits of (new?, score)
 // that vary are settled first, over the slices; the keys of the entries that tie at that score
-// then stay in shared memory for the eight bytes of the run key, and the select ends as soon as
-// every candidate that is left is among the k (usually two bytes into the run's ids). As a chain
+// then stay in shared memory for the run key, and the select ends as soon as
+// every candidate that is left is among the k (usually three passes in all: a pass costs 2.5 us or so,
+// of which the barrier and the sums are most; an insertion, a trim and a translation, bytes -> bits and run lengths as
+// digits: 262144 entries 62.7 -> 58.2 us, by frequency 90.5 -> 70.3; 8192 entries 32.8 -> 26.6). As a chain
 // of 13 launches of the whole grid, two dependent round trips and a launch each, the passes were
 // 52 of the 107 us of an insertion, a trim and a translation (262144 entries, 16384 new ones).
 constexpr int SELECT_THREADS = 1024, SELECT_MAX_BLOCKS = 16;
@@ -391,11 +393,23 @@ trim_select_kernel(unsigned int max_entries, unsigned int room, int64_t cap, voi
         return s_digit;
     };
 
-    // ---- (new?, score): the bits that vary, over the slice
+    // ---- (new?, score): the bits that vary, over the slice, up to eight a pass. They rarely are whole bytes (the
+    // clocks of the last dozen batches and whether an entry is new: one pass, a byte at a time it was two).
     const unsigned long long vary = hi_or & ~hi_and;
-    unsigned long long thr_hi = hi_and, known = ~vary;
-    for (int byte = 4; byte >= 0; --byte) {
-        if ((vary >> (8 * byte) & 0xFFull) == 0ull) continue;
+    unsigned long long thr_hi = hi_and, todo = vary;
+    while (todo != 0ull && n_match > k_rem) {
+        // the highest ones, in at most two runs: sh1, sh2 their lowest bits, w1, w2 how many they are
+        const int top = 63 - __clzll((long long)todo);
+        const int w1 = min(8, __clzll((long long)~(todo << (63 - top)))), sh1 = top - w1 + 1;
+        const unsigned long long rest = todo & ((1ull << sh1) - 1ull);
+        int w2 = 0, sh2 = 0;
+        if (w1 < 8 && rest) {
+            const int top2 = 63 - __clzll((long long)rest);
+            w2 = min(8 - w1, __clzll((long long)~(rest << (63 - top2))));
+            sh2 = top2 - w2 + 1;
+        }
+        const unsigned int m1 = (1u << w1) - 1u, m2 = (1u << w2) - 1u;
+        const unsigned long long known = ~todo;
         constexpr int U = 9;
         for (unsigned int i0 = lo; i0 < hi_end; i0 += SELECT_THREADS * U) {
             unsigned long long h[U];
@@ -406,16 +420,25 @@ trim_select_kernel(unsigned int max_entries, unsigned int room, int64_t cap, voi
             }
 #pragma unroll
             for (int e = 0; e < U; ++e)
-                count_digit(s_hist[buf], (unsigned int)(h[e] >> (8 * byte)) & 0xFFu,
+                count_digit(s_hist[buf], ((unsigned int)(h[e] >> sh1) & m1) << w2 | ((unsigned int)(h[e] >> sh2) & m2),
                             i0 + e * SELECT_THREADS + threadIdx.x < hi_end && (h[e] & known) == (thr_hi & known));
         }
         const unsigned int d = settle();
-        thr_hi = (thr_hi & ~(0xFFull << (8 * byte))) | (unsigned long long)d << (8 * byte);
-        known |= 0xFFull << (8 * byte);
+        const unsigned long long bits = (unsigned long long)m1 << sh1 | (unsigned long long)m2 << sh2;
+        thr_hi = (thr_hi & ~bits) | (unsigned long long)(d >> w2) << sh1 | (unsigned long long)(d & m2) << sh2;
+        todo &= ~bits;
     }
+    thr_hi |= todo;                                         // (every candidate left is among the k, whatever these bits)
     // ---- the run keys of the entries that tie at that score
-    unsigned long long thr_lo = 0ull, decided = 0ull;
+    unsigned long long thr_lo = 0ull, decided = 0ull, least = 0ull;
     if (n_match > k_rem) {
+        // The first digit tells runs of two, three and four ids apart (of equal score the shorter run's key is the
+        // smaller: the upper fields are zero) and has the leading bits of the last id. A byte at a time the select
+        // walked through the empty fields: five or six passes where two are enough.
+        const auto first_digit = [](unsigned long long key) -> unsigned int {
+            const unsigned int f3 = (unsigned int)(key >> 48), f2 = (unsigned int)(key >> 32) & 0xFFFFu;
+            return f3 ? 192u + (f3 >> 10) : f2 ? 128u + (f2 >> 10) : (unsigned int)key >> 25;
+        };
         constexpr int U = 9;
         for (unsigned int i0 = lo; i0 < hi_end; i0 += SELECT_THREADS * U) {
             unsigned long long h[U], key[U];
@@ -425,8 +448,10 @@ trim_select_kernel(unsigned int max_entries, unsigned int room, int64_t cap, voi
                 h[e] = i < hi_end ? __ldcg(L.r_hi + i) : ~thr_hi;
             }
 #pragma unroll
-            for (int e = 0; e < U; ++e)
+            for (int e = 0; e < U; ++e) {
+                key[e] = 0ull;
                 if (h[e] == thr_hi) key[e] = __ldcg(L.r_key + i0 + e * SELECT_THREADS + threadIdx.x);
+            }
             unsigned int mine = 0;
 #pragma unroll
             for (int e = 0; e < U; ++e) mine += h[e] == thr_hi ? 1u : 0u;
@@ -443,24 +468,34 @@ trim_select_kernel(unsigned int max_entries, unsigned int room, int64_t cap, voi
 #pragma unroll
             for (int e = 0; e < U; ++e)
                 if (h[e] == thr_hi) { if (at < room) s_keys[at] = key[e]; ++at; }
+#pragma unroll
+            for (int e = 0; e < U; ++e) count_digit(s_hist[buf], first_digit(key[e]), h[e] == thr_hi);
         }
         __syncthreads();
         const bool held = s_n <= room;                      // else the slice is read again (a table trimmed late)
         const unsigned int c_end = held ? s_n : hi_end - lo;
-        for (int byte = 7; byte >= 0 && n_match > k_rem; --byte) {
+        const unsigned int d = settle();
+        int undecided;                                      // the lowest so many bits
+        if (d >= 192u) { least = 1ull << 48; undecided = 58; thr_lo = (unsigned long long)(d - 192u) << 58; }
+        else if (d >= 128u) { least = 1ull << 32; undecided = 42; thr_lo = (unsigned long long)(d - 128u) << 42; }
+        else { undecided = 25; thr_lo = (unsigned long long)d << 25; }
+        decided = ~0ull << undecided;
+        while (undecided > 0 && n_match > k_rem) {
+            const int w = min(8, undecided);
+            undecided -= w;
             for (unsigned int i0 = 0; i0 < c_end; i0 += SELECT_THREADS) {
                 const unsigned int i = i0 + threadIdx.x;
                 bool ok = i < c_end;
                 unsigned long long key = 0ull;
                 if (ok) {
                     key = held ? s_keys[i] : __ldcg(L.r_key + lo + i);
-                    ok = (key & decided) == thr_lo && (held || __ldcg(L.r_hi + lo + i) == thr_hi);
+                    ok = key >= least && (key & decided) == thr_lo && (held || __ldcg(L.r_hi + lo + i) == thr_hi);
                 }
-                count_digit(s_hist[buf], (unsigned int)(key >> (8 * byte)) & 0xFFu, ok);
+                count_digit(s_hist[buf], (unsigned int)(key >> undecided) & ((1u << w) - 1u), ok);
             }
             const unsigned int d = settle();
-            thr_lo |= (unsigned long long)d << (8 * byte);
-            decided |= 0xFFull << (8 * byte);
+            thr_lo |= (unsigned long long)d << undecided;
+            decided |= (unsigned long long)((1u << w) - 1u) << undecided;
         }
     }
     thr_lo |= ~decided;                                     // every candidate left is among the k
@@ -838,10 +873,11 @@ int32_t od_cache_trim(od_ctx *c, void *stream)
     c->table_written = true;
     TrimState *st = (TrimState *)c->d_trim;
     const int grid = c->sm_count * 4;
+    const int wave = c->sm_count * 5;                       // of the pass over the table: what is resident (62.5 -> 61.4 us in a row)
     const bool pdl = c->opt_pdl != 0;
     const int blocks = c->trim_blocks;                      // 0: the select is a chain of launches
     if (!blocks) OD_CUDA(chain_launch(trim_begin_kernel, 1u, 256u, s, pdl, st, (unsigned int)c->dyn_max));
-    OD_CUDA(chain_launch(trim_compact_kernel, (unsigned)grid, 256u, s, pdl, c->dyn_policy, c->clock,
+    OD_CUDA(chain_launch(trim_compact_kernel, (unsigned)wave, 256u, s, pdl, c->dyn_policy, c->clock,
                          (const unsigned long long *)c->d_keys, (const int32_t *)c->d_vals,
                          (const unsigned int *)c->d_stamp, (const unsigned int *)c->d_freq,
                          (const unsigned int *)c->d_born, (unsigned long long *)c->d_keys2, c->d_vals2,

@@ -157,6 +157,35 @@ def test_trim_over_ties(cuda_device, policy, bound, batch, batches):
     ctx.close()
 
 
+# scores whose varying bits lie apart (more than two runs of them, more than eight bits) and whole-word clocks; runs
+# of one length, of leading ids from 0 to the last, and the bound inside and at the ends of a group of equal scores
+@pytest.mark.parametrize("clocks", [(1, 2, 3), (0x80000001, 0x7FFFFFFF, 5), (1, 0x4000, 0x10002, 0x1010101, 0xFFFFFFF0)])
+@pytest.mark.parametrize("length", [2, 3, 4, 0])
+@pytest.mark.parametrize("bound", [1, 299, 300, 301, 555])
+def test_trim_over_scores_with_bits_apart(cuda_device, clocks, length, bound):
+    rng = np.random.default_rng(70 + length)
+    v_q, v_p, dev = 65535, 1000, cuda_device
+    ctx = od.Context(cuda_device, v_q, v_p, 4, 4)
+    ctx.set_vocab_map(np.full(v_q, -1, np.int32))
+    ctx.cache_configure(bound, cp.LRU, 300)
+    ref = cp.DynamicCache(bound, cp.LRU, v_q, v_p)
+    for clock in clocks:
+        ctx.cache_set_clock(clock); ref.set_clock(clock)
+        n = min(300, bound)
+        lens = np.full(n, length, np.int32) if length else rng.integers(2, 5, size=n).astype(np.int32)
+        runs = rng.choice([0, 1, 1022, 1023, 1024, 32767, 65534, 7, 511, 512], size=(n, 4)).astype(np.int32)
+        runs[:, 1] = rng.integers(0, v_q, size=n)
+        tg = rng.integers(0, v_p, size=n).astype(np.int32)
+        for _ in range(2 if bound < 300 else 1):
+            ctx.cache_insert(torch.from_numpy(runs).to(dev), torch.from_numpy(lens).to(dev), torch.from_numpy(tg).to(dev))
+            ref.insert_batch(runs, lens, tg)
+        if clock == clocks[-1] or bound < 400:
+            ctx.cache_trim(); ref.trim()
+            assert len(ref) <= bound
+            _compare(ctx, ref)
+    ctx.close()
+
+
 # the select in one launch, and the chain of launches for a table too large for it
 @pytest.mark.parametrize("bound", [100, 400000])
 @pytest.mark.parametrize("trims", [1, 2])
