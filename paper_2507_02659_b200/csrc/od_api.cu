@@ -608,7 +608,7 @@ int32_t od_exit_rule(od_ctx *c, int32_t B, int32_t K_max, const float *head_logi
     DeviceGuard g(c->device);
     if (!g.ok) return OD_ERR_CUDA;
     c->last_was_map = false;
-    OD_CUDA(od_launch_exit(B, K_max, head_logits, avail_len, gamma, draft_len, reject_prob, exit_flags,
+    OD_CUDA(od_launch_exit(B, K_max, head_logits, avail_len, gamma, draft_len, reject_prob, exit_flags, c->opt_pdl != 0,
                            (cudaStream_t)stream));
     return OD_OK;
 }

@@ -300,7 +300,7 @@ cudaError_t od_distill_prepare_device(int32_t v_q);
 void od_cache_free_dynamic(od_ctx *c);   // frees what od_cache_configure allocated beyond keys / vals
 
 cudaError_t od_launch_exit(int32_t B, int32_t K_max, const float *head_logits, const int32_t *avail_len,
-                           float gamma, int32_t *draft_len, float *reject_prob, uint32_t *flags,
+                           float gamma, int32_t *draft_len, float *reject_prob, uint32_t *flags, bool pdl,
                            cudaStream_t s);
 
 // 64-bit key of a run of draft ids: (id + 1) in 16 bits per position, first id
