@@ -24,6 +24,7 @@
 //           histogram, and a digit of (new?, score) that is the same in every live entry
 //           costs no histogram. Then the survivors are re-inserted from the dense list
 //           into the spare table, which becomes the table. No kernel waits for another.
+#include <algorithm>
 #include <stddef.h>
 #include <string.h>
 #include <utility>
@@ -133,13 +134,14 @@ __global__ void insert_claim_kernel(int32_t N, int32_t v_q, int32_t v_p, const i
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= N) return;
     cand_slot[i] = -1;
-    const int L = len[i];
-    bool ok = L >= 2 && L <= OD_NGRAM_MAX && target[i] >= 0 && target[i] < v_p;
+    // one round trip: every load goes out before the first is looked at
+    const int L = len[i], tgt = target[i];
     int32_t ids[OD_NGRAM_MAX];
-    for (int j = 0; j < OD_NGRAM_MAX; ++j) {
-        ids[j] = j < L && ok ? runs[(size_t)i * OD_NGRAM_MAX + j] : 0;
-        if (j < L && ok && (ids[j] < 0 || ids[j] >= v_q)) ok = false;
-    }
+#pragma unroll
+    for (int j = 0; j < OD_NGRAM_MAX; ++j) ids[j] = runs[(size_t)i * OD_NGRAM_MAX + j];
+    bool ok = L >= 2 && L <= OD_NGRAM_MAX && tgt >= 0 && tgt < v_p;
+#pragma unroll
+    for (int j = 0; j < OD_NGRAM_MAX; ++j) ok = ok && (j >= L || (ids[j] >= 0 && ids[j] < v_q));
     if (!ok) { atomicAdd(&st->invalid, 1u); return; }
     const unsigned long long key = od_pack_run(ids, L);
     const uint64_t ngroups = (uint64_t)cap / OD_GROUP;
@@ -193,11 +195,11 @@ __global__ void insert_commit_kernel(int32_t N, const int32_t *__restrict__ targ
     chain_wait();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= N) return;
-    const int32_t slot = cand_slot[i];
+    const int32_t slot = cand_slot[i], tgt = target[i];
     if (slot < 0 || owner[slot] != (unsigned int)i) return; // a candidate with a lower index carries this run
     stamp[slot] = clock; freq[slot] = 1u; born[slot] = clock;
     __threadfence();
-    vals[slot] = target[i];                                  // the entry exists from here on
+    vals[slot] = tgt;                                        // the entry exists from here on
     owner[slot] = 0xFFFFFFFFu;
     atomicAdd(&st->size, 1u);
 }
@@ -675,10 +677,11 @@ __global__ void trim_rebuild_kernel(unsigned long long *nkeys, int32_t *nvals, u
     }
     const uint64_t ngroups = (uint64_t)cap / OD_GROUP;
     for (unsigned int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-        const unsigned long long hi = L.r_hi[i], key = L.r_key[i];
+        // (all of it at once, though some are dropped: one round trip)
+        const unsigned long long hi = __ldcg(L.r_hi + i), key = __ldcg(L.r_key + i);
+        const int32_t v = __ldcg(L.r_val + i);
+        const unsigned int s = __ldcg(L.r_stamp + i), f = __ldcg(L.r_freq + i), b = __ldcg(L.r_born + i);
         if (k > 0u && (hi < thr_hi || (hi == thr_hi && key <= thr_lo))) continue;   // among the k first: dropped
-        const int32_t v = L.r_val[i];
-        const unsigned int s = L.r_stamp[i], f = L.r_freq[i], b = L.r_born[i];
         uint64_t g = od_hash64(key) & (ngroups - 1);
         // A group is filled from its slot 0 without holes (od_cache_insert stops at the first
         // empty slot). Every placement takes the next slot of its group from the group's
@@ -872,8 +875,10 @@ int32_t od_cache_trim(od_ctx *c, void *stream)
     c->last_was_map = false;
     c->table_written = true;
     TrimState *st = (TrimState *)c->d_trim;
-    const int grid = c->sm_count * 4;
-    const int wave = c->sm_count * 5;                       // of the pass over the table: what is resident (62.5 -> 61.4 us in a row)
+    // What is resident at a time, and no more blocks than have anything to do (4 or 5 to a multiprocessor: the pass
+    // over the table with 5 in place of 4 makes 62.5 us in a row 61.4, the rebuild with 8 in place of 4 57.0 -> 57.4)
+    const int wave = (int)std::min<int64_t>(c->sm_count * 5, (c->cap + 1023) / 1024);
+    const int grid = (int)std::min<int64_t>(c->sm_count * 4, (c->dyn_max + c->dyn_max_insert + 255) / 256);
     const bool pdl = c->opt_pdl != 0;
     const int blocks = c->trim_blocks;                      // 0: the select is a chain of launches
     if (!blocks) OD_CUDA(chain_launch(trim_begin_kernel, 1u, 256u, s, pdl, st, (unsigned int)c->dyn_max));
