@@ -402,16 +402,18 @@ int level_within(const od_ctx *c, int32_t B, int32_t K_max, int32_t v_len, int32
     const int64_t bytes = (int64_t)od_sample_part_tiles(v_len, level) * OD_SAMPLE_TILE * (dtype == OD_BF16 ? 2 : 4);
     return bytes * (K_max + 1) <= most ? level : -1;
 }
-// A cluster streams its sequence's rows by itself, 60 GB/s a block (the special-function unit's rate), however
-// few rows others have; three launches spread all rows over all multiprocessors. The line lies where a block may
-// have 360 KB to stream (device time of a step, three launches -> one; sequences x K_max, target ids, blocks: KB):
-//   1 x 6, 128256 bf16, 16: 112 KB  13.8 -> 12.0      15 x 6, 8: 224 KB  18.6 -> 15.4     24 x 6, 5: 354 KB  20.3 -> 19.8
-//   15 x 12, 8: 417 KB  19.8 -> 19.3                  28 x 6, 4: 449 KB  21.5 -> 21.7     22 x 12, 6: 556 KB  23.2 -> 23.4
-//   36 x 4, 50001 fp32, 3: 333 KB  20.4 -> 17.6       7 x 3, 152064, 16: 76 KB  16.4 -> 12.4
+// A cluster streams its sequence's rows by itself, at most 60 GB/s a block (the special-function unit's rate; 40 from
+// HBM with what it has in flight), however few rows others have; three launches spread all rows over all
+// multiprocessors. The line lies where a block may have 320 KB to stream (device time of a step, three launches -> one;
+// sequences x K_max, target ids, blocks: KB; in brackets with inputs that change from pass to pass, from HBM):
+//   1 x 6, 128256 bf16, 16: 112 KB  13.8 -> 12.0 (13.3 -> 10.9)     15 x 6, 8: 221 KB  18.6 -> 15.4 (19.7 -> 16.7)
+//   22 x 6, 6: 294 KB  20.0 -> 18.0 (20.9 -> 19.6)                  24 x 6, 5: 354 KB  20.3 -> 19.8 (21.3 -> 21.5)
+//   15 x 12, 8: 410 KB  19.8 -> 19.3                  28 x 6, 4: 441 KB  21.5 -> 21.7     22 x 12, 6: 546 KB  23.2 -> 23.4
+//   36 x 4, 50001 fp32, 3: 330 KB  20.4 -> 17.6       7 x 3, 152064, 16: 76 KB  16.4 -> 12.4
 // and batches of two blocks a sequence gain little (60 x 8, 32000: 16.0 -> 15.3; 60 x 6, 128256: 30.0 -> 34.8).
 int step_level(const od_ctx *c, int32_t B, int32_t K_max, int32_t v_len, int32_t dtype)
 {
-    return level_within(c, B, K_max, v_len, dtype, 3, 360 * 1024);
+    return level_within(c, B, K_max, v_len, dtype, 3, 320 * 1024);
 }
 // Step 2 alone takes the place of two launches, not three, and its blocks leave no room for those of the next call:
 // 200 KB (the three calls: 20 x 4, 50001 fp32, 6: 167 KB  18.3 -> 18.2; 44 x 4, 40000, 3: 133 KB  20.7 -> 20.0; 15 x 6,
