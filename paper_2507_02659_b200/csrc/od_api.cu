@@ -97,21 +97,39 @@ int32_t check_shard(const od_ctx *c, int32_t shard_lo, int32_t shard_len)
     return OD_OK;
 }
 
-// The kernels' limits, set for every context (they are lost with the device's primary context), and how many
-// clusters of each size are resident at a time, asked for once per device (sixteen occupancy questions, most of what a context cost).
+// The unique number of the current CUDA context, 0 if the driver does not say.
+unsigned long long cuda_context_id()
+{
+    typedef int (*GetId)(void *, unsigned long long *);
+    void *fn = nullptr;
+    cudaDriverEntryPointQueryResult found;
+    unsigned long long id = 0;
+    if (cudaFree(nullptr) != cudaSuccess ||                 // (there is a context from here on)
+        cudaGetDriverEntryPointByVersion("cuCtxGetId", &fn, 12000, cudaEnableDefault, &found) != cudaSuccess || !fn ||
+        ((GetId)fn)(nullptr, &id) != 0) {
+        cudaGetLastError();
+        return 0;
+    }
+    return id;
+}
+
+// The kernels' limits, and how many clusters of each size are resident at a time: once per CUDA context (limits are
+// lost with it, after cudaDeviceReset for instance), not in every od_create, which they made 1 ms and more longer.
 bool prepare_kernels(od_ctx *c)
 {
-    struct Resident { bool known; int32_t sample[OD_SAMPLE_LEVELS], step[OD_SAMPLE_LEVELS]; };
+    struct Resident { unsigned long long context; int32_t sample[OD_SAMPLE_LEVELS], step[OD_SAMPLE_LEVELS]; };
     constexpr int DEVICES = 64;
     static std::mutex mutex;
     static Resident of[DEVICES];
     std::lock_guard<std::mutex> lock(mutex);
     Resident here = {};
     Resident &r = c->device < DEVICES ? of[c->device] : here;
-    if (od_sample_prepare_device(r.known ? nullptr : r.sample) != cudaSuccess ||
-        od_step_prepare_device(r.known ? nullptr : r.step) != cudaSuccess)
-        return false;
-    r.known = true;
+    const unsigned long long id = cuda_context_id();
+    if (id == 0 || r.context != id) {
+        r.context = 0;
+        if (od_sample_prepare_device(r.sample) != cudaSuccess || od_step_prepare_device(r.step) != cudaSuccess) return false;
+        r.context = id;
+    }
     memcpy(c->sample_clusters, r.sample, sizeof(r.sample));
     memcpy(c->step_clusters, r.step, sizeof(r.step));
     return true;

@@ -445,7 +445,7 @@ cudaError_t od_sample_prepare_device(int32_t *clusters)
     cudaError_t e = prepare_kernels<OD_BF16>();
     if (e == cudaSuccess) e = prepare_kernels<OD_F32>();
     if (e != cudaSuccess) return e;
-    for (int level = 0; clusters && level < OD_SAMPLE_LEVELS; ++level)
+    for (int level = 0; level < OD_SAMPLE_LEVELS; ++level)
         clusters[level] = resident_clusters(od_sample_kernel<OD_BF16, true, STAGED>, od_sample_parts(level), 64 * 1024);
     return cudaSuccess;
 }

@@ -442,13 +442,13 @@ cudaError_t launch_step(int source, int parts, size_t smem, cudaStream_t s, bool
 
 }  // namespace
 
-// clusters: [levels] resident at a time with a multiprocessor to every block (null: not asked)
+// clusters: [levels] resident at a time with a multiprocessor to every block
 cudaError_t od_step_prepare_device(int32_t *clusters)
 {
     cudaError_t e = allow_all<OD_BF16>();
     if (e == cudaSuccess) e = allow_all<OD_F32>();
     if (e != cudaSuccess) return e;
-    for (int level = 0; clusters && level < OD_SAMPLE_LEVELS; ++level)
+    for (int level = 0; level < OD_SAMPLE_LEVELS; ++level)
         clusters[level] = resident_clusters(od_step_kernel<OD_BF16, STAGED>, od_sample_parts(level), 64 * 1024);
     return cudaSuccess;
 }
