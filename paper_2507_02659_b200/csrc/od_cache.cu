@@ -851,7 +851,6 @@ int32_t od_cache_insert(od_ctx *c, int32_t N, const int32_t *runs, const int32_t
     Guard g(c->device);
     if (!g.ok) return OD_ERR_CUDA;
     cudaStream_t s = (cudaStream_t)stream;
-    c->last_was_map = false;
     c->table_written = true;
     const int threads = 128, blocks = (N + threads - 1) / threads;
     const bool pdl = c->opt_pdl != 0;
@@ -872,7 +871,6 @@ int32_t od_cache_trim(od_ctx *c, void *stream)
     Guard g(c->device);
     if (!g.ok) return OD_ERR_CUDA;
     cudaStream_t s = (cudaStream_t)stream;
-    c->last_was_map = false;
     c->table_written = true;
     TrimState *st = (TrimState *)c->d_trim;
     // What is resident at a time, and no more blocks than have anything to do (4 or 5 to a multiprocessor: the pass

@@ -87,9 +87,11 @@ struct od_ctx {
     bool verify_early;
     bool table_written;             // a kernel that writes the n-gram table was launched since the last translation kernel
 
-    // the last launch on this context was the translation kernel, which lets the next
-    // kernel start before its own outputs exist (see od_sample.cu)
-    bool last_was_map;
+    // The last launch on this context that a draw's inputs depend on was a verification's, which let the next kernel
+    // start only after the translation was complete: the draw behind it may read the translation's outputs before
+    // griddepcontrol.wait. Not behind a translation, nor behind a fetch of rows that the draw reads, nor behind
+    // anything the library did not launch itself for this step.
+    bool translation_complete;
 
     // last launch info
     int64_t info[4];

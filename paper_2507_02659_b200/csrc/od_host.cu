@@ -96,7 +96,6 @@ bool od_host_rows_readable(const void *logits, size_t logits_bytes, const void *
 
 cudaError_t od_launch_fetch_logits(od_ctx *c, int32_t B, int32_t K_max, const char *src, size_t row_bytes, cudaStream_t s)
 {
-    c->last_was_map = false;
     const unsigned pieces = (unsigned)((row_bytes + FETCH_BYTES - 1) / FETCH_BYTES);
     fetch_logits_kernel<<<dim3(pieces, (unsigned)K_max + 1, (unsigned)B), FETCH_THREADS, 0, s>>>((char *)c->s_logits, src, (int64_t)row_bytes,
                                                                                          K_max, c->s_m);
@@ -105,6 +104,7 @@ cudaError_t od_launch_fetch_logits(od_ctx *c, int32_t B, int32_t K_max, const ch
 
 cudaError_t od_launch_fetch_drafter(od_ctx *c, int32_t B, int32_t K_max, const char *src, cudaStream_t s)
 {
+    c->translation_complete = false;                        // the draw behind this launch waits for it before it reads anything
     const int64_t row_bytes = (int64_t)c->v_q * 4;
     const unsigned pieces = (unsigned)((row_bytes + FETCH_BYTES - 1) / FETCH_BYTES);
     fetch_drafter_kernel<<<dim3(pieces, (unsigned)B), FETCH_THREADS, 0, s>>>((char *)c->s_q_rows, src, row_bytes, K_max, c->s_m, c->s_tail,

@@ -90,7 +90,7 @@ cudaError_t od_launch_map(od_ctx *c, int32_t B, int32_t K_max, const int32_t *dr
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = c->opt_pdl ? 1 : 0;
-    c->last_was_map = true;
+    c->translation_complete = false;
     // A kernel that writes the table (insert, trim) may be the launch in front of this one: then
     // the probes stay behind the wait. A translation kernel releases its successor after its
     // wait, or (inside od_step) that successor is the streaming pass, which does: either way

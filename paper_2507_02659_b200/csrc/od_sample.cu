@@ -94,7 +94,7 @@ od_sample_kernel(const SampleArgs a)
 
     // Under programmatic dependent launch this grid is resident while the verification
     // kernels still run. What the translation kernel wrote (it finished before them) is
-    // read now. (a.early = 0: the launch before this one was not od_verify; everything waits.)
+    // read now. (a.early = 0: no verification is in front of this launch; everything waits.)
     asm volatile("griddepcontrol.launch_dependents;");
     if (!a.early) asm volatile("griddepcontrol.wait;" ::: "memory");
     const int32_t map_serial = SOURCE == FROM_ROW ? __ldg(a.map_serial_now) : a.map_serial;
@@ -511,16 +511,14 @@ static cudaError_t launch_sample(od_ctx *c, int mode, int32_t B, int32_t K_max, 
     context_args(c, a);
     a.tile_lo = tile_lo; a.tile_hi = tile_hi; a.col0 = mode == 0 ? 0 : shard_lo;
     a.n_shards = n_shards; a.shard_index = shard_index; a.mass_all = mass_all; a.mass_out = mass_out;
-    // the translation kernel releases its successor before it has written anything: directly
-    // after it, nothing may be read early
-    a.early = c->last_was_map ? 0 : 1;
+    a.early = c->translation_complete ? 1 : 0;
     if (fuse) {
         a.plan.W = fuse->W; a.plan.n_chunks = fuse->n_chunks; a.plan.span_min = fuse->span_min;
         a.plan.span_a = fuse->span_a; a.plan.seg_warps = fuse->seg_warps; a.plan.partials = c->d_partials;
         a.w_row_max = fuse->row_max; a.w_row_sum = fuse->row_sum; a.w_p_sel = fuse->p_sel; a.w_ratio = fuse->ratio;
         a.w_n_accepted = fuse->n_accepted; a.w_n_draft = fuse->n_draft_accepted; a.w_vflags = fuse->flags;
     }
-    c->last_was_map = false;
+    if (mode != 1) c->translation_complete = false;         // of this step; the next one has its own
     const DrawPlan plan = mode == 0 ? plan_draw(c, level, a) : DrawPlan{};
     if (mode != 2) {
         c->info[2] = (int64_t)blocks_x * B;

@@ -487,7 +487,7 @@ cudaError_t od_launch_step(od_ctx *c, int32_t B, int32_t K_max, const int32_t *d
     const DrawPlan plan = plan_draw(c, level, a);
     cut_rows(level, dtype, a);
     c->table_written = false;
-    c->last_was_map = true;                                 // (it releases the next launch before it has written anything)
+    c->translation_complete = false;                        // (it releases the next launch before it has written anything)
     const int parts = od_sample_parts(level);
     c->info[0] = (int64_t)parts * B; c->info[1] = a.part_units;
     c->info[2] = (int64_t)parts * B; c->info[3] = a.tiles_per_warp;
@@ -511,7 +511,7 @@ cudaError_t od_launch_verify_rows(od_ctx *c, int32_t B, int32_t K_max, const voi
     a.w_n_accepted = out->n_accepted; a.w_n_draft = out->n_draft_accepted; a.w_vflags = out->flags;
     a.inputs_early = early && c->opt_pdl != 0;
     cut_rows(level, dtype, a);
-    c->last_was_map = false;
+    c->translation_complete = true;
     const int parts = od_sample_parts(level);
     c->info[0] = (int64_t)parts * B; c->info[1] = a.part_units;
     const bool pdl = c->opt_pdl != 0;
@@ -532,7 +532,7 @@ cudaError_t od_launch_shard_rows(od_ctx *c, int32_t B, int32_t K_max, int32_t sh
     a.stats = (float4 *)stats;
     a.inputs_early = early && c->opt_pdl != 0;
     cut_rows(level, dtype, a);
-    c->last_was_map = false;
+    c->translation_complete = true;
     const int parts = od_sample_parts(level);
     c->info[0] = (int64_t)parts * B; c->info[1] = a.part_units;
     const bool pdl = c->opt_pdl != 0;

@@ -573,7 +573,7 @@ cudaError_t od_launch_verify_stream(od_ctx *c, int32_t B, int32_t K_max, const v
                                     int64_t row_stride, int64_t seq_stride, const int32_t *m,
                                     const float *temperature, od_fused_verify *plan, cudaStream_t s)
 {
-    c->last_was_map = false;
+    c->translation_complete = true;
     VerifyArgs a = {};
     plan_stream(c, B, K_max, c->v_p, dtype, c->verify_early, a);
     a.logits = logits; a.row_stride = row_stride; a.seq_stride = seq_stride;
@@ -599,7 +599,7 @@ cudaError_t od_launch_verify(od_ctx *c, int32_t B, int32_t K_max, const void *lo
 {
     const int64_t esz = dtype == OD_BF16 ? 2 : 4;
     const int32_t slice = slice_of(K_max, c->v_p, dtype);
-    c->last_was_map = false;
+    c->translation_complete = true;
     for (int32_t b0 = 0; b0 < B; b0 += slice) {
         const int32_t nb = B - b0 < slice ? B - b0 : slice;
         VerifyArgs a = {};
@@ -641,7 +641,7 @@ cudaError_t od_launch_verify_shard_stats(od_ctx *c, int32_t B, int32_t K_max, in
 {
     const int64_t esz = dtype == OD_BF16 ? 2 : 4;
     const int32_t slice = slice_of(K_max, shard_len, dtype);
-    c->last_was_map = false;
+    c->translation_complete = true;
     for (int32_t b0 = 0; b0 < B; b0 += slice) {
         const int32_t nb = B - b0 < slice ? B - b0 : slice;
         VerifyArgs a = {};
@@ -678,7 +678,7 @@ cudaError_t od_launch_verify_shard_finish(od_ctx *c, int32_t B, int32_t K_max, i
                                           int32_t *n_accepted, int32_t *n_draft_accepted, uint32_t *flags,
                                           cudaStream_t s)
 {
-    c->last_was_map = false;
+    c->translation_complete = true;
     if (B == 0) return cudaSuccess;
     VerifyArgs a = {};
     a.B = B; a.K_max = K_max; a.v_p = c->v_p;

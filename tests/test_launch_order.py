@@ -1,0 +1,154 @@
+"""Which kernels the library launches, in which order and with what they may read before the launch in front of
+them is done: the host code on a CUDA runtime that runs nothing (tests/helpers/fake_cudart.cu)."""
+import ctypes as C
+
+import numpy as np
+import pytest
+
+import helpers
+
+V_Q, V_P, B, K = 1000, 4000, 40, 4
+
+
+def _aligned(n):
+    raw = np.zeros(n + 64, np.uint8)
+    at = -raw.ctypes.data % 64
+    return raw[at:at + n]
+
+
+class Lib:
+    """One context of the library on the fake runtime. Every array is zeros, or what a call was given."""
+
+    def __init__(self, v_q=V_Q, v_p=V_P, max_batch=B, k=K, vocab_map=None):
+        self.L, self.k, self.v_q, self.v_p, self.kept = helpers.fake_runtime_lib(), k, v_q, v_p, []
+        self.L.fake_unpin_all()
+        self.L.fake_no_driver_functions(0)
+        h = C.c_void_p()
+        self.call("od_create", C.byref(h), 0, v_q, v_p, max_batch, k)
+        self.ctx = h
+        if vocab_map is None:
+            vocab_map = np.where(np.arange(v_q) % 10 < 7, np.arange(v_q) + 1, -1)
+        self.call("od_set_vocab_map", h, self.array(vocab_map.astype(np.int32)))
+        self.call("od_cache_build", h, None, None, None, C.c_int64(0))
+        self.log()
+
+    def close(self):
+        self.call("od_destroy", self.ctx)
+
+    def call(self, name, *args):
+        assert getattr(self.L, name)(*args) == 0, name
+
+    def array(self, a):
+        b = _aligned(a.nbytes).view(a.dtype)[:a.size]
+        b[:] = a.ravel()
+        self.kept.append(b)
+        return C.c_void_p(b.ctypes.data)
+
+    def zeros(self, n, dtype=np.int32):
+        return self.array(np.zeros(n, dtype))
+
+    def log(self):
+        """(kernel, grid, early) of every launch, (direction, bytes) of every copy, since the last call."""
+        out = []
+        for line in self.L.fake_log().decode().splitlines():
+            w = line.split()
+            out.append((w[0], tuple(map(int, w[1:4])), int(w[4])) if len(w) == 5 else (w[0], int(w[1])))
+        return out
+
+    def early(self, *kernels):
+        """The launches' names and their `early`, copies left out."""
+        return [(x[0], x[2]) for x in self.log() if len(x) == 3 and (not kernels or x[0] in kernels)]
+
+    def inputs(self, n=B):
+        """Pointers that the calls below share: outputs and inputs of a step for n sequences."""
+        K, z = self.k, self.zeros
+        self.n = n
+        names = dict(draft_ids=n * K, draft_len=n, q_sel=n * K, temperature=n, seed=2 * n, tgt_ids=n * K, q_prime=n * K,
+                     span_start=n * K, span_len=n * K, m=n, tail=n, row_max=n * (K + 1), row_sum=n * (K + 1), p_sel=n * K,
+                     ratio=n * K, n_acc=n, n_draft=n, vflags=n, token=n, mass=n, sflags=n, counters=8)
+        self.p = {name: z(count) for name, count in names.items()}
+        self.p["q_rows"] = z(n * K * self.v_q)
+        self.p["logits"] = z(n * (K + 1) * self.v_p, np.uint16)
+        return self.p
+
+    def strides(self):
+        return C.c_int64(self.v_p), C.c_int64(self.v_p * (self.k + 1))
+
+    def map(self):
+        p = self.p
+        self.call("od_map_proposals", self.ctx, self.n, self.k, p["draft_ids"], p["draft_len"], p["q_sel"], p["tgt_ids"], p["q_prime"],
+                  p["span_start"], p["span_len"], p["m"], p["tail"], p["counters"], None)
+
+    def verify(self):
+        p = self.p
+        self.call("od_verify", self.ctx, self.n, self.k, p["logits"], 1, *self.strides(), p["tgt_ids"], p["q_prime"], p["span_len"], p["m"],
+                  p["temperature"], p["seed"], C.c_uint64(0), p["row_max"], p["row_sum"], p["p_sel"], p["ratio"], p["n_acc"],
+                  p["n_draft"], p["vflags"], None)
+
+    def sample(self):
+        p = self.p
+        self.call("od_sample_residual", self.ctx, self.n, self.k, p["logits"], 1, *self.strides(), p["row_max"], p["row_sum"], p["q_rows"],
+                  p["draft_ids"], p["tgt_ids"], p["q_prime"], p["span_start"], p["span_len"], p["m"], p["tail"], p["n_acc"],
+                  p["temperature"], p["seed"], C.c_uint64(0), p["token"], p["mass"], p["sflags"], None)
+
+    def step(self):
+        p = self.p
+        self.call("od_step", self.ctx, self.n, self.k, p["draft_ids"], p["draft_len"], p["q_sel"], p["q_rows"], p["logits"], 1,
+                  *self.strides(), p["temperature"], p["seed"], C.c_uint64(0), p["tgt_ids"], p["q_prime"], p["span_start"],
+                  p["span_len"], p["m"], p["tail"], p["counters"], p["row_max"], p["row_sum"], p["p_sel"], p["ratio"], p["n_acc"],
+                  p["n_draft"], p["vflags"], p["token"], p["mass"], p["sflags"], None)
+
+    def step_host(self):
+        p = self.p
+        self.call("od_step_host", self.ctx, self.n, self.k, p["draft_ids"], p["draft_len"], p["q_sel"], p["q_rows"], p["logits"], 1,
+                  p["temperature"], p["seed"], C.c_uint64(0), p["n_acc"], p["n_draft"], p["token"], p["tgt_ids"], p["m"],
+                  p["vflags"], p["sflags"], None)
+
+    def pin(self, name, bytes_=None):
+        a = next(a for a in self.kept if a.ctypes.data == self.p[name].value)
+        self.L.fake_pin(a.ctypes.data, a.nbytes if bytes_ is None else bytes_)
+
+
+@pytest.fixture
+def lib():
+    made = []
+
+    def make(**kw):
+        made.append(Lib(**kw))
+        return made[-1]
+    yield make
+    for x in made:
+        x.close()
+
+
+# ---- what the sampler may read ahead: the translation's outputs, where the launch in front let it start only after
+# the translation was complete
+
+@pytest.mark.parametrize("pinned", [True, False])
+@pytest.mark.parametrize("grid", [0, 100])
+def test_the_draw_from_host_buffers_reads_nothing_ahead_of_the_rows_that_are_fetched(lib, pinned, grid):
+    c = lib()
+    c.inputs()
+    c.call("od_set_option", c.ctx, b"verify_grid", C.c_int64(grid))
+    c.call("od_host_step_reserve", c.ctx, 1)
+    if pinned:
+        c.pin("logits"); c.pin("q_rows")
+    c.step_host()
+    step2 = [("od_verify_stream_kernel", -1), ("od_verify_decide_kernel", -1)] if grid else [("od_verify_rows_kernel", -1)]
+    fetch = lambda name: [(name, -1)] if pinned else []
+    assert c.early() == ([("od_map_kernel", 0)] + fetch("fetch_logits_kernel") + step2 + fetch("fetch_drafter_kernel") +
+                         [("od_sample_kernel", 0 if pinned else 1)])
+
+
+@pytest.mark.parametrize("calls,early", [("sample", [0]), ("map sample", [0]), ("map verify sample", [1]), ("map verify sample sample", [1, 0]),
+                                         ("map verify map sample", [0]), ("step sample", [0]), ("map verify step sample", [0])])
+@pytest.mark.parametrize("n", [1, B])
+def test_a_draw_reads_the_translation_ahead_only_behind_a_verification(lib, calls, early, n):
+    c = lib()
+    c.inputs(n)
+    c.call("od_set_option", c.ctx, b"early_inputs", C.c_int64(0))
+    for name in calls.split():
+        getattr(c, name)()
+    seen = c.early("od_sample_kernel", "od_step_kernel")
+    assert [e for k, e in seen if k == "od_sample_kernel"] == early
+    assert ("od_step_kernel" in [k for k, _ in seen]) == ("step" in calls)
