@@ -42,7 +42,9 @@
  *     translation kernel is the launch in front of the streaming kernel and has
  *     itself waited for everything earlier in the stream before letting it
  *     start (logits and temperatures, by the streaming kernel; where od_step is
- *     one launch it reads nothing of the caller's early); and when the
+ *     one launch it reads nothing of the caller's early; what the calls of one
+ *     step have read already, its temperatures and draft ids, the later calls may
+ *     read early again, the drafter's distributions they may not); and when the
  *     caller has set option "early_inputs" = 1, which is the caller's promise
  *     that the inputs of a call were complete before the launch that precedes
  *     the call was enqueued (a producer two launches back, or data resident

@@ -538,7 +538,7 @@ struct Ahead {
 __device__ __forceinline__ void prepare_positions(const SampleArgs &a, Ahead &h, int b, int lane, int s0, int32_t d1)
 {
     const int K = a.K_max;
-    h.s0 = 0; h.len = 1; h.tgt = -1; h.d1 = -1; h.pm = -1; h.qp = 0.f; h.qd1 = 0.f;
+    h.s0 = 0; h.len = 1; h.tgt = -1; h.d1 = -1; h.pm = -1; h.qp = 0.f;
     if (lane < K && lane <= h.mb) {
         h.s0 = s0;
         h.len = lane < h.mb ? h.l_len : 1;
@@ -549,9 +549,15 @@ __device__ __forceinline__ void prepare_positions(const SampleArgs &a, Ahead &h,
         if (d1 >= 0 && d1 < a.v_q) {
             h.d1 = d1;
             h.pm = __ldg(a.vocab_map + d1);
-            h.qd1 = __ldg(a.q_rows + ((size_t)b * K + h.s0) * a.v_q + d1);
         }
     }
+}
+// Its probability, from the drafter's row. The rows are the first thing of the caller's that a draw alone reads: whatever
+// is directly in front of it may write them, so this is behind griddepcontrol.wait. (With the loads of the rows'
+// statistics, which wait as well, it costs no trip of its own.)
+__device__ __forceinline__ void load_first_probability(const SampleArgs &a, Ahead &h, int b)
+{
+    h.qd1 = h.d1 >= 0 ? __ldg(a.q_rows + ((size_t)b * a.K_max + h.s0) * a.v_q + h.d1) : 0.f;
 }
 __device__ __forceinline__ Ahead load_ahead(const SampleArgs &a, int b, int lane)
 {

@@ -98,7 +98,8 @@ od_sample_kernel(const SampleArgs a)
     asm volatile("griddepcontrol.launch_dependents;");
     if (!a.early) asm volatile("griddepcontrol.wait;" ::: "memory");
     const int32_t map_serial = SOURCE == FROM_ROW ? __ldg(a.map_serial_now) : a.map_serial;
-    const Ahead h = load_ahead(a, b, lane);
+    Ahead h = load_ahead(a, b, lane);
+    if (FUSED) load_first_probability(a, h, b);             // (the step's inputs were complete before its translation)
     const int mb = h.mb;
 
     // FUSED, still before the wait: where the rows' partials will be (sums of m), and position
@@ -136,6 +137,7 @@ od_sample_kernel(const SampleArgs a)
 
     // n_accepted and the row statistics come from the verification kernels
     if (a.early) asm volatile("griddepcontrol.wait;" ::: "memory");
+    if (!FUSED) load_first_probability(a, h, b);
 
     int j = 0;
     float rm = 0.f, rs = 0.f;                      // lane k: statistics of row k
@@ -195,7 +197,7 @@ od_sample_shard_kernel(const SampleArgs a)
 
     asm volatile("griddepcontrol.launch_dependents;");
     if (!a.early) asm volatile("griddepcontrol.wait;" ::: "memory");
-    const Ahead h = load_ahead(a, b, lane);
+    Ahead h = load_ahead(a, b, lane);
     const int mb = h.mb;
     const float T = h.T;
     const bool planned = __ldg(a.map_serial_now) == a.map_serial;   // (as in od_sample_kernel)
@@ -212,6 +214,7 @@ od_sample_shard_kernel(const SampleArgs a)
 
     // n_accepted and the row statistics come from the verification kernels
     if (a.early) asm volatile("griddepcontrol.wait;" ::: "memory");
+    load_first_probability(a, h, b);
 
     if (!(T > 0.f)) {                              // every block of the sequence leaves here
         if (part == 0 && threadIdx.x == 0) {

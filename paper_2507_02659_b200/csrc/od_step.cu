@@ -271,6 +271,7 @@ od_step_kernel(const __grid_constant__ StepArgs a)
     rows_from_one<DTYPE>(a, slice, b, mb, warp, lane, scale, s_rec);
     // (what the draw starts with travels during the exchange)
     prepare_positions(a, h, b, lane, w.start, w.first_id);
+    load_first_probability(a, h, b);
     Part<SOURCE> mine;
     mine.prepare(a, (int)part, warp, lane);
     float rm, rs;
