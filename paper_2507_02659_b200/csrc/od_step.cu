@@ -221,11 +221,10 @@ od_step_kernel(const __grid_constant__ StepArgs a)
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     float *s_q = (float *)s_dyn, *s_val = s_q + (SOURCE == STAGED ? a.slots : 0) + warp * a.tiles_per_warp;
 
-    // Under the caller's promise (inputs_early) everything but the writes runs before the wait. The next
-    // launch is released before it only where this one reads the n-gram table before it as well: a later launch
-    // may then find the table as this one did (see od_launch_map).
+    // Under the caller's promise (inputs_early) everything but the writes runs before the wait (the table's lookups
+    // where no writer of it may be at work). The next launch is released behind the wait all the same: it may be a
+    // step that reads its own inputs early, and the promise is that what is two launches back is complete.
     const bool all_early = a.inputs_early && a.table_early;
-    if (all_early) release_next();
     const int32_t map_serial = SOURCE == FROM_ROW ? __ldg(a.map_serial_now) : a.map_serial;
     if (threadIdx.x == 0) s_bad = 0;
     od_cluster_arrive_relaxed();                            // this block runs: the others may store to it
@@ -276,7 +275,7 @@ od_step_kernel(const __grid_constant__ StepArgs a)
     mine.prepare(a, (int)part, warp, lane);
     float rm, rs;
     exchange_rows(slice, mb, part, nparts, warp, lane, scale, s_rec, s_all, s_M, s_S, &s_bad, rm, rs);
-    if (all_early) wait_for_earlier();                      // nothing has been written yet
+    if (all_early) { wait_for_earlier(); release_next(); }  // nothing has been written yet
     const bool writes = part == 0 && warp == 0;
     if (writes) {
         store_walk(a.out, w, b, K, a.v_q, lane);

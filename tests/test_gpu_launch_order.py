@@ -62,3 +62,37 @@ def test_the_drafters_rows_may_be_written_directly_in_front_of_the_draw(cuda_dev
         for a, b in zip(want, got):
             assert torch.equal(a, b)
     ctx.close()
+
+
+@pytest.mark.parametrize("late", ["logits", "draft_ids", "q_rows"])
+@pytest.mark.parametrize("between", [1, 3])
+def test_inputs_written_two_launches_back_are_complete(cuda_device, late, between):
+    """Under early_inputs a step reads its inputs while the launch in front of it runs: that launch must not have let it
+    start before the producer in front of itself was done."""
+    w = _workload(B=2, k_max=3)
+    st = synth.make_static(w)
+    ctx = parity.make_context(w, st, cuda_device)
+    first, s = (synth.make_step(w, st, i, device=cuda_device) for i in range(2))
+
+    def step(x, **kw):
+        return od.od_step(ctx, *(kw.get(n, getattr(x, n)) for n in ("draft_ids", "draft_len", "q_sel", "q_rows", "logits", "temperature", "seed")), x.step)
+    flat = lambda out: [t.clone() for o, names in zip(out, (("m", "tail_kind"), ("n_accepted", "n_draft_accepted", "flags"), ("out_token", "resid_mass", "flags")))
+                        for t in (getattr(o, n) for n in names)]
+    src = getattr(s, late)
+    n = src.numel() + -src.numel() % 8                      # (whole 16-byte pieces)
+    padded, dst = torch.zeros(n, dtype=src.dtype, device=cuda_device), torch.zeros(n, dtype=src.dtype, device=cuda_device)
+    padded[:src.numel()] = src.flatten()
+    view = dst[:src.numel()].view(src.shape)
+    want = flat(step(s))
+    ctx.set_option("early_inputs", 1)
+    for _ in range(4):
+        dst.fill_(1 if late == "draft_ids" else float("nan"))
+        torch.cuda.synchronize()
+        _produce(dst, padded)
+        for _ in range(between):
+            step(first)
+        got = flat(step(s, **{late: view}))
+        torch.cuda.synchronize()
+        for a, b in zip(want, got):
+            assert torch.equal(a, b)
+    ctx.close()
