@@ -104,11 +104,14 @@ __device__ __forceinline__ unsigned int digit_of(int pass, unsigned long long hi
 
 // The kernels of an insertion and of a trim form chains in which each needs what the one
 // before it wrote. They are launched with programmatic stream serialization and wait at once:
-// the launch latency of a kernel is spent while its predecessor still runs.
-__device__ __forceinline__ void chain_wait()
+// the launch latency of a kernel is spent while its predecessor still runs. The first kernel of a chain releases the
+// next behind its wait: what runs behind the chain may read its inputs early, and is promised that what was in front of
+// the chain is done.
+__device__ __forceinline__ void chain_wait(bool first = false)
 {
-    asm volatile("griddepcontrol.launch_dependents;");
+    if (!first) asm volatile("griddepcontrol.launch_dependents;");
     asm volatile("griddepcontrol.wait;" ::: "memory");
+    if (first) asm volatile("griddepcontrol.launch_dependents;");
 }
 
 // launch with or without programmatic stream serialization (the context's "pdl" option)
@@ -130,7 +133,7 @@ __global__ void insert_claim_kernel(int32_t N, int32_t v_q, int32_t v_p, const i
                                     unsigned long long *keys, const int32_t *vals, int64_t cap,
                                     unsigned int *owner, int32_t *cand_slot, TrimState *st)
 {
-    chain_wait();
+    chain_wait(true);
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= N) return;
     cand_slot[i] = -1;
@@ -208,7 +211,7 @@ __device__ __forceinline__ void reset_live(TrimState::Live &l) { l.n = 0u; l.hi_
 
 __global__ void trim_begin_kernel(TrimState *st, unsigned int max_entries)
 {
-    chain_wait();
+    chain_wait(true);
     const unsigned int k = st->size > max_entries ? st->size - max_entries : 0u;
     if (threadIdx.x == 0) {
         st->k = k;
@@ -256,7 +259,7 @@ __global__ void trim_compact_kernel(int policy, unsigned int clock, const unsign
     __shared__ unsigned int s_warp[32];
     __shared__ unsigned int s_base;
     __shared__ unsigned long long s_and, s_or;
-    chain_wait();
+    chain_wait(true);
     const TrimLists L = trim_lists(lists, cap);
     if (threadIdx.x == 0) { s_and = ~0ull; s_or = 0ull; }
     unsigned long long t_and = ~0ull, t_or = 0ull;

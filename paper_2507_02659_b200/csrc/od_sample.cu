@@ -95,7 +95,9 @@ od_sample_kernel(const SampleArgs a)
     // Under programmatic dependent launch this grid is resident while the verification
     // kernels still run. What the translation kernel wrote (it finished before them) is
     // read now. (a.early = 0: no verification is in front of this launch; everything waits.)
-    asm volatile("griddepcontrol.launch_dependents;");
+    // Inside od_step the next launch is released at once (the streaming pass in front has waited). A call of its own
+    // releases behind its wait: the launch in front may be anything, and what is behind may read its inputs early.
+    if (FUSED) asm volatile("griddepcontrol.launch_dependents;");
     if (!a.early) asm volatile("griddepcontrol.wait;" ::: "memory");
     const int32_t map_serial = SOURCE == FROM_ROW ? __ldg(a.map_serial_now) : a.map_serial;
     Ahead h = load_ahead(a, b, lane);
@@ -137,6 +139,7 @@ od_sample_kernel(const SampleArgs a)
 
     // n_accepted and the row statistics come from the verification kernels
     if (a.early) asm volatile("griddepcontrol.wait;" ::: "memory");
+    if (!FUSED) asm volatile("griddepcontrol.launch_dependents;");
     if (!FUSED) load_first_probability(a, h, b);
 
     int j = 0;
@@ -195,7 +198,6 @@ od_sample_shard_kernel(const SampleArgs a)
     const int K = a.K_max;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 
-    asm volatile("griddepcontrol.launch_dependents;");
     if (!a.early) asm volatile("griddepcontrol.wait;" ::: "memory");
     Ahead h = load_ahead(a, b, lane);
     const int mb = h.mb;
@@ -214,6 +216,7 @@ od_sample_shard_kernel(const SampleArgs a)
 
     // n_accepted and the row statistics come from the verification kernels
     if (a.early) asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;");      // (behind the wait, as in od_sample_kernel)
     load_first_probability(a, h, b);
 
     if (!(T > 0.f)) {                              // every block of the sequence leaves here

@@ -96,3 +96,54 @@ def test_inputs_written_two_launches_back_are_complete(cuda_device, late, betwee
         for a, b in zip(want, got):
             assert torch.equal(a, b)
     ctx.close()
+
+
+@pytest.mark.parametrize("call", ["map", "verify", "noalloc", "sample", "stats", "finish", "mass", "pick", "distill", "exit", "insert", "trim"])
+def test_no_call_lets_the_next_one_start_before_its_own_wait(cuda_device, call):
+    """The same with each other call in between: a translation behind it reads its proposal early."""
+    w = _workload(B=2, k_max=3)
+    st = synth.make_static(w)
+    ctx = parity.make_context(w, st, cuda_device)
+    ctx.cache_configure(1000, 0, len(st.runs))              # nothing is evicted
+    dev = lambda x: torch.as_tensor(np.ascontiguousarray(x), dtype=torch.int32, device=cuda_device)
+    cached = [dev(x) for x in (st.runs, st.run_len, st.run_target)]
+    ctx.cache_set_clock(1)
+    ctx.cache_insert(*cached)
+    a, s = (synth.make_step(w, st, i, device=cuda_device) for i in range(2))
+    mp = od.od_map_proposals(ctx, a.draft_ids, a.draft_len, a.q_sel)
+    vo = od.od_verify(ctx, a.logits, mp, a.temperature, a.seed, 0)
+    shard = (0, a.logits)
+    stats = od.od_verify_shard_stats(ctx, *shard, mp, a.temperature)[None]
+    mass = od.od_sample_shard_mass(ctx, *shard, vo, a.q_rows, a.draft_ids, mp, a.temperature)[None]
+    vo2 = od.alloc_verify_out(ctx, w.B, w.k_max)
+    head = torch.zeros(w.B, w.k_max, device=cuda_device)
+    calls = {
+        "map": lambda: od.od_map_proposals(ctx, a.draft_ids, a.draft_len, a.q_sel),
+        "verify": lambda: od.od_verify(ctx, a.logits, mp, a.temperature, a.seed, 0, out=vo2),
+        "noalloc": lambda: od.od_verify_noalloc(w.v_p, a.logits, mp, a.temperature, a.seed, 0, vo2),
+        "sample": lambda: od.od_sample_residual(ctx, a.logits, vo, a.q_rows, a.draft_ids, mp, a.temperature, a.seed, 0),
+        "stats": lambda: od.od_verify_shard_stats(ctx, *shard, mp, a.temperature),
+        "finish": lambda: od.od_verify_shard_finish(ctx, stats, mp, a.temperature, a.seed, 0),
+        "mass": lambda: od.od_sample_shard_mass(ctx, *shard, vo, a.q_rows, a.draft_ids, mp, a.temperature),
+        "pick": lambda: od.od_sample_shard_pick(ctx, 0, 0, mass, a.logits, vo, a.q_rows, a.draft_ids, mp, a.temperature, a.seed, 0),
+        "distill": lambda: od.od_distill_loss(ctx, a.q_rows, a.draft_ids, mp, a.logits, vo, a.temperature, 0.2, 0),
+        "exit": lambda: od.od_exit_rule(ctx, head, None, 0.5),
+        "insert": lambda: ctx.cache_insert(*cached),
+        "trim": lambda: ctx.cache_trim(),
+    }
+    want = od.od_map_proposals(ctx, s.draft_ids, s.draft_len, s.q_sel)
+    source = torch.zeros(s.draft_ids.numel() + -s.draft_ids.numel() % 4, dtype=torch.int32, device=cuda_device)
+    late = torch.zeros_like(source)
+    source[:s.draft_ids.numel()] = s.draft_ids.flatten()
+    ctx.set_option("early_inputs", 1)
+    for _ in range(3):
+        late.fill_(1)
+        torch.cuda.synchronize()
+        _produce(late, source)
+        calls[call]()
+        got = od.od_map_proposals(ctx, late[:s.draft_ids.numel()].view(s.draft_ids.shape), s.draft_len, s.q_sel)
+        torch.cuda.synchronize()
+        assert torch.equal(got.m, want.m) and torch.equal(got.tail_kind, want.tail_kind)
+        for b, m in enumerate(want.m.tolist()):
+            assert torch.equal(got.tgt_ids[b, :m], want.tgt_ids[b, :m]) and torch.equal(got.span_len[b, :m], want.span_len[b, :m])
+    ctx.close()
