@@ -102,6 +102,7 @@ od_sample_kernel(const SampleArgs a)
     const int32_t map_serial = SOURCE == FROM_ROW ? __ldg(a.map_serial_now) : a.map_serial;
     Ahead h = load_ahead(a, b, lane);
     if (FUSED) load_first_probability(a, h, b);             // (the step's inputs were complete before its translation)
+    else request_first_probability(a, h, b);
     const int mb = h.mb;
 
     // FUSED, still before the wait: where the rows' partials will be (sums of m), and position
@@ -200,6 +201,7 @@ od_sample_shard_kernel(const SampleArgs a)
 
     if (!a.early) asm volatile("griddepcontrol.wait;" ::: "memory");
     Ahead h = load_ahead(a, b, lane);
+    request_first_probability(a, h, b);
     const int mb = h.mb;
     const float T = h.T;
     const bool planned = __ldg(a.map_serial_now) == a.map_serial;   // (as in od_sample_kernel)
