@@ -457,7 +457,7 @@ od_verify_finish_kernel(const VerifyArgs a)
     const float T = a.temperature[b];
     const bool bad_T = !(T > 0.f);
     const float scale = bad_T ? 0.f : 1.4426950408889634f / T;
-    float q = 0.f, u = 0.f;
+    float q = 0.f;
     bool t_ok = false;
     int32_t my_span = 0;
     if (r == 0 && lane < mb) my_span = a.span_len[(size_t)b * a.K_max + lane];
@@ -466,12 +466,13 @@ od_verify_finish_kernel(const VerifyArgs a)
         const int32_t t = a.tgt_ids[o];
         t_ok = t >= 0 && t < a.v_p;
         q = a.q_prime[o];
-        u = od_uniform(a.seed[b], a.step, (uint32_t)r, 0u);
     }
     __syncthreads();
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;");
     if (r <= mb) {
+        // (the seeds are what no earlier call of the step has read: a launch directly in front may write them)
+        const uint64_t seed = lane == 0 && r < mb ? a.seed[b] : 0ull;
         const int row_slot = b * (a.K_max + 1) + r;
         float c = -FLT_MAX, s = 0.f, mx = -INFINITY, x_t = -INFINITY;
         for (int k = lane; k < a.n_shards; k += 32) {
@@ -483,6 +484,7 @@ od_verify_finish_kernel(const VerifyArgs a)
 #pragma unroll
         for (int off = 16; off > 0; off >>= 1) x_t = fmaxf(x_t, __shfl_xor_sync(0xFFFFFFFFu, x_t, off));
         warp_merge(c, s, mx);
+        const float u = od_uniform(seed, a.step, (uint32_t)r, 0u);
         if (lane == 0) decide_row(a, b, r, mb, c, s, mx, scale, t_ok, x_t, q, u, s_bits);
     }
     __syncthreads();

@@ -64,6 +64,31 @@ def test_the_drafters_rows_may_be_written_directly_in_front_of_the_draw(cuda_dev
     ctx.close()
 
 
+def test_the_seeds_may_be_written_directly_in_front_of_the_shards_decisions(cuda_device):
+    """od_verify_shard_finish is the first call of a sharded step that reads them."""
+    w = _workload(B=24)
+    st = synth.make_static(w)
+    ctx = parity.make_context(w, st, cuda_device)
+    s = synth.make_step(w, st, 0, device=cuda_device)
+    mp = od.od_map_proposals(ctx, s.draft_ids, s.draft_len, s.q_sel)
+    stats = od.od_verify_shard_stats(ctx, 0, s.logits, mp, s.temperature)[None]
+    # acceptances that the uniforms decide: a ratio of a half everywhere
+    mp.q_prime.copy_(2 * od.od_verify(ctx, s.logits, mp, s.temperature, s.seed, s.step).p_sel)
+    finish = lambda seed: od.od_verify_shard_finish(ctx, stats, mp, s.temperature, seed, s.step)
+    want, other = finish(s.seed), finish(s.seed + 1)
+    torch.cuda.synchronize()
+    assert not torch.equal(want.flags, other.flags) or not torch.equal(want.n_accepted, other.n_accepted)
+    late = torch.empty_like(s.seed)
+    for _ in range(4):
+        late.copy_(s.seed + 1)
+        torch.cuda.synchronize()
+        _produce(late, s.seed)
+        got = finish(late)
+        torch.cuda.synchronize()
+        assert torch.equal(got.n_accepted, want.n_accepted) and torch.equal(got.flags, want.flags)
+    ctx.close()
+
+
 @pytest.mark.parametrize("late", ["logits", "draft_ids", "q_rows"])
 @pytest.mark.parametrize("between", [1, 3])
 def test_inputs_written_two_launches_back_are_complete(cuda_device, late, between):
