@@ -1040,7 +1040,8 @@ inline int draw_level(const od_ctx *c, int32_t B)
         }
     }
     // staged probabilities of over 100 KB would leave room for one block per multiprocessor
-    while (level < most && !c->map_same_ids && c->sample_slots[level] * 4 > 100 * 1024) ++level;
+    for (int next = level + 1; next <= most && !c->map_same_ids && c->sample_slots[level] * 4 > 100 * 1024; ++next)
+        if (od_sample_parts(next) != 5) level = next;
     return level;
 }
 

@@ -152,3 +152,16 @@ def test_a_draw_reads_the_translation_ahead_only_behind_a_verification(lib, call
     seen = c.early("od_sample_kernel", "od_step_kernel")
     assert [e for k, e in seen if k == "od_sample_kernel"] == early
     assert ("od_step_kernel" in [k for k, _ in seen]) == ("step" in calls)
+
+
+# ---- how many blocks draw for a sequence
+
+@pytest.mark.parametrize("v_p,blocks", [(102400, 4), (128000, 6), (153600, 6), (160000, 8)])
+def test_a_part_with_more_mapped_ids_than_two_blocks_can_stage_is_cut_in_the_samplers_own_steps(lib, v_p, blocks):
+    """Most of the ids of a part mapped: 25600 of them are 100 KB. Five blocks would do for 128000 ids; they are the
+    one-launch step's."""
+    c = lib(v_q=65000, v_p=v_p, max_batch=200, k=1, vocab_map=np.arange(65000, dtype=np.int32) + 1)
+    c.inputs(200)
+    c.map(); c.verify(); c.log()
+    c.sample()
+    assert [x for x in c.log() if x[0] == "od_sample_kernel"] == [("od_sample_kernel", (blocks, 200, 1), 1)]
