@@ -464,8 +464,8 @@ int32_t od_host_step_reserve(od_ctx *ctx, int32_t logit_dtype);
  * the dense ones above (logits [B, K_max+1, target_vocab]). Where logits and
  * q_rows are page-locked (16-byte aligned, each inside one page-locked range) the
  * device reads the rows that the step needs from them: rows 0..m_b of the logits
- * and the one drafter row of a sequence's draw. Of other buffers the rows that the
- * step can read are copied (rows 0..K_b and
+ * and the one drafter row of a sequence's draw. Of other buffers, and of large ones with
+ * one token proposed by every sequence, the rows that the step can read are copied (rows 0..K_b and
  * 0..K_b-1 of sequence b, K_b = draft_len[b] read on the host). Outputs: host
  * int32[B] each for n_accepted, n_draft_accepted, out_token; int32[B,K_max]
  * tgt_ids; int32[B] m; uint32[B] verify_flags and sample_flags (any output may

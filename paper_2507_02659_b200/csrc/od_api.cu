@@ -702,7 +702,8 @@ int32_t od_step_host(od_ctx *c, int32_t B, int32_t K_max, const int32_t *draft_i
     // no kernel looks at.
     const size_t lrow = (size_t)c->v_p * esz, qrow = (size_t)c->v_q * 4;
     const char *d_logits, *d_q_rows;
-    const bool fetched = od_host_rows_readable(logits, nB * (K + 1) * lrow, q_rows, nB * K * qrow, &d_logits, &d_q_rows);
+    const bool fetched = !od_host_better_copied(c, B, K_max, draft_len, lrow, qrow) &&
+                         od_host_rows_readable(logits, nB * (K + 1) * lrow, q_rows, nB * K * qrow, &d_logits, &d_q_rows);
     if (!fetched) {
         size_t l_from = 0, l_bytes = 0, q_from = 0, q_bytes = 0;   // pending runs (byte offsets)
         for (size_t b = 0; b <= nB; ++b) {

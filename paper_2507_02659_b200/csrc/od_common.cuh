@@ -150,7 +150,8 @@ cudaError_t od_launch_verify_rows(od_ctx *c, int32_t B, int32_t K_max, const voi
 cudaError_t od_launch_shard_rows(od_ctx *c, int32_t B, int32_t K_max, int32_t shard_lo, int32_t shard_len, const void *logits,
                                  int32_t dtype, int64_t row_stride, int64_t seq_stride, const int32_t *tgt_ids, const int32_t *m,
                                  const float *temperature, float *stats, bool early, cudaStream_t s);
-// od_step_host (od_host.cu): page-locked buffers that the device reads itself
+// od_step_host (od_host.cu): page-locked buffers that the device reads itself, where that is not slower than copies
+bool od_host_better_copied(const od_ctx *c, int32_t B, int32_t K_max, const int32_t *draft_len, size_t lrow, size_t qrow);
 bool od_host_rows_readable(const void *logits, size_t logits_bytes, const void *q_rows, size_t q_bytes, const char **d_logits,
                            const char **d_q_rows);
 cudaError_t od_launch_fetch_logits(od_ctx *c, int32_t B, int32_t K_max, const char *src, size_t row_bytes, cudaStream_t s);

@@ -5,7 +5,8 @@
 // translation has found m_b, and the ONE drafter row that the draw needs once step 2 has decided where it is,
 // not the K_b rows that the step might have needed. (32 sequences x up to 6 tokens, 128256 bf16 ids: 51 MB in 59
 // copies of about 1 MB, which themselves run at 45 GB/s where one large copy reaches 55; fetched 41 MB: 1278 -> 870 us, 833 on another machine.)
-// Buffers that the device cannot read are copied, rows 0..K_b and 0..K_b-1 of every sequence.
+// Buffers that the device cannot read, and those of which all is likely needed (od_host_better_copied), are copied, rows
+// 0..K_b and 0..K_b-1 of every sequence.
 #include "od_common.cuh"
 
 namespace {
@@ -85,6 +86,19 @@ const char *device_view(const void *p, size_t bytes)
 }
 
 }  // namespace
+
+// One token from every sequence, of another vocabulary and with rows no longer than the target's: all of both buffers is
+// likely needed, and two large copies bring it at 55 GB/s. (128256 bf16 ids, sequences: copied, fetched us: 4: 138, 139;
+// 8: 182, 189; 32: 472, 486; 128: 1595, 1675. fp32 4: 175, 178; 64: 1437, 1527. 64000 bf16 8: 147, 144; 32: 316, 326. With
+// one vocabulary the accepted sequences' drafter rows are not fetched: 32000 fp32 32: 315, 274. Two tokens each: 32
+// sequences of 128256 bf16 ids 690, 638, fp32 1137, 1110.)
+bool od_host_better_copied(const od_ctx *c, int32_t B, int32_t K_max, const int32_t *draft_len, size_t lrow, size_t qrow)
+{
+    if (K_max != 1 || c->map_same_ids || qrow > lrow || (size_t)B * (2 * lrow + qrow) < (size_t)4 << 20) return false;
+    for (int32_t b = 0; b < B; ++b)
+        if (draft_len[b] < 1) return false;
+    return true;
+}
 
 bool od_host_rows_readable(const void *logits, size_t logits_bytes, const void *q_rows, size_t q_bytes, const char **d_logits,
                            const char **d_q_rows)

@@ -1,5 +1,7 @@
 """Calls whose inputs are written by a launch that is still at work when the library's kernels become resident: a producer
 that releases its dependents first and writes half a millisecond later (tests/helpers/early_producer.cu)."""
+import ctypes as C
+
 import numpy as np
 import pytest
 import torch
@@ -172,3 +174,23 @@ def test_no_call_lets_the_next_one_start_before_its_own_wait(cuda_device, call):
         for b, m in enumerate(want.m.tolist()):
             assert torch.equal(got.tgt_ids[b, :m], want.tgt_ids[b, :m]) and torch.equal(got.span_len[b, :m], want.span_len[b, :m])
     ctx.close()
+
+
+def test_the_driver_says_which_host_buffers_the_device_can_read(cuda_device):
+    """od_step_host fetches rows from page-locked memory and copies from other; both give the same results, so this asks
+    the rule itself, with the driver's answers: all of a range, and one byte more than is left of it."""
+    lib = C.CDLL(od.lib()._name)
+    readable = lib._Z21od_host_rows_readablePKvmS0_mPPKcS3_
+    readable.restype = C.c_bool
+    pinned = torch.empty(1 << 20, dtype=torch.uint8, pin_memory=True)
+    other = torch.empty(1 << 20, dtype=torch.uint8)
+    on_device = torch.empty(1 << 20, dtype=torch.uint8, device=cuda_device)
+    a, b = C.c_void_p(), C.c_void_p()
+
+    def ask(t, at, n):
+        return readable(C.c_void_p(t.data_ptr() + at), C.c_size_t(n), C.c_void_p(pinned.data_ptr()), C.c_size_t(16), C.byref(a), C.byref(b))
+    assert ask(pinned, 0, 1 << 20) and a.value == pinned.data_ptr() and b.value == pinned.data_ptr()
+    assert ask(pinned, 4096, (1 << 20) - 4096)
+    assert not ask(pinned, 8, 64)                           # not 16-byte aligned
+    assert not ask(pinned, 0, 1 << 40)                      # beyond any page-locked range
+    assert not ask(other, 0, 64) and not ask(on_device, 0, 64)

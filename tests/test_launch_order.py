@@ -140,6 +140,45 @@ def test_the_draw_from_host_buffers_reads_nothing_ahead_of_the_rows_that_are_fet
                          [("od_sample_kernel", 0 if pinned else 1)])
 
 
+@pytest.mark.parametrize("kw,lens,fetched", [
+    (dict(v_q=1000, v_p=4000, k=2), 1, True), (dict(v_q=7000, v_p=40000, k=1), 1, False), (dict(v_q=7000, v_p=40000, k=1), 2, False),
+    (dict(v_q=7000, v_p=40000, k=1), 0, True), (dict(v_q=7000, v_p=40000, k=2), 2, True), (dict(v_q=7000, v_p=14000, k=1), 1, True),
+    (dict(v_q=7000, v_p=13992, k=1), 1, True), (dict(v_q=30000, v_p=59992, k=1), 1, True), (dict(v_q=30000, v_p=60000, k=1), 1, False),
+    (dict(v_q=40000, v_p=80000, k=1, vocab_map=np.arange(40000)), 1, True)])
+def test_large_buffers_with_one_token_from_every_sequence_are_copied(lib, kw, lens, fetched):
+    """And not: small ones, an empty proposal among them, two tokens, drafter rows longer than the target's, one vocabulary."""
+    c = lib(max_batch=40, **kw)
+    p = c.inputs(40)
+    next(a for a in c.kept if a.ctypes.data == p["draft_len"].value)[:] = [1] * 20 + [lens] + [1] * 19
+    c.call("od_host_step_reserve", c.ctx, 1)
+    c.pin("logits"); c.pin("q_rows")
+    c.log()
+    c.step_host()
+    log = c.log()
+    assert [x[0] for x in log if x[0].startswith("fetch")] == (["fetch_logits_kernel", "fetch_drafter_kernel"] if fetched else [])
+    rows = [x[1] for x in log if x[0] == "to_device" and x[1] >= 1 << 20]
+    assert sorted(rows) == ([] if fetched else sorted([40 * 2 * kw["v_p"] * 2, 40 * kw["v_q"] * 4]))
+
+
+# page-locked only in part (the range ends inside), off 16 bytes, and a driver that does not say how far the range goes
+@pytest.mark.parametrize("how", ["short", "offset", "no_driver", "one_pageable"])
+def test_buffers_that_the_device_cannot_read_for_certain_are_copied(lib, how):
+    c = lib()
+    p = c.inputs()
+    c.call("od_host_step_reserve", c.ctx, 1)
+    n = B * (K + 1) * V_P * 2
+    if how == "offset":
+        p["logits"] = C.c_void_p(c.zeros(n + 64, np.uint8).value + 8)
+        c.L.fake_pin(p["logits"], n)
+    else:
+        c.pin("logits", n - 1 if how == "short" else None)
+    if how != "one_pageable":
+        c.pin("q_rows")
+    c.L.fake_no_driver_functions(how == "no_driver")
+    c.step_host()
+    assert not any(x[0].startswith("fetch") for x in c.log())
+
+
 @pytest.mark.parametrize("calls,early", [("sample", [0]), ("map sample", [0]), ("map verify sample", [1]), ("map verify sample sample", [1, 0]),
                                          ("map verify map sample", [0]), ("step sample", [0]), ("map verify step sample", [0])])
 @pytest.mark.parametrize("n", [1, B])
