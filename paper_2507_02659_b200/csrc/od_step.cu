@@ -130,8 +130,9 @@ __device__ __forceinline__ void rows_from_one(const StepArgs &a, const Slice &s,
 }
 
 // 2^d for d <= 0, to fp32's last place or so (Taylor's series of e^(f ln 2), |f| <= 1/2, to f^7: 5e-9), 0 below 2^-125.
-// Every level of the merge multiplies whole sums by it, ever fewer and larger ones: with ex2.approx (2^-22) there the row
-// sums were 1.5 to 3 times as far from 64 bits as those of the streaming pass, which has one such level of 64 partials.
+// Every level of the merge multiplies whole sums by it, ever fewer and larger ones, and ex2.approx (2^-22) errs on one side:
+// mean error of 600 row sums against 64 bits, 15 sequences of 50001 bf16 ids: -5.6e-8 with ex2.approx, -0.3e-8 so; 60 of
+// 8000 fp32 ids -4.5e-8, -0.4e-8 (root mean square 9.5e-8, 8.0e-8; the streaming pass, one such level: -4.1e-8, 8.8e-8).
 __device__ __forceinline__ float exp2_to_last_place(float d)
 {
     const float m = d + 12582912.f, f = d - (m - 12582912.f);   // 1.5 * 2^23: the nearest whole number n in m's low bits

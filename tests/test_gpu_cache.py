@@ -287,6 +287,62 @@ def test_translation_directly_behind_cache_writers_with_early_inputs(cuda_device
     ctx.close()
 
 
+@pytest.mark.parametrize("B,grid", [(2, 0), (2, 100), (20, 0)])
+def test_steps_directly_behind_cache_writers_with_early_inputs(cuda_device, B, grid):
+    """The same for od_step: in one launch, which reads all its inputs and the table before its wait unless a writer of the
+    table may be at work, and in three."""
+    rng = np.random.default_rng(78)
+    v_q, v_p, K, dev = 60, 8000, 6, cuda_device
+    vocab_map = np.where(rng.random(v_q) < 0.7, rng.permutation(v_p)[:v_q], -1).astype(np.int32)
+    ctx = od.Context(dev, v_q, v_p, B, K)
+    ctx.set_vocab_map(vocab_map)
+    ctx.cache_configure(40, cp.LRU, 64)
+    ctx.set_option("early_inputs", 1)
+    ctx.set_option("verify_grid", grid)
+    ref = cp.DynamicCache(40, cp.LRU, v_q, v_p)
+    uruns, ulens = _universe(rng, 120, v_q)
+    utgt = rng.integers(0, v_p, size=120).astype(np.int32)
+    g = torch.Generator(device=dev).manual_seed(3)
+    logits = torch.randn(B, K + 1, v_p, generator=g, device=dev).bfloat16()
+    q_rows = torch.softmax(torch.randn(B, K, v_q, generator=g, device=dev), -1)
+    T, seed = torch.ones(B, device=dev), torch.arange(B, device=dev)
+    for tick in range(1, 13):
+        ctx.cache_set_clock(tick); ref.set_clock(tick)
+        props = []
+        for _ in range(4):
+            d = rng.integers(0, v_q, size=(B, K)).astype(np.int32)
+            klen = rng.integers(0, K + 1, size=B).astype(np.int32)
+            for b in range(B):
+                e = int(rng.integers(0, 120)); L = int(ulens[e])
+                if L <= klen[b] and rng.random() < 0.9:
+                    o = int(rng.integers(0, klen[b] - L + 1)); d[b, o:o + L] = uruns[e, :L]
+            q = rng.random((B, K)).astype(np.float32)
+            props.append((d, klen, q, torch.from_numpy(d).to(dev), torch.from_numpy(klen).to(dev), torch.from_numpy(q).to(dev)))
+        pick = rng.integers(0, 120, size=30)
+        runs, lens, tg = uruns[pick].copy(), ulens[pick].copy(), utgt[pick].copy()
+        d_runs, d_lens, d_tg = (torch.from_numpy(x).to(dev) for x in (runs, lens, tg))
+        torch.cuda.synchronize()                              # every input is resident from here on
+        step = lambda i: od.od_step(ctx, *props[i][3:], q_rows, logits, T, seed, tick)[0]
+        ctx.cache_insert(d_runs, d_lens, d_tg)
+        got = [step(0), step(1)]                              # directly behind the insertion, behind another step
+        ctx.cache_trim()
+        got += [step(2), step(3)]
+        torch.cuda.synchronize()
+        if B == 2:
+            assert (ctx.last_launch_info(0) == ctx.last_launch_info(2)) == (grid == 0)
+        ref.insert_batch(runs, lens, tg)
+        for i, mp in enumerate(got):
+            if i == 2:
+                ref.trim()
+            d, klen, q = props[i][:3]
+            for b in range(B):
+                tgt, qp, ss, sl, m, stop = ref.map_sequence(vocab_map, d[b, :klen[b]], q[b])
+                assert int(mp.m[b]) == m and bool(mp.tail_kind[b]) == stop, (tick, i, b)
+                assert mp.tgt_ids[b, :m].tolist() == tgt and mp.span_len[b, :m].tolist() == sl
+        _compare(ctx, ref)
+    ctx.close()
+
+
 def test_a_full_table_counts_what_it_loses(cuda_device):
     """Insertions without a trim until the table (64 slots for a bound of 8 + 8) is full: every
     candidate is either in the cache or counted as lost, and malformed ones are counted too."""

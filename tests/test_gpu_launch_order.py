@@ -194,3 +194,59 @@ def test_the_driver_says_which_host_buffers_the_device_can_read(cuda_device):
     assert not ask(pinned, 8, 64)                           # not 16-byte aligned
     assert not ask(pinned, 0, 1 << 40)                      # beyond any page-locked range
     assert not ask(other, 0, 64) and not ask(on_device, 0, 64)
+
+
+# The tests of the order in three launches that are elsewhere take whichever path the chip's resident clusters give at
+# their sizes; the same here with the streaming pass for certain.
+@pytest.mark.parametrize("early", [0, 1])
+def test_three_launches_equal_the_three_calls(cuda_device, early):
+    w = _workload(B=40, v_p=30011, cache_entries=800)
+    st = synth.make_static(w)
+    ctx = parity.make_context(w, st, cuda_device)
+    ctx.set_option("verify_grid", 148)
+    s = synth.make_step(w, st, 3, device=cuda_device)
+    lg = parity.pad_rows(s.logits)
+    want = parity.gpu_step(ctx, s, logits=lg)
+    ctx.set_option("early_inputs", early)
+    torch.cuda.synchronize()
+    runs = [od.od_step(ctx, s.draft_ids, s.draft_len, s.q_sel, s.q_rows, lg, s.temperature, s.seed, s.step) for _ in range(4)]
+    torch.cuda.synchronize()
+    rows = torch.arange(w.k_max + 1, device=cuda_device)[None, :] <= want[0].m[:, None]
+    pos = rows[:, 1:]
+    for got in runs:
+        for o, names, where in ((0, ("tgt_ids", "q_prime"), pos), (1, ("row_max", "row_sum"), rows), (1, ("p_sel", "ratio"), pos),
+                                (0, ("m", "tail_kind"), ...), (1, ("n_accepted", "n_draft_accepted", "flags"), ...),
+                                (2, ("out_token", "resid_mass", "flags"), ...)):
+            for n in names:
+                assert torch.equal(getattr(got[o], n)[where], getattr(want[o], n)[where]), n
+    ctx.close()
+
+
+@pytest.mark.parametrize("grid", [0, 148])
+@pytest.mark.parametrize("B", [2, 48])
+@pytest.mark.parametrize("call", ["step", "verify"])
+def test_logits_may_be_written_directly_in_front(cuda_device, grid, B, call):
+    w = _workload(B=B)
+    st = synth.make_static(w)
+    ctx = parity.make_context(w, st, cuda_device)
+    ctx.set_option("verify_grid", grid)
+    s = synth.make_step(w, st, 0, device=cuda_device)
+    mp = od.od_map_proposals(ctx, s.draft_ids, s.draft_len, s.q_sel)
+    late = torch.empty_like(s.logits)
+
+    def run(lg):
+        if call == "verify":
+            vo = od.od_verify(ctx, lg, mp, s.temperature, s.seed, s.step)
+            return [vo.n_accepted, vo.flags]
+        _, vo, so = od.od_step(ctx, s.draft_ids, s.draft_len, s.q_sel, s.q_rows, lg, s.temperature, s.seed, s.step)
+        return [vo.n_accepted, vo.flags, so.out_token, so.resid_mass, so.flags]
+    want = run(s.logits)
+    for _ in range(4):
+        late.fill_(float("nan"))
+        torch.cuda.synchronize()
+        _produce(late, s.logits)
+        got = run(late)
+        torch.cuda.synchronize()
+        for a, b in zip(want, got):
+            assert torch.equal(a, b)
+    ctx.close()

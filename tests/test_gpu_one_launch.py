@@ -146,3 +146,84 @@ def test_host_buffers(cuda_device, v_q, where):
                           ("m", mp.m), ("verify_flags", vo.flags), ("sample_flags", so.flags)):
             assert torch.equal(getattr(out, name), ref.cpu()), name
     ctx.close()
+
+
+def test_the_step_takes_every_number_of_blocks_per_sequence(cuda_device):
+    """Which of the batches above were one launch, and of how many blocks, differs from chip to chip; all of them occur."""
+    w = _workload(B=50, k_max=2)
+    st = synth.make_static(w)
+    ctx = parity.make_context(w, st, cuda_device)
+    s = synth.make_step(w, st, 0, device=cuda_device)
+    parts = set()
+    for B in range(1, 51):
+        cut = dataclasses.replace(s, **{k: getattr(s, k)[:B].contiguous() for k in ("draft_ids", "draft_len", "q_sel", "q_rows", "logits", "temperature", "seed")})
+        _step(ctx, cut, parity.pad_rows(cut.logits))
+        if ctx.last_launch_info(0) == ctx.last_launch_info(2):             # one grid
+            parts.add(ctx.last_launch_info(0) // B)
+    assert parts >= {16, 8, 6, 5, 4, 3}, parts
+    ctx.close()
+
+
+# Each of a sum's terms is within 2^-22, its partial sums within 2^-24 of themselves, errors of both signs: 600 sums of
+# thousands of terms come to 1e-7 or less on average, and to a mean error that says what is on one side. 2^-25 is six times
+# what the merge has and half of what it had with ex2.approx (-4.5e-8 to -5.6e-8).
+@pytest.mark.parametrize("B,V,K", [(15, 50001, 4), (60, 8000, 4)])
+@pytest.mark.parametrize("dtype", ["bf16", "f32"])
+def test_row_sums_are_not_off_to_one_side(cuda_device, B, V, K, dtype):
+    dev, dt, per = cuda_device, torch.bfloat16 if dtype == "bf16" else torch.float32, 8 if dtype == "bf16" else 4
+    g = torch.Generator(device=dev).manual_seed(1)
+    ctx = od.Context(dev, 1000, V, B, K)
+    ctx.set_vocab_map(np.arange(1000, dtype=np.int32) + 1)
+    T = torch.tensor([0.5, 0.7, 1.0], device=dev).repeat(B)[:B].contiguous()
+    seed, ln = torch.arange(B, device=dev), torch.full((B,), K, dtype=torch.int32, device=dev)
+    err = {"step": [], "verify": [], "shard": []}
+    for step in range(600 // (B * (K + 1))):
+        lg = torch.zeros(B, K + 1, -(-V // per) * per, dtype=dt, device=dev)[:, :, :V]
+        lg.copy_(torch.randn(B, K + 1, V, generator=g, device=dev) * 3)
+        ids = torch.randint(0, 1000, (B, K), generator=g, device=dev, dtype=torch.int32)
+        q = torch.full((B, K, 1000), 1e-3, device=dev)
+        x = lg.double()
+        want = torch.exp((x - x.amax(-1, keepdim=True)) / T.double()[:, None, None]).sum(-1)
+        mp, vo, _ = od.od_step(ctx, ids, ln, q[:, :, 0].contiguous(), q, lg, T, seed, step)
+        assert ctx.last_launch_info(0) == ctx.last_launch_info(2)          # one grid
+        err["step"].append(vo.row_sum / want - 1)
+        err["verify"].append(od.od_verify(ctx, lg, mp, T, seed, step).row_sum / want - 1)
+        stats = od.od_verify_shard_stats(ctx, 0, lg, mp, T)[None]
+        err["shard"].append(od.od_verify_shard_finish(ctx, stats, mp, T, seed, step).row_sum / want - 1)
+    for name, e in err.items():
+        e = torch.cat(e)
+        assert e.abs().max() <= 2.0 ** -20 and e.pow(2).mean().sqrt() <= 2.0 ** -23, name
+        assert abs(float(e.mean())) <= 2.0 ** -25, name
+    ctx.close()
+
+
+@pytest.mark.parametrize("late", [False, True])
+def test_a_draw_behind_a_step_in_one_launch_waits_for_its_outputs(cuda_device, late):
+    """od_sample_residual on the outputs of the od_step directly in front, over garbage; `late`: that step itself waits
+    half a millisecond for its logits."""
+    import helpers
+    w = _workload(B=4, v_p=40000)
+    st = synth.make_static(w)
+    ctx = parity.make_context(w, st, cuda_device)
+    s = synth.make_step(w, st, 0, device=cuda_device)
+    _, _, want = _step(ctx, s, s.logits)
+    mp, vo, so = od.alloc_map_out(ctx, w.B, w.k_max), od.alloc_verify_out(ctx, w.B, w.k_max), od.alloc_sample_out(ctx, w.B)
+    logits = s.logits.clone()
+    stream = torch.cuda.current_stream(cuda_device).cuda_stream
+    for _ in range(4):
+        for t in (mp.tgt_ids, mp.span_start, mp.span_len, mp.m, vo.n_accepted):
+            t.fill_(-1)
+        vo.row_sum.fill_(float("nan"))
+        if late:
+            logits.fill_(float("nan"))
+        torch.cuda.synchronize()
+        if late:
+            assert helpers.early_producer_lib().early_producer(logits.data_ptr(), s.logits.data_ptr(), logits.numel() * 2, 1000000, stream) == 0
+        od.od_step(ctx, s.draft_ids, s.draft_len, s.q_sel, s.q_rows, logits, s.temperature, s.seed, s.step, mp=mp, vo=vo, so=so)
+        assert ctx.last_launch_info(0) == ctx.last_launch_info(2)
+        again = od.od_sample_residual(ctx, logits, vo, s.q_rows, s.draft_ids, mp, s.temperature, s.seed, s.step)
+        torch.cuda.synchronize()
+        for got in (so, again):
+            assert torch.equal(got.out_token, want.out_token) and torch.equal(got.flags, want.flags)
+            torch.testing.assert_close(got.resid_mass, want.resid_mass, rtol=2.0 ** -22, atol=0)   # (other cuts: fp64 sums, one rounding)
+    ctx.close()
