@@ -144,12 +144,14 @@ def ncu_traffic(workload: str):
     """Per-launch DRAM bytes (read + write) of the stream kernel from the committed ncu
     summary profiles/traffic.txt, or None when there is no figure for this workload or
     the kernel source has changed since the counters were taken. Line format:
-    <workload> <bytes per launch> <sha256 of od_verify.cu at capture time>."""
+    <workload> <bytes per launch> <sha256 of od_verify.cu and od_stream.cuh, one behind the other, at capture time>."""
     import hashlib
     try:
-        src = os.path.join(ROOT, "paper_2507_02659_b200", "csrc", "od_verify.cu")
-        with open(src, "rb") as f:
-            digest = hashlib.sha256(f.read()).hexdigest()
+        digest = hashlib.sha256()
+        for name in ("od_verify.cu", "od_stream.cuh"):
+            with open(os.path.join(ROOT, "paper_2507_02659_b200", "csrc", name), "rb") as f:
+                digest.update(f.read())
+        digest = digest.hexdigest()
         with open(os.path.join(ROOT, "profiles", "traffic.txt")) as f:
             for line in f:
                 t = line.split()
