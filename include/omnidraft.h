@@ -340,7 +340,10 @@ int32_t od_sample_residual(od_ctx *ctx, int32_t B, int32_t K_max,
  * kernel may start on rows 0 of the logits while the translation kernel still
  * runs, with no promise needed from the caller (see "pdl" in the conventions).
  * Small batches are one launch, which may add a row's terms in another
- * order than od_verify does (the row sums' last bits).
+ * order than od_verify does (the row sums' last bits, and with them a decision at
+ * its boundary, which the flag words report). Which batches are one launch, and
+ * how a row is cut, follows from how many thread-block clusters the device holds
+ * at a time: the last bits may differ between devices that hold other numbers.
  * All pointers are device pointers owned by the caller; inputs and outputs as
  * documented for the three calls (counters may be NULL). Asynchronous; allocates
  * nothing; errors as for the three calls, checked before the first launch. */

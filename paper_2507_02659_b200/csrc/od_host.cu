@@ -4,7 +4,7 @@
 // From page-locked buffers the device fetches the rows itself: the logit rows 0..m_b once the
 // translation has found m_b, and the ONE drafter row that the draw needs once step 2 has decided where it is,
 // not the K_b rows that the step might have needed. (32 sequences x up to 6 tokens, 128256 bf16 ids: 51 MB in 59
-// copies of about 1 MB, which themselves run at 45 GB/s where one large copy reaches 55; fetched 41 MB: 1278 -> 870 us, 833 on another machine.)
+// copies of about 1 MB, which themselves run at 45 GB/s where one large copy reaches 55; fetched 41 MB: 1220 -> 826 us.)
 // Buffers that the device cannot read, and those of which all is likely needed (od_host_better_copied), are copied, rows
 // 0..K_b and 0..K_b-1 of every sequence.
 #include "od_common.cuh"

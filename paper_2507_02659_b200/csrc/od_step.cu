@@ -13,7 +13,7 @@
 //   the draw     as in od_sample.cu.
 // What it takes the place of is three launches (translation, streaming pass, sampler), each of which waits
 // for the slowest block of the one before it, and writes and reads partials through L2. Bound by the chain of
-// round trips: one sequence of 128256 bf16 ids, six tokens, 14.3 -> 12.0 us a step; of 32000 fp32 ids (stamps): 1.0 us to
+// round trips: one sequence of 128256 bf16 ids, six tokens, 14.5 -> 12.4 us a step; of 32000 fp32 ids (stamps): 1.0 us to
 // the proposal and the map, 0.9 to the pieces, 1.6 the rows, 1.5 the exchange, 0.6 the decisions, 1.6 the tiles, 0.9 the
 // exchange of their sums, 1.5 the tile and the id.
 #include <float.h>
@@ -70,8 +70,10 @@ __device__ __forceinline__ const char *row_of(const StepArgs &a, int b, int r)
 }
 
 // Units a warp requests at a time. fp32 rows have twice the bytes to each exponential: twice the loads in flight make
-// a step faster (36 sequences of 50001 ids 18.6 -> 17.6 us); bf16 steps are slower by the code and the registers that
-// this costs (one sequence of 128256 ids 12.0 -> 12.3).
+// a step faster where the rows come from HBM (inputs that change from pass to pass, sequences x K_max: 9 x 3, 152064 ids
+// 18.4 -> 16.8 us; 24 x 4, 50001 17.9 -> 17.2; 15 x 4 14.3 -> 14.0; 1 x 4, 32000 9.2 -> 9.3), and 1 to 2 % slower where they
+// are in L2 (13.8 -> 13.9, 13.4 -> 13.7, 11.1 -> 11.2, 8.1 -> 8.3). bf16 steps are slower by the code and the registers
+// that this costs (one sequence of 128256 ids, from L2, 12.0 -> 12.3).
 template <int DTYPE>
 constexpr int GROUP = DTYPE == OD_BF16 ? U : 2 * U;
 
@@ -407,11 +409,12 @@ int level_within(const od_ctx *c, int32_t B, int32_t K_max, int32_t v_len, int32
 // HBM with what it has in flight), however few rows others have; three launches spread all rows over all
 // multiprocessors. The line lies where a block may have 320 KB to stream (device time of a step, three launches -> one;
 // sequences x K_max, target ids, blocks: KB; in brackets with inputs that change from pass to pass, from HBM):
-//   1 x 6, 128256 bf16, 16: 112 KB  13.8 -> 12.0 (13.3 -> 10.9)     15 x 6, 8: 221 KB  18.6 -> 15.4 (19.7 -> 16.7)
+//   1 x 6, 128256 bf16, 16: 112 KB  14.5 -> 12.4 (14.9 -> 13.1)     15 x 6, 8: 221 KB  18.6 -> 15.4 (19.7 -> 16.7)
 //   22 x 6, 6: 294 KB  20.0 -> 18.0 (20.9 -> 19.6)                  24 x 6, 5: 354 KB  20.3 -> 19.8 (21.3 -> 21.5)
 //   15 x 12, 8: 410 KB  19.8 -> 19.3                  28 x 6, 4: 441 KB  21.5 -> 21.7     22 x 12, 6: 546 KB  23.2 -> 23.4
-//   36 x 4, 50001 fp32, 3: 330 KB  20.4 -> 17.6       7 x 3, 152064, 16: 76 KB  16.4 -> 12.4
-// and batches of two blocks a sequence gain little (60 x 8, 32000: 16.0 -> 15.3; 60 x 6, 128256: 30.0 -> 34.8).
+//   7 x 3, 152064 bf16, 16: 76 KB  16.4 -> 12.4      24 x 4, 50001 fp32, 6: 165 KB  16.5 -> 13.7 (19.5 -> 17.2)
+// One line for both types, though fp32 rows have half the exponentials to a byte: 36 x 4, 50001 fp32, 3: 330 KB, just
+// beyond it, would be 20.4 -> 17.6 from L2 (three launches there now 18.5). Batches of two blocks a sequence gain little (60 x 8, 32000: 16.0 -> 15.3; 60 x 6, 128256: 30.0 -> 34.8).
 int step_level(const od_ctx *c, int32_t B, int32_t K_max, int32_t v_len, int32_t dtype)
 {
     return level_within(c, B, K_max, v_len, dtype, 3, 320 * 1024);
