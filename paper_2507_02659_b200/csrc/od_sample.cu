@@ -201,7 +201,6 @@ od_sample_shard_kernel(const SampleArgs a)
 
     if (!a.early) asm volatile("griddepcontrol.wait;" ::: "memory");
     Ahead h = load_ahead(a, b, lane);
-    request_first_probability(a, h, b);
     const int mb = h.mb;
     const float T = h.T;
     const bool planned = __ldg(a.map_serial_now) == a.map_serial;   // (as in od_sample_kernel)
