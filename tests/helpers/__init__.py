@@ -32,11 +32,11 @@ def fake_runtime_lib():
     src = os.path.join(_HERE, "fake_cudart.cu")
     if not os.path.exists(_FAKE) or os.path.getmtime(_FAKE) < max(build._newest_source(), os.path.getmtime(src)):
         with tempfile.TemporaryDirectory() as tmp:
-            jobs, objects = [], []
+            nvcc, jobs, objects = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc"), [], []
             for path in [os.path.join(build.CSRC, f) for f in build.SOURCES] + [src]:
                 objects.append(os.path.join(tmp, os.path.basename(path) + ".o"))
                 # (host code only: the device code is parsed and not compiled)
-                jobs.append(subprocess.Popen(["nvcc", "-gencode", "arch=compute_100a,code=sm_100a", "-std=c++17", "-Xcompiler", "-fPIC",
+                jobs.append(subprocess.Popen([nvcc, "-gencode", "arch=compute_100a,code=sm_100a", "-std=c++17", "-Xcompiler", "-fPIC",
                                               "--fdevice-syntax-only", "-I", os.path.join(build.ROOT, "include"), "-I", build.CSRC,
                                               "-c", "-o", objects[-1], path]))
             assert [j.wait() for j in jobs] == [0] * len(jobs)
