@@ -190,8 +190,8 @@ int32_t od_cache_build(od_ctx *ctx, const int32_t *host_runs,
  * synchronous. Needs draft_vocab <= 65535 (UNSUPPORTED otherwise). Device memory:
  * the table has S = the next power of two >= 2 * (max_entries + max_insert) slots;
  * two copies of it (24 bytes per slot each, the second one is the table a trim
- * builds), a claim word per slot and 68 bytes per slot of trim scratch are
- * allocated here, 120 * S bytes in all (NOMEM if that fails); nothing is
+ * builds), a claim word per slot, 52 bytes per slot of trim scratch and a word per 32 slots of each copy are
+ * allocated here, 104.25 * S bytes in all (NOMEM if that fails); nothing is
  * allocated later. */
 int32_t od_cache_configure(od_ctx *ctx, int64_t max_entries, int32_t policy,
                            int32_t max_insert);

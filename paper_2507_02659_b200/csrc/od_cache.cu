@@ -13,17 +13,19 @@
 //           the result does not depend on thread timing.
 //   trim    with k = size - max_entries > 0 entries too many, the k entries that
 //           come first in the order (inserted at the current clock?, score, run key)
-//           are dropped, score = last-access clock (LRU) or frequency (LFU). One
-//           pass over the table packs the live entries into a dense list (and clears
-//           the spare table); the k-th smallest is found by a most-significant-digit
-//           radix select over the 104-bit order key, by one cluster of blocks
-//           (trim_select_kernel). Tables too large for that take a chain of 13 histogram
-//           launches over the CANDIDATES only: a pass copies the entries that still match
+//           are dropped, score = last-access clock (LRU) or frequency (LFU). A first
+//           pass counts the entries by score, in 256 bins (trim_count_kernel); that
+//           says for almost every entry whether it stays: a second pass copies those
+//           that do straight into their own group of the spare table (trim_split_kernel)
+//           and lists the entries of the one bin in which the k-th falls. The k-th of
+//           those is found by a most-significant-digit radix select over the 104-bit order
+//           key, by one cluster of blocks (trim_select_kernel). Tables too large for that take
+//           a chain of 13 histogram launches: a pass copies the entries that still match
 //           the decided prefix into the next list whenever that at least halves it, every
 //           block works out the digit the pass before it decided from that pass's 256-bin
-//           histogram, and a digit of (new?, score) that is the same in every live entry
-//           costs no histogram. Then the survivors are re-inserted from the dense list
-//           into the spare table, which becomes the table. No kernel waits for another.
+//           histogram, and a digit of (new?, score) that is the same in every listed entry
+//           costs no histogram. Then the rest of the survivors go from the list
+//           into the spare table (trim_place_kernel), which becomes the table. No kernel waits for another.
 #include <algorithm>
 #include <stddef.h>
 #include <string.h>
@@ -51,27 +53,25 @@ struct TrimState {
     unsigned int k;             // entries to drop in this trim
     unsigned int invalid;       // malformed candidates seen by od_cache_insert
     unsigned int dropped;       // candidates that found no free slot on their whole probe sequence
-    // what the pass over the table finds out; empty again when a trim has read it, so that a
-    // trim that is replayed from a CUDA graph starts like the one that was captured
-    struct Live {
-        unsigned int n;         // entries of the dense list
-        unsigned long long hi_and, hi_or;   // AND / OR of (new?, score) over the live entries: bits that never vary
-    } live;
-    unsigned int n_list;        // trim_select_kernel: live.n as it was, for the rebuild,
-    unsigned long long thr_hi, thr_lo;      // and the k-th order key
+    // The pass that counts sets these back, and the last kernel the bins: a trim that is replayed from a CUDA
+    // graph starts like the one that was captured.
+    unsigned int k_rem;         // of the listed entries, how many to drop
+    unsigned int n_list;        // entries listed because their bin has both kinds
+    unsigned int n_late;        // survivors that are not in the group their run hashes to, listed from the other end
+    unsigned long long hi_and, hi_or;       // AND / OR of (new?, score) over the listed entries: bits that never vary
+    unsigned long long thr_hi, thr_lo;      // trim_select_kernel: the k-th order key
+    unsigned int bins[256];     // live entries by score (score_bin)
     SelState sel[PASSES + 1];   // sel[p]: written by block 0 of pass p (sel[PASSES]: by the rebuild)
     unsigned int n_out[PASSES]; // entries pass p copied into its output list
     unsigned int hist[PASSES][256];
 };
 
-// Trim scratch for a table of `cap` slots: the dense list of live entries (order key and
-// payload) and two lists of (hi, lo) candidates.
+// Trim scratch for a table of `cap` slots: the listed entries (order key and slot in the old table)
+// and two lists of (hi, lo) candidates.
 struct TrimLists {
     unsigned long long *r_hi, *r_key;
-    int32_t *r_val;
-    unsigned int *r_stamp, *r_freq, *r_born;
+    unsigned int *r_slot;
     unsigned long long *l_hi[2], *l_lo[2];
-    unsigned int *grp_fill;             // [cap / OD_GROUP] slots handed out in each group of the table being built
 };
 __host__ __device__ inline TrimLists trim_lists(void *base, int64_t cap)
 {
@@ -80,12 +80,12 @@ __host__ __device__ inline TrimLists trim_lists(void *base, int64_t cap)
     t.r_hi = q; t.r_key = q + cap;
     t.l_hi[0] = q + 2 * cap; t.l_lo[0] = q + 3 * cap;
     t.l_hi[1] = q + 4 * cap; t.l_lo[1] = q + 5 * cap;
-    unsigned int *w = (unsigned int *)(q + 6 * cap);
-    t.r_val = (int32_t *)w; t.r_stamp = w + cap; t.r_freq = w + 2 * cap; t.r_born = w + 3 * cap;
-    t.grp_fill = w + 4 * cap;
+    t.r_slot = (unsigned int *)(q + 6 * cap);
     return t;
 }
-constexpr size_t TRIM_LIST_BYTES_PER_SLOT = 6 * 8 + 5 * 4;   // (the last array needs a 32nd of its share)
+constexpr size_t TRIM_LIST_BYTES_PER_SLOT = 6 * 8 + 4;
+// Slots taken in each group (a count may run past the group's 32), for a table of `cap` slots: read four groups at a time
+inline size_t fill_words(int64_t cap) { return (size_t)(cap / OD_GROUP < 4 ? 4 : cap / OD_GROUP); }
 
 // order key of a live entry: hi = (inserted at the current clock) << 32 | score, lo = run key
 __device__ __forceinline__ void order_key(int policy, unsigned int clock, unsigned long long key,
@@ -131,7 +131,7 @@ cudaError_t chain_launch(void (*kernel)(Params...), unsigned grid, unsigned bloc
 __global__ void insert_claim_kernel(int32_t N, int32_t v_q, int32_t v_p, const int32_t *__restrict__ runs,
                                     const int32_t *__restrict__ len, const int32_t *__restrict__ target,
                                     unsigned long long *keys, const int32_t *vals, int64_t cap,
-                                    unsigned int *owner, int32_t *cand_slot, TrimState *st)
+                                    unsigned int *owner, int32_t *cand_slot, unsigned int *fill, TrimState *st)
 {
     chain_wait(true);
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -176,6 +176,7 @@ __global__ void insert_claim_kernel(int32_t N, int32_t v_q, int32_t v_p, const i
                 seen = keys[slot];
             }
             const unsigned long long cur = seen == 0ull ? atomicCAS(keys + slot, 0ull, key) : seen;
+            if (cur == 0ull) atomicAdd(fill + g, 1u);
             if (cur == 0ull || cur == key) {
                 // an entry with a value was there before this batch: nothing to add
                 if (seen == 0ull || ((volatile const int32_t *)vals)[slot] < 0) {
@@ -207,19 +208,10 @@ __global__ void insert_commit_kernel(int32_t N, const int32_t *__restrict__ targ
     atomicAdd(&st->size, 1u);
 }
 
-__device__ __forceinline__ void reset_live(TrimState::Live &l) { l.n = 0u; l.hi_and = ~0ull; l.hi_or = 0ull; }
-
 __global__ void trim_begin_kernel(TrimState *st, unsigned int max_entries)
 {
     chain_wait(true);
-    const unsigned int k = st->size > max_entries ? st->size - max_entries : 0u;
-    if (threadIdx.x == 0) {
-        st->k = k;
-        reset_live(st->live);
-        SelState z = {};
-        z.k_rem = k;
-        st->sel[0] = z;
-    }
+    if (threadIdx.x == 0) st->k = st->size > max_entries ? st->size - max_entries : 0u;
     for (int p = 0; p < PASSES; ++p) st->hist[p][threadIdx.x] = 0u;
     if (threadIdx.x < PASSES) st->n_out[threadIdx.x] = 0u;
 }
@@ -246,90 +238,37 @@ __device__ __forceinline__ unsigned int block_offsets(unsigned int n, unsigned i
     return base + inc - n;
 }
 
-// One pass over the table: every live entry goes into the dense list (in no particular
-// order: one append per block and iteration), and the spare table is cleared: its keys and values,
-// which say whether a slot is taken and set (stamp, freq and born of a free slot are never read,
-// and written with the entry). Bound by L2 traffic, of which the empty slots were most: four
-// slots without a key cost no more than their keys.
-__global__ void trim_compact_kernel(int policy, unsigned int clock, const unsigned long long *keys,
-                                    const int32_t *vals, const unsigned int *stamp, const unsigned int *freq,
-                                    const unsigned int *born, unsigned long long *nkeys, int32_t *nvals,
-                                    int64_t cap, void *lists, TrimState *st)
-{
-    __shared__ unsigned int s_warp[32];
-    __shared__ unsigned int s_base;
-    __shared__ unsigned long long s_and, s_or;
-    chain_wait(true);
-    const TrimLists L = trim_lists(lists, cap);
-    if (threadIdx.x == 0) { s_and = ~0ull; s_or = 0ull; }
-    unsigned long long t_and = ~0ull, t_or = 0ull;
-    // four slots per thread and iteration
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x * 4;
-    for (int64_t slot0 = (int64_t)blockIdx.x * blockDim.x * 4; slot0 < cap; slot0 += stride) {
-        const int64_t slot = slot0 + (int64_t)threadIdx.x * 4;
-        unsigned long long kk[4] = {0ull, 0ull, 0ull, 0ull};
-        int vv[4] = {-1, -1, -1, -1};
-        uint4 ss, ff, bb;
-        if (slot < cap) {                                   // cap is a multiple of 64
-            const ulonglong2 k01 = __ldg((const ulonglong2 *)(keys + slot));
-            const ulonglong2 k23 = __ldg((const ulonglong2 *)(keys + slot) + 1);
-            kk[0] = k01.x; kk[1] = k01.y; kk[2] = k23.x; kk[3] = k23.y;
-            *(ulonglong2 *)(nkeys + slot) = make_ulonglong2(0ull, 0ull);
-            *((ulonglong2 *)(nkeys + slot) + 1) = make_ulonglong2(0ull, 0ull);
-            *(int4 *)(nvals + slot) = make_int4(-1, -1, -1, -1);
-            if ((slot & (OD_GROUP - 1)) == 0) L.grp_fill[slot / OD_GROUP] = 0u;
-        }
-        if ((kk[0] | kk[1] | kk[2] | kk[3]) != 0ull) {
-            const int4 v4 = __ldg((const int4 *)(vals + slot));
-            ss = __ldg((const uint4 *)(stamp + slot));
-            ff = __ldg((const uint4 *)(freq + slot));
-            bb = __ldg((const uint4 *)(born + slot));
-            vv[0] = v4.x; vv[1] = v4.y; vv[2] = v4.z; vv[3] = v4.w;
-        }
-        unsigned int n = 0;
-#pragma unroll
-        for (int e = 0; e < 4; ++e) n += (kk[e] != 0ull && vv[e] >= 0) ? 1u : 0u;
-        unsigned int total;
-        unsigned int at = block_offsets(n, s_warp, total);
-        if (threadIdx.x == 0) s_base = total ? atomicAdd(&st->live.n, total) : 0u;
-        __syncthreads();
-        at += s_base;
-        const unsigned int s4[4] = {ss.x, ss.y, ss.z, ss.w}, f4[4] = {ff.x, ff.y, ff.z, ff.w}, b4[4] = {bb.x, bb.y, bb.z, bb.w};
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            if (kk[e] == 0ull || vv[e] < 0 || at >= cap) continue;   // (never beyond the list)
-            unsigned long long hi, lo;
-            order_key(policy, clock, kk[e], s4[e], f4[e], b4[e], hi, lo);
-            t_and &= hi; t_or |= hi;
-            L.r_hi[at] = hi; L.r_key[at] = lo;
-            L.r_val[at] = vv[e]; L.r_stamp[at] = s4[e]; L.r_freq[at] = f4[e]; L.r_born[at] = b4[e];
-            ++at;
-        }
-    }
-    // which bits of (new?, score) vary at all: AND and OR over the live entries
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
-        t_and &= __shfl_xor_sync(0xFFFFFFFFu, t_and, off);
-        t_or |= __shfl_xor_sync(0xFFFFFFFFu, t_or, off);
-    }
-    if ((threadIdx.x & 31) == 0) { atomicAnd(&s_and, t_and); atomicOr(&s_or, t_or); }
-    __syncthreads();
-    if (threadIdx.x == 0) { atomicAnd(&st->live.hi_and, s_and); atomicOr(&st->live.hi_or, s_or); }
-}
-
-// ---- the k-th order key in one launch ------------------------------------------------------
+// ---- the two passes over the table ---------------------------------------------------------
 //
-// One cluster of P blocks, each with a slice of the dense list: a most-significant-digit radix
-// select in which a pass is a histogram in shared memory, ONE cluster barrier and the sum of the
-// P histograms over distributed shared memory, by every block alike. The bits of (new?, score)
-// that vary are settled first, over the slices; the keys of the entries that tie at that score
-// then stay in shared memory for the run key, and the select ends as soon as
-// every candidate that is left is among the k (usually three passes in all: a pass costs 2.5 us or so,
-// of which the barrier and the sums are most; an insertion, a trim and a translation, bytes -> bits and run lengths as
-// digits: 262144 entries 62.7 -> 58.2 us, by frequency 90.5 -> 70.3; 8192 entries 32.8 -> 26.6). As a chain
-// of 13 launches of the whole grid, two dependent round trips and a launch each, the passes were
-// 52 of the 107 us of an insertion, a trim and a translation (262144 entries, 16384 new ones).
-constexpr int SELECT_THREADS = 1024, SELECT_MAX_BLOCKS = 16;
+// Sixteen lanes take a group's first sixteen slots (a table at most half full often has no more: a group is filled from
+// slot 0), then the rest where the sixteenth is taken, four groups at a time. How far a group is filled is kept for
+// each, so that no slot is cleared that was not taken. Neither pass has an atomic per entry: a survivor stays in the
+// group it is in. Bound by the chain of round trips and by L2 (262144 entries: 13 MB read, 12 MB written). Before,
+// one pass packed all live entries into a list, the select walked through it, and a rebuild put every survivor into the slot that
+// its group's counter gave. Device time of an insertion, a trim and a translation, before -> now: 262144 entries and 16384 new
+// ones 53.7 -> 37.5 us, by frequency 70.1 -> 64.8; 4096 and 512 24.4 -> 23.1; 32768 and 4096 by frequency 35.3 -> 34.7. (The
+// whole trim in one cluster of 1 to 16 blocks, for tables of up to 131072 slots: 26.5 and 37.7 us on the last two; a step
+// of it is a chain of trips as long as a launch's.)
+constexpr int TRIM_THREADS = 256, TRIM_HALVES = TRIM_THREADS / 16, QUAD = 4;   // groups of a half-warp at a time
+
+// (new?, score) to one of 256 bins, in the order of trims: 255 new; else by age (LRU) or frequency (LFU), exact up to 127,
+// four bins to an octave beyond. (A stamp past the clock, which the caller may set back, counts as of now.)
+__device__ __forceinline__ unsigned int log_bin(unsigned int v)
+{
+    const int e = 31 - __clz((int)v);
+    return v < 128u ? v : 128u + ((unsigned int)(e - 7) << 2) + (v >> (e - 2) & 3u);   // at most 227
+}
+__device__ __forceinline__ unsigned int score_bin(int policy, unsigned int clock, unsigned int score, bool is_new)
+{
+    if (is_new) return 255u;
+    return policy == 0 ? 254u - log_bin(score <= clock ? clock - score : 0u) : log_bin(score);
+}
+// whether all of a bin's entries have one (new?, score), and which
+__device__ __forceinline__ bool exact_bin(int policy, unsigned int clock, unsigned int bin, unsigned long long &hi)
+{
+    hi = policy == 0 ? (unsigned long long)(clock - (254u - bin)) : (unsigned long long)bin;
+    return policy == 0 ? bin < 254u && bin > 254u - 128u && 254u - bin <= clock : bin < 128u;
+}
 
 // Count digit `d` of the lanes with `ok` into hist: digits are heavily tied (scores, the upper
 // bytes of short runs), so lanes that agree count as one add.
@@ -339,23 +278,244 @@ __device__ __forceinline__ void count_digit(unsigned int *hist, unsigned int d, 
     if (ok && __ffs(same) - 1 == (int)(threadIdx.x & 31)) atomicAdd(hist + d, (unsigned int)__popc(same));
 }
 
+// The live entries by score.
+__global__ void __launch_bounds__(TRIM_THREADS)
+trim_count_kernel(int policy, unsigned int clock, const int32_t *vals, const unsigned int *score, const unsigned int *born,
+                  int64_t cap, TrimState *st)
+{
+    __shared__ unsigned int s_bins[256];
+    s_bins[threadIdx.x] = 0u;
+    const int64_t quads = (cap / OD_GROUP + QUAD - 1) / QUAD;
+    const int at = threadIdx.x & 15;
+    chain_wait(true);
+    if (blockIdx.x == 0 && threadIdx.x == 0) { st->n_list = 0u; st->n_late = 0u; st->hi_and = ~0ull; st->hi_or = 0ull; }
+    __syncthreads();
+    for (int64_t q0 = (int64_t)blockIdx.x * TRIM_HALVES; q0 < quads; q0 += (int64_t)gridDim.x * TRIM_HALVES) {
+        const int64_t quad = q0 + (threadIdx.x >> 4);
+        bool more = false;                                  // a group's sixteenth slot is taken: the others too
+        for (int s = at; s < OD_GROUP && (s < 16 || __any_sync(0xFFFFFFFFu, more)); s += 16) {
+            int32_t v[QUAD];
+            unsigned int sc[QUAD], bn[QUAD];
+#pragma unroll
+            for (int e = 0; e < QUAD; ++e) {
+                const int64_t slot = (quad * QUAD + e) * OD_GROUP + s;
+                v[e] = -1;
+                if (slot < cap) { v[e] = __ldcg(vals + slot); sc[e] = __ldcg(score + slot); bn[e] = __ldcg(born + slot); }
+            }
+#pragma unroll
+            for (int e = 0; e < QUAD; ++e) {
+                count_digit(s_bins, score_bin(policy, clock, sc[e], bn[e] == clock), v[e] >= 0);   // (a slot without a value is no entry)
+                more = more || (at == 15 && v[e] >= 0);
+            }
+        }
+    }
+    __syncthreads();
+    if (s_bins[threadIdx.x]) atomicAdd(st->bins + threadIdx.x, s_bins[threadIdx.x]);
+}
+
+// A slot of the old table, as it goes into the new one
+struct Entry {
+    unsigned long long key;
+    int32_t v;
+    unsigned int stamp, freq, born;
+};
+struct Table {
+    unsigned long long *keys;                               // an empty slot has no value (-1)
+    int32_t *vals;
+    unsigned int *stamp, *freq, *born, *fill;
+    __device__ __forceinline__ Entry load(int64_t slot) const
+    {
+        return Entry{__ldcg(keys + slot), __ldcg(vals + slot), __ldcg(stamp + slot), __ldcg(freq + slot), __ldcg(born + slot)};
+    }
+    __device__ __forceinline__ void store(int64_t slot, const Entry &e) const
+    {
+        keys[slot] = e.key; vals[slot] = e.v; stamp[slot] = e.stamp; freq[slot] = e.freq; born[slot] = e.born;
+    }
+};
+
+// An entry into the new table. A group is filled from its slot 0 without holes (od_cache_insert stops at the first empty
+// slot). Every placement takes the next slot of its group from the group's count: no two entries ever want the same
+// slot, so there is nothing to retry. A full group (32 entries: rare in a table at most half full) sends
+// the entry on to the next group, as a probe would go.
+__device__ __forceinline__ void place_entry(const Table &to, int64_t cap, const Entry &en)
+{
+    const uint64_t ngroups = (uint64_t)cap / OD_GROUP;
+    uint64_t g = od_hash64(en.key) & (ngroups - 1);
+    for (uint64_t step = 0; step < ngroups; ++step) {
+        const unsigned int at = atomicAdd(to.fill + g, 1u);
+        if (at < (unsigned int)OD_GROUP) { to.store((int64_t)(g * OD_GROUP + at), en); break; }
+        g = (g + 1) & (ngroups - 1);
+    }
+}
+
+// Which bin the k-th entry is in; then every group's survivors into the same group of the new table, and into the list what
+// cannot be said yet. The table has not been written since before the pass that counts waited, so the first
+// groups are loaded in front of this kernel's own wait.
+__global__ void __launch_bounds__(TRIM_THREADS, 4)
+trim_split_kernel(int policy, unsigned int clock, unsigned int max_entries, const Table from, const Table to, int64_t cap,
+                  void *lists, TrimState *st)
+{
+    __shared__ unsigned int s_warp[TRIM_THREADS / 32], s_base[2], s_bin, s_rem, s_in;
+    __shared__ unsigned long long s_and, s_or;
+    asm volatile("griddepcontrol.launch_dependents;");
+    const int64_t groups = cap / OD_GROUP, quads = (groups + QUAD - 1) / QUAD;
+    const int at = threadIdx.x & 15, half = threadIdx.x >> 4 & 1;
+    const TrimLists L = trim_lists(lists, cap);
+    unsigned int run[QUAD];
+    Entry en[QUAD];
+    int64_t q0 = (int64_t)blockIdx.x * TRIM_HALVES, quad = q0 + (threadIdx.x >> 4);
+    const auto load = [&](int s) {
+#pragma unroll
+        for (int e = 0; e < QUAD; ++e) {
+            const int64_t slot = (quad * QUAD + e) * OD_GROUP + s;
+            en[e].v = -1;
+            if (slot < cap) en[e] = from.load(slot);
+        }
+    };
+    load(at);
+    if (threadIdx.x == 0) { s_and = ~0ull; s_or = 0ull; s_bin = 256u; s_rem = 0u; s_in = 0u; }
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+
+    // ---- the first bin at which the running count reaches k (none: everything goes)
+    const unsigned int size = __ldcg(&st->size), k = size > max_entries ? size - max_entries : 0u;
+    const unsigned int mine = __ldcg(st->bins + threadIdx.x);
+    unsigned int total;
+    const unsigned int before = block_offsets(mine, s_warp, total);
+    if (k > before && k - before <= mine) { s_bin = threadIdx.x; s_rem = k - before; s_in = mine; }
+    __syncthreads();
+    const bool whole = s_rem == s_in;                       // the bin goes as a whole: nothing is left to find out
+    const unsigned int first_kept = k == 0u ? 0u : s_bin + (whole ? 1u : 0u), mixed = k == 0u || whole ? 512u : s_bin;
+    unsigned long long bin_hi;
+    const bool exact = exact_bin(policy, clock, mixed & 255u, bin_hi);
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        st->k = k; st->k_rem = mixed < 256u ? s_rem : 0u;
+        if (exact) { st->hi_and = bin_hi; st->hi_or = bin_hi; }
+    }
+
+    for (;;) {
+        const bool in = quad < quads;
+        unsigned int had[QUAD];
+#pragma unroll
+        for (int e = 0; e < QUAD; ++e) run[e] = 0u;
+        // (where a group's sixteenth slot is taken: the others too)
+        const int rounds = __syncthreads_or(at == 15 && max(max(en[0].v, en[1].v), max(en[2].v, en[3].v)) >= 0) ? 2 : 1;
+        for (int round = 0; round < rounds; ++round) {
+            const int s = at + 16 * round;
+            if (round) load(s);
+            const uint4 taken = round + 1 == rounds && in ? __ldcg((const uint4 *)to.fill + quad) : make_uint4(0u, 0u, 0u, 0u);
+            had[0] = taken.x; had[1] = taken.y; had[2] = taken.z; had[3] = taken.w;
+            unsigned int listed = 0u, late = 0u;            // of this thread's four: bit e
+            unsigned long long t_and = ~0ull, t_or = 0ull;
+#pragma unroll
+            for (int e = 0; e < QUAD; ++e) {
+                const int64_t g = quad * QUAD + e;
+                const bool is_new = en[e].born == clock;
+                const unsigned int score = policy == 0 ? en[e].stamp : en[e].freq;
+                const unsigned int bin = en[e].v >= 0 ? score_bin(policy, clock, score, is_new) : 0u;
+                const bool live = en[e].v >= 0, home = live && (int64_t)(od_hash64(en[e].key) & (uint64_t)(groups - 1)) == g;
+                const bool keep = live && bin >= first_kept && bin != mixed;
+                if (live && bin == mixed) {
+                    listed |= 1u << e;
+                    unsigned long long hi, lo;
+                    order_key(policy, clock, en[e].key, en[e].stamp, en[e].freq, en[e].born, hi, lo);
+                    t_and &= hi; t_or |= hi;
+                }
+                if (keep && !home) late |= 1u << e;
+                const unsigned int stays = __ballot_sync(0xFFFFFFFFu, keep && home) >> (16 * half) & 0xFFFFu;
+                if (keep && home) to.store(g * OD_GROUP + run[e] + __popc(stays & ((1u << at) - 1u)), en[e]);
+                run[e] += __popc(stays);
+            }
+            // ---- the lists: one append per block
+            unsigned int sum;
+            unsigned int ofs = block_offsets(__popc(listed) | __popc(late) << 16, s_warp, sum);
+            if (sum == 0u) continue;                        // (the same for every thread of the block)
+            if (threadIdx.x == 0) s_base[0] = sum & 0xFFFFu ? atomicAdd(&st->n_list, sum & 0xFFFFu) : 0u;
+            if (threadIdx.x == 32) s_base[1] = sum >> 16 ? atomicAdd(&st->n_late, sum >> 16) : 0u;
+            if (!exact && (sum & 0xFFFFu)) {
+#pragma unroll
+                for (int off = 16; off > 0; off >>= 1) {
+                    t_and &= __shfl_xor_sync(0xFFFFFFFFu, t_and, off);
+                    t_or |= __shfl_xor_sync(0xFFFFFFFFu, t_or, off);
+                }
+                if ((threadIdx.x & 31) == 0) { atomicAnd(&s_and, t_and); atomicOr(&s_or, t_or); }
+            }
+            __syncthreads();
+            int64_t i_list = (int64_t)s_base[0] + (ofs & 0xFFFFu), i_late = cap - 1 - ((int64_t)s_base[1] + (ofs >> 16));
+#pragma unroll
+            for (int e = 0; e < QUAD; ++e) {
+                const unsigned int slot = (unsigned int)((quad * QUAD + e) * OD_GROUP + s);
+                if (listed >> e & 1u) {
+                    if (i_list < cap) {                     // (never beyond the list)
+                        order_key(policy, clock, en[e].key, en[e].stamp, en[e].freq, en[e].born, L.r_hi[i_list], L.r_key[i_list]);
+                        L.r_slot[i_list] = slot;
+                    }
+                    ++i_list;
+                }
+                if (late >> e & 1u) {
+                    if (i_late >= 0) L.r_slot[i_late] = slot;
+                    --i_late;
+                }
+            }
+        }
+        // ---- the slots that are free now and were taken, and how far each group is filled
+#pragma unroll
+        for (int e = 0; e < QUAD; ++e)
+            for (unsigned int s = run[e] + at; s < min(had[e], (unsigned int)OD_GROUP); s += 16) {
+                const int64_t slot = (quad * QUAD + e) * OD_GROUP + s;
+                to.keys[slot] = 0ull; to.vals[slot] = -1;
+            }
+        if (in && at == 0) ((uint4 *)to.fill)[quad] = make_uint4(run[0], run[1], run[2], run[3]);
+        q0 += (int64_t)gridDim.x * TRIM_HALVES;
+        if (q0 >= quads) break;
+        quad = q0 + (threadIdx.x >> 4);
+        load(at);
+    }
+    if (!exact && threadIdx.x == 0 && (s_and != ~0ull || s_or != 0ull)) { atomicAnd(&st->hi_and, s_and); atomicOr(&st->hi_or, s_or); }
+}
+
+// ---- the k-th order key in one launch ------------------------------------------------------
+//
+// One cluster of P blocks, each with a slice of the list: a most-significant-digit radix
+// select in which a pass is a histogram in shared memory, ONE cluster barrier and the sum of the
+// P histograms over distributed shared memory, by every block alike. The bits of (new?, score)
+// that vary are settled first, over the slices; the keys of the entries that tie at that score
+// then stay in shared memory for the run key, and the select ends as soon as
+// every candidate that is left is among the k (usually two passes in all, three by frequency: a pass costs 2.5 us or so,
+// of which the barrier and the sums are most). As a chain of 13 launches of the whole grid the passes took
+// 52 us for the 262144 entries of a table. The cluster then places the entries of its list that stay (without a launch of
+// its own for that, and with a list that a thread holds in registers: 40.8 -> 37.5 us).
+constexpr int SELECT_THREADS = 1024, SELECT_MAX_BLOCKS = 16;
+
 __global__ void __launch_bounds__(SELECT_THREADS, 1)
-trim_select_kernel(unsigned int max_entries, unsigned int room, int64_t cap, void *lists, TrimState *st)
+trim_select_kernel(unsigned int room, const Table from, const Table to, int64_t cap, void *lists, TrimState *st, int place)
 {
     extern __shared__ __align__(16) unsigned long long s_keys[];   // [room]
     __shared__ unsigned int s_hist[2][256], s_sum[256];
     __shared__ unsigned int s_n, s_digit, s_run, s_in;
     const unsigned int P = gridDim.x, rank = blockIdx.x, lane = threadIdx.x & 31u;
-    chain_wait();
-    const unsigned int size = __ldcg(&st->size), k = size > max_entries ? size - max_entries : 0u;
-    const unsigned int n = (unsigned int)min((int64_t)__ldcg(&st->live.n), cap);
-    const unsigned long long hi_and = __ldcg(&st->live.hi_and), hi_or = __ldcg(&st->live.hi_or);
-    if (k == 0u) {                                          // nothing to drop: every block leaves (the others use none of what block 0 resets)
-        if (rank == 0 && threadIdx.x == 0) { st->k = 0u; st->n_list = n; reset_live(st->live); }
-        return;
-    }
+    chain_wait(true);                                       // (the next kernel reads the list in front of its own wait)
+    const unsigned int n = (unsigned int)min((int64_t)__ldcg(&st->n_list), cap), k = __ldcg(&st->k_rem);
+    const unsigned long long hi_and = __ldcg(&st->hi_and), hi_or = __ldcg(&st->hi_or);
     const TrimLists L = trim_lists(lists, cap);
+    if (rank == 0 && threadIdx.x == 0) st->size = __ldcg(&st->size) - __ldcg(&st->k);
+    if (place) {
+        if (rank == 0 && threadIdx.x < 256) st->bins[threadIdx.x] = 0u;   // for the next trim
+        const unsigned int late = __ldcg(&st->n_late);
+        for (unsigned int i = rank * SELECT_THREADS + threadIdx.x; i < late; i += P * SELECT_THREADS)
+            place_entry(to, cap, from.load(__ldcg(L.r_slot + (cap - 1 - (int64_t)i))));
+    }
+    if (n == 0u) return;                                    // nothing to find out: every block leaves
     const unsigned int per = (n + P - 1) / P, lo = min(rank * per, n), hi_end = min(lo + per, n);
+    // An entry for a thread at most (the clock of one batch, as a rule): it stays in registers, and what goes into the
+    // new table is on its way while the digits are counted.
+    const bool one = per <= SELECT_THREADS, have = one && lo + threadIdx.x < hi_end;
+    unsigned long long my_hi = 0ull;
+    Entry mine = {};
+    if (have) {
+        my_hi = __ldcg(L.r_hi + lo + threadIdx.x);
+        mine.key = __ldcg(L.r_key + lo + threadIdx.x);
+        if (place) mine = from.load(__ldcg(L.r_slot + lo + threadIdx.x));
+    }
     for (int i = threadIdx.x; i < 512; i += SELECT_THREADS) s_hist[i >> 8][i & 255] = 0u;
     if (threadIdx.x == 0) s_n = 0u;
     __syncthreads();
@@ -415,8 +575,10 @@ trim_select_kernel(unsigned int max_entries, unsigned int room, int64_t cap, voi
         }
         const unsigned int m1 = (1u << w1) - 1u, m2 = (1u << w2) - 1u;
         const unsigned long long known = ~todo;
+        const auto digit = [&](unsigned long long h) { return ((unsigned int)(h >> sh1) & m1) << w2 | ((unsigned int)(h >> sh2) & m2); };
         constexpr int U = 9;
-        for (unsigned int i0 = lo; i0 < hi_end; i0 += SELECT_THREADS * U) {
+        if (one) count_digit(s_hist[buf], digit(my_hi), have && (my_hi & known) == (thr_hi & known));
+        for (unsigned int i0 = one ? hi_end : lo; i0 < hi_end; i0 += SELECT_THREADS * U) {
             unsigned long long h[U];
 #pragma unroll
             for (int e = 0; e < U; ++e) {
@@ -425,8 +587,7 @@ trim_select_kernel(unsigned int max_entries, unsigned int room, int64_t cap, voi
             }
 #pragma unroll
             for (int e = 0; e < U; ++e)
-                count_digit(s_hist[buf], ((unsigned int)(h[e] >> sh1) & m1) << w2 | ((unsigned int)(h[e] >> sh2) & m2),
-                            i0 + e * SELECT_THREADS + threadIdx.x < hi_end && (h[e] & known) == (thr_hi & known));
+                count_digit(s_hist[buf], digit(h[e]), i0 + e * SELECT_THREADS + threadIdx.x < hi_end && (h[e] & known) == (thr_hi & known));
         }
         const unsigned int d = settle();
         const unsigned long long bits = (unsigned long long)m1 << sh1 | (unsigned long long)m2 << sh2;
@@ -445,7 +606,8 @@ trim_select_kernel(unsigned int max_entries, unsigned int room, int64_t cap, voi
             return f3 ? 192u + (f3 >> 10) : f2 ? 128u + (f2 >> 10) : (unsigned int)key >> 25;
         };
         constexpr int U = 9;
-        for (unsigned int i0 = lo; i0 < hi_end; i0 += SELECT_THREADS * U) {
+        if (one) count_digit(s_hist[buf], first_digit(mine.key), have && my_hi == thr_hi);
+        for (unsigned int i0 = one ? hi_end : lo; i0 < hi_end; i0 += SELECT_THREADS * U) {
             unsigned long long h[U], key[U];
 #pragma unroll
             for (int e = 0; e < U; ++e) {
@@ -478,7 +640,7 @@ trim_select_kernel(unsigned int max_entries, unsigned int room, int64_t cap, voi
         }
         __syncthreads();
         const bool held = s_n <= room;                      // else the slice is read again (a table trimmed late)
-        const unsigned int c_end = held ? s_n : hi_end - lo;
+        const unsigned int c_end = one ? 0u : held ? s_n : hi_end - lo;
         const unsigned int d = settle();
         int undecided;                                      // the lowest so many bits
         if (d >= 192u) { least = 1ull << 48; undecided = 58; thr_lo = (unsigned long long)(d - 192u) << 58; }
@@ -488,6 +650,8 @@ trim_select_kernel(unsigned int max_entries, unsigned int room, int64_t cap, voi
         while (undecided > 0 && n_match > k_rem) {
             const int w = min(8, undecided);
             undecided -= w;
+            if (one) count_digit(s_hist[buf], (unsigned int)(mine.key >> undecided) & ((1u << w) - 1u),
+                                 have && my_hi == thr_hi && mine.key >= least && (mine.key & decided) == thr_lo);
             for (unsigned int i0 = 0; i0 < c_end; i0 += SELECT_THREADS) {
                 const unsigned int i = i0 + threadIdx.x;
                 bool ok = i < c_end;
@@ -504,18 +668,21 @@ trim_select_kernel(unsigned int max_entries, unsigned int room, int64_t cap, voi
         }
     }
     thr_lo |= ~decided;                                     // every candidate left is among the k
-    od_cluster_arrive(); od_cluster_wait();                 // nobody leaves while its histogram may still be read
-    if (rank == 0 && threadIdx.x == 0) {
-        st->k = k; st->size = size - k;
-        st->thr_hi = thr_hi; st->thr_lo = thr_lo;
-        st->n_list = n;
-        reset_live(st->live);                               // (read by every block before its first barrier)
-    }
+    od_cluster_arrive();                                    // (waited for below: nobody leaves while its histogram may still be read)
+    if (place && have && (my_hi > thr_hi || (my_hi == thr_hi && mine.key > thr_lo))) place_entry(to, cap, mine);
+    if (place && !one)
+        for (unsigned int i = lo + threadIdx.x; i < hi_end; i += SELECT_THREADS) {
+            const unsigned long long hi = __ldcg(L.r_hi + i), key = __ldcg(L.r_key + i);
+            const Entry en = from.load(__ldcg(L.r_slot + i));   // (though some are dropped: one round trip less)
+            if (hi > thr_hi || (hi == thr_hi && key > thr_lo)) place_entry(to, cap, en);
+        }
+    od_cluster_wait();
+    if (rank == 0 && threadIdx.x == 0) { st->thr_hi = thr_hi; st->thr_lo = thr_lo; }
 }
 
 // ---- the same as a chain of launches, for tables too large for one cluster -----------------
 
-// Is digit `pass` the same in every live entry? Only asked for the five bytes of (new?, score).
+// Is digit `pass` the same in every listed entry? Only asked for the five bytes of (new?, score).
 __device__ __forceinline__ bool digit_is_constant(int pass, unsigned long long hi_and, unsigned long long hi_or)
 {
     return pass < 5 && (((hi_or & ~hi_and) >> (8 * (4 - pass))) & 0xFFull) == 0ull;
@@ -526,10 +693,10 @@ __device__ __forceinline__ bool digit_is_constant(int pass, unsigned long long h
 // same numbers. All threads of the block call; s_hist (256 words) and s_sel are its scratch.
 __device__ __forceinline__ SelState select_state(int pass, const TrimState *st, unsigned int *s_hist, SelState *s_sel)
 {
-    const TrimState::Live &live = st->live;
     if (pass == 0) {
-        SelState z = st->sel[0];
-        z.n_in = z.n_match = __ldcg(&live.n);
+        SelState z = {};
+        z.k_rem = __ldcg(&st->k_rem);
+        z.n_in = z.n_match = __ldcg(&st->n_list);
         return z;
     }
     const int q = pass - 1;                                  // the digit to settle
@@ -541,10 +708,9 @@ __device__ __forceinline__ SelState select_state(int pass, const TrimState *st, 
         t.mask_hi = __ldcg(&g->mask_hi); t.mask_lo = __ldcg(&g->mask_lo);
         t.k_rem = __ldcg(&g->k_rem); t.n_in = __ldcg(&g->n_in);
         t.n_match = __ldcg(&g->n_match); t.cur = __ldcg(&g->cur);
-        if (q == 0) t.n_in = t.n_match = __ldcg(&live.n);
         *s_sel = t;
     }
-    const unsigned long long hi_and = __ldcg(&live.hi_and), hi_or = __ldcg(&live.hi_or);
+    const unsigned long long hi_and = __ldcg(&st->hi_and), hi_or = __ldcg(&st->hi_or);
     const unsigned int n_out = __ldcg(&st->n_out[q]);
     __syncthreads();
     if (threadIdx.x < 32) {
@@ -608,10 +774,10 @@ __global__ void trim_hist_kernel(int pass, int64_t cap, void *lists, TrimState *
     __shared__ unsigned int s_base;
     __shared__ SelState s_sel;
     chain_wait();
-    if (st->k == 0u) return;                                 // nothing to drop: every block leaves
+    if (__ldcg(&st->n_list) == 0u) return;                   // nothing to find out: every block leaves
     const SelState S = select_state(pass, st, s_hist, &s_sel);
     if (blockIdx.x == 0 && threadIdx.x == 0) st->sel[pass] = S;
-    if (digit_is_constant(pass, __ldcg(&st->live.hi_and), __ldcg(&st->live.hi_or))) return;   // the next pass fills it in
+    if (digit_is_constant(pass, __ldcg(&st->hi_and), __ldcg(&st->hi_or))) return;   // the next pass fills it in
     __syncthreads();
     s_hist[threadIdx.x] = 0u;
     __syncthreads();
@@ -658,49 +824,43 @@ __global__ void trim_hist_kernel(int pass, int64_t cap, void *lists, TrimState *
     if (s_hist[threadIdx.x]) atomicAdd(&st->hist[pass][threadIdx.x], s_hist[threadIdx.x]);
 }
 
-// survivors of the dense list go into the (cleared) new table; which slot of its group an
-// entry gets depends on timing, the set of entries does not
-__global__ void trim_rebuild_kernel(unsigned long long *nkeys, int32_t *nvals, unsigned int *nstamp,
-                                    unsigned int *nfreq, unsigned int *nborn, int64_t cap, void *lists,
-                                    const TrimState *st, int selected)
+// The listed entries that stay, and the survivors that were not in the group their run hashes to, go into the new table;
+// which slot of its group an entry gets depends on timing, the set of entries does not.
+__global__ void __launch_bounds__(TRIM_THREADS)
+trim_place_kernel(const Table from, const Table to, int64_t cap, void *lists, TrimState *st, int selected)
 {
     __shared__ unsigned int s_hist[256];
     __shared__ SelState s_sel;
-    chain_wait();
+    asm volatile("griddepcontrol.launch_dependents;");
     const TrimLists L = trim_lists(lists, cap);
-    const unsigned int n = __ldcg(selected ? &st->n_list : &st->live.n), k = st->k;
-    unsigned long long thr_hi = 0ull, thr_lo = 0ull;
-    if (k > 0u) {                                           // block-uniform
-        if (selected) {
-            thr_hi = st->thr_hi; thr_lo = st->thr_lo;
-        } else {
+    const unsigned int i0 = blockIdx.x * TRIM_THREADS + threadIdx.x, stride = gridDim.x * TRIM_THREADS;
+    unsigned int n = 0u;
+    unsigned long long hi = 0ull;
+    Entry en = {};
+    const auto load = [&](unsigned int i) { hi = __ldcg(L.r_hi + i); en = from.load(__ldcg(L.r_slot + i)); };
+    if (selected) {                                         // the list was complete when trim_select_kernel let this kernel start
+        n = __ldcg(&st->n_list);
+        if (i0 < n) load(i0);
+    }
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    if (blockIdx.x == 0) st->bins[threadIdx.x] = 0u;        // for the next trim
+    unsigned long long thr_hi, thr_lo;
+    if (selected) {
+        thr_hi = __ldcg(&st->thr_hi); thr_lo = __ldcg(&st->thr_lo);
+    } else {
+        n = __ldcg(&st->n_list);
+        if (n > 0u) {                                       // block-uniform
             const SelState S = select_state(PASSES, st, s_hist, &s_sel);
             thr_hi = S.pre_hi; thr_lo = S.pre_lo;
+            if (i0 < n) load(i0);
         }
     }
-    const uint64_t ngroups = (uint64_t)cap / OD_GROUP;
-    for (unsigned int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-        // (all of it at once, though some are dropped: one round trip)
-        const unsigned long long hi = __ldcg(L.r_hi + i), key = __ldcg(L.r_key + i);
-        const int32_t v = __ldcg(L.r_val + i);
-        const unsigned int s = __ldcg(L.r_stamp + i), f = __ldcg(L.r_freq + i), b = __ldcg(L.r_born + i);
-        if (k > 0u && (hi < thr_hi || (hi == thr_hi && key <= thr_lo))) continue;   // among the k first: dropped
-        uint64_t g = od_hash64(key) & (ngroups - 1);
-        // A group is filled from its slot 0 without holes (od_cache_insert stops at the first
-        // empty slot). Every placement takes the next slot of its group from the group's
-        // counter: no two entries ever want the same slot, so there is nothing to retry and
-        // a placement is one atomic add and five stores. A full group (32 entries: rare in a
-        // table at most half full) sends the entry on to the next group, as a probe would go.
-        for (uint64_t step = 0; step < ngroups; ++step) {
-            const unsigned int at = atomicAdd(L.grp_fill + g, 1u);
-            if (at < (unsigned int)OD_GROUP) {
-                const int64_t ns = (int64_t)(g * OD_GROUP + at);
-                nkeys[ns] = key; nvals[ns] = v; nstamp[ns] = s; nfreq[ns] = f; nborn[ns] = b;
-                break;
-            }
-            g = (g + 1) & (ngroups - 1);
-        }
+    for (unsigned int i = i0; i < n; i += stride) {
+        if (i != i0) load(i);
+        if (hi > thr_hi || (hi == thr_hi && en.key > thr_lo)) place_entry(to, cap, en);   // the others are among the k first: dropped
     }
+    const unsigned int late = __ldcg(&st->n_late);
+    for (unsigned int i = i0; i < late; i += stride) place_entry(to, cap, from.load(__ldcg(L.r_slot + (cap - 1 - (int64_t)i))));
 }
 
 __global__ void trim_end_kernel(TrimState *st)
@@ -750,8 +910,11 @@ void select_config(cudaLaunchConfig_t &cfg, cudaLaunchAttribute *attr, const od_
     cfg.attrs = attr; cfg.numAttrs = 1;
 }
 
-// Blocks of the one-launch select: a cluster of 16, or of the portable 8, whose shared memory holds
-// the tying keys (393216 / 196608 entries); 0 = the table is too large for it.
+// Blocks of the one-launch select, 0 = the table is too large for it (393216 entries; 196608 where clusters of 16 are not
+// to be had): the list's keys have to fit in their shared memory. As few as give every thread an entry of the list, which
+// by LRU is one batch as a rule and by LFU most of the table (two a thread), and at most 16384 entries of the table to a
+// block in any case: a pass over a cluster of 1 to 4 blocks is shorter than one of 16 (4096 entries, 512 new ones: 23.9 us
+// with 16, 23.1 with 1; 32768 by LFU 35.6 with 8, 34.5 with 16).
 int select_blocks(const od_ctx *c)
 {
     if (cudaFuncSetAttribute(trim_select_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||
@@ -759,16 +922,24 @@ int select_blocks(const od_ctx *c)
         cudaGetLastError();
         return 0;
     }
-    for (int blocks = SELECT_MAX_BLOCKS; blocks >= 8; blocks /= 2) {
+    const int64_t entries = c->dyn_max + c->dyn_max_insert;
+    const int64_t want = c->dyn_policy == 0 ? std::max<int64_t>((c->dyn_max_insert + SELECT_THREADS - 1) / SELECT_THREADS, (entries + 16383) / 16384)
+                                            : (entries + 2 * SELECT_THREADS - 1) / (2 * SELECT_THREADS);
+    int blocks = 1, best = 0;
+    for (; blocks <= SELECT_MAX_BLOCKS; blocks *= 2) {
         if (select_room(c, blocks) > SELECT_ROOM_MAX) continue;
         cudaLaunchConfig_t cfg = {};
         cudaLaunchAttribute attr[2];
         select_config(cfg, attr, c, blocks);
         int n = 0;
-        if (cudaOccupancyMaxActiveClusters(&n, trim_select_kernel, &cfg) == cudaSuccess && n > 0) return blocks;
-        cudaGetLastError();
+        if (cudaOccupancyMaxActiveClusters(&n, trim_select_kernel, &cfg) != cudaSuccess || n < 1) {
+            cudaGetLastError();
+            continue;
+        }
+        best = blocks;
+        if (blocks >= want) break;
     }
-    return 0;
+    return best;
 }
 
 }  // namespace
@@ -776,10 +947,11 @@ int select_blocks(const od_ctx *c)
 void od_cache_free_dynamic(od_ctx *c)
 {
     void *ptrs[] = {c->d_stamp, c->d_freq, c->d_born, c->d_keys2, c->d_vals2, c->d_stamp2, c->d_freq2,
-                    c->d_born2, c->d_owner, c->d_cand_slot, c->d_trim, c->d_trim_lists};
+                    c->d_born2, c->d_fill, c->d_fill2, c->d_owner, c->d_cand_slot, c->d_trim, c->d_trim_lists};
     for (void *p : ptrs)
         if (p) cudaFree(p);
     c->d_stamp = c->d_freq = c->d_born = c->d_stamp2 = c->d_freq2 = c->d_born2 = c->d_owner = nullptr;
+    c->d_fill = c->d_fill2 = nullptr;
     c->d_keys2 = nullptr; c->d_vals2 = nullptr; c->d_cand_slot = nullptr; c->d_trim = nullptr;
     c->d_trim_lists = nullptr;
     c->dyn = false;
@@ -812,6 +984,8 @@ int32_t od_cache_configure(od_ctx *c, int64_t max_entries, int32_t policy, int32
     if (st == OD_OK) st = alloc_zero(&c->d_stamp2, (size_t)cap);
     if (st == OD_OK) st = alloc_zero(&c->d_freq2, (size_t)cap);
     if (st == OD_OK) st = alloc_zero(&c->d_born2, (size_t)cap);
+    if (st == OD_OK) st = alloc_zero(&c->d_fill, fill_words(cap));
+    if (st == OD_OK) st = alloc_zero(&c->d_fill2, fill_words(cap));
     if (st == OD_OK) st = alloc_zero(&c->d_owner, (size_t)cap);
     if (st == OD_OK) st = alloc_zero(&c->d_cand_slot, (size_t)max_insert);
     TrimState *ts = nullptr;
@@ -826,9 +1000,6 @@ int32_t od_cache_configure(od_ctx *c, int64_t max_entries, int32_t policy, int32
     OD_CUDA(cudaMemset(c->d_owner, 0xFF, (size_t)cap * sizeof(uint32_t)));
     c->cap = cap;
     c->table_written = true;
-    TrimState *dst = (TrimState *)c->d_trim;
-    const TrimState::Live empty = {0u, ~0ull, 0ull};
-    OD_CUDA(cudaMemcpy(&dst->live, &empty, sizeof(empty), cudaMemcpyHostToDevice));
     c->dyn = true; c->dyn_policy = policy; c->dyn_max = max_entries; c->dyn_max_insert = max_insert;
     c->clock = 0;
     c->trim_blocks = select_blocks(c);
@@ -859,7 +1030,7 @@ int32_t od_cache_insert(od_ctx *c, int32_t N, const int32_t *runs, const int32_t
     const bool pdl = c->opt_pdl != 0;
     OD_CUDA(chain_launch(insert_claim_kernel, (unsigned)blocks, (unsigned)threads, s, pdl, N, c->v_q, c->v_p, runs, len,
                          target, (unsigned long long *)c->d_keys, (const int32_t *)c->d_vals, c->cap,
-                         c->d_owner, c->d_cand_slot, (TrimState *)c->d_trim));
+                         c->d_owner, c->d_cand_slot, c->d_fill, (TrimState *)c->d_trim));
     OD_CUDA(chain_launch(insert_commit_kernel, (unsigned)blocks, (unsigned)threads, s, pdl, N, target, c->d_vals,
                          c->d_stamp, c->d_freq, c->d_born, c->d_owner, (const int32_t *)c->d_cand_slot,
                          c->clock, (TrimState *)c->d_trim));
@@ -876,38 +1047,43 @@ int32_t od_cache_trim(od_ctx *c, void *stream)
     cudaStream_t s = (cudaStream_t)stream;
     c->table_written = true;
     TrimState *st = (TrimState *)c->d_trim;
-    // What is resident at a time, and no more blocks than have anything to do (4 or 5 to a multiprocessor: the pass
-    // over the table with 5 in place of 4 makes 62.5 us in a row 61.4, the rebuild with 8 in place of 4 57.0 -> 57.4)
-    const int wave = (int)std::min<int64_t>(c->sm_count * 5, (c->cap + 1023) / 1024);
-    const int grid = (int)std::min<int64_t>(c->sm_count * 4, (c->dyn_max + c->dyn_max_insert + 255) / 256);
+    // one resident wave at most, and no more blocks than have anything to do
+    const int64_t most = c->sm_count * 4;
+    const unsigned passes = (unsigned)std::min<int64_t>(most, (c->cap / OD_GROUP + QUAD * TRIM_HALVES - 1) / (QUAD * TRIM_HALVES));
+    const unsigned place = (unsigned)std::min<int64_t>(most, (c->dyn_max + c->dyn_max_insert + TRIM_THREADS - 1) / TRIM_THREADS);
     const bool pdl = c->opt_pdl != 0;
     const int blocks = c->trim_blocks;                      // 0: the select is a chain of launches
+    // The select's cluster places what it leaves of the list by itself, which spares a launch, but by LFU, where the list
+    // is long: most entries have a frequency of one, where a clock is that of one batch.
+    const bool placed = blocks && c->dyn_policy == 0;
+    const Table from = {(unsigned long long *)c->d_keys, c->d_vals, c->d_stamp, c->d_freq, c->d_born, c->d_fill};
+    const Table to = {(unsigned long long *)c->d_keys2, c->d_vals2, c->d_stamp2, c->d_freq2, c->d_born2, c->d_fill2};
     if (!blocks) OD_CUDA(chain_launch(trim_begin_kernel, 1u, 256u, s, pdl, st, (unsigned int)c->dyn_max));
-    OD_CUDA(chain_launch(trim_compact_kernel, (unsigned)wave, 256u, s, pdl, c->dyn_policy, c->clock,
-                         (const unsigned long long *)c->d_keys, (const int32_t *)c->d_vals,
-                         (const unsigned int *)c->d_stamp, (const unsigned int *)c->d_freq,
-                         (const unsigned int *)c->d_born, (unsigned long long *)c->d_keys2, c->d_vals2,
-                         c->cap, c->d_trim_lists, st));
+    OD_CUDA(chain_launch(trim_count_kernel, passes, (unsigned)TRIM_THREADS, s, pdl, c->dyn_policy, c->clock, from.vals,
+                         c->dyn_policy == 0 ? from.stamp : from.freq, from.born, c->cap, st));
+    OD_CUDA(chain_launch(trim_split_kernel, passes, (unsigned)TRIM_THREADS, s, pdl, c->dyn_policy, c->clock,
+                         (unsigned int)c->dyn_max, from, to, c->cap, c->d_trim_lists, st));
     if (blocks) {
         cudaLaunchConfig_t cfg = {};
         cudaLaunchAttribute attr[2];
         select_config(cfg, attr, c, blocks);
         cfg.stream = s;
         cfg.numAttrs = pdl ? 2 : 1;
-        OD_CUDA(cudaLaunchKernelEx(&cfg, trim_select_kernel, (unsigned int)c->dyn_max, select_room(c, blocks), c->cap,
-                                   c->d_trim_lists, st));
+        OD_CUDA(cudaLaunchKernelEx(&cfg, trim_select_kernel, select_room(c, blocks), from, to, c->cap, c->d_trim_lists, st,
+                                   placed ? 1 : 0));
     } else {
         for (int pass = 0; pass < PASSES; ++pass)
             OD_CUDA(chain_launch(trim_hist_kernel, (unsigned)c->sm_count, 256u, s, pdl, pass, c->cap,
                                  c->d_trim_lists, st));
     }
-    OD_CUDA(chain_launch(trim_rebuild_kernel, (unsigned)grid, 256u, s, pdl, (unsigned long long *)c->d_keys2,
-                         c->d_vals2, c->d_stamp2, c->d_freq2, c->d_born2, c->cap, c->d_trim_lists,
-                         (const TrimState *)st, blocks ? 1 : 0));
+    if (!placed)
+        OD_CUDA(chain_launch(trim_place_kernel, place, (unsigned)TRIM_THREADS, s, pdl, from, to, c->cap, c->d_trim_lists,
+                             st, blocks ? 1 : 0));
     if (!blocks) OD_CUDA(chain_launch(trim_end_kernel, 1u, 1u, s, pdl, st));
     // the rebuilt table is the table for every call enqueued from now on
     std::swap(c->d_keys, c->d_keys2); std::swap(c->d_vals, c->d_vals2);
     std::swap(c->d_stamp, c->d_stamp2); std::swap(c->d_freq, c->d_freq2); std::swap(c->d_born, c->d_born2);
+    std::swap(c->d_fill, c->d_fill2);
     return OD_OK;
 }
 

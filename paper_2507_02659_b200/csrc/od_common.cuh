@@ -62,11 +62,12 @@ struct od_ctx {
     uint32_t *d_stamp, *d_freq, *d_born;            // [cap]
     uint64_t *d_keys2; int32_t *d_vals2;            // [cap] spare table
     uint32_t *d_stamp2, *d_freq2, *d_born2;
+    uint32_t *d_fill, *d_fill2;     // [cap / 32] slots taken in each group, of the table and of the spare one
     uint32_t *d_owner;              // [cap] first-wins claims of a batch (0xFFFFFFFF = none)
     int32_t *d_cand_slot;           // [dyn_max_insert]
     void *d_trim;                   // trim / size state (device)
     int32_t trim_blocks;            // blocks of the one-launch select, 0 = the table is too large for it
-    void *d_trim_lists;             // trim scratch: the live entries' records and two candidate lists, 64 bytes per slot
+    void *d_trim_lists;             // trim scratch: the listed entries and two candidate lists, 52 bytes per slot
 
     // od_verify scratch
     float4 *d_partials;             // [rows][OD_VERIFY_SEG_MAX] (c, sum, max, -), rows of one launch

@@ -375,3 +375,43 @@ def test_a_full_table_counts_what_it_loses(cuda_device):
     assert set(held) <= seen
     ctx.close()
 
+
+
+@pytest.mark.parametrize("policy", [cp.LRU, cp.LFU])
+@pytest.mark.parametrize("bound, batch", [(100, 28), (8, 24), (2000, 48), (60000, 30000)])
+def test_trim_of_a_table_filled_to_the_brim(cuda_device, policy, bound, batch):
+    """Insertions without a trim until almost every slot is taken: entries stand in groups that their run does not hash
+    to, and groups beyond their first sixteen slots; clocks far enough apart for bins of many scores."""
+    rng = np.random.default_rng(90 + bound)
+    v_q, v_p, dev = 60, 300, cuda_device
+    cap = 64
+    while cap < 2 * (bound + batch):
+        cap *= 2
+    ctx = od.Context(dev, v_q, v_p, 64, 4)
+    ctx.set_vocab_map(np.full(v_q, -1, np.int32))
+    ctx.cache_configure(bound, policy, batch)
+    ref = cp.DynamicCache(bound, policy, v_q, v_p)
+    clock = 1
+    for turn in range(3):
+        while len(ref) + batch <= cap * 31 // 32:
+            clock += int(rng.choice([1, 3, 40, 200, 5000]))
+            ctx.cache_set_clock(clock); ref.set_clock(clock)
+            runs, lens = _universe(rng, batch, v_q)
+            tg = rng.integers(0, v_p, size=batch).astype(np.int32)
+            ctx.cache_insert(torch.from_numpy(runs).to(dev), torch.from_numpy(lens).to(dev), torch.from_numpy(tg).to(dev))
+            ref.insert_batch(runs, lens, tg)
+            # accesses: a few runs often, up to 150 times a batch
+            d = np.zeros((64, 4), np.int32)
+            klen = np.zeros(64, np.int32)
+            for b in range(64):
+                i = int(rng.integers(0, batch)) if b < 60 else 0
+                klen[b] = lens[i]; d[b] = runs[i]
+            for _ in range(int(rng.choice([1, 1, 30]))):
+                od.od_map_proposals(ctx, torch.from_numpy(d).to(dev), torch.from_numpy(klen).to(dev), torch.rand(64, 4, device=dev))
+                for b in range(64):
+                    ref.map_sequence(np.full(v_q, -1, np.int32), d[b, :klen[b]], np.ones(4, np.float32))
+        _compare(ctx, ref)
+        ctx.cache_trim(); ref.trim()
+        assert len(ref) == bound and ctx.cache_stats() == (bound, 0, 0)
+        _compare(ctx, ref)
+    ctx.close()
