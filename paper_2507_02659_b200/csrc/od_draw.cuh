@@ -274,6 +274,15 @@ struct WarpTiles {                                          // the warp's own ru
         if ((lane & 15) == 0 && (lane == 0 || two)) val[t - t_lo + (lane >> 4)] = v;
         total += (double)v;
     }
+    // tile t's value is another
+    __device__ __forceinline__ void replace(int t, float v)
+    {
+        v = fmaxf(0.f, v);
+        __syncwarp();
+        if (lane < 16) total += (double)v - (double)val[t - t_lo];
+        __syncwarp();
+        if (lane == 0) val[t - t_lo] = v;
+    }
     __device__ __forceinline__ double sum() const
     {
         return __shfl_sync(0xFFFFFFFFu, total, 0) + __shfl_sync(0xFFFFFFFFu, total, 16);
@@ -321,8 +330,10 @@ __device__ __forceinline__ void load_tile(const SeqState &q, int tile, int lane,
 // A lane's eight ids of a whole tile: the sum of their residuals, or of e alone. A tile is 256
 // ids of work for one warp, and its instructions bound a large batch: 276 a tile and 66.8 us for
 // 296 staged rows of 152064 ids with a branch per id, 195 and 51.9 us with a select per id,
-// 154 and 44.8 us so: an unmapped id's multiply-add is predicated off, and Eq. (2)'s two ids are
-// looked for only in the tiles that hold them. (The clamp at zero as the multiply-add's own .sat is 0.8 % of
+// 154 and 44.8 us with an unmapped id's multiply-add predicated off and Eq. (2)'s two ids looked for in every tile. Now
+// those tiles are evaluated once more behind the pass (a test less in each tile), and the staging does without a base
+// for each group of its list: the step of 296 such rows 89.9 -> 87.4 us, 512 with eight tokens 271.4 -> 266.8, 64 of 128256 ids
+// 28.65 -> 28.1, 100 of 90001 fp32 ids 43.0 -> 41.8. (The clamp at zero as the multiply-add's own .sat is 0.8 % of
 // the step faster, but clamps at one too, which e(M) may exceed by c's rounding; with the residuals as
 // halves, to allow for that, it is no faster than the maximum.)
 template <int DTYPE>
@@ -386,7 +397,7 @@ __device__ __forceinline__ float tile_lane_sum_staged(const SeqState &q, const S
             "@p fma.rn.f32 %0, v, %2, %0;\n\t"
             "@p add.u32 %1, %1, 4; max.f32 %0, %0, 0f00000000;}"
             : "+f"(r[k]), "+r"(rank_at) : "f"(nS), "r"(oct), "r"(1u << k) : "memory");
-    return with_eq2_ids<DTYPE>(q, a, tile, lane, r);
+    return sum_of_eight(r);
 }
 
 // The lanes' sums of two tiles: lanes 0..15 end with the first tile's value, lanes 16..31 with the second's.
@@ -805,18 +816,13 @@ struct Part {
     int p_lo, p_hi, p_hi_w;
     int4 ni[2][2];
     uint32_t word[EB];
-    int32_t base[EB];
     int4 list;
-    int g_at;
+    int g_at;                                               // the group of word[0]
     __device__ __forceinline__ void load_words(const SampleArgs &a, int lane)
     {
 #pragma unroll
-        for (int e = 0; e < EB; ++e) {
-            const bool in = g_at + e * CWARPS < list.y;
-            word[e] = in ? __ldg(a.list_word + (size_t)(g_at + e * CWARPS) * 32 + lane) : 0xFFFFu;
-            base[e] = in ? __ldg(a.list_base + g_at + e * CWARPS) : 0;
-        }
-        g_at += EB * CWARPS;
+        for (int e = 0; e < EB; ++e)
+            word[e] = g_at + e * CWARPS < list.y ? __ldg(a.list_word + (size_t)(g_at + e * CWARPS) * 32 + lane) : 0xFFFFu;
     }
     __device__ __forceinline__ void prepare(const SampleArgs &a, int part, int warp, int lane)
     {
@@ -899,8 +905,12 @@ __device__ __forceinline__ void draw(const SampleArgs &a, const Ahead &h, Part<S
 #pragma unroll
             for (int e = 0; e < EB; ++e) {
                 at[e] = my.word[e] & 0xFFFFu;
-                if (at[e] != 0xFFFFu) x[e] = __ldg(q.q_row + my.base[e] + (int)(my.word[e] >> 16));
+                if (at[e] == 0xFFFFu) continue;
+                const float *from = q.q_row + (my.word[e] >> 16);
+                if (a.v_q > 65536) from += __ldg(a.list_base + my.g_at + e * CWARPS);   // (else there is one page of draft ids)
+                x[e] = __ldg(from);
             }
+            my.g_at += EB * CWARPS;
             const bool more = my.g_at < my.list.y;             // the same for every lane of a warp
             if (more) my.load_words(a, lane);
 #pragma unroll
@@ -910,6 +920,15 @@ __device__ __forceinline__ void draw(const SampleArgs &a, const Ahead &h, Part<S
         }
         __syncthreads();
         warp_tiles_ahead<DTYPE, STAGED>(q, a, sr, p_lo, hi_w, lane, out, cur);
+        // Eq. (2)'s two ids, which the pass above does not look for: their tiles once more
+#pragma unroll 1
+        for (int i = 0; i < 2; ++i) {
+            const int id = i == 0 ? q.prefix_token : q.ngram_token, t = id / OD_SAMPLE_TILE;
+            if (id < 0 || t < p_lo || t >= hi_w) continue;
+            float r[EPT];
+            tile_values<DTYPE>(q, a, true, t, lane, r, &sr);
+            out.replace(t, warp_sum_f32(sum_of_eight(r)));
+        }
         if (hi_w < p_hi) warp_tiles_dense<DTYPE, 1>(q, a, true, max(hi_w, p_lo), p_hi, lane, out);
     } else {
         warp_run<DTYPE, SOURCE>(q, a, p_lo, p_hi, hi_w, lane, out, my.ni);

@@ -132,3 +132,11 @@ def test_a_smaller_context_made_after_a_larger_one(cuda_device):
     assert int((so.flags | sh.flags)[0]) & od.OD_SF_BOUNDARY or torch.equal(sh.out_token, so.out_token)
     other.close()
     ctx.close()
+
+
+@pytest.mark.parametrize("dtype", ["bf16", "f32"])
+def test_staged_ids_beyond_one_page_of_draft_ids(cuda_device, dtype):
+    """Over 65536 draft ids: the groups of the staging lists have bases of their own."""
+    w = _workload(B=5, k_max=3, v_q=70001, v_p=90001, mapped_frac=0.6, cache_entries=0, logit_dtype=dtype)
+    st = synth.make_static(w)
+    assert {2, 16} <= {b for tiles in (0, 3, 1000) for b in _check(w, st, cuda_device, tiles, 2)}
