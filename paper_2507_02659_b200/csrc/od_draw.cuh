@@ -324,8 +324,13 @@ template <int DTYPE>
 __device__ __forceinline__ void load_tile(const SeqState &q, int tile, int lane, uint4 *raw)
 {
     const uint4 *src = (const uint4 *)(q.row + (size_t)(tile * OD_SAMPLE_TILE + lane * EPT) * (DTYPE == OD_BF16 ? 2 : 4));
-    raw[0] = ld_once(src);
-    if (DTYPE != OD_BF16) raw[1] = ld_once(src + 1);
+    // (fp32 rows through L1, where the draw finds its tile again: three calls of 19 sequences of 100277 ids 20.9 -> 20.3 us;
+    // bf16 rows gain nothing by it, a batch of 296 loses 2.5 %)
+    if (DTYPE == OD_BF16) {
+        raw[0] = ld_once(src);
+    } else {
+        raw[0] = __ldg(src); raw[RAW<DTYPE> - 1] = __ldg(src + 1);
+    }
 }
 // A lane's eight ids of a whole tile: the sum of their residuals, or of e alone. A tile is 256
 // ids of work for one warp, and its instructions bound a large batch: 276 a tile and 66.8 us for
@@ -493,7 +498,8 @@ struct TileLoads {
 // Pass 1 over whole tiles [t_lo, t_hi) without the inverse map: the loads of the next tiles are
 // issued before the current ones are worked on. cur: the first two tiles', which the caller
 // requested (FROM_ROW keeps one tile ahead only, for its registers).
-template <int DTYPE, int SOURCE, typename Sink>
+// LONE: many warps have one tile alone (the step in one launch), and do not work on it twice.
+template <int DTYPE, int SOURCE, bool LONE, typename Sink>
 __device__ __forceinline__ void warp_tiles_ahead(const SeqState &q, const SampleArgs &a, const StagedRow &sr, int t_lo, int t_hi,
                                                  int lane, Sink &out, TileLoads<DTYPE, SOURCE> (&cur)[SOURCE == FROM_ROW ? 1 : 2])
 {
@@ -503,10 +509,10 @@ __device__ __forceinline__ void warp_tiles_ahead(const SeqState &q, const Sample
         float s0, s1;
         if (SOURCE == FROM_ROW) {
             TileLoads<DTYPE, SOURCE> nx;
-            nx.load(q, a, two ? t + 1 : t, lane);
+            if (!LONE || two) nx.load(q, a, two ? t + 1 : t, lane);
             s0 = cur[0].sum(q, a, sr, t, lane);
             if (t + 2 < t_hi) cur[0].load(q, a, t + 2, lane);
-            s1 = nx.sum(q, a, sr, t + 1, lane);
+            s1 = !LONE || two ? nx.sum(q, a, sr, t + 1, lane) : 0.f;
         } else {
             TileLoads<DTYPE, SOURCE> nx[2];
             if (t + 2 < t_hi) {
@@ -514,7 +520,7 @@ __device__ __forceinline__ void warp_tiles_ahead(const SeqState &q, const Sample
                 nx[1].load(q, a, min(t + 3, t_hi - 1), lane);
             }
             s0 = cur[0].sum(q, a, sr, t, lane);
-            s1 = cur[SOURCE == FROM_ROW ? 0 : 1].sum(q, a, sr, t + 1, lane);
+            s1 = !LONE || two ? cur[SOURCE == FROM_ROW ? 0 : 1].sum(q, a, sr, t + 1, lane) : 0.f;
             cur[0] = nx[0]; cur[SOURCE == FROM_ROW ? 0 : 1] = nx[1];
         }
         out.pair(t, pair_sum(s0, s1, lane), two);
@@ -539,7 +545,8 @@ __device__ __forceinline__ void first_tiles(const SeqState &q, const SampleArgs 
 struct Ahead {
     int mb;
     bool stop;
-    float T;
+    float T, scale;                     // scale: log2(e) / T
+    float u_draw;                       // the uniform of a draw at position `lane` (where it was worked out ahead)
     int32_t l_len, l_tgt;               // piece `lane`: its length, target id
     float l_qp;                         // and q'
     int32_t s0, len, tgt, d1, pm;       // position `lane`: row of the drafter, length of the piece there (1 at a stop);
@@ -587,6 +594,7 @@ __device__ __forceinline__ Ahead load_ahead(const SampleArgs &a, int b, int lane
     int mb = a.m[b];
     h.stop = a.tail_kind[b] == OD_TAIL_UNMAPPED_STOP;
     h.T = a.temperature[b];
+    h.scale = 1.4426950408889634f / h.T;
     int32_t l_s0 = 0, l_did = -1;
     h.l_len = 1; h.l_tgt = -1; h.l_qp = 0.f;
     if (lane < K) {
@@ -612,7 +620,7 @@ __device__ __forceinline__ SeqState seq_state(const SampleArgs &a, const Ahead &
     const size_t esz = DTYPE == OD_BF16 ? 2 : 4;
     SeqState q;
     q.row = (const char *)a.logits + ((size_t)b * a.seq_stride + (size_t)j * a.row_stride) * esz - (size_t)col0 * esz;
-    q.scale = 1.4426950408889634f / h.T;
+    q.scale = h.scale;
     {
         // reference exponent c = fl(M*scale), od_verify's own, so that the errors of e(t) are those of the
         // row sum (a margin on it, to keep e(t) below one, made the residual mass's mean error 5 to 10 %
@@ -660,7 +668,7 @@ __device__ __forceinline__ void prefetch_q_row(const SampleArgs &a, const SeqSta
 
 // A warp's run of tiles [t_lo, t_hi): whole tiles pipelined, the row's ragged last tile (if it is
 // this warp's) on its own. ni: the first pair's inverse-map entries (not read where ids are shared).
-template <int DTYPE, int SOURCE, typename Sink>
+template <int DTYPE, int SOURCE, bool LONE, typename Sink>
 __device__ __forceinline__ void warp_run(const SeqState &q, const SampleArgs &a, int t_lo, int t_hi, int hi_w, int lane,
                                          Sink &out, int4 (&ni)[2][2])
 {
@@ -669,11 +677,11 @@ __device__ __forceinline__ void warp_run(const SeqState &q, const SampleArgs &a,
     if (!q.residual) {
         TileLoads<DTYPE, FREE> cur[2];
         first_tiles<DTYPE, FREE>(q, a, t_lo, hi_w, lane, cur);
-        warp_tiles_ahead<DTYPE, FREE>(q, a, none, t_lo, hi_w, lane, out, cur);
+        warp_tiles_ahead<DTYPE, FREE, LONE>(q, a, none, t_lo, hi_w, lane, out, cur);
     } else if (SOURCE == FROM_ROW) {
         TileLoads<DTYPE, FROM_ROW> cur[1];
         first_tiles<DTYPE, FROM_ROW>(q, a, t_lo, hi_w, lane, cur);
-        warp_tiles_ahead<DTYPE, FROM_ROW>(q, a, none, t_lo, hi_w, lane, out, cur);
+        warp_tiles_ahead<DTYPE, FROM_ROW, LONE>(q, a, none, t_lo, hi_w, lane, out, cur);
     } else if (SOURCE == FROM_MAP && t_lo < hi_w) {
         warp_tiles_dense_piped<DTYPE>(q, a, t_lo, hi_w, lane, out, ni);
     }
@@ -711,12 +719,7 @@ __device__ __forceinline__ bool pick_in_tile(const SeqState &q, const SampleArgs
         if (my_pick == 0x7FFFFFFF && nc > target) { my_pick = t0 + e; lo = c; hi = nc; }
         c = nc;
     }
-    int pick = my_pick, last = my_last;
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
-        pick = min(pick, __shfl_xor_sync(0xFFFFFFFFu, pick, off));
-        last = max(last, __shfl_xor_sync(0xFFFFFFFFu, last, off));
-    }
+    const int pick = __reduce_min_sync(0xFFFFFFFFu, my_pick), last = __reduce_max_sync(0xFFFFFFFFu, my_last);
     const float R = (float)(Rn / (double)q.S);              // residual mass (1 for the free token)
     if (pick != 0x7FFFFFFF) {
         if (my_pick == pick) {                              // exactly one lane owns the picked id
@@ -746,6 +749,10 @@ __device__ __forceinline__ bool pick_in_tile(const SeqState &q, const SampleArgs
 // them block-wide; 3.2 with all P * 16 run sums exchanged and scanned by every warp).
 // The whole step, device time: one sequence of 32000 fp32 ids 13.3 -> 12.0 us, 24 of 128256 bf16
 // ids 24.2 -> 22.6, 64 31.7 -> 29.7, 512 of 152064 286 -> 273, 256 of 32000 (same tokenizer) 44.2 -> 37.0.
+// A block costs about 10 us whatever its share of the tiles (512 sequences with 1, 2, 4 parts: 270, 278, 308 us), and every
+// warp of it goes through the same chain, so its instructions count sixteen times: integer sums and
+// minima in one instruction, the draw's uniform for every position ahead of the wait, the divisions that find a row's
+// partials too, no second tile for a warp with one: 256 of 32000 34.7 -> 33.8, 64 of 128256 28.1 -> 27.5, one of 32000 fp32 8.66 -> 8.3.
 // FUSED: the launch in front is the streaming pass of od_verify itself; its decide kernel is
 // folded into this kernel's prologue (see SampleArgs).
 constexpr int CWARPS = 16, CTHREADS = CWARPS * 32;
@@ -853,19 +860,15 @@ __device__ __forceinline__ int decide(const SampleArgs &a, const Ahead &h, int b
     bool acc = false, bnd = false;
     Acceptance d = {};
     if (lane < mb) {
-        d = accept_position(rm, rs, bad_T ? 0.f : 1.4426950408889634f / h.T, t_ok, x_t, h.l_qp, u);
+        d = accept_position(rm, rs, bad_T ? 0.f : h.scale, t_ok, x_t, h.l_qp, u);
         acc = d.accept; bnd = d.boundary;
     }
     const unsigned int accmask = __ballot_sync(0xFFFFFFFFu, acc);
-    int j = 0;
-    while (j < mb && (accmask >> j & 1u)) ++j;
-    if (bad_T) j = 0;
+    const int j = bad_T ? 0 : __ffs((int)~accmask) - 1;     // (no position beyond mb <= OD_MAX_K is accepted)
     if (store) {
         if (lane < mb) { a.w_p_sel[(size_t)b * K + lane] = d.p; a.w_ratio[(size_t)b * K + lane] = d.ratio; }
         const unsigned int bndmask = __ballot_sync(0xFFFFFFFFu, bnd);
-        int nd = lane < j ? h.l_len : 0;
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) nd += __shfl_xor_sync(0xFFFFFFFFu, nd, off);
+        const int nd = __reduce_add_sync(0xFFFFFFFFu, lane < j ? h.l_len : 0);
         if (lane == 0) {
             uint32_t f = bndmask & OD_VF_BOUNDARY_MASK;
             if (vbits & 1u) f |= OD_VF_NONFINITE;
@@ -878,7 +881,8 @@ __device__ __forceinline__ int decide(const SampleArgs &a, const Ahead &h, int b
 
 // The draw at position j by the cluster of a sequence (every thread calls). STARTED: the cluster has met at
 // a barrier already, so every block of it runs; else the caller has arrived (relaxed) at the first one.
-template <int DTYPE, int SOURCE, bool STARTED>
+// AHEAD: h.u_draw is there.
+template <int DTYPE, int SOURCE, bool STARTED, bool AHEAD>
 __device__ __forceinline__ void draw(const SampleArgs &a, const Ahead &h, Part<SOURCE> &my, int b, unsigned part, unsigned nparts,
                                      int warp, int lane, int j, float rm, float rs, bool planned, float *s_q, float *s_val)
 {
@@ -893,7 +897,7 @@ __device__ __forceinline__ void draw(const SampleArgs &a, const Ahead &h, Part<S
     // ---- pass 1: the value of every tile; the ragged last one (all of them, if the map is another) one by one ----
     WarpTiles out = {s_val, lane, p_lo, 0.0};
     const int hi_w = planned ? my.p_hi_w : p_lo;
-    const uint64_t seed_b = a.seed[b];
+    const uint64_t seed_b = AHEAD ? 0ull : a.seed[b];
     const StagedRow sr = {s_q, a.octet, (uint32_t)my.list.z};
     if (SOURCE == STAGED && q.residual) {
         TileLoads<DTYPE, STAGED> cur[2];
@@ -919,7 +923,7 @@ __device__ __forceinline__ void draw(const SampleArgs &a, const Ahead &h, Part<S
             if (!more) break;
         }
         __syncthreads();
-        warp_tiles_ahead<DTYPE, STAGED>(q, a, sr, p_lo, hi_w, lane, out, cur);
+        warp_tiles_ahead<DTYPE, STAGED, STARTED>(q, a, sr, p_lo, hi_w, lane, out, cur);
         // Eq. (2)'s two ids, which the pass above does not look for: their tiles once more
 #pragma unroll 1
         for (int i = 0; i < 2; ++i) {
@@ -931,9 +935,9 @@ __device__ __forceinline__ void draw(const SampleArgs &a, const Ahead &h, Part<S
         }
         if (hi_w < p_hi) warp_tiles_dense<DTYPE, 1>(q, a, true, max(hi_w, p_lo), p_hi, lane, out);
     } else {
-        warp_run<DTYPE, SOURCE>(q, a, p_lo, p_hi, hi_w, lane, out, my.ni);
+        warp_run<DTYPE, SOURCE, STARTED>(q, a, p_lo, p_hi, hi_w, lane, out, my.ni);
     }
-    const float u = od_uniform(seed_b, a.step, (uint32_t)j, 1u);
+    const float u = AHEAD ? __shfl_sync(0xFFFFFFFFu, h.u_draw, j) : od_uniform(seed_b, a.step, (uint32_t)j, 1u);
 
     // ---- the sums: of the runs inside the block, of the block to every block of the cluster
     const double run_sum = out.sum();

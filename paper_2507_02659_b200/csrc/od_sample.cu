@@ -107,7 +107,7 @@ od_sample_kernel(const SampleArgs a)
 
     // FUSED, still before the wait: where the rows' partials will be (sums of m), and position
     // k's inputs of the acceptance test in lane k
-    int before = 0, total = 0;
+    int before = 0, total = 0, segments = 0;
     float d_xt = 0.f, d_u = 0.f;
     bool d_tok = false;
     if (threadIdx.x == 0) s_vbits = 0;
@@ -117,22 +117,22 @@ od_sample_kernel(const SampleArgs a)
             total += v;
             if (i < b) before += v;
         }
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) {
-            before += __shfl_xor_sync(0xFFFFFFFFu, before, off);
-            total += __shfl_xor_sync(0xFFFFFFFFu, total, off);
-        }
+        before = __reduce_add_sync(0xFFFFFFFFu, before);
+        total = __reduce_add_sync(0xFFFFFFFFu, total);
         if (lane == 0) { s_red[0][warp] = before; s_red[1][warp] = total; }
         if (lane < mb) {
             d_tok = h.l_tgt >= 0 && h.l_tgt < a.v_p;
             const char *row_k = (const char *)a.logits +
                                 ((size_t)b * a.seq_stride + (size_t)lane * a.row_stride) * (DTYPE == OD_BF16 ? 2 : 4);
             if (d_tok) d_xt = od_load_logit<DTYPE>(row_k, h.l_tgt);
-            d_u = od_uniform(a.seed[b], a.step, (uint32_t)lane, 0u);
         }
+        const uint64_t seed = a.seed[b];
+        d_u = od_uniform(seed, a.step, (uint32_t)lane, 0u);
+        h.u_draw = od_uniform(seed, a.step, (uint32_t)lane, 1u);
         __syncthreads();
-        before = 0; total = 0;
-        for (int w = 0; w < CWARPS; ++w) { before += s_red[0][w]; total += s_red[1][w]; }
+        before = __reduce_add_sync(0xFFFFFFFFu, lane < CWARPS ? s_red[0][lane] : 0);
+        total = __reduce_add_sync(0xFFFFFFFFu, lane < CWARPS ? s_red[1][lane] : 0);
+        segments = row_partial_segments(a.plan, b, warp, before, total);   // (of the row this warp merges first)
     }
 
     Part<SOURCE> mine;
@@ -148,11 +148,11 @@ od_sample_kernel(const SampleArgs a)
     if (FUSED) {
         // ---- step 2's decisions (what od_verify_decide_kernel does, same arithmetic, same order)
         const bool bad_T = !(h.T > 0.f);
-        const float dscale = bad_T ? 0.f : 1.4426950408889634f / h.T;
+        const float dscale = bad_T ? 0.f : h.scale;
         for (int r = warp; r <= mb; r += CWARPS) {
             const int row_slot = b * (K + 1) + r;
             float c, sum, mx;
-            merge_row_partials(a.plan, row_slot, row_partial_segments(a.plan, b, r, before, total), lane, c, sum, mx);
+            merge_row_partials(a.plan, row_slot, r == warp ? segments : row_partial_segments(a.plan, b, r, before, total), lane, c, sum, mx);
             if (lane == 0) {
                 const float S = row_sum_of(c, sum, mx, dscale);
                 s_M[r] = mx; s_S[r] = S;
@@ -175,7 +175,7 @@ od_sample_kernel(const SampleArgs a)
     // FROM_ROW: the map is still the one this launch was laid out for
     const bool planned = map_serial == a.map_serial;
     od_cluster_arrive_relaxed();                   // this block runs: the others may store to it (waited for below)
-    draw<DTYPE, SOURCE, false>(a, h, mine, b, part, nparts, warp, lane, j, rm, rs, planned, s_q, s_val);
+    draw<DTYPE, SOURCE, false, FUSED>(a, h, mine, b, part, nparts, warp, lane, j, rm, rs, planned, s_q, s_val);
 }
 
 // ---- vocabulary shards: MODE 1, a shard's mass shares; MODE 2, a shard's pick ---------------
@@ -247,8 +247,8 @@ od_sample_shard_kernel(const SampleArgs a)
     if (MODE != 2) {
         // ---- pass 1: the value of every tile ----
         const int hi_w = planned || !a.same_ids ? p_hi_w : p_lo;
-        if (a.same_ids) warp_run<DTYPE, FROM_ROW>(q, a, p_lo, p_hi, hi_w, lane, out, ni);
-        else warp_run<DTYPE, FROM_MAP>(q, a, p_lo, p_hi, hi_w, lane, out, ni);
+        if (a.same_ids) warp_run<DTYPE, FROM_ROW, false>(q, a, p_lo, p_hi, hi_w, lane, out, ni);
+        else warp_run<DTYPE, FROM_MAP, false>(q, a, p_lo, p_hi, hi_w, lane, out, ni);
         // The tile values are read by another block: the barrier orders this block's stores
         // before thread 0's fence, the fence before its ticket (release); the block that
         // draws the last ticket fences again before anyone in it reads (acquire).

@@ -52,7 +52,9 @@ __device__ __forceinline__ void cluster_store4(float4 *p, uint32_t rank, float4 
 // A block's slice [u0, u1) of a row, in units
 struct Slice {
     int u0, u1, full;                   // full: units of a row that are whole
+    uint32_t inv;                       // ceil(2^32 / units): f / units for f < 2^32 / units, without a division behind the walk
     __device__ __forceinline__ int units() const { return u1 - u0; }
+    __device__ __forceinline__ int rows_before(int f) const { return units() > 1 ? (int)__umulhi((uint32_t)f, inv) : f; }
 };
 template <int DTYPE>
 __device__ __forceinline__ Slice slice_of(const StepArgs &a, int part)
@@ -61,6 +63,7 @@ __device__ __forceinline__ Slice slice_of(const StepArgs &a, int part)
     s.u0 = min(part * a.part_units, a.W);
     s.u1 = min(s.u0 + a.part_units, a.W);
     s.full = full_units_of<DTYPE>(a.v_p);
+    s.inv = s.u1 > s.u0 ? 0xFFFFFFFFu / (uint32_t)(s.u1 - s.u0) + 1u : 0u;
     return s;
 }
 template <int DTYPE>
@@ -120,7 +123,7 @@ __device__ __forceinline__ void rows_from_one(const StepArgs &a, const Slice &s,
     int f = warp * per;
     const int f_hi = min(f + per, total);
     if (f >= f_hi) return;
-    int r = 1 + f / n, v = f - (r - 1) * n;
+    int r = 1 + s.rows_before(f), v = f - (r - 1) * n;  // (f < OD_MAX_K * n, and a block has at most 320 KB of rows)
     while (f < f_hi) {
         const int cnt = min(n - v, f_hi - f), v0 = s.u0 + v, v1 = v0 + cnt;
         const char *row = row_of<DTYPE>(a, b, r);
@@ -165,13 +168,10 @@ __device__ __forceinline__ void exchange_rows(const Slice &s, int mb, unsigned p
     __syncthreads();
     od_cluster_wait();                                      // every block runs
     for (int r = warp; r <= mb; r += CWARPS) {
-        int first = 0, end = 0;                             // the warps that had units of the row
-        if (n > 0) {
-            first = r == 0 ? 0 : (r - 1) * n / per;
-            end = r == 0 ? (n - 1) / per0 + 1 : (r * n - 1) / per + 1;
-        }
+        // the warps that had units of the row: from unit lane * per on, per of them
+        const bool held = r == 0 ? lane * per0 < n : lane * per < r * n && (lane + 1) * per > (r - 1) * n;
         float c = -FLT_MAX, sum = 0.f, mx = -INFINITY;
-        if (lane >= first && lane < end) {
+        if (held) {
             const float4 v = s_rec[r * CWARPS + lane];
             c = v.x; sum = v.y; mx = v.z;
         }
@@ -250,12 +250,14 @@ od_step_kernel(const __grid_constant__ StepArgs a)
     if (a.inputs_early && !all_early) { wait_for_earlier(); release_next(); }
     Kb = Kb < 0 ? 0 : (Kb > K ? K : Kb);
     const float u = od_uniform(seed, a.step, (uint32_t)lane, 0u);
+    h.u_draw = od_uniform(seed, a.step, (uint32_t)lane, 1u);
     // ---- the piece that begins at offset `warp`: the longest cached run, else the direct map
     if (warp < Kb) {
         const int4 piece = look_up_piece(id, qs, warp, Kb, a.v_q, a.vocab_map, a.keys, a.vals, a.cap, lane);
         if (lane == 0) s_piece[warp] = piece;
     }
-    const float scale = h.T > 0.f ? 1.4426950408889634f / h.T : 0.f;
+    h.scale = 1.4426950408889634f / h.T;
+    const float scale = h.T > 0.f ? h.scale : 0.f;
     zero.finish(a, slice, b, warp, lane, scale, s_rec);
     __syncthreads();
 
@@ -292,7 +294,7 @@ od_step_kernel(const __grid_constant__ StepArgs a)
         if (part == 0 && threadIdx.x == 0) { a.out_token[b] = -1; a.resid_mass[b] = 0.f; a.flags[b] = OD_SF_BAD_TEMPERATURE; }
         return;
     }
-    draw<DTYPE, SOURCE, true>(a, h, mine, b, part, nparts, warp, lane, j, rm, rs, map_serial == a.map_serial, s_q, s_val);
+    draw<DTYPE, SOURCE, true, true>(a, h, mine, b, part, nparts, warp, lane, j, rm, rs, map_serial == a.map_serial, s_q, s_val);
 }
 
 // Step 2 alone, with the same slices and the same order of reduction. SHARD: the rows are the columns [col0,
@@ -313,7 +315,8 @@ od_verify_rows_kernel(const __grid_constant__ StepArgs a)
     if (!a.inputs_early) { wait_for_earlier(); release_next(); }
     Ahead h = {};
     h.T = a.temperature[b];
-    const float scale = h.T > 0.f ? 1.4426950408889634f / h.T : 0.f;
+    h.scale = 1.4426950408889634f / h.T;
+    const float scale = h.T > 0.f ? h.scale : 0.f;
     const Slice slice = slice_of<DTYPE>(a, (int)part);
     RowZero<DTYPE> zero;
     zero.begin(a, slice, b, warp, lane);
