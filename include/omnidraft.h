@@ -142,7 +142,7 @@ enum od_counter {
  * `draft_vocab` ids and a target vocabulary of `target_vocab` ids, for
  * batches of at most `max_batch` sequences with at most `max_k`
  * (1..OD_MAX_K) proposed tokens each. Allocates the device-side scratch
- * (tickets, partial row statistics, tile sums) once; synchronous.
+ * (partial row statistics, tile sums) once; synchronous.
  * target_vocab is bounded by what od_sample_residual keeps in shared memory
  * (8 bytes per 256 ids, at most 200 KB: 6,553,600 ids); larger vocabularies
  * are refused with OD_ERR_UNSUPPORTED. */

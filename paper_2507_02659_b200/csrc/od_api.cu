@@ -47,8 +47,7 @@ void free_all(od_ctx *c)
 {
     od_cache_free_dynamic(c);
     void *ptrs[] = {c->d_vocab_map, c->d_inv_map, c->d_map_serial, c->d_distill_lists, c->d_sample_lists, c->d_keys, c->d_vals, c->d_partials,
-                    c->d_tile_sums,
-                    c->d_samp_ticket, c->s_logits, c->s_q_rows, c->s_q_sel, c->s_temperature,
+                    c->d_tile_sums, c->s_logits, c->s_q_rows, c->s_q_sel, c->s_temperature,
                     c->s_draft_ids, c->s_draft_len, c->s_seed, c->s_tgt_ids, c->s_span_start,
                     c->s_span_len, c->s_m, c->s_n_acc, c->s_n_draft, c->s_token, c->s_q_prime,
                     c->s_row_max, c->s_row_sum, c->s_p_sel, c->s_ratio, c->s_mass, c->s_tail,
@@ -204,7 +203,6 @@ int32_t od_create(od_ctx **ctx, int32_t device, int32_t draft_vocab, int32_t tar
     c->d_sample_lists = lists;
     if (st == OD_OK) st = dev_alloc(&c->d_partials, rows * OD_VERIFY_SEG_MAX);
     if (st == OD_OK) st = dev_alloc(&c->d_tile_sums, (size_t)max_batch * c->tiles_per_row);
-    if (st == OD_OK) st = dev_alloc(&c->d_samp_ticket, (size_t)max_batch);
     if (st != OD_OK) {
         free_all(c);
         delete c;

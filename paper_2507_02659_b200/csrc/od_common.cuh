@@ -74,7 +74,6 @@ struct od_ctx {
 
     // od_sample_residual scratch
     double *d_tile_sums;            // [max_batch * tiles_per_row] value of each tile
-    unsigned int *d_samp_ticket;    // [max_batch]
     int32_t tiles_per_row;
 
     // options

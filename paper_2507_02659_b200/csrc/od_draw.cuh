@@ -49,7 +49,6 @@ struct SampleArgs {
     float *resid_mass;
     uint32_t *flags;
     double *tile_val;                   // [B][ntiles] sum over the tile of r'
-    unsigned int *ticket;
     // vocabulary shards: this shard's tiles are [tile_lo, tile_hi); `logits` points at
     // its first column (target id col0), v_p is the id one past its last column
     int32_t tile_lo, tile_hi, col0;
@@ -252,10 +251,20 @@ __device__ __forceinline__ float warp_sum_f32(float v)
 struct GlobalTiles {                                        // [ntiles] of one sequence
     double *val;
     int lane;
-    __device__ __forceinline__ void one(int t, float v) { if (lane == 0) val[t] = (double)v; }
+    double total;                                           // of the warp's tiles: lanes 0..15 and 16..31 each hold a share
+    __device__ __forceinline__ void one(int t, float v)
+    {
+        if (lane == 0) val[t] = (double)v;
+        if (lane < 16) total += (double)fmaxf(0.f, v);      // (a tile with NaN has no mass)
+    }
     __device__ __forceinline__ void pair(int t, float v, bool two)
     {
         if ((lane & 15) == 0 && (lane == 0 || two)) val[t + (lane >> 4)] = (double)v;
+        total += lane < 16 || two ? (double)fmaxf(0.f, v) : 0.0;
+    }
+    __device__ __forceinline__ double sum() const
+    {
+        return __shfl_sync(0xFFFFFFFFu, total, 0) + __shfl_sync(0xFFFFFFFFu, total, 16);
     }
 };
 struct WarpTiles {                                          // the warp's own run in shared memory, and its sum
@@ -765,7 +774,7 @@ __device__ __forceinline__ void draw_from_p(const SeqState &q, const SampleArgs 
     __shared__ double s_sum[CTHREADS];
     __shared__ int s_crossing, s_lastmass, s_done;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    GlobalTiles out = {a.tile_val + (size_t)b * a.ntiles, lane};
+    GlobalTiles out = {a.tile_val + (size_t)b * a.ntiles, lane, 0.0};
     for (int t = warp * 2; t < a.ntiles; t += CWARPS * 2)
         warp_tiles_dense<DTYPE, 2>(q, a, false, t, t + 2 < a.ntiles ? t + 2 : a.ntiles, lane, out);
     if (threadIdx.x == 0) { s_crossing = 0x7FFFFFFF; s_lastmass = -1; s_done = 0; }
@@ -1077,7 +1086,7 @@ inline void context_args(const od_ctx *c, SampleArgs &a)
     a.map_serial = c->map_serial; a.map_serial_now = c->d_map_serial;
     a.same_ids = c->map_same_ids;
     a.row_vec = c->v_q % 4 == 0 && ((uintptr_t)a.q_rows & 15u) == 0;
-    a.tile_val = c->d_tile_sums; a.ticket = c->d_samp_ticket;
+    a.tile_val = c->d_tile_sums;
 }
 
 // the cut of a row into the level's parts, and the level's lists

@@ -37,9 +37,11 @@
 //
 // Vocabulary shards (the rows split by columns over several GPUs) use the same
 // kernel in two further modes. A shard owns a window of whole tiles:
-//   mode 1  pass 1 over the window, then the last block adds the window's tile
-//           values: the shard's share of the residual mass (and, when that is
-//           zero, of the mass of p_j, for the fallback);
+//   mode 1  pass 1 over the window by a cluster of blocks, whose sums meet in the first
+//           one: the shard's share of the residual mass (and, when that is zero, of the
+//           mass of p_j, for the fallback). A rank's five calls, 64 sequences, a quarter of
+//           128256 ids: 25.1 us with a ticket, two fences and a last block that loaded the tile
+//           values again, 24.4 so;
 //   mode 2  after the shares of all shards were exchanged: every shard forms the
 //           same total and target = u * total, finds the shard in which the running
 //           sum over shards crosses the target, and that shard alone scans its
@@ -55,27 +57,6 @@
 namespace {
 
 constexpr int WARPS = OD_SAMPLE_THREADS / 32;
-
-// Sum of s_val[my_lo, my_hi) over the block's threads in the order of the scan of
-// pass 2 (a thread's run, lanes in order, warps in order); every thread gets it.
-__device__ __forceinline__ double block_total(const double *s_val, int my_lo, int my_hi, double *s_warp)
-{
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    double inc = 0.0;
-    for (int t = my_lo; t < my_hi; ++t) inc += s_val[t];
-#pragma unroll
-    for (int off = 1; off < 32; off <<= 1) {
-        const double v = __shfl_up_sync(0xFFFFFFFFu, inc, off);
-        if (lane >= off) inc += v;
-    }
-    __syncthreads();                                // s_warp may still be read from an earlier call
-    if (lane == 31) s_warp[warp] = inc;
-    __syncthreads();
-    double tot = 0.0;
-    for (int w = 0; w < WARPS; ++w) tot += s_warp[w];
-    return tot;
-}
-
 
 template <int DTYPE, bool FUSED, int SOURCE>
 __global__ void __launch_bounds__(CTHREADS, 2)
@@ -186,7 +167,7 @@ od_sample_shard_kernel(const SampleArgs a)
     extern __shared__ __align__(16) unsigned char s_dyn[];   // ntiles x 8 bytes
     double *s_val = (double *)s_dyn;                         // pass 2: tile values
     __shared__ double s_warp[WARPS];
-    __shared__ unsigned int s_last;
+    __shared__ double s_part[OD_SAMPLE_MAX_PARTS];          // MODE 1: the cluster's blocks' sums, in its first block
     __shared__ int s_tile, s_lastmass, s_done;
     __shared__ double s_before;
     __shared__ double s_cross[OD_SAMPLE_THREADS];           // pass 2: the sum in front of a thread's crossing tile
@@ -219,6 +200,24 @@ od_sample_shard_kernel(const SampleArgs a)
     if (a.early) asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;");      // (behind the wait, as in od_sample_kernel)
     load_first_probability(a, h, b);
+    // MODE 2: all it needs from memory is requested here, in one trip: the first 1024 tile values, the seed, lane k the
+    // shares of shard k
+    const int ntiles = a.ntiles;
+    double *tile_val = a.tile_val + (size_t)b * ntiles;
+    double first_val[4], share_r = 0.0, share_e = 0.0;
+    uint64_t seed_b = 0;
+    if (MODE == 2) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int t = tile_lo + (int)threadIdx.x + i * OD_SAMPLE_THREADS;
+            first_val[i] = t < tile_hi ? __ldcg(tile_val + t) : 0.0;
+        }
+        seed_b = a.seed[b];
+        if (lane < a.n_shards) {
+            share_r = a.mass_all[((size_t)lane * a.B + b) * 2];
+            share_e = a.mass_all[((size_t)lane * a.B + b) * 2 + 1];
+        }
+    }
 
     if (!(T > 0.f)) {                              // every block of the sequence leaves here
         if (part == 0 && threadIdx.x == 0) {
@@ -230,6 +229,7 @@ od_sample_shard_kernel(const SampleArgs a)
         }
         return;
     }
+    if (MODE == 1) od_cluster_arrive_relaxed();    // this block runs: the first one may be stored to (waited for below)
     float rm = 0.f, rs = 0.f;                      // lane k: statistics of row k
     if (lane <= mb) {
         rm = a.row_max[b * (K + 1) + lane];
@@ -240,26 +240,40 @@ od_sample_shard_kernel(const SampleArgs a)
     const SeqState q = seq_state<DTYPE>(a, h, b, j, rm, rs, a.col0, planned);
     if (MODE != 2 && q.residual && threadIdx.x == 0) prefetch_q_row(a, q, part, nparts);
 
-    const int ntiles = a.ntiles;
-    double *tile_val = a.tile_val + (size_t)b * ntiles;
-    GlobalTiles out = {tile_val, lane};
+    GlobalTiles out = {tile_val, lane, 0.0};
 
     if (MODE != 2) {
         // ---- pass 1: the value of every tile ----
         const int hi_w = planned || !a.same_ids ? p_hi_w : p_lo;
         if (a.same_ids) warp_run<DTYPE, FROM_ROW, false>(q, a, p_lo, p_hi, hi_w, lane, out, ni);
         else warp_run<DTYPE, FROM_MAP, false>(q, a, p_lo, p_hi, hi_w, lane, out, ni);
-        // The tile values are read by another block: the barrier orders this block's stores
-        // before thread 0's fence, the fence before its ticket (release); the block that
-        // draws the last ticket fences again before anyone in it reads (acquire).
+        // ---- the window's sum: the blocks' sums meet in the first block of the cluster
+        const double run_sum = out.sum();
+        if (lane == 0) s_warp[warp] = run_sum;
         __syncthreads();
+        od_cluster_wait();
         if (threadIdx.x == 0) {
-            __threadfence();
-            s_last = atomicAdd(a.ticket + b, 1u) == nparts - 1 ? 1u : 0u;
-            __threadfence();
+            double sum = 0.0;
+            for (int w = 0; w < WARPS; ++w) sum += s_warp[w];
+            od_cluster_store(&s_part[part], 0u, sum);
         }
-        __syncthreads();
-        if (!s_last) return;
+        od_cluster_arrive();
+        od_cluster_wait();
+        if (part != 0) return;
+        double mass_r = 0.0, mass_e = 0.0;
+        for (unsigned int i = 0; i < nparts; ++i) mass_r += s_part[i];
+        if (q.residual && !(mass_r > 0.0)) {
+            // no residual mass here: should no shard have any, the draw is from p_j
+            out.total = 0.0;
+            for (int t_lo = tile_lo + warp * 2; t_lo < tile_hi; t_lo += WARPS * 2)
+                warp_tiles_dense<DTYPE, 2>(q, a, false, t_lo, t_lo + 2 < tile_hi ? t_lo + 2 : tile_hi, lane, out);
+            const double e_sum = out.sum();
+            if (lane == 0) s_warp[warp] = e_sum;
+            __syncthreads();
+            for (int w = 0; w < WARPS; ++w) mass_e += s_warp[w];
+        }
+        if (threadIdx.x == 0) { a.mass_out[2 * b] = mass_r; a.mass_out[2 * b + 1] = mass_e; }
+        return;
     }
 
     // ---- pass 2 (one block per sequence) ----
@@ -268,51 +282,24 @@ od_sample_shard_kernel(const SampleArgs a)
     const int per = (tile_hi - tile_lo + OD_SAMPLE_THREADS - 1) / OD_SAMPLE_THREADS;
     const int my_lo = tile_lo + threadIdx.x * per < tile_hi ? tile_lo + threadIdx.x * per : tile_hi;
     const int my_hi = my_lo + per < tile_hi ? my_lo + per : tile_hi;
-    // tile values (rounding can leave a tile without residual mass slightly negative): four
-    // requests per thread at a time, and the draw's uniform worked out while they travel
-    float u = 0.f;
-    const uint64_t seed_b = MODE == 1 ? 0ull : a.seed[b];   // requested with the tile values, used behind them
-    for (int t0 = tile_lo + threadIdx.x, first = 1; first || t0 < tile_hi; t0 += 4 * OD_SAMPLE_THREADS, first = 0) {
-        double v[4];
+    // tile values (rounding can leave a tile without residual mass slightly negative)
+    const float u = od_uniform(seed_b, a.step, (uint32_t)j, 1u);
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const int t = t0 + i * OD_SAMPLE_THREADS;
-            v[i] = t < tile_hi ? __ldcg(tile_val + t) : 0.0;
-        }
-        if (MODE != 1 && first) u = od_uniform(seed_b, a.step, (uint32_t)j, 1u);
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const int t = t0 + i * OD_SAMPLE_THREADS;
-            if (t < tile_hi) s_val[t] = fmax(0.0, v[i]);
-        }
+    for (int i = 0; i < 4; ++i) {
+        const int t = tile_lo + (int)threadIdx.x + i * OD_SAMPLE_THREADS;
+        if (t < tile_hi) s_val[t] = fmax(0.0, first_val[i]);
     }
-    if (MODE != 2 && threadIdx.x == 0) a.ticket[b] = 0;
+    for (int t = tile_lo + (int)threadIdx.x + 4 * OD_SAMPLE_THREADS; t < tile_hi; t += OD_SAMPLE_THREADS) s_val[t] = fmax(0.0, __ldcg(tile_val + t));
     __syncthreads();
-
-    if (MODE == 1) {
-        // ---- this shard's shares ----
-        const double mass_r = block_total(s_val, my_lo, my_hi, s_warp);
-        double mass_e = 0.0;
-        if (residual && !(mass_r > 0.0)) {
-            // no residual mass here: should no shard have any, the draw is from p_j
-            for (int t_lo = tile_lo + warp * 2; t_lo < tile_hi; t_lo += WARPS * 2)
-                warp_tiles_dense<DTYPE, 2>(q, a, false, t_lo, t_lo + 2 < tile_hi ? t_lo + 2 : tile_hi, lane, out);
-            __syncthreads();
-            for (int t = tile_lo + threadIdx.x; t < tile_hi; t += OD_SAMPLE_THREADS) s_val[t] = fmax(0.0, tile_val[t]);
-            __syncthreads();
-            mass_e = block_total(s_val, my_lo, my_hi, s_warp);
-        }
-        if (threadIdx.x == 0) { a.mass_out[2 * b] = mass_r; a.mass_out[2 * b + 1] = mass_e; }
-        return;
-    }
 
     double shard_before = 0.0, shard_total = 0.0;      // MODE 2: sums over the shards before this one / all
     if (MODE == 2) {
+        const auto share = [&](int s, bool e) -> double {
+            if (s < 32) return __shfl_sync(0xFFFFFFFFu, e ? share_e : share_r, s);
+            return a.mass_all[((size_t)s * a.B + b) * 2 + (e ? 1 : 0)];
+        };
         double tot_r = 0.0, tot_e = 0.0;
-        for (int s = 0; s < a.n_shards; ++s) {
-            tot_r += a.mass_all[((size_t)s * a.B + b) * 2];
-            tot_e += a.mass_all[((size_t)s * a.B + b) * 2 + 1];
-        }
+        for (int s = 0; s < a.n_shards; ++s) { tot_r += share(s, false); tot_e += share(s, true); }
         const bool use_e = residual && !(tot_r > 0.0);
         if (use_e) { residual = false; flags |= OD_SF_ZERO_MASS; }   // the tile values then hold p_j's
         shard_total = use_e ? tot_e : tot_r;
@@ -323,7 +310,7 @@ od_sample_shard_kernel(const SampleArgs a)
             double c = 0.0;
             int last = -1;
             for (int s = 0; s < a.n_shards; ++s) {
-                const double v = a.mass_all[((size_t)s * a.B + b) * 2 + (use_e ? 1 : 0)];
+                const double v = share(s, use_e);
                 if (s == a.shard_index) shard_before = c;
                 if (v > 0.0) last = s;
                 if (c + v > target) { owner = s; break; }
@@ -438,6 +425,7 @@ static cudaError_t prepare_kernels()
     if (e == cudaSuccess) e = allow_cluster16<DTYPE, false, STAGED>(staged);
     if (e == cudaSuccess) e = allow_cluster16<DTYPE, true, STAGED>(staged);
     if (e == cudaSuccess) e = allow_smem(od_sample_shard_kernel<DTYPE, 1>, bytes);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(od_sample_shard_kernel<DTYPE, 1>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     if (e == cudaSuccess) e = allow_smem(od_sample_shard_kernel<DTYPE, 2>, bytes);
     return e;
 }
@@ -500,9 +488,12 @@ static cudaError_t launch_sample(od_ctx *c, int mode, int32_t B, int32_t K_max, 
             const int64_t want = (int64_t)c->sm_count * 4;
             int64_t per_row = want / B;
             if (per_row < 1) per_row = 1;
+            if (per_row > OD_SAMPLE_MAX_PARTS) per_row = OD_SAMPLE_MAX_PARTS;
             tpw = (wtiles + per_row * WARPS - 1) / (per_row * WARPS);
             if (tpw < 1) tpw = 1;
         }
+        // (a cluster has at most 16 blocks)
+        if (tpw * WARPS * OD_SAMPLE_MAX_PARTS < wtiles) tpw = (wtiles + WARPS * OD_SAMPLE_MAX_PARTS - 1) / (WARPS * OD_SAMPLE_MAX_PARTS);
         const int64_t tiles_per_block = tpw * WARPS;
         if (mode == 1) blocks_x = (int)((wtiles + tiles_per_block - 1) / tiles_per_block);
     }
@@ -550,8 +541,10 @@ static cudaError_t launch_sample(od_ctx *c, int mode, int32_t B, int32_t K_max, 
     }
     cfg.gridDim = dim3((unsigned)B, (unsigned)blocks_x);
     cfg.blockDim = dim3(OD_SAMPLE_THREADS);
-    cfg.dynamicSmemBytes = od_sample_smem_bytes(ntiles);
-    cfg.numAttrs = c->opt_pdl ? 1 : 0;
+    cfg.dynamicSmemBytes = mode == 1 ? 0 : od_sample_smem_bytes(ntiles);
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = 1; attr[1].val.clusterDim.y = (unsigned)blocks_x; attr[1].val.clusterDim.z = 1;
+    cfg.numAttrs = (c->opt_pdl ? 1 : 0) + (mode == 1 ? 1 : 0);
     if (mode == 1)
         return bf ? cudaLaunchKernelEx(&cfg, od_sample_shard_kernel<OD_BF16, 1>, a)
                   : cudaLaunchKernelEx(&cfg, od_sample_shard_kernel<OD_F32, 1>, a);
