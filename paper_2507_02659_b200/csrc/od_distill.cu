@@ -88,17 +88,21 @@ __device__ __forceinline__ float kl_term(const KlRow &r, float qd, float x, floa
 }
 
 // What a block finds out about its position (b, j) first: the piece of the translated proposal
-// that covers it, if any (thread i looks at piece i, so the loads go out together).
+// that covers it, if any. Thread i looks at piece i, whether or not there is one (i < K_max keeps the address inside the
+// arrays): one round trip, not one for m and another for the pieces.
 __device__ __forceinline__ void find_piece(const DistillArgs &a, int b, int j, int *s_piece, int &piece, int &plen)
 {
-    int mb = a.m[b];
-    mb = mb < 0 ? 0 : (mb > a.K_max ? a.K_max : mb);
-    if (threadIdx.x == 0) { s_piece[0] = -1; s_piece[1] = 0; }
-    __syncthreads();
-    if ((int)threadIdx.x < mb) {
-        const size_t o = (size_t)b * a.K_max + threadIdx.x;
-        const int s0 = a.span_start[o], L = a.span_len[o];
-        if (j >= s0 && j < s0 + L) { s_piece[0] = (int)threadIdx.x; s_piece[1] = L; }
+    if (threadIdx.x < 32) {
+        const int i = (int)threadIdx.x;
+        int s0 = 0, L = 0;
+        if (i < a.K_max) {
+            const size_t o = (size_t)b * a.K_max + i;
+            s0 = a.span_start[o]; L = a.span_len[o];
+        }
+        const unsigned covers = __ballot_sync(0xFFFFFFFFu, i < a.m[b] && i < a.K_max && j >= s0 && j < s0 + L);
+        const int p = covers ? 31 - __clz(covers) : -1;
+        L = __shfl_sync(0xFFFFFFFFu, L, p & 31);
+        if (i == 0) { s_piece[0] = p; s_piece[1] = p < 0 ? 0 : L; }
     }
     __syncthreads();
     piece = s_piece[0]; plen = s_piece[1];
@@ -240,7 +244,7 @@ od_distill_kernel(const __grid_constant__ DistillArgs a)
     float *grad = a.grad ? a.grad + ((size_t)b * a.K_max + j) * a.v_q : nullptr;
     // The chunk's list: groups of 32 entries, one per lane (od_distill_lists). It belongs to the
     // context: the first entries are requested before the wait, the others a batch ahead.
-    constexpr int EB = 4;                                   // groups per warp and batch
+    constexpr int EB = DTYPE == OD_BF16 ? 5 : 4;            // groups per warp and batch (as many as 40 registers hold; fp32 1 to 2 % slower with 5)
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int2 groups = SAME ? make_int2(0, 0) : __ldg((const int2 *)a.list_ofs + rank);
     const int g_hi = groups.y;
