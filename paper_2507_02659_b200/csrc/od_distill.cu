@@ -42,6 +42,8 @@ namespace {
 
 constexpr int THREADS = 512;                     // three blocks to a multiprocessor at 40 registers
 constexpr int WARPS = THREADS / 32;
+constexpr int FEW_EB = 6, FEW_PQ = 4;             // two blocks to a multiprocessor, 64 registers: more in flight (see the launcher)
+constexpr int FEW_CHUNK = FEW_PQ * THREADS * 4;
 
 struct DistillArgs {
     int32_t B, K_max, v_q, v_p;
@@ -228,8 +230,8 @@ __device__ __noinline__ void looked_up_position(const DistillArgs &a, int b, int
 // rows are 16-byte aligned, so the coalesced accesses (q, gradient) move four ids per
 // instruction; chunks are multiples of 32 ids. SAME: target ids are draft ids, nothing is
 // gathered; the logits wait in shared memory for the gradient.
-template <int DTYPE, bool VEC4, bool SAME>
-__global__ void __launch_bounds__(THREADS, 3)
+template <int DTYPE, bool VEC4, bool SAME, int RESIDENT>
+__global__ void __launch_bounds__(THREADS, RESIDENT)
 od_distill_kernel(const __grid_constant__ DistillArgs a)
 {
     extern __shared__ __align__(16) unsigned char s_dyn[];   // [chunk] the logit of each mapped id, at its draft id
@@ -244,7 +246,8 @@ od_distill_kernel(const __grid_constant__ DistillArgs a)
     float *grad = a.grad ? a.grad + ((size_t)b * a.K_max + j) * a.v_q : nullptr;
     // The chunk's list: groups of 32 entries, one per lane (od_distill_lists). It belongs to the
     // context: the first entries are requested before the wait, the others a batch ahead.
-    constexpr int EB = DTYPE == OD_BF16 ? 5 : 4;            // groups per warp and batch (as many as 40 registers hold; fp32 1 to 2 % slower with 5)
+    // groups per warp and batch: as many as the registers hold (fp32 1 to 2 % slower with 5 in 40)
+    constexpr int EB = RESIDENT == 2 ? FEW_EB : DTYPE == OD_BF16 ? 5 : 4;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int2 groups = SAME ? make_int2(0, 0) : __ldg((const int2 *)a.list_ofs + rank);
     const int g_hi = groups.y;
@@ -300,11 +303,19 @@ od_distill_kernel(const __grid_constant__ DistillArgs a)
         loss_t += l; qg_t += g;
     };
     const raw_t *xrow = (const raw_t *)row;
+    constexpr bool KEEP = RESIDENT == 2;                     // the chunk's probabilities stay in registers
+    float4 kept[KEEP ? FEW_PQ : 1];
     if (!SAME) {
         // (the first probabilities travel meanwhile)
         constexpr int PQ = 2;                                // vectors of four probabilities in flight per thread
         float4 qv[PQ];
-        if (VEC4) {
+        if (KEEP) {
+#pragma unroll
+            for (int i = 0; i < FEW_PQ; ++i) {
+                const int d = lo + (int)threadIdx.x * 4 + i * THREADS * 4;
+                if (d < hi) kept[KEEP ? i : 0] = __ldg((const float4 *)(q + d));
+            }
+        } else if (VEC4) {
 #pragma unroll
             for (int i = 0; i < PQ; ++i) {
                 const int d = lo + (int)threadIdx.x * 4 + i * THREADS * 4;
@@ -330,7 +341,13 @@ od_distill_kernel(const __grid_constant__ DistillArgs a)
         kl.lg2_S = lg2_approx(S);
         __syncthreads();
         // ---- the loss and sum_e q(e) g(e)
-        if (VEC4) {
+        if (KEEP) {
+#pragma unroll
+            for (int i = 0; i < FEW_PQ; ++i) {
+                const int d = lo + (int)threadIdx.x * 4 + i * THREADS * 4;
+                if (d < hi) sum4(mapped4(d, kept[KEEP ? i : 0]), Logit<DTYPE>::load4(s_x + (d - lo)));
+            }
+        } else if (VEC4) {
             const int d0 = lo + (int)threadIdx.x * 4;
             for (int d1 = d0; d1 < hi; d1 += PQ * THREADS * 4) {
                 float4 nx[PQ];
@@ -409,7 +426,21 @@ od_distill_kernel(const __grid_constant__ DistillArgs a)
     if (!grad) return;
     // ---- the gradient: q(d) (g(d) - sum_e q(e) g(e))
     const float gbar = (float)qg;
-    if (VEC4) {
+    if (KEEP) {
+#pragma unroll
+        for (int i = 0; i < FEW_PQ; ++i) {
+            const int d = lo + (int)threadIdx.x * 4 + i * THREADS * 4;
+            if (d >= hi) continue;
+            const float4 v = kept[KEEP ? i : 0], u = mapped4(d, v);
+            const float4 x = Logit<DTYPE>::load4(s_x + (d - lo));
+            float4 o;
+            o.x = fmaf(-v.x, gbar, v.x * kl_term(kl, u.x, x.x, loss_t, qg_t));
+            o.y = fmaf(-v.y, gbar, v.y * kl_term(kl, u.y, x.y, loss_t, qg_t));
+            o.z = fmaf(-v.z, gbar, v.z * kl_term(kl, u.z, x.z, loss_t, qg_t));
+            o.w = fmaf(-v.w, gbar, v.w * kl_term(kl, u.w, x.w, loss_t, qg_t));
+            __stcs((float4 *)(grad + d), o);
+        }
+    } else if (VEC4) {
 #pragma unroll 4
         for (int d = lo + (int)threadIdx.x * 4; d < hi; d += THREADS * 4) {
             const float4 v = __ldg((const float4 *)(q + d)), u = mapped4(d, v);
@@ -547,7 +578,7 @@ od_distill_position_kernel(const DistillArgs a)
     }
 }
 
-template <int DTYPE, bool VEC4, bool SAME>
+template <int DTYPE, bool VEC4, bool SAME, int RESIDENT>
 cudaError_t launch_chunks(const DistillArgs &a, int C, bool pdl, cudaStream_t s)
 {
     cudaLaunchConfig_t cfg = {};
@@ -562,16 +593,19 @@ cudaError_t launch_chunks(const DistillArgs &a, int C, bool pdl, cudaStream_t s)
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = pdl ? 2 : 1;
-    return cudaLaunchKernelEx(&cfg, od_distill_kernel<DTYPE, VEC4, SAME>, a);
+    return cudaLaunchKernelEx(&cfg, od_distill_kernel<DTYPE, VEC4, SAME, RESIDENT>, a);
 }
 template <int DTYPE, bool VEC4>
-cudaError_t launch(const DistillArgs &a, int C, bool same, bool pdl, cudaStream_t s)
+cudaError_t launch(const DistillArgs &a, int C, bool same, bool few, bool pdl, cudaStream_t s)
 {
     if (C == 0) {
         od_distill_position_kernel<DTYPE, VEC4><<<dim3((unsigned)a.K_max, (unsigned)a.B), THREADS, 0, s>>>(a);
         return cudaGetLastError();
     }
-    return same ? launch_chunks<DTYPE, VEC4, true>(a, C, pdl, s) : launch_chunks<DTYPE, VEC4, false>(a, C, pdl, s);
+    if (same) return launch_chunks<DTYPE, VEC4, true, 3>(a, C, pdl, s);
+    if constexpr (VEC4)
+        if (few) return launch_chunks<DTYPE, true, false, 2>(a, C, pdl, s);
+    return launch_chunks<DTYPE, VEC4, false, 3>(a, C, pdl, s);
 }
 
 // draft ids per chunk for a vocabulary cut into C = 1 << level chunks: whole words of the mapped
@@ -609,6 +643,10 @@ cudaError_t od_launch_distill(od_ctx *c, int32_t B, int32_t K_max, const float *
     while (more(level) && !(same && !grad) && chunk_ids(c->v_q, level) * (bf ? 2 : 4) > (same ? 2 : 1) * CHUNK_BYTES) ++level;
     while (more(level) && positions * 2 << level <= wave) ++level;
     a.chunk = chunk_ids(c->v_q, level);
+    // Where two blocks to a multiprocessor hold them all, they have 64 registers instead of 40: six groups of the list in
+    // flight, and a thread's probabilities stay in registers from the sums to the gradient (128256 bf16 / 152064 fp32 ids, 1 x 4
+    // 6.55 -> 6.05 us / 6.6 -> 6.3, 5 x 5 8.3 -> 7.6 / 8.6 -> 8.1, 12 x 6 11.8 -> 10.3 / 12.2 -> 11.1; 8 or 10 groups spill).
+    const bool few = !same && vec4 && a.chunk <= FEW_CHUNK && positions << level <= (int64_t)c->sm_count * 2;
     // One block per position instead where the chunks would not fit, or where the target row is so
     // short that the gather in draft order finds its lines in L1 and there are positions enough
     // (128 x 10, v_q = 32000, 22400 ids mapped, v_p = 34330 / 45000 / 64000 / 128000: without a gradient
@@ -622,8 +660,8 @@ cudaError_t od_launch_distill(od_ctx *c, int32_t B, int32_t K_max, const float *
     const OdDistillLists l = od_distill_lists(c->d_distill_lists, c->v_q, c->v_p);
     a.list_word = l.word + (size_t)level * l.groups * 32; a.list_base = l.base + (size_t)level * l.groups;
     a.list_ofs = l.ofs + level * OD_DISTILL_MAX_CHUNKS * 2; a.mapped_bits = l.bits;
-    if (vec4) return bf ? launch<OD_BF16, true>(a, C, same, pdl, s) : launch<OD_F32, true>(a, C, same, pdl, s);
-    return bf ? launch<OD_BF16, false>(a, C, same, pdl, s) : launch<OD_F32, false>(a, C, same, pdl, s);
+    if (vec4) return bf ? launch<OD_BF16, true>(a, C, same, few, pdl, s) : launch<OD_F32, true>(a, C, same, few, pdl, s);
+    return bf ? launch<OD_BF16, false>(a, C, same, few, pdl, s) : launch<OD_F32, false>(a, C, same, few, pdl, s);
 }
 
 // The kernels' dynamic shared memory (a chunk of a draft vocabulary of v_q ids): opt in where it
@@ -632,14 +670,14 @@ cudaError_t od_distill_prepare_device(int32_t v_q)
 {
     const int n = OD_DISTILL_MAX_CHUNK_IDS * 4;
     if (chunk_ids(v_q, 0) * 4 <= 48 * 1024) return cudaSuccess;
-    cudaError_t e = cudaFuncSetAttribute(od_distill_kernel<OD_BF16, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, n);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(od_distill_kernel<OD_F32, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, n);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(od_distill_kernel<OD_BF16, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, n);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(od_distill_kernel<OD_F32, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, n);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(od_distill_kernel<OD_BF16, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, n);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(od_distill_kernel<OD_F32, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, n);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(od_distill_kernel<OD_BF16, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, n);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(od_distill_kernel<OD_F32, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, n);
+    cudaError_t e = cudaFuncSetAttribute(od_distill_kernel<OD_BF16, true, false, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize, n);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(od_distill_kernel<OD_F32, true, false, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize, n);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(od_distill_kernel<OD_BF16, false, false, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize, n);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(od_distill_kernel<OD_F32, false, false, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize, n);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(od_distill_kernel<OD_BF16, true, true, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize, n);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(od_distill_kernel<OD_F32, true, true, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize, n);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(od_distill_kernel<OD_BF16, false, true, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize, n);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(od_distill_kernel<OD_F32, false, true, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize, n);
     return e;
 }
 

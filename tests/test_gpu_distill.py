@@ -156,3 +156,14 @@ def test_shared_ids_and_short_target_rows(cuda_device, kind, v_q, v_p, B, k_max,
     # the same terms, in another order where the two take different kernels
     torch.testing.assert_close(lone, loss, rtol=2e-5, atol=2e-6)
     ctx.close()
+
+
+# few positions of whole vectors: two blocks to a multiprocessor, a thread's probabilities kept; chunks of 8192 ids and
+# just beyond, most positions for each number of chunks and one more, ragged ends of chunks
+@pytest.mark.parametrize("v_q, v_p, B, k_max", [(65532, 66001, 2, 3), (65540, 66001, 2, 3), (16388, 20011, 9, 4), (16388, 20011, 19, 2),
+                                                (32764, 40003, 37, 2), (32764, 40003, 25, 3), (4, 40, 1, 1)])
+def test_few_positions(cuda_device, v_q, v_p, B, k_max):
+    """Tolerances as above."""
+    for dtype in ("bf16", "f32"):
+        w = _small(B=B, k_max=k_max, v_q=v_q, v_p=v_p, cache_entries=0, logit_dtype=dtype, gen_seed=0xBEEFFA)
+        _check(w, cuda_device, [0], 0.2, ds.LAMBDA_CONSTANT, positions=sorted({0, B // 2, B - 1}))
