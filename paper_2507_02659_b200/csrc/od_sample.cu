@@ -155,7 +155,7 @@ od_sample_kernel(const SampleArgs a)
     }
     // FROM_ROW: the map is still the one this launch was laid out for
     const bool planned = map_serial == a.map_serial;
-    od_cluster_arrive_relaxed();                   // this block runs: the others may store to it (waited for below)
+    if (SOURCE != FROM_ROW || nparts > 1) od_cluster_arrive_relaxed();   // this block runs: the others may store to it (waited for below)
     draw<DTYPE, SOURCE, false, FUSED>(a, h, mine, b, part, nparts, warp, lane, j, rm, rs, planned, s_q, s_val);
 }
 
