@@ -246,7 +246,7 @@ __device__ __forceinline__ unsigned int block_offsets(unsigned int n, unsigned i
 // group it is in. Bound by the chain of round trips and by L2 (262144 entries: 13 MB read, 12 MB written). Before,
 // one pass packed all live entries into a list, the select walked through it, and a rebuild put every survivor into the slot that
 // its group's counter gave. Device time of an insertion, a trim and a translation, before -> now: 262144 entries and 16384 new
-// ones 53.7 -> 37.5 us, by frequency 70.1 -> 64.8; 4096 and 512 24.4 -> 23.1; 32768 and 4096 by frequency 35.3 -> 34.7. (The
+// ones 53.7 -> 36.5 us, by frequency 70.1 -> 64.6; 4096 and 512 24.4 -> 22.7; 32768 and 4096 by frequency 35.2 -> 34.2. (The
 // whole trim in one cluster of 1 to 16 blocks, for tables of up to 131072 slots: 26.5 and 37.7 us on the last two; a step
 // of it is a chain of trips as long as a launch's.)
 constexpr int TRIM_THREADS = 256, TRIM_HALVES = TRIM_THREADS / 16, QUAD = 4;   // groups of a half-warp at a time
@@ -373,6 +373,15 @@ trim_split_kernel(int policy, unsigned int clock, unsigned int max_entries, cons
         }
     };
     load(at);
+    // An entry is in another group than its run hashes to only if all groups from there on were full: where none of the
+    // four groups in front of the half-warp's is, nobody asks (the hash is a third of the pass's instructions).
+    const auto behind_a_full_group = [&]() {
+        if (quad >= quads) return false;
+        const uint4 f = __ldcg((const uint4 *)from.fill + quad);
+        const unsigned int before = __ldcg(from.fill + ((quad * QUAD - 1) & (groups - 1)));
+        return max(max(before, f.x), max(f.y, f.z)) >= (unsigned int)OD_GROUP;
+    };
+    bool ask = behind_a_full_group();
     if (threadIdx.x == 0) { s_and = ~0ull; s_or = 0ull; s_bin = 256u; s_rem = 0u; s_in = 0u; }
     asm volatile("griddepcontrol.wait;" ::: "memory");
 
@@ -393,7 +402,7 @@ trim_split_kernel(int policy, unsigned int clock, unsigned int max_entries, cons
     }
 
     for (;;) {
-        const bool in = quad < quads;
+        const bool in = quad < quads, ask_here = __any_sync(0xFFFFFFFFu, ask);
         unsigned int had[QUAD];
 #pragma unroll
         for (int e = 0; e < QUAD; ++e) run[e] = 0u;
@@ -412,7 +421,9 @@ trim_split_kernel(int policy, unsigned int clock, unsigned int max_entries, cons
                 const bool is_new = en[e].born == clock;
                 const unsigned int score = policy == 0 ? en[e].stamp : en[e].freq;
                 const unsigned int bin = en[e].v >= 0 ? score_bin(policy, clock, score, is_new) : 0u;
-                const bool live = en[e].v >= 0, home = live && (int64_t)(od_hash64(en[e].key) & (uint64_t)(groups - 1)) == g;
+                const bool live = en[e].v >= 0;
+                bool home = true;
+                if (ask_here) home = (int64_t)(od_hash64(en[e].key) & (uint64_t)(groups - 1)) == g;
                 const bool keep = live && bin >= first_kept && bin != mixed;
                 if (live && bin == mixed) {
                     listed |= 1u << e;
@@ -469,6 +480,7 @@ trim_split_kernel(int policy, unsigned int clock, unsigned int max_entries, cons
         if (q0 >= quads) break;
         quad = q0 + (threadIdx.x >> 4);
         load(at);
+        ask = behind_a_full_group();
     }
     if (!exact && threadIdx.x == 0 && (s_and != ~0ull || s_or != 0ull)) { atomicAnd(&st->hi_and, s_and); atomicOr(&st->hi_or, s_or); }
 }
