@@ -246,7 +246,7 @@ __device__ __forceinline__ unsigned int block_offsets(unsigned int n, unsigned i
 // group it is in. Bound by the chain of round trips and by L2 (262144 entries: 13 MB read, 12 MB written). Before,
 // one pass packed all live entries into a list, the select walked through it, and a rebuild put every survivor into the slot that
 // its group's counter gave. Device time of an insertion, a trim and a translation, before -> now: 262144 entries and 16384 new
-// ones 53.7 -> 36.5 us, by frequency 70.1 -> 64.6; 4096 and 512 24.4 -> 22.7; 32768 and 4096 by frequency 35.2 -> 34.2. (The
+// ones 53.7 -> 36.1 us, by frequency 70.1 -> 64.0; 4096 and 512 24.4 -> 22.9; 32768 and 4096 by frequency 35.2 -> 34.3. (The
 // whole trim in one cluster of 1 to 16 blocks, for tables of up to 131072 slots: 26.5 and 37.7 us on the last two; a step
 // of it is a chain of trips as long as a launch's.)
 constexpr int TRIM_THREADS = 256, TRIM_HALVES = TRIM_THREADS / 16, QUAD = 4;   // groups of a half-warp at a time
@@ -364,15 +364,15 @@ trim_split_kernel(int policy, unsigned int clock, unsigned int max_entries, cons
     unsigned int run[QUAD];
     Entry en[QUAD];
     int64_t q0 = (int64_t)blockIdx.x * TRIM_HALVES, quad = q0 + (threadIdx.x >> 4);
-    const auto load = [&](int s) {
+    const auto load = [&](int s, unsigned int which) {
 #pragma unroll
         for (int e = 0; e < QUAD; ++e) {
             const int64_t slot = (quad * QUAD + e) * OD_GROUP + s;
             en[e].v = -1;
-            if (slot < cap) en[e] = from.load(slot);
+            if (slot < cap && (which >> e & 1u)) en[e] = from.load(slot);
         }
     };
-    load(at);
+    load(at, 0xFu);
     // An entry is in another group than its run hashes to only if all groups from there on were full: where none of the
     // four groups in front of the half-warp's is, nobody asks (the hash is a third of the pass's instructions).
     const auto behind_a_full_group = [&]() {
@@ -406,36 +406,42 @@ trim_split_kernel(int policy, unsigned int clock, unsigned int max_entries, cons
         unsigned int had[QUAD];
 #pragma unroll
         for (int e = 0; e < QUAD; ++e) run[e] = 0u;
-        // (where a group's sixteenth slot is taken: the others too)
-        const int rounds = __syncthreads_or(at == 15 && max(max(en[0].v, en[1].v), max(en[2].v, en[3].v)) >= 0) ? 2 : 1;
+        // the groups whose sixteenth slot is taken: their other slots too
+        unsigned int more = 0u;
+        if (at == 15) {
+#pragma unroll
+            for (int e = 0; e < QUAD; ++e) more |= en[e].v >= 0 ? 1u << e : 0u;
+        }
+        const int rounds = __syncthreads_or((int)more) ? 2 : 1;
         for (int round = 0; round < rounds; ++round) {
             const int s = at + 16 * round;
-            if (round) load(s);
+            if (round) { more = __shfl_sync(0xFFFFFFFFu, more, 16 * half + 15); load(s, more); }
             const uint4 taken = round + 1 == rounds && in ? __ldcg((const uint4 *)to.fill + quad) : make_uint4(0u, 0u, 0u, 0u);
             had[0] = taken.x; had[1] = taken.y; had[2] = taken.z; had[3] = taken.w;
             unsigned int listed = 0u, late = 0u;            // of this thread's four: bit e
             unsigned long long t_and = ~0ull, t_or = 0ull;
+            if (round == 0 || __any_sync(0xFFFFFFFFu, more != 0u))
 #pragma unroll
-            for (int e = 0; e < QUAD; ++e) {
-                const int64_t g = quad * QUAD + e;
-                const bool is_new = en[e].born == clock;
-                const unsigned int score = policy == 0 ? en[e].stamp : en[e].freq;
-                const unsigned int bin = en[e].v >= 0 ? score_bin(policy, clock, score, is_new) : 0u;
-                const bool live = en[e].v >= 0;
-                bool home = true;
-                if (ask_here) home = (int64_t)(od_hash64(en[e].key) & (uint64_t)(groups - 1)) == g;
-                const bool keep = live && bin >= first_kept && bin != mixed;
-                if (live && bin == mixed) {
-                    listed |= 1u << e;
-                    unsigned long long hi, lo;
-                    order_key(policy, clock, en[e].key, en[e].stamp, en[e].freq, en[e].born, hi, lo);
-                    t_and &= hi; t_or |= hi;
+                for (int e = 0; e < QUAD; ++e) {
+                    const int64_t g = quad * QUAD + e;
+                    const bool is_new = en[e].born == clock;
+                    const unsigned int score = policy == 0 ? en[e].stamp : en[e].freq;
+                    const unsigned int bin = en[e].v >= 0 ? score_bin(policy, clock, score, is_new) : 0u;
+                    const bool live = en[e].v >= 0;
+                    bool home = true;
+                    if (ask_here) home = (int64_t)(od_hash64(en[e].key) & (uint64_t)(groups - 1)) == g;
+                    const bool keep = live && bin >= first_kept && bin != mixed;
+                    if (live && bin == mixed) {
+                        listed |= 1u << e;
+                        unsigned long long hi, lo;
+                        order_key(policy, clock, en[e].key, en[e].stamp, en[e].freq, en[e].born, hi, lo);
+                        t_and &= hi; t_or |= hi;
+                    }
+                    if (keep && !home) late |= 1u << e;
+                    const unsigned int stays = __ballot_sync(0xFFFFFFFFu, keep && home) >> (16 * half) & 0xFFFFu;
+                    if (keep && home) to.store(g * OD_GROUP + run[e] + __popc(stays & ((1u << at) - 1u)), en[e]);
+                    run[e] += __popc(stays);
                 }
-                if (keep && !home) late |= 1u << e;
-                const unsigned int stays = __ballot_sync(0xFFFFFFFFu, keep && home) >> (16 * half) & 0xFFFFu;
-                if (keep && home) to.store(g * OD_GROUP + run[e] + __popc(stays & ((1u << at) - 1u)), en[e]);
-                run[e] += __popc(stays);
-            }
             // ---- the lists: one append per block
             unsigned int sum;
             unsigned int ofs = block_offsets(__popc(listed) | __popc(late) << 16, s_warp, sum);
@@ -479,7 +485,7 @@ trim_split_kernel(int policy, unsigned int clock, unsigned int max_entries, cons
         q0 += (int64_t)gridDim.x * TRIM_HALVES;
         if (q0 >= quads) break;
         quad = q0 + (threadIdx.x >> 4);
-        load(at);
+        load(at, 0xFu);
         ask = behind_a_full_group();
     }
     if (!exact && threadIdx.x == 0 && (s_and != ~0ull || s_or != 0ull)) { atomicAnd(&st->hi_and, s_and); atomicOr(&st->hi_or, s_or); }
