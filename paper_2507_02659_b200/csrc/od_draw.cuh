@@ -283,14 +283,19 @@ struct WarpTiles {                                          // the warp's own ru
         if ((lane & 15) == 0 && (lane == 0 || two)) val[t - t_lo + (lane >> 4)] = v;
         total += (double)v;
     }
-    // tile t's value is another
+    // tile t's value is another; then, with all tiles as they stay, the sum of the run's first n anew, in the order of the
+    // pass: correcting it by the difference would lose what is small beside the old value (and give NaN where that is infinite)
     __device__ __forceinline__ void replace(int t, float v)
     {
-        v = fmaxf(0.f, v);
         __syncwarp();
-        if (lane < 16) total += (double)v - (double)val[t - t_lo];
+        if (lane == 0) val[t - t_lo] = fmaxf(0.f, v);
+    }
+    __device__ __forceinline__ void sum_anew(int n)
+    {
         __syncwarp();
-        if (lane == 0) val[t - t_lo] = v;
+        total = 0.0;
+#pragma unroll 1                                            // (unrolled by eight: 0.8 % of the step of 296, in the pass's registers)
+        for (int i = lane >> 4; i < n; i += 2) total += (double)val[i];
     }
     __device__ __forceinline__ double sum() const
     {
@@ -934,6 +939,7 @@ __device__ __forceinline__ void draw(const SampleArgs &a, const Ahead &h, Part<S
         __syncthreads();
         warp_tiles_ahead<DTYPE, STAGED, STARTED>(q, a, sr, p_lo, hi_w, lane, out, cur);
         // Eq. (2)'s two ids, which the pass above does not look for: their tiles once more
+        bool other = false;
 #pragma unroll 1
         for (int i = 0; i < 2; ++i) {
             const int id = i == 0 ? q.prefix_token : q.ngram_token, t = id / OD_SAMPLE_TILE;
@@ -941,7 +947,9 @@ __device__ __forceinline__ void draw(const SampleArgs &a, const Ahead &h, Part<S
             float r[EPT];
             tile_values<DTYPE>(q, a, true, t, lane, r, &sr);
             out.replace(t, warp_sum_f32(sum_of_eight(r)));
+            other = true;
         }
+        if (other) out.sum_anew(hi_w - p_lo);
         if (hi_w < p_hi) warp_tiles_dense<DTYPE, 1>(q, a, true, max(hi_w, p_lo), p_hi, lane, out);
     } else {
         warp_run<DTYPE, SOURCE, STARTED>(q, a, p_lo, p_hi, hi_w, lane, out, my.ni);

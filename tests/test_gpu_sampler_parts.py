@@ -140,3 +140,39 @@ def test_staged_ids_beyond_one_page_of_draft_ids(cuda_device, dtype):
     w = _workload(B=5, k_max=3, v_q=70001, v_p=90001, mapped_frac=0.6, cache_entries=0, logit_dtype=dtype)
     st = synth.make_static(w)
     assert {2, 16} <= {b for tiles in (0, 3, 1000) for b in _check(w, st, cuda_device, tiles, 2)}
+
+
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+@pytest.mark.parametrize("v_p", [4096, 70001])
+def test_residual_that_is_small_beside_the_n_gram_token(cuda_device, dtype, v_p):
+    """Eq. (2) takes the n-gram's token, which has all but 1e-17 of the target's mass, off the residual: what is left
+    is e^-50 for every other id, and it is drawn as any other mass, the ids around that token too. Bounds: an exponent
+    of 72 is off by half an ulp (4e-6), a term by ln 2 of that, the fp32 sums by less; 1e-5 of up to 70000 ids moves a
+    draw by less than one id, so a draw near an id's end may be its neighbour."""
+    v_q, B, gram = 64, 256, 300
+    ctx = od.Context(cuda_device, v_q, v_p, B, 2)
+    vmap = np.full(v_q, -1, np.int32)
+    vmap[3:40] = 1000 + 7 * np.arange(37)
+    ctx.set_vocab_map(vmap)
+    ctx.cache_build(np.array([[1, 2, -1, -1]], np.int32), np.array([2], np.int32), np.array([gram], np.int32))
+    ids = torch.tensor([[1, 2]], dtype=torch.int32, device=cuda_device).repeat(B, 1)
+    q_sel, q_rows = torch.ones(B, 2, device=cuda_device), torch.zeros(B, 2, v_q, device=cuda_device)
+    q_rows[:, 0, 1] = q_rows[:, 1, 2] = 1.0
+    logits = parity.pad_rows(torch.full((B, 3, v_p), -50.0, dtype=dtype, device=cuda_device))
+    logits[:, :, gram] = 0.0
+    T = torch.ones(B, device=cuda_device)
+    seed = torch.arange(B, device=cuda_device)
+    mp = od.od_map_proposals(ctx, ids, torch.full((B,), 2, dtype=torch.int32, device=cuda_device), q_sel)
+    vo = od.od_verify(ctx, logits, mp, T, seed, 0)
+    assert (mp.m == 1).all() and (mp.tgt_ids[:, 0] == gram).all()
+    vo.n_accepted.zero_()                                   # (p = q' = 1: a verification accepts it)
+    so = od.od_sample_residual(ctx, logits, vo, q_rows, ids, mp, T, seed, 0)
+    assert (so.flags & ~od.OD_SF_BOUNDARY == 0).all()
+    want = (v_p - 1) * np.exp(-50.0)
+    np.testing.assert_allclose(so.resid_mass.cpu().numpy(), want, rtol=1e-5)
+    at = np.array([oracle.uniform(b, 0, 0, 1) for b in range(B)]) * (v_p - 1)
+    token = so.out_token.cpu().numpy()
+    index = token - (token > gram)
+    assert (token != gram).all() and (np.abs(index - np.floor(at)) <= (np.abs(at - np.round(at)) < 1e-5 * at + 1e-3)).all()
+    assert (at < 4000).sum() > 4                            # ids around the n-gram's token are drawn
+    ctx.close()
