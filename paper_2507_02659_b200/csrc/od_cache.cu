@@ -24,8 +24,8 @@
 //           the decided prefix into the next list whenever that at least halves it, every
 //           block works out the digit the pass before it decided from that pass's 256-bin
 //           histogram, and a digit of (new?, score) that is the same in every listed entry
-//           costs no histogram. Then the rest of the survivors go from the list
-//           into the spare table (trim_place_kernel), which becomes the table. No kernel waits for another.
+//           costs no histogram. Then the rest of the survivors go from the list into the
+//           spare table (by that cluster, or trim_place_kernel), which becomes the table. No kernel waits for another.
 #include <algorithm>
 #include <stddef.h>
 #include <string.h>
@@ -500,39 +500,47 @@ trim_split_kernel(int policy, unsigned int clock, unsigned int max_entries, cons
 // then stay in shared memory for the run key, and the select ends as soon as
 // every candidate that is left is among the k (usually two passes in all, three by frequency: a pass costs 2.5 us or so,
 // of which the barrier and the sums are most). As a chain of 13 launches of the whole grid the passes took
-// 52 us for the 262144 entries of a table. The cluster then places the entries of its list that stay (without a launch of
-// its own for that, and with a list that a thread holds in registers: 40.8 -> 37.5 us).
+// 52 us for the 262144 entries of a table.
+// How long the list is, only the device knows: one batch where a clock is one batch's, but most of the table where it was
+// loaded at one clock, and by LFU as a rule. As many blocks take part as the list gives an entry a thread to; the others leave (4096
+// entries and 512 new ones: 23.9 us with 16 blocks, 22.8 with one). Such a list stays in registers, and the cluster places what
+// stays of it. A longer one is left to trim_place_kernel on the whole chip, which is launched where the table may have one
+// (`follow`). An insertion and a trim by LRU of 262144 entries that were loaded at one clock, 16384 new ones: 72.1 us placed by the
+// cluster, 54.9 so; 16000 and 256: 62.3 -> 31.6. (As many clusters as are resident, each with the whole select and a
+// share of the placing, in place of the second launch: 58.3 and 32.1, and 39.3 where the list is short: 37.0.)
 constexpr int SELECT_THREADS = 1024, SELECT_MAX_BLOCKS = 16;
 
 __global__ void __launch_bounds__(SELECT_THREADS, 1)
-trim_select_kernel(unsigned int room, const Table from, const Table to, int64_t cap, void *lists, TrimState *st, int place)
+trim_select_kernel(unsigned int room, const Table from, const Table to, int64_t cap, void *lists, TrimState *st, int follow)
 {
     extern __shared__ __align__(16) unsigned long long s_keys[];   // [room]
     __shared__ unsigned int s_hist[2][256], s_sum[256];
     __shared__ unsigned int s_n, s_digit, s_run, s_in;
-    const unsigned int P = gridDim.x, rank = blockIdx.x, lane = threadIdx.x & 31u;
+    const unsigned int rank = blockIdx.x, lane = threadIdx.x & 31u;
     chain_wait(true);                                       // (the next kernel reads the list in front of its own wait)
     const unsigned int n = (unsigned int)min((int64_t)__ldcg(&st->n_list), cap), k = __ldcg(&st->k_rem);
     const unsigned long long hi_and = __ldcg(&st->hi_and), hi_or = __ldcg(&st->hi_or);
     const TrimLists L = trim_lists(lists, cap);
     if (rank == 0 && threadIdx.x == 0) st->size = __ldcg(&st->size) - __ldcg(&st->k);
+    if (rank == 0 && threadIdx.x < 256) st->bins[threadIdx.x] = 0u;   // for the next trim
+    const bool one = n <= gridDim.x * SELECT_THREADS, place = one || !follow;
     if (place) {
-        if (rank == 0 && threadIdx.x < 256) st->bins[threadIdx.x] = 0u;   // for the next trim
         const unsigned int late = __ldcg(&st->n_late);
-        for (unsigned int i = rank * SELECT_THREADS + threadIdx.x; i < late; i += P * SELECT_THREADS)
+        for (unsigned int i = rank * SELECT_THREADS + threadIdx.x; i < late; i += gridDim.x * SELECT_THREADS)
             place_entry(to, cap, from.load(__ldcg(L.r_slot + (cap - 1 - (int64_t)i))));
     }
-    if (n == 0u) return;                                    // nothing to find out: every block leaves
+    // the blocks that take part: a cluster's barrier waits for the threads that have not left
+    const unsigned int P = min(gridDim.x, (n + SELECT_THREADS - 1) / SELECT_THREADS);
+    if (rank >= P) return;
     const unsigned int per = (n + P - 1) / P, lo = min(rank * per, n), hi_end = min(lo + per, n);
-    // An entry for a thread at most (the clock of one batch, as a rule): it stays in registers, and what goes into the
-    // new table is on its way while the digits are counted.
-    const bool one = per <= SELECT_THREADS, have = one && lo + threadIdx.x < hi_end;
+    // An entry for a thread at most: it stays in registers, and what goes into the new table is on its way while the
+    // digits are counted.
+    const bool have = one && lo + threadIdx.x < hi_end;
     unsigned long long my_hi = 0ull;
     Entry mine = {};
     if (have) {
         my_hi = __ldcg(L.r_hi + lo + threadIdx.x);
-        mine.key = __ldcg(L.r_key + lo + threadIdx.x);
-        if (place) mine = from.load(__ldcg(L.r_slot + lo + threadIdx.x));
+        mine = from.load(__ldcg(L.r_slot + lo + threadIdx.x));
     }
     for (int i = threadIdx.x; i < 512; i += SELECT_THREADS) s_hist[i >> 8][i & 255] = 0u;
     if (threadIdx.x == 0) s_n = 0u;
@@ -687,7 +695,7 @@ trim_select_kernel(unsigned int room, const Table from, const Table to, int64_t 
     }
     thr_lo |= ~decided;                                     // every candidate left is among the k
     od_cluster_arrive();                                    // (waited for below: nobody leaves while its histogram may still be read)
-    if (place && have && (my_hi > thr_hi || (my_hi == thr_hi && mine.key > thr_lo))) place_entry(to, cap, mine);
+    if (have && (my_hi > thr_hi || (my_hi == thr_hi && mine.key > thr_lo))) place_entry(to, cap, mine);
     if (place && !one)
         for (unsigned int i = lo + threadIdx.x; i < hi_end; i += SELECT_THREADS) {
             const unsigned long long hi = __ldcg(L.r_hi + i), key = __ldcg(L.r_key + i);
@@ -843,9 +851,11 @@ __global__ void trim_hist_kernel(int pass, int64_t cap, void *lists, TrimState *
 }
 
 // The listed entries that stay, and the survivors that were not in the group their run hashes to, go into the new table;
-// which slot of its group an entry gets depends on timing, the set of entries does not.
+// which slot of its group an entry gets depends on timing, the set of entries does not. `held`: behind trim_select_kernel,
+// which has placed lists of at most so many entries itself (then one block waits for it, so that what waits for this launch
+// waits for it too); 0: behind the chain of histograms.
 __global__ void __launch_bounds__(TRIM_THREADS)
-trim_place_kernel(const Table from, const Table to, int64_t cap, void *lists, TrimState *st, int selected)
+trim_place_kernel(const Table from, const Table to, int64_t cap, void *lists, TrimState *st, unsigned int held)
 {
     __shared__ unsigned int s_hist[256];
     __shared__ SelState s_sel;
@@ -856,14 +866,18 @@ trim_place_kernel(const Table from, const Table to, int64_t cap, void *lists, Tr
     unsigned long long hi = 0ull;
     Entry en = {};
     const auto load = [&](unsigned int i) { hi = __ldcg(L.r_hi + i); en = from.load(__ldcg(L.r_slot + i)); };
-    if (selected) {                                         // the list was complete when trim_select_kernel let this kernel start
+    if (held) {                                             // the list was complete when trim_select_kernel let this kernel start
         n = __ldcg(&st->n_list);
+        if (n <= held) {
+            if (blockIdx.x == 0) asm volatile("griddepcontrol.wait;" ::: "memory");
+            return;
+        }
         if (i0 < n) load(i0);
     }
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    if (blockIdx.x == 0) st->bins[threadIdx.x] = 0u;        // for the next trim
+    if (!held && blockIdx.x == 0) st->bins[threadIdx.x] = 0u;   // for the next trim
     unsigned long long thr_hi, thr_lo;
-    if (selected) {
+    if (held) {
         thr_hi = __ldcg(&st->thr_hi); thr_lo = __ldcg(&st->thr_lo);
     } else {
         n = __ldcg(&st->n_list);
@@ -928,11 +942,10 @@ void select_config(cudaLaunchConfig_t &cfg, cudaLaunchAttribute *attr, const od_
     cfg.attrs = attr; cfg.numAttrs = 1;
 }
 
-// Blocks of the one-launch select, 0 = the table is too large for it (393216 entries; 196608 where clusters of 16 are not
-// to be had): the list's keys have to fit in their shared memory. As few as give every thread an entry of the list, which
-// by LRU is one batch as a rule and by LFU most of the table (two a thread), and at most 16384 entries of the table to a
-// block in any case: a pass over a cluster of 1 to 4 blocks is shorter than one of 16 (4096 entries, 512 new ones: 23.9 us
-// with 16, 23.1 with 1; 32768 by LFU 35.6 with 8, 34.5 with 16).
+// Blocks of the one-launch select, 0 = the table is too large for it: the keys of a list of all its entries have to fit in
+// the blocks' shared memory (16 blocks: 393216 entries; 196608 where clusters of 16 are not to be had). As few as give every
+// entry of the table a thread of its own, and two to a thread by LFU, where the list is most of the table as a rule (32768
+// entries: 35.6 us with 8 blocks, 34.5 with 16).
 int select_blocks(const od_ctx *c)
 {
     if (cudaFuncSetAttribute(trim_select_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||
@@ -941,8 +954,8 @@ int select_blocks(const od_ctx *c)
         return 0;
     }
     const int64_t entries = c->dyn_max + c->dyn_max_insert;
-    const int64_t want = c->dyn_policy == 0 ? std::max<int64_t>((c->dyn_max_insert + SELECT_THREADS - 1) / SELECT_THREADS, (entries + 16383) / 16384)
-                                            : (entries + 2 * SELECT_THREADS - 1) / (2 * SELECT_THREADS);
+    const int64_t per_thread = c->dyn_policy == 0 ? 1 : 2;
+    const int64_t want = (entries + per_thread * SELECT_THREADS - 1) / (per_thread * SELECT_THREADS);
     int blocks = 1, best = 0;
     for (; blocks <= SELECT_MAX_BLOCKS; blocks *= 2) {
         if (select_room(c, blocks) > SELECT_ROOM_MAX) continue;
@@ -1068,12 +1081,14 @@ int32_t od_cache_trim(od_ctx *c, void *stream)
     // one resident wave at most, and no more blocks than have anything to do
     const int64_t most = c->sm_count * 4;
     const unsigned passes = (unsigned)std::min<int64_t>(most, (c->cap / OD_GROUP + QUAD * TRIM_HALVES - 1) / (QUAD * TRIM_HALVES));
-    const unsigned place = (unsigned)std::min<int64_t>(most, (c->dyn_max + c->dyn_max_insert + TRIM_THREADS - 1) / TRIM_THREADS);
     const bool pdl = c->opt_pdl != 0;
     const int blocks = c->trim_blocks;                      // 0: the select is a chain of launches
-    // The select's cluster places what it leaves of the list by itself, which spares a launch, but by LFU, where the list
-    // is long: most entries have a frequency of one, where a clock is that of one batch.
-    const bool placed = blocks && c->dyn_policy == 0;
+    // whether the list may be longer than what the select's cluster places by itself
+    const int64_t entries = c->dyn_max + c->dyn_max_insert;
+    const bool follow = !blocks || entries > (int64_t)blocks * SELECT_THREADS;
+    // (without a long list that launch costs a trim 0.9 us with four blocks to a multiprocessor, 0.7 with two, 0.5 with one; with
+    // 262144 entries to place four and two take the same, one 2.5 us more)
+    const unsigned place = (unsigned)std::min<int64_t>(blocks ? c->sm_count * 2 : most, (entries + TRIM_THREADS - 1) / TRIM_THREADS);
     const Table from = {(unsigned long long *)c->d_keys, c->d_vals, c->d_stamp, c->d_freq, c->d_born, c->d_fill};
     const Table to = {(unsigned long long *)c->d_keys2, c->d_vals2, c->d_stamp2, c->d_freq2, c->d_born2, c->d_fill2};
     if (!blocks) OD_CUDA(chain_launch(trim_begin_kernel, 1u, 256u, s, pdl, st, (unsigned int)c->dyn_max));
@@ -1088,15 +1103,15 @@ int32_t od_cache_trim(od_ctx *c, void *stream)
         cfg.stream = s;
         cfg.numAttrs = pdl ? 2 : 1;
         OD_CUDA(cudaLaunchKernelEx(&cfg, trim_select_kernel, select_room(c, blocks), from, to, c->cap, c->d_trim_lists, st,
-                                   placed ? 1 : 0));
+                                   follow ? 1 : 0));
     } else {
         for (int pass = 0; pass < PASSES; ++pass)
             OD_CUDA(chain_launch(trim_hist_kernel, (unsigned)c->sm_count, 256u, s, pdl, pass, c->cap,
                                  c->d_trim_lists, st));
     }
-    if (!placed)
+    if (follow)
         OD_CUDA(chain_launch(trim_place_kernel, place, (unsigned)TRIM_THREADS, s, pdl, from, to, c->cap, c->d_trim_lists,
-                             st, blocks ? 1 : 0));
+                             st, (unsigned)blocks * SELECT_THREADS));
     if (!blocks) OD_CUDA(chain_launch(trim_end_kernel, 1u, 1u, s, pdl, st));
     // the rebuilt table is the table for every call enqueued from now on
     std::swap(c->d_keys, c->d_keys2); std::swap(c->d_vals, c->d_vals2);

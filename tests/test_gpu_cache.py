@@ -415,3 +415,31 @@ def test_trim_of_a_table_filled_to_the_brim(cuda_device, policy, bound, batch):
         assert len(ref) == bound and ctx.cache_stats() == (bound, 0, 0)
         _compare(ctx, ref)
     ctx.close()
+
+
+# lists of one clock's entries from more than a cluster of the select holds down to none, over every number of its blocks
+@pytest.mark.parametrize("policy", [cp.LRU, cp.LFU])
+@pytest.mark.parametrize("bound, batch, tick", [(500, 90, 1), (3000, 170, 1), (3000, 170, 1000), (20000, 1100, 1)])
+def test_trims_while_the_entries_of_one_clock_run_out(cuda_device, policy, bound, batch, tick):
+    rng = np.random.default_rng(70)
+    v_q, v_p, dev = 32000, 128256, cuda_device
+    ctx = od.Context(cuda_device, v_q, v_p, 4, 4)
+    ctx.set_vocab_map(np.full(v_q, -1, np.int32))
+    ctx.cache_configure(bound, policy, batch)
+    ref = cp.DynamicCache(bound, policy, v_q, v_p)
+    clock = 5
+    while True:
+        ctx.cache_set_clock(clock); ref.set_clock(clock)
+        runs, lens = _universe(rng, batch, v_q)
+        tg = rng.integers(0, v_p, size=batch).astype(np.int32)
+        ctx.cache_insert(torch.from_numpy(runs).to(dev), torch.from_numpy(lens).to(dev), torch.from_numpy(tg).to(dev))
+        ref.insert_batch(runs, lens, tg)
+        if clock == 5 and len(ref) < bound:
+            continue                                        # the first clock's entries, without a trim between
+        ctx.cache_trim(); ref.trim()
+        _compare(ctx, ref)
+        assert ctx.cache_stats()[0] == len(ref)
+        if clock > 5 + tick * (bound // batch + 2):
+            break
+        clock += tick
+    ctx.close()
