@@ -61,6 +61,9 @@ struct TrimState {
     unsigned long long hi_and, hi_or;       // AND / OR of (new?, score) over the listed entries: bits that never vary
     unsigned long long thr_hi, thr_lo;      // trim_select_kernel: the k-th order key
     unsigned int bins[256];     // live entries by score (score_bin)
+    // LRU: hardly an entry was accessed before this clock (what the last trim dropped was, if none has been set back since), and what
+    // it is behind a trim without a list. Where the bins begin: what stays and what goes does not depend on it.
+    unsigned int oldest, next_oldest;
     SelState sel[PASSES + 1];   // sel[p]: written by block 0 of pass p (sel[PASSES]: by the rebuild)
     unsigned int n_out[PASSES]; // entries pass p copied into its output list
     unsigned int hist[PASSES][256];
@@ -251,23 +254,31 @@ __device__ __forceinline__ unsigned int block_offsets(unsigned int n, unsigned i
 // of it is a chain of trips as long as a launch's.)
 constexpr int TRIM_THREADS = 256, TRIM_HALVES = TRIM_THREADS / 16, QUAD = 4;   // groups of a half-warp at a time
 
-// (new?, score) to one of 256 bins, in the order of trims: 255 new; else by age (LRU) or frequency (LFU), exact up to 127,
-// four bins to an octave beyond. (A stamp past the clock, which the caller may set back, counts as of now.)
+// (new?, score) to one of 256 bins, in the order of trims: 255 new; else by frequency (LFU), or by the clock from the oldest
+// on (LRU), exact for 128 of them, four bins to an octave beyond. LRU drops the oldest, so their clocks have bins of their own
+// whatever the step of the clock: by age, exact for the last 127 clocks, the entries of several batches shared the bin where
+// the k-th is (16384 entries, 256 new ones, an insertion and a trim, with a clock that goes on by 1000: 25.9 us by age, 18.0 so).
 __device__ __forceinline__ unsigned int log_bin(unsigned int v)
 {
     const int e = 31 - __clz((int)v);
     return v < 128u ? v : 128u + ((unsigned int)(e - 7) << 2) + (v >> (e - 2) & 3u);   // at most 227
 }
-__device__ __forceinline__ unsigned int score_bin(int policy, unsigned int clock, unsigned int score, bool is_new)
+// the least value of a bin (of one beyond the last: 2^32)
+__device__ __forceinline__ unsigned long long log_bin_floor(unsigned int bin)
+{
+    return bin < 128u ? bin : (unsigned long long)(4u + (bin & 3u)) << (((bin - 128u) >> 2) + 5u);
+}
+__device__ __forceinline__ unsigned int score_bin(int policy, unsigned int oldest, unsigned int score, bool is_new)
 {
     if (is_new) return 255u;
-    return policy == 0 ? 254u - log_bin(score <= clock ? clock - score : 0u) : log_bin(score);
+    if (policy != 0) return log_bin(score);
+    return score < oldest ? 0u : 1u + log_bin(score - oldest);
 }
 // whether all of a bin's entries have one (new?, score), and which
-__device__ __forceinline__ bool exact_bin(int policy, unsigned int clock, unsigned int bin, unsigned long long &hi)
+__device__ __forceinline__ bool exact_bin(int policy, unsigned int oldest, unsigned int bin, unsigned long long &hi)
 {
-    hi = policy == 0 ? (unsigned long long)(clock - (254u - bin)) : (unsigned long long)bin;
-    return policy == 0 ? bin < 254u && bin > 254u - 128u && 254u - bin <= clock : bin < 128u;
+    hi = policy == 0 ? (unsigned long long)(oldest + bin - 1u) : (unsigned long long)bin;
+    return policy == 0 ? bin >= 1u && bin <= 128u : bin < 128u;
 }
 
 // Count digit `d` of the lanes with `ok` into hist: digits are heavily tied (scores, the upper
@@ -288,6 +299,7 @@ trim_count_kernel(int policy, unsigned int clock, const int32_t *vals, const uns
     const int64_t quads = (cap / OD_GROUP + QUAD - 1) / QUAD;
     const int at = threadIdx.x & 15;
     chain_wait(true);
+    const unsigned int oldest = __ldcg(&st->oldest);
     if (blockIdx.x == 0 && threadIdx.x == 0) { st->n_list = 0u; st->n_late = 0u; st->hi_and = ~0ull; st->hi_or = 0ull; }
     __syncthreads();
     for (int64_t q0 = (int64_t)blockIdx.x * TRIM_HALVES; q0 < quads; q0 += (int64_t)gridDim.x * TRIM_HALVES) {
@@ -304,7 +316,7 @@ trim_count_kernel(int policy, unsigned int clock, const int32_t *vals, const uns
             }
 #pragma unroll
             for (int e = 0; e < QUAD; ++e) {
-                count_digit(s_bins, score_bin(policy, clock, sc[e], bn[e] == clock), v[e] >= 0);   // (a slot without a value is no entry)
+                count_digit(s_bins, score_bin(policy, oldest, sc[e], bn[e] == clock), v[e] >= 0);   // (a slot without a value is no entry)
                 more = more || (at == 15 && v[e] >= 0);
             }
         }
@@ -386,7 +398,7 @@ trim_split_kernel(int policy, unsigned int clock, unsigned int max_entries, cons
     asm volatile("griddepcontrol.wait;" ::: "memory");
 
     // ---- the first bin at which the running count reaches k (none: everything goes)
-    const unsigned int size = __ldcg(&st->size), k = size > max_entries ? size - max_entries : 0u;
+    const unsigned int oldest = __ldcg(&st->oldest), size = __ldcg(&st->size), k = size > max_entries ? size - max_entries : 0u;
     const unsigned int mine = __ldcg(st->bins + threadIdx.x);
     unsigned int total;
     const unsigned int before = block_offsets(mine, s_warp, total);
@@ -395,9 +407,11 @@ trim_split_kernel(int policy, unsigned int clock, unsigned int max_entries, cons
     const bool whole = s_rem == s_in;                       // the bin goes as a whole: nothing is left to find out
     const unsigned int first_kept = k == 0u ? 0u : s_bin + (whole ? 1u : 0u), mixed = k == 0u || whole ? 512u : s_bin;
     unsigned long long bin_hi;
-    const bool exact = exact_bin(policy, clock, mixed & 255u, bin_hi);
+    const bool exact = exact_bin(policy, oldest, mixed & 255u, bin_hi);
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         st->k = k; st->k_rem = mixed < 256u ? s_rem : 0u;
+        // (bins up to s_bin went: the least clock of the next)
+        st->next_oldest = k == 0u || s_bin >= 256u ? oldest : (unsigned int)min((unsigned long long)clock, oldest + log_bin_floor(s_bin));
         if (exact) { st->hi_and = bin_hi; st->hi_or = bin_hi; }
     }
 
@@ -426,7 +440,7 @@ trim_split_kernel(int policy, unsigned int clock, unsigned int max_entries, cons
                     const int64_t g = quad * QUAD + e;
                     const bool is_new = en[e].born == clock;
                     const unsigned int score = policy == 0 ? en[e].stamp : en[e].freq;
-                    const unsigned int bin = en[e].v >= 0 ? score_bin(policy, clock, score, is_new) : 0u;
+                    const unsigned int bin = en[e].v >= 0 ? score_bin(policy, oldest, score, is_new) : 0u;
                     const bool live = en[e].v >= 0;
                     bool home = true;
                     if (ask_here) home = (int64_t)(od_hash64(en[e].key) & (uint64_t)(groups - 1)) == g;
@@ -521,7 +535,10 @@ trim_select_kernel(unsigned int room, const Table from, const Table to, int64_t 
     const unsigned int n = (unsigned int)min((int64_t)__ldcg(&st->n_list), cap), k = __ldcg(&st->k_rem);
     const unsigned long long hi_and = __ldcg(&st->hi_and), hi_or = __ldcg(&st->hi_or);
     const TrimLists L = trim_lists(lists, cap);
-    if (rank == 0 && threadIdx.x == 0) st->size = __ldcg(&st->size) - __ldcg(&st->k);
+    if (rank == 0 && threadIdx.x == 0) {
+        st->size = __ldcg(&st->size) - __ldcg(&st->k);
+        if (n == 0u) st->oldest = __ldcg(&st->next_oldest);
+    }
     if (rank == 0 && threadIdx.x < 256) st->bins[threadIdx.x] = 0u;   // for the next trim
     const bool one = n <= gridDim.x * SELECT_THREADS, place = one || !follow;
     if (place) {
@@ -703,7 +720,7 @@ trim_select_kernel(unsigned int room, const Table from, const Table to, int64_t 
             if (hi > thr_hi || (hi == thr_hi && key > thr_lo)) place_entry(to, cap, en);
         }
     od_cluster_wait();
-    if (rank == 0 && threadIdx.x == 0) { st->thr_hi = thr_hi; st->thr_lo = thr_lo; }
+    if (rank == 0 && threadIdx.x == 0) { st->thr_hi = thr_hi; st->thr_lo = thr_lo; st->oldest = (unsigned int)thr_hi; }
 }
 
 // ---- the same as a chain of launches, for tables too large for one cluster -----------------
@@ -885,6 +902,7 @@ trim_place_kernel(const Table from, const Table to, int64_t cap, void *lists, Tr
             const SelState S = select_state(PASSES, st, s_hist, &s_sel);
             thr_hi = S.pre_hi; thr_lo = S.pre_lo;
             if (i0 < n) load(i0);
+            if (i0 == 0) st->next_oldest = (unsigned int)thr_hi;
         }
     }
     for (unsigned int i = i0; i < n; i += stride) {
@@ -898,7 +916,7 @@ trim_place_kernel(const Table from, const Table to, int64_t cap, void *lists, Tr
 __global__ void trim_end_kernel(TrimState *st)
 {
     chain_wait();
-    st->size -= st->k; st->k = 0u;
+    st->size -= st->k; st->k = 0u; st->oldest = st->next_oldest;
 }
 
 #define OD_CUDA(call)                                  \

@@ -443,3 +443,44 @@ def test_trims_while_the_entries_of_one_clock_run_out(cuda_device, policy, bound
             break
         clock += tick
     ctx.close()
+
+
+def _clocks(kind, n):
+    if kind == "steps of 1000":
+        return [4000 + 1000 * i for i in range(n)]
+    if kind == "any":
+        return list(np.cumsum(np.random.default_rng(3).choice([1, 2, 130, 5000, 70000000], size=n)))
+    if kind == "set back":                                  # and on from there, and behind the end of 32 bits
+        return [100000 + 10 * i for i in range(n // 3)] + [50 + i for i in range(n // 3)] + [0xFFFFFFF0 + i for i in range(15)]
+    return [7 + i // 4 for i in range(n)]                   # four insertions to a tick
+
+
+# the bins by clock begin where the last trim left off, which says nothing about entries that the caller dates back
+@pytest.mark.parametrize("kind, bound, batch", [(kind, *size) for kind in ("steps of 1000", "any", "set back", "four a tick")
+                                                for size in ((200, 30), (2048, 256), (5000, 900))] + [("steps of 1000", 400000, 50000)])
+def test_trims_by_clocks_of_any_step(cuda_device, kind, bound, batch):
+    rng = np.random.default_rng(77)
+    v_q, v_p, dev = 3000, 30000, cuda_device
+    ctx = od.Context(cuda_device, v_q, v_p, 64, 4)
+    ctx.set_vocab_map(np.full(v_q, -1, np.int32))
+    ctx.cache_configure(bound, cp.LRU, batch)
+    ref = cp.DynamicCache(bound, cp.LRU, v_q, v_p)
+    for clock in _clocks(kind, bound // batch + (4 if bound > 100000 else 30)):
+        ctx.cache_set_clock(int(clock)); ref.set_clock(int(clock))
+        runs, lens = _universe(rng, batch, v_q)
+        tg = rng.integers(0, v_p, size=batch).astype(np.int32)
+        ctx.cache_insert(torch.from_numpy(runs).to(dev), torch.from_numpy(lens).to(dev), torch.from_numpy(tg).to(dev))
+        ref.insert_batch(runs, lens, tg)
+        # some of the entries are accessed
+        held = list(ref.entries)
+        picked = [held[i] for i in rng.integers(0, len(held), size=64)]
+        d, klen = np.zeros((64, 4), np.int32), np.zeros(64, np.int32)
+        for b, run in enumerate(picked):
+            klen[b] = len(run); d[b, :len(run)] = run
+        od.od_map_proposals(ctx, torch.from_numpy(d).to(dev), torch.from_numpy(klen).to(dev), torch.ones(64, 4, device=dev))
+        for b in range(64):
+            ref.map_sequence(np.full(v_q, -1, np.int32), d[b, :klen[b]], np.ones(4, np.float32))
+        ctx.cache_trim(); ref.trim()
+        assert ctx.cache_stats()[0] == len(ref)
+    _compare(ctx, ref)
+    ctx.close()
