@@ -116,7 +116,7 @@ unsigned long long cuda_context_id()
 // lost with it, after cudaDeviceReset for instance), not in every od_create, which they made 1 ms and more longer.
 bool prepare_kernels(od_ctx *c)
 {
-    struct Resident { unsigned long long context; int32_t sample[OD_SAMPLE_LEVELS], step[OD_SAMPLE_LEVELS]; };
+    struct Resident { unsigned long long context; int32_t sample[OD_SAMPLE_LEVELS], step[OD_SAMPLE_LEVELS], shard[OD_SHARD_SIZES][OD_SAMPLE_MAX_PARTS + 1]; };
     constexpr int DEVICES = 64;
     static std::mutex mutex;
     static Resident of[DEVICES];
@@ -126,11 +126,12 @@ bool prepare_kernels(od_ctx *c)
     const unsigned long long id = cuda_context_id();
     if (id == 0 || r.context != id) {
         r.context = 0;
-        if (od_sample_prepare_device(r.sample) != cudaSuccess || od_step_prepare_device(r.step) != cudaSuccess) return false;
+        if (od_sample_prepare_device(r.sample, r.shard) != cudaSuccess || od_step_prepare_device(r.step) != cudaSuccess) return false;
         r.context = id;
     }
     memcpy(c->sample_clusters, r.sample, sizeof(r.sample));
     memcpy(c->step_clusters, r.step, sizeof(r.step));
+    memcpy(c->shard_clusters, r.shard, sizeof(r.shard));
     return true;
 }
 

@@ -13,7 +13,9 @@
 #define OD_WARP 32
 #define OD_GROUP 32                 // slots of one hash-table probe group
 #define OD_SAMPLE_TILE 256          // elements of one residual-sampler tile (8 per lane of a warp)
-#define OD_SAMPLE_THREADS 256       // of the vocabulary shards' sampler
+#define OD_SAMPLE_THREADS 256       // of the vocabulary shards' sampler; a shard's mass by blocks of 256, 512 or 1024
+#define OD_SHARD_SIZES 3
+#define OD_SHARD_MAX_THREADS (OD_SAMPLE_THREADS << (OD_SHARD_SIZES - 1))
 #define OD_SAMPLE_LEVELS 8          // 1, 2, 3, 4, 5, 6, 8 or 16 blocks draw for one sequence
 #define OD_SAMPLE_MAX_PARTS 16      // (over 8: a non-portable cluster)
 #define OD_SAMPLE_MAX_SLOTS 53248   // mapped ids of a part: 208 KB of shared memory
@@ -38,6 +40,7 @@ struct od_ctx {
     int32_t sample_slots[OD_SAMPLE_LEVELS];   // most mapped ids of a part
     int32_t sample_clusters[OD_SAMPLE_LEVELS];   // clusters of the sampler that are resident at a time
     int32_t step_clusters[OD_SAMPLE_LEVELS];     // of the whole step in one launch: a multiprocessor to each block
+    int32_t shard_clusters[OD_SHARD_SIZES][OD_SAMPLE_MAX_PARTS + 1];   // of a shard's mass, by threads and blocks
     bool have_map;
     bool distill_lists;             // some map had gather lists: every later one has the distillation kernel's
     // The map's serial number. A launch is laid out for the map of its time (where ids are shared, how many
@@ -174,7 +177,7 @@ cudaError_t od_launch_sample(od_ctx *c, int32_t B, int32_t K_max, const void *lo
 
 size_t od_sample_smem_bytes(int32_t ntiles);            // dynamic shared memory of the shard sampler's kernel
 // opt in to the dynamic shared memory and the cluster size that the sampler's kernels may ask for
-cudaError_t od_sample_prepare_device(int32_t *clusters);   // clusters: [levels] resident at a time
+cudaError_t od_sample_prepare_device(int32_t *clusters, int32_t (*shard_clusters)[OD_SAMPLE_MAX_PARTS + 1]);   // resident at a time
 
 // The pairs of a vocabulary map in target-id order (host).
 struct OdMappedIds {

@@ -251,20 +251,49 @@ __device__ __forceinline__ float warp_sum_f32(float v)
 struct GlobalTiles {                                        // [ntiles] of one sequence
     double *val;
     int lane;
-    double total;                                           // of the warp's tiles: lanes 0..15 and 16..31 each hold a share
-    __device__ __forceinline__ void one(int t, float v)
-    {
-        if (lane == 0) val[t] = (double)v;
-        if (lane < 16) total += (double)fmaxf(0.f, v);      // (a tile with NaN has no mass)
-    }
+    __device__ __forceinline__ void one(int t, float v) { if (lane == 0) val[t] = (double)v; }
     __device__ __forceinline__ void pair(int t, float v, bool two)
     {
         if ((lane & 15) == 0 && (lane == 0 || two)) val[t + (lane >> 4)] = (double)v;
-        total += lane < 16 || two ? (double)fmaxf(0.f, v) : 0.0;
+    }
+};
+// The same, and the sum of the warp's. With fp32 rows the tile loop spills by it, so it is kept in shared memory (a rank's
+// mass of 256 sequences, half of 152064 ids, in registers and in shared memory: fp32 28.8 and 27.3 us, bf16 23.4 and 24.6).
+template <int DTYPE>
+struct SummedTiles {
+    double *val, *s_sum;                                    // s_sum: two of the warp's own (fp32)
+    int lane;
+    double total;                                           // (bf16) lanes 0..15 and 16..31 each hold a share
+    __device__ __forceinline__ void clear()
+    {
+        total = 0.0;
+        if (DTYPE == OD_BF16) return;
+        __syncwarp();
+        if (lane < 2) s_sum[lane] = 0.0;
+        __syncwarp();
+    }
+    __device__ __forceinline__ void one(int t, float v)
+    {
+        if (lane == 0) val[t] = (double)v;
+        v = fmaxf(0.f, v);                                  // (a tile with NaN has no mass)
+        if (DTYPE == OD_BF16) {
+            if (lane < 16) total += (double)v;
+        } else if (lane == 0) {
+            s_sum[0] += (double)v;
+        }
+    }
+    __device__ __forceinline__ void pair(int t, float v, bool two)
+    {
+        if (DTYPE == OD_BF16) total += lane < 16 || two ? (double)fmaxf(0.f, v) : 0.0;
+        if ((lane & 15) != 0 || (lane != 0 && !two)) return;
+        val[t + (lane >> 4)] = (double)v;
+        if (DTYPE != OD_BF16) s_sum[lane >> 4] += (double)fmaxf(0.f, v);
     }
     __device__ __forceinline__ double sum() const
     {
-        return __shfl_sync(0xFFFFFFFFu, total, 0) + __shfl_sync(0xFFFFFFFFu, total, 16);
+        if (DTYPE == OD_BF16) return __shfl_sync(0xFFFFFFFFu, total, 0) + __shfl_sync(0xFFFFFFFFu, total, 16);
+        __syncwarp();
+        return s_sum[0] + s_sum[1];
     }
 };
 struct WarpTiles {                                          // the warp's own run in shared memory, and its sum
@@ -779,7 +808,7 @@ __device__ __forceinline__ void draw_from_p(const SeqState &q, const SampleArgs 
     __shared__ double s_sum[CTHREADS];
     __shared__ int s_crossing, s_lastmass, s_done;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    GlobalTiles out = {a.tile_val + (size_t)b * a.ntiles, lane, 0.0};
+    GlobalTiles out = {a.tile_val + (size_t)b * a.ntiles, lane};
     for (int t = warp * 2; t < a.ntiles; t += CWARPS * 2)
         warp_tiles_dense<DTYPE, 2>(q, a, false, t, t + 2 < a.ntiles ? t + 2 : a.ntiles, lane, out);
     if (threadIdx.x == 0) { s_crossing = 0x7FFFFFFF; s_lastmass = -1; s_done = 0; }
@@ -1044,12 +1073,12 @@ __device__ __forceinline__ void draw(const SampleArgs &a, const Ahead &h, Part<S
 
 // ---- host: how many blocks draw for one of B sequences, and what a launch of that many is told ----
 
-// clusters of `parts` blocks of CTHREADS that are resident at a time (0: the device has no room for one)
+// clusters of `parts` blocks that are resident at a time (0: the device has no room for one)
 template <typename Kern>
-int resident_clusters(Kern kern, int parts, size_t smem)
+int resident_clusters(Kern kern, int parts, size_t smem, int threads = CTHREADS)
 {
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)parts); cfg.blockDim = dim3(CTHREADS); cfg.dynamicSmemBytes = smem;
+    cfg.gridDim = dim3((unsigned)parts); cfg.blockDim = dim3((unsigned)threads); cfg.dynamicSmemBytes = smem;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = (unsigned)parts; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;

@@ -39,9 +39,7 @@
 // kernel in two further modes. A shard owns a window of whole tiles:
 //   mode 1  pass 1 over the window by a cluster of blocks, whose sums meet in the first
 //           one: the shard's share of the residual mass (and, when that is zero, of the
-//           mass of p_j, for the fallback). A rank's five calls, 64 sequences, a quarter of
-//           128256 ids: 25.1 us with a ticket, two fences and a last block that loaded the tile
-//           values again, 24.4 so;
+//           mass of p_j, for the fallback);
 //   mode 2  after the shares of all shards were exchanged: every shard forms the
 //           same total and target = u * total, finds the shard in which the running
 //           sum over shards crosses the target, and that shard alone scans its
@@ -160,13 +158,16 @@ od_sample_kernel(const SampleArgs a)
 }
 
 // ---- vocabulary shards: MODE 1, a shard's mass shares; MODE 2, a shard's pick ---------------
+// 64 registers in both: four blocks of 256 threads to a multiprocessor; MODE 1 may have blocks of up to 1024.
 template <int DTYPE, int MODE>
-__global__ void __launch_bounds__(OD_SAMPLE_THREADS, 4)
+__global__ void __launch_bounds__(MODE == 1 ? OD_SHARD_MAX_THREADS : OD_SAMPLE_THREADS, MODE == 1 ? 1 : 4)
 od_sample_shard_kernel(const SampleArgs a)
 {
     extern __shared__ __align__(16) unsigned char s_dyn[];   // ntiles x 8 bytes
     double *s_val = (double *)s_dyn;                         // pass 2: tile values
-    __shared__ double s_warp[WARPS];
+    __shared__ double s_warp[MODE == 1 ? OD_SHARD_MAX_THREADS / 32 : WARPS];
+    __shared__ double s_sums[MODE == 1 && DTYPE != OD_BF16 ? OD_SHARD_MAX_THREADS / 32 * 2 : 1];
+    const int warps = MODE == 1 ? (int)(blockDim.x >> 5) : WARPS;
     __shared__ double s_part[OD_SAMPLE_MAX_PARTS];          // MODE 1: the cluster's blocks' sums, in its first block
     __shared__ int s_tile, s_lastmass, s_done;
     __shared__ double s_before;
@@ -189,7 +190,7 @@ od_sample_shard_kernel(const SampleArgs a)
     // a shard's tiles and ids keep their numbers of the full row
     const int tile_lo = a.tile_lo, tile_hi = a.tile_hi;
     // pass 1's whole tiles of this warp, and the inverse-map entries of their first pair
-    const int p_lo = tile_lo + ((int)part * WARPS + warp) * a.tiles_per_warp;
+    const int p_lo = tile_lo + ((int)part * warps + warp) * a.tiles_per_warp;
     int p_hi = p_lo + a.tiles_per_warp;
     if (p_hi > tile_hi) p_hi = tile_hi;
     const int p_hi_w = p_hi < a.v_p / OD_SAMPLE_TILE ? p_hi : a.v_p / OD_SAMPLE_TILE;
@@ -240,9 +241,9 @@ od_sample_shard_kernel(const SampleArgs a)
     const SeqState q = seq_state<DTYPE>(a, h, b, j, rm, rs, a.col0, planned);
     if (MODE != 2 && q.residual && threadIdx.x == 0) prefetch_q_row(a, q, part, nparts);
 
-    GlobalTiles out = {tile_val, lane, 0.0};
-
     if (MODE != 2) {
+        SummedTiles<DTYPE> out = {tile_val, s_sums + (DTYPE == OD_BF16 ? 0 : 2 * warp), lane, 0.0};
+        out.clear();
         // ---- pass 1: the value of every tile ----
         const int hi_w = planned || !a.same_ids ? p_hi_w : p_lo;
         if (a.same_ids) warp_run<DTYPE, FROM_ROW, false>(q, a, p_lo, p_hi, hi_w, lane, out, ni);
@@ -254,7 +255,7 @@ od_sample_shard_kernel(const SampleArgs a)
         od_cluster_wait();
         if (threadIdx.x == 0) {
             double sum = 0.0;
-            for (int w = 0; w < WARPS; ++w) sum += s_warp[w];
+            for (int w = 0; w < warps; ++w) sum += s_warp[w];
             od_cluster_store(&s_part[part], 0u, sum);
         }
         od_cluster_arrive();
@@ -264,13 +265,13 @@ od_sample_shard_kernel(const SampleArgs a)
         for (unsigned int i = 0; i < nparts; ++i) mass_r += s_part[i];
         if (q.residual && !(mass_r > 0.0)) {
             // no residual mass here: should no shard have any, the draw is from p_j
-            out.total = 0.0;
-            for (int t_lo = tile_lo + warp * 2; t_lo < tile_hi; t_lo += WARPS * 2)
+            out.clear();
+            for (int t_lo = tile_lo + warp * 2; t_lo < tile_hi; t_lo += warps * 2)
                 warp_tiles_dense<DTYPE, 2>(q, a, false, t_lo, t_lo + 2 < tile_hi ? t_lo + 2 : tile_hi, lane, out);
             const double e_sum = out.sum();
             if (lane == 0) s_warp[warp] = e_sum;
             __syncthreads();
-            for (int w = 0; w < WARPS; ++w) mass_e += s_warp[w];
+            for (int w = 0; w < warps; ++w) mass_e += s_warp[w];
         }
         if (threadIdx.x == 0) { a.mass_out[2 * b] = mass_r; a.mass_out[2 * b + 1] = mass_e; }
         return;
@@ -435,14 +436,46 @@ static cudaError_t prepare_kernels()
 // context (it is the kernel's: a smaller one would take it from a context made earlier), and ask how many
 // clusters of each size are resident at a time (0: the device has no room for one; the device must be
 // current; allocates nothing).
-cudaError_t od_sample_prepare_device(int32_t *clusters)
+cudaError_t od_sample_prepare_device(int32_t *clusters, int32_t (*shard_clusters)[OD_SAMPLE_MAX_PARTS + 1])
 {
     cudaError_t e = prepare_kernels<OD_BF16>();
     if (e == cudaSuccess) e = prepare_kernels<OD_F32>();
     if (e != cudaSuccess) return e;
     for (int level = 0; level < OD_SAMPLE_LEVELS; ++level)
         clusters[level] = resident_clusters(od_sample_kernel<OD_BF16, true, STAGED>, od_sample_parts(level), 64 * 1024);
+    for (int size = 0; size < OD_SHARD_SIZES; ++size) {
+        shard_clusters[size][0] = 0;
+        for (int parts = 1; parts <= OD_SAMPLE_MAX_PARTS; ++parts)
+            shard_clusters[size][parts] = resident_clusters(od_sample_shard_kernel<OD_F32, 1>, parts, 0, OD_SAMPLE_THREADS << size);
+    }
     return cudaSuccess;
+}
+
+// How a shard's window of `tiles` tiles is cut for B sequences (MODE 1): blocks of a cluster, their threads, tiles of a warp
+struct ShardCut {
+    int blocks, threads;
+    int64_t tiles_per_warp;
+};
+// As few tiles a warp as give every sequence a cluster that is resident at once, which is asked of the device for every size:
+// a cluster is placed as a whole, and those that find no place wait for a whole round (45 sequences, half of 152064 bf16 ids, a
+// rank's five calls: 28.0 us with 13 blocks of 256 threads, of which 38 clusters are resident, 24.7 with 10 and 56). A sixteenth of
+// the room is left free, or the last ones are placed late (70 sequences, a quarter of 128256 ids: 8 blocks with 71 places
+// 23.8, 2 of 1024 threads 22.6). An even number of tiles, since warps work on pairs. Larger blocks where they give each warp
+// fewer tiles: in windows that 16 blocks of 256 threads cannot share so finely (one sequence, half of a million ids: 23.2
+// and 20.8 with 1024) and for numbers of sequences between theirs (145, half of 152064: 43.5 with 3 of 256, 40.4 with 2 of 512).
+static ShardCut shard_cut(const od_ctx *c, int32_t B, int64_t tiles)
+{
+    const int64_t asked = c->opt_sample_tiles_per_warp;
+    for (int64_t tpw = asked > 0 ? asked : 2;; tpw += asked > 0 ? 1 : 2)
+        for (int size = 0; size < OD_SHARD_SIZES; ++size) {
+            const int threads = OD_SAMPLE_THREADS << size, warps = threads / 32;
+            const int64_t blocks = (tiles + tpw * warps - 1) / (tpw * warps);
+            if (blocks > OD_SAMPLE_MAX_PARTS) continue;
+            const int32_t room = c->shard_clusters[size][blocks];
+            const bool fits = asked > 0 ? room > 0 : B <= (blocks > 2 ? room - room / 16 : room);
+            if (!fits && (size > 0 || blocks > 1)) continue;    // (single blocks, whatever their number)
+            return {(int)blocks, threads, asked > 0 ? tpw : (tiles + blocks * warps - 1) / (blocks * warps)};
+        }
 }
 
 template <int DTYPE>
@@ -476,31 +509,18 @@ static cudaError_t launch_sample(od_ctx *c, int mode, int32_t B, int32_t K_max, 
     const int ntiles = c->tiles_per_row;
     const int tile_lo = mode == 0 ? 0 : shard_lo / OD_SAMPLE_TILE;
     const int tile_hi = mode == 0 ? ntiles : (shard_lo + shard_len + OD_SAMPLE_TILE - 1) / OD_SAMPLE_TILE;
-    const int wtiles = tile_hi - tile_lo;
-    int64_t tpw = c->opt_sample_tiles_per_warp;
-    int blocks_x = 1, level = 0;
+    ShardCut cut = {1, OD_SAMPLE_THREADS, 1};
+    int level = 0;
     if (mode == 0) {
         level = draw_level(c, B);
-        blocks_x = od_sample_parts(level);
-    } else {
-        if (tpw <= 0) {
-            // one resident wave (four 256-thread blocks per SM) over the whole batch
-            const int64_t want = (int64_t)c->sm_count * 4;
-            int64_t per_row = want / B;
-            if (per_row < 1) per_row = 1;
-            if (per_row > OD_SAMPLE_MAX_PARTS) per_row = OD_SAMPLE_MAX_PARTS;
-            tpw = (wtiles + per_row * WARPS - 1) / (per_row * WARPS);
-            if (tpw < 1) tpw = 1;
-        }
-        // (a cluster has at most 16 blocks)
-        if (tpw * WARPS * OD_SAMPLE_MAX_PARTS < wtiles) tpw = (wtiles + WARPS * OD_SAMPLE_MAX_PARTS - 1) / (WARPS * OD_SAMPLE_MAX_PARTS);
-        const int64_t tiles_per_block = tpw * WARPS;
-        if (mode == 1) blocks_x = (int)((wtiles + tiles_per_block - 1) / tiles_per_block);
+        cut.blocks = od_sample_parts(level);
+    } else if (mode == 1) {
+        cut = shard_cut(c, B, tile_hi - tile_lo);
     }
     SampleArgs a = {};
     a.logits = logits; a.row_stride = row_stride; a.seq_stride = seq_stride;
     a.B = B; a.K_max = K_max; a.v_p = mode == 0 ? c->v_p : shard_lo + shard_len;
-    a.tiles_per_warp = (int32_t)tpw;
+    a.tiles_per_warp = (int32_t)cut.tiles_per_warp;
     a.row_max = row_max; a.row_sum = row_sum; a.q_rows = q_rows;
     a.draft_ids = draft_ids; a.tgt_ids = tgt_ids; a.q_prime = q_prime;
     a.span_start = span_start; a.span_len = span_len; a.m = m; a.tail_kind = tail_kind;
@@ -519,7 +539,7 @@ static cudaError_t launch_sample(od_ctx *c, int mode, int32_t B, int32_t K_max, 
     if (mode != 1) c->translation_complete = false;         // of this step; the next one has its own
     const DrawPlan plan = mode == 0 ? plan_draw(c, level, a) : DrawPlan{};
     if (mode != 2) {
-        c->info[2] = (int64_t)blocks_x * B;
+        c->info[2] = (int64_t)cut.blocks * B;
         c->info[3] = a.tiles_per_warp;
     }
 
@@ -531,19 +551,19 @@ static cudaError_t launch_sample(od_ctx *c, int mode, int32_t B, int32_t K_max, 
     cfg.attrs = c->opt_pdl ? attr : attr + 1;
     const bool bf = dtype == OD_BF16;
     if (mode == 0) {
-        cfg.gridDim = dim3((unsigned)blocks_x, (unsigned)B);
+        cfg.gridDim = dim3((unsigned)cut.blocks, (unsigned)B);
         cfg.blockDim = dim3(CTHREADS);
         attr[1].id = cudaLaunchAttributeClusterDimension;
-        attr[1].val.clusterDim.x = (unsigned)blocks_x; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
+        attr[1].val.clusterDim.x = (unsigned)cut.blocks; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
         cfg.numAttrs = c->opt_pdl ? 2 : 1;
         cfg.dynamicSmemBytes = plan.smem;
         return bf ? launch_step<OD_BF16>(cfg, a, fuse != nullptr, plan.source) : launch_step<OD_F32>(cfg, a, fuse != nullptr, plan.source);
     }
-    cfg.gridDim = dim3((unsigned)B, (unsigned)blocks_x);
-    cfg.blockDim = dim3(OD_SAMPLE_THREADS);
+    cfg.gridDim = dim3((unsigned)B, (unsigned)cut.blocks);
+    cfg.blockDim = dim3((unsigned)cut.threads);
     cfg.dynamicSmemBytes = mode == 1 ? 0 : od_sample_smem_bytes(ntiles);
     attr[1].id = cudaLaunchAttributeClusterDimension;
-    attr[1].val.clusterDim.x = 1; attr[1].val.clusterDim.y = (unsigned)blocks_x; attr[1].val.clusterDim.z = 1;
+    attr[1].val.clusterDim.x = 1; attr[1].val.clusterDim.y = (unsigned)cut.blocks; attr[1].val.clusterDim.z = 1;
     cfg.numAttrs = (c->opt_pdl ? 1 : 0) + (mode == 1 ? 1 : 0);
     if (mode == 1)
         return bf ? cudaLaunchKernelEx(&cfg, od_sample_shard_kernel<OD_BF16, 1>, a)

@@ -20,6 +20,16 @@ std::string &log_text() { static std::string s; return s; }
 struct Range { const char *p; size_t bytes; };
 std::vector<Range> &pinned() { static std::vector<Range> v; return v; }
 bool no_driver_functions = false;
+unsigned cluster_limit = 16;                                 // blocks of the largest cluster that the device has room for
+
+unsigned cluster_of(const cudaLaunchConfig_t *cfg)
+{
+    unsigned blocks = 1;
+    for (unsigned i = 0; i < cfg->numAttrs; ++i)
+        if (cfg->attrs[i].id == cudaLaunchAttributeClusterDimension)
+            blocks = cfg->attrs[i].val.clusterDim.x * cfg->attrs[i].val.clusterDim.y * cfg->attrs[i].val.clusterDim.z;
+    return blocks;
+}
 
 const char *const NAMES[] = {"od_map_kernel", "od_verify_stream_kernel", "od_verify_decide_kernel", "od_verify_finish_kernel",
                              "od_verify_rows_kernel", "od_sample_kernel", "od_sample_shard_kernel", "od_step_kernel",
@@ -63,6 +73,7 @@ const char *fake_log(void) { static std::string last; last = log_text(); log_tex
 void fake_pin(const void *p, size_t bytes) { pinned().push_back({(const char *)p, bytes}); }
 void fake_unpin_all(void) { pinned().clear(); }
 void fake_no_driver_functions(int none) { no_driver_functions = none != 0; }
+void fake_cluster_limit(int blocks) { cluster_limit = (unsigned)blocks; }
 
 // ---- the runtime
 #ifndef __CUDA_ARCH__                                        // (the device's has some of the same names)
@@ -79,7 +90,10 @@ cudaError_t __cudaPopCallConfiguration(dim3 *grid, dim3 *block, size_t *smem, vo
     return cudaSuccess;
 }
 cudaError_t cudaLaunchKernel(const void *func, dim3 grid, dim3, void **args, size_t, cudaStream_t) { return launched(func, grid, args); }
-cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t *cfg, const void *func, void **args) { return launched(func, cfg->gridDim, args); }
+cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t *cfg, const void *func, void **args)
+{
+    return cluster_of(cfg) > cluster_limit ? cudaErrorInvalidClusterSize : launched(func, cfg->gridDim, args);
+}
 cudaError_t cudaDeviceGetAttribute(int *v, cudaDeviceAttr a, int)
 {
     *v = a == cudaDevAttrMultiProcessorCount ? 148 : a == cudaDevAttrComputeCapabilityMajor ? 10 : 0;
@@ -107,9 +121,7 @@ cudaError_t cudaGetLastError(void) { return cudaSuccess; }
 cudaError_t cudaGetSymbolAddress(void **p, const void *s) { *p = const_cast<void *>(s); return cudaSuccess; }
 cudaError_t cudaOccupancyMaxActiveClusters(int *n, const void *, const cudaLaunchConfig_t *cfg)
 {
-    *n = 148;
-    for (unsigned i = 0; i < cfg->numAttrs; ++i)
-        if (cfg->attrs[i].id == cudaLaunchAttributeClusterDimension) *n = 148 / (int)cfg->attrs[i].val.clusterDim.x;
+    *n = cluster_of(cfg) > cluster_limit ? 0 : 148 / (int)cluster_of(cfg);
     return cudaSuccess;
 }
 cudaError_t cudaGetDriverEntryPointByVersion(const char *name, void **fn, unsigned, unsigned long long, cudaDriverEntryPointQueryResult *)

@@ -218,3 +218,21 @@ def test_shard_arguments_are_validated(cuda_device):
                                 s.logits[:, :, :256].contiguous(), od.alloc_verify_out(ctx, 2, w.k_max), s.q_rows,
                                 s.draft_ids, mp, s.temperature, s.seed, 0)      # shard_index >= n_shards
     ctx.close()
+
+
+# windows and batches whose mass is summed by clusters of 256, 512 and 1024 threads, of 9 to 15 and of 16 blocks, and by single blocks
+@pytest.mark.parametrize("dtype", ["bf16", "f32"])
+@pytest.mark.parametrize("v_p, n_shards, B, tiles, blocks", [(70001, 2, 1, 0, 9), (70001, 2, 3, 1, 9), (70001, 1, 2, 1, 9), (150001, 2, 4, 0, 10),
+                                                             (400001, 2, 2, 0, 13), (1000001, 2, 1, 0, 16), (5003, 2, 300, 0, 1),
+                                                             (70001, 2, 150, 0, 3), (70001, 2, 5, 200, 1)])
+def test_every_size_of_cluster_that_sums_a_shards_mass(cuda_device, dtype, v_p, n_shards, B, tiles, blocks):
+    w = _workload(f"mass{v_p}", B=B, k_max=1, v_q=300, v_p=v_p, cache_entries=20, logit_dtype=dtype)
+    st = synth.make_static(w)
+    ctx = parity.make_context(w, st, cuda_device)
+    ctx.set_option("sample_tiles_per_warp", tiles)
+    cache = oracle.Cache(st.runs, st.run_len, st.run_target)
+    s = synth.make_step(w, st, 0, device=cuda_device)
+    stats, _ = _sharded_check(ctx, cache, st, w, s, n_shards, sel=sorted({0, B // 2, B - 1}), logits=parity.pad_rows(s.logits))
+    assert stats.sample_compared > 0
+    assert ctx.last_launch_info(2) == blocks * B
+    ctx.close()

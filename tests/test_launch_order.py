@@ -204,3 +204,27 @@ def test_a_part_with_more_mapped_ids_than_two_blocks_can_stage_is_cut_in_the_sam
     c.map(); c.verify(); c.log()
     c.sample()
     assert [x for x in c.log() if x[0] == "od_sample_kernel"] == [("od_sample_kernel", (blocks, 200, 1), 1)]
+
+
+# a device that has room for no cluster of this many blocks, as the part of a divided one may; every number of a shard's
+# sequences, narrow and wide windows, and tiles per warp that the caller sets
+@pytest.mark.parametrize("limit", [1, 3, 8, 16])
+@pytest.mark.parametrize("v_p", [1000, 152064, 4000000])
+def test_a_shards_mass_asks_for_no_cluster_that_the_device_has_no_room_for(lib, limit, v_p):
+    helpers.fake_runtime_lib().fake_cluster_limit(limit)
+    try:
+        c = lib(v_q=1000, v_p=v_p, max_batch=512, k=1)
+        c.L.fake_no_driver_functions(1)                     # (the device is asked again for every context)
+        c.call("od_destroy", c.ctx)
+        c.call("od_create", C.byref(c.ctx), 0, 1000, v_p, 512, 1)
+        c.call("od_set_vocab_map", c.ctx, c.array(np.arange(1000, dtype=np.int32)[::-1].copy()))
+        p = c.zeros(64)                                     # (nothing is read)
+        for tiles in (0, 1, 1000):
+            c.call("od_set_option", c.ctx, b"sample_tiles_per_warp", C.c_int64(tiles))
+            for n in (1, 2, 37, 148, 149, 512):
+                c.log()
+                c.call("od_sample_shard_mass", c.ctx, n, 1, 0, v_p, p, 1, C.c_int64(v_p), C.c_int64(2 * v_p), *[p] * 11, p, p, None)
+                (name, grid, _), = c.log()
+                assert name == "od_sample_shard_kernel" and grid[0] == n and grid[1] <= limit
+    finally:
+        helpers.fake_runtime_lib().fake_cluster_limit(16)
