@@ -246,8 +246,9 @@ od_distill_kernel(const __grid_constant__ DistillArgs a)
     float *grad = a.grad ? a.grad + ((size_t)b * a.K_max + j) * a.v_q : nullptr;
     // The chunk's list: groups of 32 entries, one per lane (od_distill_lists). It belongs to the
     // context: the first entries are requested before the wait, the others a batch ahead.
-    // groups per warp and batch: as many as the registers hold (fp32 1 to 2 % slower with 5 in 40)
-    constexpr int EB = RESIDENT == 2 ? FEW_EB : DTYPE == OD_BF16 ? 5 : 4;
+    // groups per warp and batch (five in 40 registers: one chunk of 8000 bf16 ids 2 to 7 % slower, 32000 in four 2 to 4 %,
+    // 64 x 6 of 32000 and 128256 1 % faster)
+    constexpr int EB = RESIDENT == 2 ? FEW_EB : 4;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int2 groups = SAME ? make_int2(0, 0) : __ldg((const int2 *)a.list_ofs + rank);
     const int g_hi = groups.y;
