@@ -116,7 +116,10 @@ unsigned long long cuda_context_id()
 // lost with it, after cudaDeviceReset for instance), not in every od_create, which they made 1 ms and more longer.
 bool prepare_kernels(od_ctx *c)
 {
-    struct Resident { unsigned long long context; int32_t sample[OD_SAMPLE_LEVELS], step[OD_SAMPLE_LEVELS], shard[OD_SHARD_SIZES][OD_SAMPLE_MAX_PARTS + 1]; };
+    struct Resident {
+        unsigned long long context;
+        int32_t sample[OD_SAMPLE_LEVELS], step[OD_SAMPLE_LEVELS], shard[OD_SHARD_SIZES][OD_SAMPLE_MAX_PARTS + 1], distill[OD_DISTILL_LEVELS];
+    };
     constexpr int DEVICES = 64;
     static std::mutex mutex;
     static Resident of[DEVICES];
@@ -127,11 +130,13 @@ bool prepare_kernels(od_ctx *c)
     if (id == 0 || r.context != id) {
         r.context = 0;
         if (od_sample_prepare_device(r.sample, r.shard) != cudaSuccess || od_step_prepare_device(r.step) != cudaSuccess) return false;
+        od_distill_resident(r.distill);
         r.context = id;
     }
     memcpy(c->sample_clusters, r.sample, sizeof(r.sample));
     memcpy(c->step_clusters, r.step, sizeof(r.step));
     memcpy(c->shard_clusters, r.shard, sizeof(r.shard));
+    memcpy(c->distill_few_clusters, r.distill, sizeof(r.distill));
     return true;
 }
 

@@ -41,6 +41,7 @@ struct od_ctx {
     int32_t sample_clusters[OD_SAMPLE_LEVELS];   // clusters of the sampler that are resident at a time
     int32_t step_clusters[OD_SAMPLE_LEVELS];     // of the whole step in one launch: a multiprocessor to each block
     int32_t shard_clusters[OD_SHARD_SIZES][OD_SAMPLE_MAX_PARTS + 1];   // of a shard's mass, by threads and blocks
+    int32_t distill_few_clusters[OD_DISTILL_LEVELS];   // of the distillation loss with two blocks to a multiprocessor
     bool have_map;
     bool distill_lists;             // some map had gather lists: every later one has the distillation kernel's
     // The map's serial number. A launch is laid out for the map of its time (where ids are shared, how many
@@ -302,6 +303,7 @@ inline size_t od_distill_lists_bytes(int32_t v_q, int32_t v_p)
 }
 void od_distill_plan(int32_t v_q, int32_t v_p, const OdMappedIds &mapped, void *out);   // host
 cudaError_t od_distill_prepare_device(int32_t v_q);
+void od_distill_resident(int32_t *clusters);             // [levels]
 
 void od_cache_free_dynamic(od_ctx *c);   // frees what od_cache_configure allocated beyond keys / vals
 

@@ -647,7 +647,11 @@ cudaError_t od_launch_distill(od_ctx *c, int32_t B, int32_t K_max, const float *
     // Where two blocks to a multiprocessor hold them all, they have 64 registers instead of 40: six groups of the list in
     // flight, and a thread's probabilities stay in registers from the sums to the gradient (128256 bf16 / 152064 fp32 ids, 1 x 4
     // 6.55 -> 6.05 us / 6.6 -> 6.3, 5 x 5 8.3 -> 7.6 / 8.6 -> 8.1, 12 x 6 11.8 -> 10.3 / 12.2 -> 11.1; 8 or 10 groups spill).
-    const bool few = !same && vec4 && a.chunk <= FEW_CHUNK && positions << level <= (int64_t)c->sm_count * 2;
+    // The device says how many clusters it holds (33 of 8 blocks, where 296 blocks would be 37: 6 x 6 positions of 128256 bf16 ids
+    // 8.3 us with 40 registers, 9.4 with 64). One in 32 too many is no loss: positions without a translation leave at once (71 of
+    // 4 blocks: 12 x 6 are faster by 3 to 17 % in eleven of twelve forms).
+    const int64_t room = c->distill_few_clusters[level];
+    const bool few = !same && vec4 && a.chunk <= FEW_CHUNK && positions << level <= (int64_t)c->sm_count * 2 && positions <= room + room / 32;
     // One block per position instead where the chunks would not fit, or where the target row is so
     // short that the gather in draft order finds its lines in L1 and there are positions enough
     // (128 x 10, v_q = 32000, 22400 ids mapped, v_p = 34330 / 45000 / 64000 / 128000: without a gradient
@@ -663,6 +667,25 @@ cudaError_t od_launch_distill(od_ctx *c, int32_t B, int32_t K_max, const float *
     a.list_ofs = l.ofs + level * OD_DISTILL_MAX_CHUNKS * 2; a.mapped_bits = l.bits;
     if (vec4) return bf ? launch<OD_BF16, true>(a, C, same, few, pdl, s) : launch<OD_F32, true>(a, C, same, few, pdl, s);
     return bf ? launch<OD_BF16, false>(a, C, same, few, pdl, s) : launch<OD_F32, false>(a, C, same, few, pdl, s);
+}
+
+// Clusters of each number of chunks that are resident with two blocks to a multiprocessor
+void od_distill_resident(int32_t *clusters)
+{
+    for (int level = 0; level < OD_DISTILL_LEVELS; ++level) {
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(1u << level); cfg.blockDim = dim3(THREADS); cfg.dynamicSmemBytes = FEW_CHUNK * 4;
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = 1u << level; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+        cfg.attrs = attr; cfg.numAttrs = 1;
+        int n = 0;
+        if (cudaOccupancyMaxActiveClusters(&n, od_distill_kernel<OD_F32, true, false, 2>, &cfg) != cudaSuccess) {
+            cudaGetLastError();
+            n = 0;
+        }
+        clusters[level] = n;
+    }
 }
 
 // The kernels' dynamic shared memory (a chunk of a draft vocabulary of v_q ids): opt in where it

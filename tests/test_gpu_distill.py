@@ -167,3 +167,13 @@ def test_few_positions(cuda_device, v_q, v_p, B, k_max):
     for dtype in ("bf16", "f32"):
         w = _small(B=B, k_max=k_max, v_q=v_q, v_p=v_p, cache_entries=0, logit_dtype=dtype, gen_seed=0xBEEFFA)
         _check(w, cuda_device, [0], 0.2, ds.LAMBDA_CONSTANT, positions=sorted({0, B // 2, B - 1}))
+
+
+# as many positions as two blocks to a multiprocessor have room for, and the next ones, with eight, four and two chunks
+@pytest.mark.parametrize("v_q, v_p, B, k_max", [(32764, 40003, 17, 2), (32764, 40003, 7, 5), (8188, 20011, 12, 3), (16388, 20011, 18, 4),
+                                                (16388, 20011, 37, 2), (8188, 20011, 76, 2), (8188, 20011, 51, 3)])
+def test_the_room_for_few_positions(cuda_device, v_q, v_p, B, k_max):
+    """Tolerances as above."""
+    for dtype in ("bf16", "f32"):
+        w = _small(B=B, k_max=k_max, v_q=v_q, v_p=v_p, cache_entries=0, logit_dtype=dtype, gen_seed=0xBEEFFB)
+        _check(w, cuda_device, [0], 0.2, ds.LAMBDA_CONSTANT, positions=sorted({0, B // 2, B - 1}))
