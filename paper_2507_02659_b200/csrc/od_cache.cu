@@ -61,10 +61,10 @@ struct TrimState {
     unsigned long long hi_and, hi_or;       // AND / OR of (new?, score) over the listed entries: bits that never vary
     unsigned long long thr_hi, thr_lo;      // trim_select_kernel: the k-th order key
     unsigned int bins[256];     // live entries by score (score_bin)
-    // LRU: hardly an entry was accessed before this clock (what the last trim dropped was, if none has been set back since), and what
-    // it is behind a trim without a list. Where the bins begin: what stays and what goes does not depend on it.
+    // LRU: where the bins begin, a clock before which hardly an entry was accessed (that of the last entry which the trim before
+    // dropped), and what becomes of it behind a trim without a list. What stays and what goes does not depend on it.
     unsigned int oldest, next_oldest;
-    SelState sel[PASSES + 1];   // sel[p]: written by block 0 of pass p (sel[PASSES]: by the rebuild)
+    SelState sel[PASSES];       // sel[p]: written by block 0 of pass p
     unsigned int n_out[PASSES]; // entries pass p copied into its output list
     unsigned int hist[PASSES][256];
 };
@@ -211,10 +211,9 @@ __global__ void insert_commit_kernel(int32_t N, const int32_t *__restrict__ targ
     atomicAdd(&st->size, 1u);
 }
 
-__global__ void trim_begin_kernel(TrimState *st, unsigned int max_entries)
+__global__ void trim_begin_kernel(TrimState *st)
 {
     chain_wait(true);
-    if (threadIdx.x == 0) st->k = st->size > max_entries ? st->size - max_entries : 0u;
     for (int p = 0; p < PASSES; ++p) st->hist[p][threadIdx.x] = 0u;
     if (threadIdx.x < PASSES) st->n_out[threadIdx.x] = 0u;
 }
@@ -1109,7 +1108,7 @@ int32_t od_cache_trim(od_ctx *c, void *stream)
     const unsigned place = (unsigned)std::min<int64_t>(blocks ? c->sm_count * 2 : most, (entries + TRIM_THREADS - 1) / TRIM_THREADS);
     const Table from = {(unsigned long long *)c->d_keys, c->d_vals, c->d_stamp, c->d_freq, c->d_born, c->d_fill};
     const Table to = {(unsigned long long *)c->d_keys2, c->d_vals2, c->d_stamp2, c->d_freq2, c->d_born2, c->d_fill2};
-    if (!blocks) OD_CUDA(chain_launch(trim_begin_kernel, 1u, 256u, s, pdl, st, (unsigned int)c->dyn_max));
+    if (!blocks) OD_CUDA(chain_launch(trim_begin_kernel, 1u, 256u, s, pdl, st));
     OD_CUDA(chain_launch(trim_count_kernel, passes, (unsigned)TRIM_THREADS, s, pdl, c->dyn_policy, c->clock, from.vals,
                          c->dyn_policy == 0 ? from.stamp : from.freq, from.born, c->cap, st));
     OD_CUDA(chain_launch(trim_split_kernel, passes, (unsigned)TRIM_THREADS, s, pdl, c->dyn_policy, c->clock,

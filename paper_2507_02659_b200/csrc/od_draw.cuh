@@ -367,8 +367,9 @@ template <int DTYPE>
 __device__ __forceinline__ void load_tile(const SeqState &q, int tile, int lane, uint4 *raw)
 {
     const uint4 *src = (const uint4 *)(q.row + (size_t)(tile * OD_SAMPLE_TILE + lane * EPT) * (DTYPE == OD_BF16 ? 2 : 4));
-    // (fp32 rows through L1, where the draw finds its tile again: three calls of 19 sequences of 100277 ids 20.9 -> 20.3 us;
-    // bf16 rows gain nothing by it, a batch of 296 loses 2.5 %)
+    // (fp32 rows through L1, where the draw finds its tile again: the step of 19 sequences of 100277 ids 14.8 -> 14.3 us, 148
+    // 46.3 -> 43.9, 296 86.0 -> 79.1, 512 162 -> 148; of 32000 shared ids 100 19.6 -> 19.0, 512 64.1 -> 63.8. Only 296 of 65000 shared ids,
+    // one block to each and a whole chip of them, lose: 59.1 -> 60.5. bf16 rows gain nothing by it, a batch of 296 loses 2.5 %)
     if (DTYPE == OD_BF16) {
         raw[0] = ld_once(src);
     } else {
@@ -430,8 +431,7 @@ __device__ __forceinline__ float tile_lane_sum(const SeqState &q, const SampleAr
 // the same with the probabilities in shared memory at `rank_at` (the address of the lane's first
 // mapped id's; `oct` says which of the eight are mapped)
 template <int DTYPE>
-__device__ __forceinline__ float tile_lane_sum_staged(const SeqState &q, const SampleArgs &a, int tile, int lane, const uint4 *raw,
-                                                      uint32_t oct, uint32_t rank_at)
+__device__ __forceinline__ float tile_lane_sum_staged(const SeqState &q, const uint4 *raw, uint32_t oct, uint32_t rank_at)
 {
     float r[EPT];
     tile_e<DTYPE>(q, raw, r);
@@ -527,8 +527,7 @@ struct TileLoads {
     __device__ __forceinline__ float sum(const SeqState &q, const SampleArgs &a, const StagedRow &sr, int tile, int lane) const
     {
         if (SOURCE == STAGED)
-            return tile_lane_sum_staged<DTYPE>(q, a, tile, lane, raw, oct,
-                                               (uint32_t)__cvta_generic_to_shared(sr.q) + ((oct >> 8) - sr.rank0) * 4u);
+            return tile_lane_sum_staged<DTYPE>(q, raw, oct, (uint32_t)__cvta_generic_to_shared(sr.q) + ((oct >> 8) - sr.rank0) * 4u);
         if (SOURCE == FREE) {
             float e[EPT];
             tile_e<DTYPE>(q, raw, e);

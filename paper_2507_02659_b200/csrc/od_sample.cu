@@ -195,7 +195,7 @@ od_sample_shard_kernel(const SampleArgs a)
     if (p_hi > tile_hi) p_hi = tile_hi;
     const int p_hi_w = p_hi < a.v_p / OD_SAMPLE_TILE ? p_hi : a.v_p / OD_SAMPLE_TILE;
     int4 ni[2][2] = {};
-    if (MODE != 2 && !a.same_ids && p_lo < p_hi_w) first_pair_entries(a, p_lo, p_hi_w, lane, ni);
+    if (MODE == 1 && !a.same_ids && p_lo < p_hi_w) first_pair_entries(a, p_lo, p_hi_w, lane, ni);
 
     // n_accepted and the row statistics come from the verification kernels
     if (a.early) asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -239,9 +239,9 @@ od_sample_shard_kernel(const SampleArgs a)
     int j = a.n_accepted[b];
     j = j < 0 ? 0 : (j > mb ? mb : j);
     const SeqState q = seq_state<DTYPE>(a, h, b, j, rm, rs, a.col0, planned);
-    if (MODE != 2 && q.residual && threadIdx.x == 0) prefetch_q_row(a, q, part, nparts);
+    if (MODE == 1 && q.residual && threadIdx.x == 0) prefetch_q_row(a, q, part, nparts);
 
-    if (MODE != 2) {
+    if (MODE == 1) {
         SummedTiles<DTYPE> out = {tile_val, s_sums + (DTYPE == OD_BF16 ? 0 : 2 * warp), lane, 0.0};
         out.clear();
         // ---- pass 1: the value of every tile ----
@@ -293,41 +293,39 @@ od_sample_shard_kernel(const SampleArgs a)
     for (int t = tile_lo + (int)threadIdx.x + 4 * OD_SAMPLE_THREADS; t < tile_hi; t += OD_SAMPLE_THREADS) s_val[t] = fmax(0.0, __ldcg(tile_val + t));
     __syncthreads();
 
-    double shard_before = 0.0, shard_total = 0.0;      // MODE 2: sums over the shards before this one / all
-    if (MODE == 2) {
-        const auto share = [&](int s, bool e) -> double {
-            if (s < 32) return __shfl_sync(0xFFFFFFFFu, e ? share_e : share_r, s);
-            return a.mass_all[((size_t)s * a.B + b) * 2 + (e ? 1 : 0)];
-        };
-        double tot_r = 0.0, tot_e = 0.0;
-        for (int s = 0; s < a.n_shards; ++s) { tot_r += share(s, false); tot_e += share(s, true); }
-        const bool use_e = residual && !(tot_r > 0.0);
-        if (use_e) { residual = false; flags |= OD_SF_ZERO_MASS; }   // the tile values then hold p_j's
-        shard_total = use_e ? tot_e : tot_r;
-        // the shard in which the running sum crosses the target (else the last one with mass)
-        int owner = -1;
-        if (shard_total > 0.0) {
-            const double target = (double)u * shard_total;
-            double c = 0.0;
-            int last = -1;
-            for (int s = 0; s < a.n_shards; ++s) {
-                const double v = share(s, use_e);
-                if (s == a.shard_index) shard_before = c;
-                if (v > 0.0) last = s;
-                if (c + v > target) { owner = s; break; }
-                c += v;
-            }
-            if (owner < 0) owner = last;
+    double shard_before = 0.0, shard_total = 0.0;      // sums over the shards before this one / all
+    const auto share = [&](int s, bool e) -> double {
+        if (s < 32) return __shfl_sync(0xFFFFFFFFu, e ? share_e : share_r, s);
+        return a.mass_all[((size_t)s * a.B + b) * 2 + (e ? 1 : 0)];
+    };
+    double tot_r = 0.0, tot_e = 0.0;
+    for (int s = 0; s < a.n_shards; ++s) { tot_r += share(s, false); tot_e += share(s, true); }
+    const bool use_e = residual && !(tot_r > 0.0);
+    if (use_e) { residual = false; flags |= OD_SF_ZERO_MASS; }   // the tile values then hold p_j's
+    shard_total = use_e ? tot_e : tot_r;
+    // the shard in which the running sum crosses the target (else the last one with mass)
+    int owner = -1;
+    if (shard_total > 0.0) {
+        const double target = (double)u * shard_total;
+        double c = 0.0;
+        int last = -1;
+        for (int s = 0; s < a.n_shards; ++s) {
+            const double v = share(s, use_e);
+            if (s == a.shard_index) shard_before = c;
+            if (v > 0.0) last = s;
+            if (c + v > target) { owner = s; break; }
+            c += v;
         }
-        if (owner != a.shard_index) {
-            if (threadIdx.x == 0) {
-                const bool report = owner < 0 && a.shard_index == 0;   // no mass anywhere: shard 0 says so
-                a.out_token[b] = -1;
-                a.resid_mass[b] = report ? (float)(shard_total / (double)q.S) : 0.f;
-                a.flags[b] = report ? (flags | OD_SF_ZERO_MASS) : 0u;
-            }
-            return;
+        if (owner < 0) owner = last;
+    }
+    if (owner != a.shard_index) {
+        if (threadIdx.x == 0) {
+            const bool report = owner < 0 && a.shard_index == 0;   // no mass anywhere: shard 0 says so
+            a.out_token[b] = -1;
+            a.resid_mass[b] = report ? (float)(shard_total / (double)q.S) : 0.f;
+            a.flags[b] = report ? (flags | OD_SF_ZERO_MASS) : 0u;
         }
+        return;
     }
 
     // exclusive scan of the tile values: thread i owns `per` consecutive tiles
@@ -425,7 +423,6 @@ static cudaError_t prepare_kernels()
     if (e == cudaSuccess) e = allow_cluster16<DTYPE, true, FROM_ROW>(bytes);
     if (e == cudaSuccess) e = allow_cluster16<DTYPE, false, STAGED>(staged);
     if (e == cudaSuccess) e = allow_cluster16<DTYPE, true, STAGED>(staged);
-    if (e == cudaSuccess) e = allow_smem(od_sample_shard_kernel<DTYPE, 1>, bytes);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(od_sample_shard_kernel<DTYPE, 1>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     if (e == cudaSuccess) e = allow_smem(od_sample_shard_kernel<DTYPE, 2>, bytes);
     return e;
