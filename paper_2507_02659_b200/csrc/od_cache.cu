@@ -248,7 +248,7 @@ __device__ __forceinline__ unsigned int block_offsets(unsigned int n, unsigned i
 // group it is in. Bound by the chain of round trips and by L2 (262144 entries: 13 MB read, 12 MB written). Before,
 // one pass packed all live entries into a list, the select walked through it, and a rebuild put every survivor into the slot that
 // its group's counter gave. Device time of an insertion, a trim and a translation, before -> now: 262144 entries and 16384 new
-// ones 53.7 -> 36.1 us, by frequency 70.1 -> 64.0; 4096 and 512 24.4 -> 22.9; 32768 and 4096 by frequency 35.2 -> 34.3. (The
+// ones 53.6 -> 36.8 us, by frequency 69.9 -> 64.8; 4096 and 512 24.4 -> 22.8; 32768 and 4096 by frequency 35.1 -> 34.2. (The
 // whole trim in one cluster of 1 to 16 blocks, for tables of up to 131072 slots: 26.5 and 37.7 us on the last two; a step
 // of it is a chain of trips as long as a launch's.)
 constexpr int TRIM_THREADS = 256, TRIM_HALVES = TRIM_THREADS / 16, QUAD = 4;   // groups of a half-warp at a time

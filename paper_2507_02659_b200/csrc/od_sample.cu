@@ -458,7 +458,7 @@ struct ShardCut {
 // rank's five calls: 28.0 us with 13 blocks of 256 threads, of which 38 clusters are resident, 24.7 with 10 and 56). A sixteenth of
 // the room is left free, or the last ones are placed late (70 sequences, a quarter of 128256 ids: 8 blocks with 71 places
 // 23.8, 2 of 1024 threads 22.6). An even number of tiles, since warps work on pairs. Larger blocks where they give each warp
-// fewer tiles: in windows that 16 blocks of 256 threads cannot share so finely (one sequence, half of a million ids: 23.2
+// fewer tiles: in windows that 16 blocks of 256 threads cannot share so finely (one sequence, half of a million ids: 24.1
 // and 20.8 with 1024) and for numbers of sequences between theirs (145, half of 152064: 43.5 with 3 of 256, 40.4 with 2 of 512).
 static ShardCut shard_cut(const od_ctx *c, int32_t B, int64_t tiles)
 {
