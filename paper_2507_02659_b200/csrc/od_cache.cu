@@ -961,8 +961,8 @@ void select_config(cudaLaunchConfig_t &cfg, cudaLaunchAttribute *attr, const od_
 
 // Blocks of the one-launch select, 0 = the table is too large for it: the keys of a list of all its entries have to fit in
 // the blocks' shared memory (16 blocks: 393216 entries; 196608 where clusters of 16 are not to be had). As few as give every
-// entry of the table a thread of its own, and two to a thread by LFU, where the list is most of the table as a rule (32768
-// entries: 35.6 us with 8 blocks, 34.5 with 16).
+// entry of the table a thread of its own: by LFU the list is most of the table as a rule (16000 entries, 256 new ones, an
+// insertion and a trim: 35.4 us with two entries a thread, 32.4 so).
 int select_blocks(const od_ctx *c)
 {
     if (cudaFuncSetAttribute(trim_select_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||
@@ -971,8 +971,7 @@ int select_blocks(const od_ctx *c)
         return 0;
     }
     const int64_t entries = c->dyn_max + c->dyn_max_insert;
-    const int64_t per_thread = c->dyn_policy == 0 ? 1 : 2;
-    const int64_t want = (entries + per_thread * SELECT_THREADS - 1) / (per_thread * SELECT_THREADS);
+    const int64_t want = (entries + SELECT_THREADS - 1) / SELECT_THREADS;
     int blocks = 1, best = 0;
     for (; blocks <= SELECT_MAX_BLOCKS; blocks *= 2) {
         if (select_room(c, blocks) > SELECT_ROOM_MAX) continue;
