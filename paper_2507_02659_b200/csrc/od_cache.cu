@@ -243,15 +243,16 @@ __device__ __forceinline__ unsigned int block_offsets(unsigned int n, unsigned i
 // ---- the two passes over the table ---------------------------------------------------------
 //
 // Sixteen lanes take a group's first sixteen slots (a table at most half full often has no more: a group is filled from
-// slot 0), then the rest where the sixteenth is taken, four groups at a time. How far a group is filled is kept for
+// slot 0), then the rest where the sixteenth is taken, up to four groups at a time. How far a group is filled is kept for
 // each, so that no slot is cleared that was not taken. Neither pass has an atomic per entry: a survivor stays in the
 // group it is in. Bound by the chain of round trips and by L2 (262144 entries: 13 MB read, 12 MB written). Before,
 // one pass packed all live entries into a list, the select walked through it, and a rebuild put every survivor into the slot that
 // its group's counter gave. Device time of an insertion, a trim and a translation, before -> now: 262144 entries and 16384 new
-// ones 53.6 -> 36.8 us, by frequency 69.9 -> 64.8; 4096 and 512 24.4 -> 22.8; 32768 and 4096 by frequency 35.1 -> 34.2. (The
+// ones 53.6 -> 36.7 us, by frequency 70.0 -> 64.7; 4096 and 512 24.5 -> 20.4; 32768 and 4096 by frequency 35.0 -> 31.9. (The
 // whole trim in one cluster of 1 to 16 blocks, for tables of up to 131072 slots: 26.5 and 37.7 us on the last two; a step
 // of it is a chain of trips as long as a launch's.)
-constexpr int TRIM_THREADS = 256, TRIM_HALVES = TRIM_THREADS / 16, QUAD = 4;   // groups of a half-warp at a time
+// QUAD: groups of a half-warp at a time, 1, 2 or 4: see trim_quad.
+constexpr int TRIM_THREADS = 256, TRIM_HALVES = TRIM_THREADS / 16;
 
 // (new?, score) to one of 256 bins, in the order of trims: 255 new; else by frequency (LFU), or by the clock from the oldest
 // on (LRU), exact for 128 of them, four bins to an octave beyond. LRU drops the oldest, so their clocks have bins of their own
@@ -289,6 +290,7 @@ __device__ __forceinline__ void count_digit(unsigned int *hist, unsigned int d, 
 }
 
 // The live entries by score.
+template <int QUAD>
 __global__ void __launch_bounds__(TRIM_THREADS)
 trim_count_kernel(int policy, unsigned int clock, const int32_t *vals, const unsigned int *score, const unsigned int *born,
                   int64_t cap, TrimState *st)
@@ -359,9 +361,30 @@ __device__ __forceinline__ void place_entry(const Table &to, int64_t cap, const 
     }
 }
 
+// How far QUAD neighbouring groups are filled
+template <int QUAD> struct FillWord;
+template <> struct FillWord<1> { typedef unsigned int type; };
+template <> struct FillWord<2> { typedef uint2 type; };
+template <> struct FillWord<4> { typedef uint4 type; };
+template <int QUAD>
+__device__ __forceinline__ void load_fill(const unsigned int *fill, int64_t quad, unsigned int (&n)[QUAD])
+{
+    typedef typename FillWord<QUAD>::type Word;
+    const Word v = __ldcg((const Word *)fill + quad);
+    memcpy(n, &v, sizeof(v));
+}
+template <int QUAD>
+__device__ __forceinline__ void store_fill(unsigned int *fill, int64_t quad, const unsigned int (&n)[QUAD])
+{
+    typename FillWord<QUAD>::type v;
+    memcpy(&v, n, sizeof(v));
+    ((typename FillWord<QUAD>::type *)fill)[quad] = v;
+}
+
 // Which bin the k-th entry is in; then every group's survivors into the same group of the new table, and into the list what
 // cannot be said yet. The table has not been written since before the pass that counts waited, so the first
 // groups are loaded in front of this kernel's own wait.
+template <int QUAD>
 __global__ void __launch_bounds__(TRIM_THREADS, 4)
 trim_split_kernel(int policy, unsigned int clock, unsigned int max_entries, const Table from, const Table to, int64_t cap,
                   void *lists, TrimState *st)
@@ -385,12 +408,14 @@ trim_split_kernel(int policy, unsigned int clock, unsigned int max_entries, cons
     };
     load(at, 0xFu);
     // An entry is in another group than its run hashes to only if all groups from there on were full: where none of the
-    // four groups in front of the half-warp's is, nobody asks (the hash is a third of the pass's instructions).
+    // groups in front of the half-warp's is, nobody asks (the hash is a third of the pass's instructions).
     const auto behind_a_full_group = [&]() {
         if (quad >= quads) return false;
-        const uint4 f = __ldcg((const uint4 *)from.fill + quad);
-        const unsigned int before = __ldcg(from.fill + ((quad * QUAD - 1) & (groups - 1)));
-        return max(max(before, f.x), max(f.y, f.z)) >= (unsigned int)OD_GROUP;
+        unsigned int f[QUAD], most = __ldcg(from.fill + ((quad * QUAD - 1) & (groups - 1)));
+        load_fill<QUAD>(from.fill, quad, f);
+#pragma unroll
+        for (int e = 0; e + 1 < QUAD; ++e) most = max(most, f[e]);
+        return most >= (unsigned int)OD_GROUP;
     };
     bool ask = behind_a_full_group();
     if (threadIdx.x == 0) { s_and = ~0ull; s_or = 0ull; s_bin = 256u; s_rem = 0u; s_in = 0u; }
@@ -418,7 +443,7 @@ trim_split_kernel(int policy, unsigned int clock, unsigned int max_entries, cons
         const bool in = quad < quads, ask_here = __any_sync(0xFFFFFFFFu, ask);
         unsigned int had[QUAD];
 #pragma unroll
-        for (int e = 0; e < QUAD; ++e) run[e] = 0u;
+        for (int e = 0; e < QUAD; ++e) { run[e] = 0u; had[e] = 0u; }
         // the groups whose sixteenth slot is taken: their other slots too
         unsigned int more = 0u;
         if (at == 15) {
@@ -429,8 +454,7 @@ trim_split_kernel(int policy, unsigned int clock, unsigned int max_entries, cons
         for (int round = 0; round < rounds; ++round) {
             const int s = at + 16 * round;
             if (round) { more = __shfl_sync(0xFFFFFFFFu, more, 16 * half + 15); load(s, more); }
-            const uint4 taken = round + 1 == rounds && in ? __ldcg((const uint4 *)to.fill + quad) : make_uint4(0u, 0u, 0u, 0u);
-            had[0] = taken.x; had[1] = taken.y; had[2] = taken.z; had[3] = taken.w;
+            if (round + 1 == rounds && in) load_fill<QUAD>(to.fill, quad, had);
             unsigned int listed = 0u, late = 0u;            // of this thread's four: bit e
             unsigned long long t_and = ~0ull, t_or = 0ull;
             if (round == 0 || __any_sync(0xFFFFFFFFu, more != 0u))
@@ -494,7 +518,7 @@ trim_split_kernel(int policy, unsigned int clock, unsigned int max_entries, cons
                 const int64_t slot = (quad * QUAD + e) * OD_GROUP + s;
                 to.keys[slot] = 0ull; to.vals[slot] = -1;
             }
-        if (in && at == 0) ((uint4 *)to.fill)[quad] = make_uint4(run[0], run[1], run[2], run[3]);
+        if (in && at == 0) store_fill<QUAD>(to.fill, quad, run);
         q0 += (int64_t)gridDim.x * TRIM_HALVES;
         if (q0 >= quads) break;
         quad = q0 + (threadIdx.x >> 4);
@@ -959,6 +983,15 @@ void select_config(cudaLaunchConfig_t &cfg, cudaLaunchAttribute *attr, const od_
     cfg.attrs = attr; cfg.numAttrs = 1;
 }
 
+// Groups of a half-warp at a time in the two passes over the table: as few as leave two blocks to a multiprocessor at one,
+// four at two (an insertion and a trim with 1, 2 and 4: 4096 entries and 512 new ones 16.0, 16.6 and 18.4 us, 16000 and 256 by LFU
+// 28.8, 29.6 and 32.4, 32768 and 4096 19.7, 20.2 and 22.0, 65536 and 2048 19.9, 18.7 and 20.3, 262144 and 16384 41.6, 38.8 and 37.4).
+int trim_quad(const od_ctx *c)
+{
+    const int64_t blocks = (c->cap / OD_GROUP + TRIM_HALVES - 1) / TRIM_HALVES;   // with one
+    return blocks <= c->sm_count * 2 ? 1 : blocks <= c->sm_count * 8 ? 2 : 4;
+}
+
 // Blocks of the one-launch select, 0 = the table is too large for it: the keys of a list of all its entries have to fit in
 // the blocks' shared memory (16 blocks: 393216 entries; 196608 where clusters of 16 are not to be had). As few as give every
 // entry of the table a thread of its own: by LFU the list is most of the table as a rule (16000 entries, 256 new ones, an
@@ -1096,7 +1129,8 @@ int32_t od_cache_trim(od_ctx *c, void *stream)
     TrimState *st = (TrimState *)c->d_trim;
     // one resident wave at most, and no more blocks than have anything to do
     const int64_t most = c->sm_count * 4;
-    const unsigned passes = (unsigned)std::min<int64_t>(most, (c->cap / OD_GROUP + QUAD * TRIM_HALVES - 1) / (QUAD * TRIM_HALVES));
+    const int quad = trim_quad(c);
+    const unsigned passes = (unsigned)std::min<int64_t>(most, (c->cap / OD_GROUP + quad * TRIM_HALVES - 1) / (quad * TRIM_HALVES));
     const bool pdl = c->opt_pdl != 0;
     const int blocks = c->trim_blocks;                      // 0: the select is a chain of launches
     // whether the list may be longer than what the select's cluster places by itself
@@ -1108,9 +1142,11 @@ int32_t od_cache_trim(od_ctx *c, void *stream)
     const Table from = {(unsigned long long *)c->d_keys, c->d_vals, c->d_stamp, c->d_freq, c->d_born, c->d_fill};
     const Table to = {(unsigned long long *)c->d_keys2, c->d_vals2, c->d_stamp2, c->d_freq2, c->d_born2, c->d_fill2};
     if (!blocks) OD_CUDA(chain_launch(trim_begin_kernel, 1u, 256u, s, pdl, st));
-    OD_CUDA(chain_launch(trim_count_kernel, passes, (unsigned)TRIM_THREADS, s, pdl, c->dyn_policy, c->clock, from.vals,
+    const auto count = quad == 4 ? trim_count_kernel<4> : quad == 2 ? trim_count_kernel<2> : trim_count_kernel<1>;
+    const auto split = quad == 4 ? trim_split_kernel<4> : quad == 2 ? trim_split_kernel<2> : trim_split_kernel<1>;
+    OD_CUDA(chain_launch(count, passes, (unsigned)TRIM_THREADS, s, pdl, c->dyn_policy, c->clock, from.vals,
                          c->dyn_policy == 0 ? from.stamp : from.freq, from.born, c->cap, st));
-    OD_CUDA(chain_launch(trim_split_kernel, passes, (unsigned)TRIM_THREADS, s, pdl, c->dyn_policy, c->clock,
+    OD_CUDA(chain_launch(split, passes, (unsigned)TRIM_THREADS, s, pdl, c->dyn_policy, c->clock,
                          (unsigned int)c->dyn_max, from, to, c->cap, c->d_trim_lists, st));
     if (blocks) {
         cudaLaunchConfig_t cfg = {};
