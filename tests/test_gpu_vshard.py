@@ -236,3 +236,18 @@ def test_every_size_of_cluster_that_sums_a_shards_mass(cuda_device, dtype, v_p, 
     assert stats.sample_compared > 0
     assert ctx.last_launch_info(2) == blocks * B
     ctx.close()
+
+
+# more shards than a warp has lanes to hold their shares
+@pytest.mark.parametrize("n_shards", [32, 33, 70])
+def test_more_shards_than_lanes(cuda_device, n_shards):
+    w = _workload(f"many{n_shards}", v_p=n_shards * 256 + 77, v_q=900, cache_entries=100, gen_seed=0xBEEF70 + n_shards)
+    st = synth.make_static(w)
+    ctx = parity.make_context(w, st, cuda_device)
+    cache = oracle.Cache(st.runs, st.run_len, st.run_target)
+    total = parity.Stats()
+    for step in range(3):
+        s = synth.make_step(w, st, step, device=cuda_device)
+        total.merge(_sharded_check(ctx, cache, st, w, s, n_shards, logits=parity.pad_rows(s.logits))[0])
+    assert total.sample_compared > 30
+    ctx.close()
